@@ -95,8 +95,12 @@ typedef struct aap_params {
                             256 or 512 (whole-block tile kernel), 1024 (the
                             pipelined kernel: one block per SM with copy, sort
                             and update warps; one species per system).
-                            Automatic picks 1024 where it applies, else 512;
-                            an ensemble follows its first replica's value   */
+                            Automatic picks 1024 where it applies, else 512,
+                            and runs a system of at most one tile per SM
+                            many steps per launch (the same trajectory bit
+                            for bit; aap_get_layout reports the kernel of
+                            the single steps); an ensemble follows its
+                            first replica's value                           */
     double   capacity;   /* tile-region capacity over the mean occupancy;
                             0 = automatic (4)                                   */
     int32_t  binnum_theta;      /* bins of the orientation histogram over
@@ -256,14 +260,16 @@ int aap_get_results(aap_handle *h, aap_results *out);
 int aap_test_fail_alloc_after(int32_t n);
 
 /* Fault injection for tests of the pipelined step kernel's bounded waits
- * (its hand-offs between the copy, sort and update warps are mbarrier waits
- * that give up after a bound; the kernel then sets AAP_ETIMEOUT in the
+ * and of the many-steps kernel (the hand-offs between the copy, sort and update
+ * warps are mbarrier waits, the steps of a launch end at a grid barrier; both
+ * give up after a bound; the kernel then sets AAP_ETIMEOUT in the
  * handle's error word, every later step of that handle returns at once, and
  * the handle reports AAP_ETIMEOUT at its next synchronising call).
  * wait_cycles: the bound in SM clock cycles for kernels launched from now on
  * (<= 0: the default, about 2 s).  stall: 1 makes the copy warp of every
- * block withhold the first tile it claims (no copies, no arrival), so that
- * the waits behind it run out; 0 switches it off.  Process-wide; call only
+ * block withhold the first tile it claims (no copies, no arrival), or one
+ * block its first arrival at the barrier, so that the waits behind it run
+ * out; 0 switches it off.  Process-wide; call only
  * while no step kernel is running.  The GPU context stays usable. */
 int aap_test_pipe_wait(int64_t wait_cycles, int32_t stall);
 

@@ -69,6 +69,7 @@ struct aap_handle {
     int *d_x0tab = nullptr, *d_y0tab = nullptr;
     unsigned char *d_scratch = nullptr;
     int *d_dense = nullptr;             // pipelined step: tiles left to the whole-block routine
+    int *d_multi = nullptr;             // many steps per launch: private counters and barrier
     unsigned long long *d_obs = nullptr;
     int *d_seen = nullptr;
     unsigned long long *d_bad = nullptr;     // [2] first invalid position / orientation of aap_set_state
@@ -384,6 +385,18 @@ int set_capacity(aap_handle *h, double factor)
         if (rc) return rc;
         if (!L.pipe && p.threads == 1024) return fail(AAP_EINVAL, "the pipelined step kernel does not fit this tiling");
     }
+    // many steps per launch: a small system with the automatic choice of kernel
+    L.multi = 0;
+    if (!h->member && p.threads == 0) {
+        L.pipe_nceh = (2 * S.twmax + 4) * (S.thmax + 2);
+        AAP_CK(aapk::configure_multi(L, p.nspecies, S.ntiles, nsm, scap));
+        if (L.multi) {
+            // a scratch slice for every block, with room for the weighted records
+            L.grid_step = std::max(L.grid_step, S.ntiles);
+            L.scratch_per_block += (size_t)L.multi_wsp * 8 * L.scratch_cap;
+            L.scratch_per_block = (L.scratch_per_block + 255) / 256 * 256;
+        }
+    }
     return AAP_OK;
 }
 
@@ -610,6 +623,7 @@ int clear_buffers(aap_handle *h)
         AAP_CK(cudaMemsetAsync(S.spill_bits[b], 0, spill_bits_bytes(S), h->stream));
     AAP_CK(cudaMemsetAsync(S.acc, 0, 2 * aapk::kAccSlots * aapk::kAccWords * sizeof(unsigned long long), h->stream));
     AAP_CK(cudaMemsetAsync(S.err, 0, sizeof(int), h->stream));
+    if (h->d_multi) AAP_CK(cudaMemsetAsync(h->d_multi, 0, aapk::multi_bytes(S.ntiles), h->stream));
     return AAP_OK;
 }
 
@@ -650,6 +664,7 @@ int alloc_all(aap_handle *h)
         if ((rc = dev_alloc(h, &h->d_ctl, sizeof(Ctl)))) return rc;
         if ((rc = dev_alloc(h, &h->d_dense, (size_t)std::max(S.ntiles, 1) * sizeof(int)))) return rc;
         AAP_CK(cudaMemsetAsync(h->d_dense, 0, (size_t)std::max(S.ntiles, 1) * sizeof(int), h->stream));
+        if (h->L.multi && (rc = dev_alloc(h, &h->d_multi, aapk::multi_bytes(S.ntiles)))) return rc;
     }
     if ((rc = dev_alloc(h, &h->d_x0tab, (size_t)(S.ntx + 1) * sizeof(int)))) return rc;
     if ((rc = dev_alloc(h, &h->d_y0tab, (size_t)(S.nty + 1) * sizeof(int)))) return rc;
@@ -683,6 +698,7 @@ int alloc_all(aap_handle *h)
     L.tile_base = h->d_tile_base;
     L.ctl = h->d_ctl;
     L.dense_list = h->d_dense;
+    L.multi_cnt = h->d_multi;
     return push_sys(h);
 }
 
@@ -785,7 +801,9 @@ int run_steps_adaptive(aap_handle *h, long long nsteps)
     int rc;
     long long left = nsteps;
     while (left > 0) {
-        const long long k = std::min(left, kAdaptSteps - h->since_copy);
+        long long k = std::min(left, kAdaptSteps - h->since_copy);
+        // many steps per launch: no launch of fewer than four steps unless the call itself is that short
+        if (h->L.multi && (k < 4 || left - k < 4)) k = std::min(left, kAdaptSteps + 3);
         if ((rc = run_steps(h, k))) return rc;
         left -= k;
         h->since_copy += k;
@@ -808,6 +826,11 @@ int run_steps_adaptive(aap_handle *h, long long nsteps)
 
 int run_steps(aap_handle *h, long long nsteps)
 {
+    if (!h->timing && h->L.multi) {
+        if (nsteps > 0) AAP_CK(aapk::launch_multi(h->L, (int)nsteps, h->stream));
+        h->step += nsteps;
+        return AAP_OK;
+    }
     if (!h->timing) {
         int rc = launch_steps(h->L, h->stream, nsteps, h->cap_stream, h->gexec);
         if (rc) return rc;
@@ -1306,6 +1329,7 @@ int aap_test_pipe_wait(int64_t wait_cycles, int32_t stall)
 {
     if (stall != 0 && stall != 1) return fail(AAP_EINVAL, "stall must be 0 or 1");
     AAP_CK(aapk::set_pipe_test(wait_cycles, stall));
+    AAP_CK(aapk::set_multi_test(wait_cycles, stall));
     return AAP_OK;
 }
 

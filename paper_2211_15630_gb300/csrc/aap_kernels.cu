@@ -123,7 +123,6 @@ k_step(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_base,
 // last block to arrive advances the step.
 __global__ void k_finish(Sys *sys, int nsys, const int *__restrict__ tile_base, Ctl *ctl)
 {
-    static_assert(kAccSlots == 64, "two accumulator slots per lane");
     __shared__ int s_last;
     const long long step = ctl->step;
     const int cur = (int)(step & 1);
@@ -151,53 +150,8 @@ __global__ void k_finish(Sys *sys, int nsys, const int *__restrict__ tile_base, 
     const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nwarps = (int)((gridDim.x * blockDim.x) >> 5);
     for (int si = gw; si < nsys; si += nwarps) {
         Sys &S = sys[si];
-        unsigned long long *a = S.acc + (size_t)cur * kAccSlots * kAccWords;
-        unsigned long long x0[5], x1[5];
-#pragma unroll
-        for (int w = 0; w < 5; ++w) {
-            x0[w] = a[lane * kAccWords + w];
-            x1[w] = a[(lane + 32) * kAccWords + w];
-        }
-#pragma unroll
-        for (int w = 0; w < 5; ++w) {
-            a[lane * kAccWords + w] = 0;
-            a[(lane + 32) * kAccWords + w] = 0;
-        }
-        long long v[5];
-#pragma unroll
-        for (int w = 0; w < 5; ++w) v[w] = warp_sum_ll((long long)(x0[w] + x1[w]));   // exact, lane 0 holds it
-        if (lane != 0) continue;
-        const double n = (double)S.n;
-        const double dc = (double)v[0] / kFixStep, ds = (double)v[1] / kFixStep;
-        const double dc2 = (double)v[3] / kFixStep, ds2 = (double)v[4] / kFixStep;
-        const double phi = n > 0 ? sqrt(dc * dc + ds * ds) / n : 0.0;
-        const double q = n > 0 ? sqrt(dc2 * dc2 + ds2 * ds2) / n : 0.0;
-        const double nbar = n > 0 ? (double)v[2] / n : 0.0;
-        if (S.trace) {
-            const long long i1 = step + 1 - S.trace_base, i0 = step - S.trace_base;
-            if (i1 >= 0 && i1 < S.trace_cap) S.trace[i1] = phi;
-            if (i0 >= 0 && i0 < S.trace_cap) S.trace_nbar[i0] = nbar;
-        }
-        if (step < S.meas_until) {
-            // on-the-fly measurement (Sec. 3.4): state t contributes p(t),
-            // q(t) and the mean neighbour number measured on it
-            const double p0 = S.last[0], q0 = S.last[1];
-            double pk = 1.0, qk = 1.0, nk = 1.0;
-            for (int k = 0; k < 4; ++k) {
-                pk *= p0;
-                qk *= q0;
-                nk *= nbar;
-                S.stats[k] += pk;
-                S.stats[4 + k] += qk;
-                S.stats[8 + k] += nk;
-            }
-            S.stats[12] += 1.0;
-        }
-        S.last[0] = phi;
-        S.last[1] = q;
-        S.last[2] = nbar;
-        S.last[3] = (double)(step + 1);
-        S.spill_cnt[cur] = 0;
+        close_sums(S, step, lane);
+        if (lane == 0) S.spill_cnt[cur] = 0;
     }
     __syncthreads();
     if (threadIdx.x == 0) {

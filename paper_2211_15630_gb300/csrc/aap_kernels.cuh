@@ -31,6 +31,9 @@ struct LaunchCfg {
     int pipe_cap, pipe_cap_own, pipe_grid;
     int pipe_nceh;               // half cells (split along x) of the largest extended tile, (2 tw + 4)(th + 2)
     int *dense_list;
+    // many steps per launch (a small system, one block per tile, all resident)
+    int multi, multi_species, multi_cap, multi_tiles, multi_threads, multi_wsp;
+    int *multi_cnt;              // device: three private counter sets and two barrier words, zero between launches
     // metric-free step (knn > 0): cell count, scan, scatter, k-nearest update
     int knn;
     long long mf_n, mf_ncell;
@@ -52,6 +55,15 @@ cudaError_t configure_pipe_kernel(int model, size_t smem);
 cudaError_t set_pipe_test(long long wait_cycles, int stall);
 // The pipelined step kernel alone (launch_step adds k_finish).
 cudaError_t launch_step_pipe(const LaunchCfg &L, cudaStream_t st);
+
+// Ints of one private counter set: a line per tile and one for the spill count.
+inline int multi_stride(int ntiles) { return (ntiles + 1) * kCntStride; }
+inline size_t multi_bytes(int ntiles) { return (3 * (size_t)multi_stride(ntiles) + 4) * sizeof(int); }
+// Decide whether a system of ntiles tiles can run many steps per launch (L.multi): all its blocks resident with at
+// least min_cap staged records each.
+cudaError_t configure_multi(LaunchCfg &L, int nspecies, int ntiles, int sm_count, int min_cap);
+cudaError_t launch_multi(const LaunchCfg &L, int nsteps, cudaStream_t st);
+cudaError_t set_multi_test(long long wait_cycles, int stall);
 
 // One full step: k_step (or the pipelined step kernel) then k_finish.  With ev != nullptr, ev[0..2] are
 // recorded before k_step, after k_step and after k_finish.

@@ -118,15 +118,6 @@ struct RawMeta {
     unsigned char spill_seg[kPipeMaxSpill]; // segment of staged spill record j
 };
 
-// What the update warps need of a sorted tile.
-struct OutMeta {
-    int tile;                   // -1: no more tiles, -2: skip (the buffer holds part of a wide tile)
-    int rbuf, rwide;            // raw buffer of the tile's staged records, and whether it spans the next one too
-    int n_own, tx, ty, tw, th, W2, twL, twR, thD, thU;   // W2: half cells per extended row, 2 tw + 4
-    int wide;                   // a half cell holds enough particles for 512 candidates
-    int dense;                  // more than 1.5 staged records per half cell on average
-};
-
 struct PipeShared {
     Sys os[2];                  // system of the tile in each output buffer (read by the update warps)
     int osys[2];                // its index, -1: none yet
@@ -541,165 +532,6 @@ __device__ __forceinline__ void sort_order(PipeShared &sh, const PipeBufs &B, in
     }
 }
 
-// ----------------------------------------------------------- update warps --
-// The neighbour sum of one particle over three rows of five half cells,
-// each row contiguous in the half-cell order.  The particle itself is
-// included (it adds e^{i theta_i} to the VM/NVM sum and sin 0 to the
-// Langevin sum; cnt counts it).  The staged (cos, sin) are integers in units
-// of 2^-22, so the sums are exact and order-free; ACC is int below 512
-// candidates and long long beyond.
-template <int MODEL, typename ACC, int UNR>
-__device__ __forceinline__ void neighbour_sum_h(const float4 *__restrict__ P, const unsigned short *cstart, int ec,
-                                                int W2, float4 pi, float r2, ACC &sc, ACC &ss, int &cnt)
-{
-    sc = 0;
-    ss = 0;
-    cnt = 0;
-    const float pcf = (float)__float_as_int(pi.z), psf = (float)__float_as_int(pi.w);
-#pragma unroll
-    for (int dy = -1; dy <= 1; ++dy) {
-        const int c0 = ec + dy * W2 - 2;
-        const int a = cstart[c0], b = cstart[c0 + 5];
-#pragma unroll UNR
-        for (int j = a; j < b; ++j) {
-            const float4 pj = P[j];
-            const float dx = pj.x - pi.x, dyy = pj.y - pi.y;
-            const float d2 = fmaf(dx, dx, dyy * dyy);
-            if (d2 <= r2) {
-                int cj = __float_as_int(pj.z), sj = __float_as_int(pj.w);
-                if (MODEL == 2 && fmaf(pcf, (float)cj, psf * (float)sj) < 0.f) {
-                    cj = -cj;                         // Eq. (collision_NVM): the reversed direction
-                    sj = -sj;
-                }
-                sc += cj;
-                ss += sj;
-                ++cnt;
-            }
-        }
-    }
-}
-
-struct Acc {
-    long long c, s, n, c2, s2;
-};
-
-// One particle per lane (own index o, inactive when o >= n_own); every lane
-// of the warp must call (the scatter is warp-aggregated).
-template <int MODEL>
-__device__ __forceinline__ void update_one(const Sys &S, const OutMeta &O, const float4 *__restrict__ P,
-                                           const unsigned short *cstart, const int4 *RB, const unsigned short *OR,
-                                           const unsigned short *OQ,
-                                           int o, long long step, bool measure, int *mhist, Acc &acc)
-{
-    const int nxt = (int)(step & 1) ^ 1;
-    const bool act = o < O.n_own;
-    int4 rec = make_int4(0, 0, 0, 0);
-    int dtile = 0, region = 0;
-    if (act) {
-        const int tw = O.tw, th = O.th, W2 = O.W2;
-        const int4 rk = RB[OR[o]];                // own regions map to themselves (no shift, no mirror)
-        const int X = rk.x, Y = rk.y;
-        const float thi = __int_as_float(rk.z);
-        const unsigned id = (unsigned)rk.w;
-        const int ec = ((Y >> S.sy) + 1) * W2 + (X >> (S.sx - 1)) + 2;      // extended half cell
-        const float4 pi = P[OQ[o]];
-        float sc, ss;                    // neighbour sums in units of 2^-22
-        int cnt;
-        bool narrow = !O.wide;
-        if (!narrow) {
-            const int ncand = cstart[ec - W2 + 3] - cstart[ec - W2 - 2] + cstart[ec + 3] - cstart[ec - 2] +
-                              cstart[ec + W2 + 3] - cstart[ec + W2 - 2];
-            narrow = ncand < 512;
-        }
-        if (narrow) {
-            // short candidate rows run faster unrolled twice, long ones
-            // (dense tiles) four times
-            int a, b;
-            if (O.dense) neighbour_sum_h<MODEL, int, 4>(P, cstart, ec, W2, pi, S.r2, a, b, cnt);
-            else neighbour_sum_h<MODEL, int, 2>(P, cstart, ec, W2, pi, S.r2, a, b, cnt);
-            sc = (float)a;
-            ss = (float)b;
-        } else {
-            long long a, b;
-            neighbour_sum_h<MODEL, long long, 4>(P, cstart, ec, W2, pi, S.r2, a, b, cnt);
-            sc = (float)a;
-            ss = (float)b;
-        }
-        const int nb = cnt - 1;          // the particle itself was counted
-        if (measure) {
-            int bt = (int)floorf((thi + AAP_PI_F) * ((float)S.bins_theta * (1.0f / AAP_2PI_F)));
-            bt = min(max(bt, 0), S.bins_theta - 1);
-            atomicAdd(&mhist[bt], 1);
-            atomicAdd(&mhist[S.bins_theta + min(nb, S.bins_nbr - 1)], 1);
-        }
-        uint32_t c4[4] = {id, (uint32_t)step, (uint32_t)((unsigned long long)step >> 32), 0u};
-        philox4x32_10(c4, S.seed_lo, S.seed_hi);
-        const float u0 = u01f(c4[0]);
-        float thn, cn, sn;
-        int dX, dY;
-        if (MODEL != 1) {
-            // Eq. (collision_VM) / (collision_NVM) + noise; Eq. (streaming)
-            thn = arg2(ss, sc) + S.omega_step + S.eta_pi * (2.0f * u0 - 1.0f);
-            __sincosf(thn, &sn, &cn);
-            dX = __float2int_rn(S.kx * cn);
-            dY = __float2int_rn(S.ky * sn);
-        } else {
-            // Eq. (Langevin_dynamics), one Euler-Maruyama step
-            const float u1 = u01f(c4[1]);
-            const float h = S.wlen > 0 ? S.wtab[min(nb, S.wlen - 1)]
-                                       : (S.weight ? 1.0f : 1.0f / (1.0f + (float)nb));
-            // sum_j sin(o (theta_j - theta_i)) from the exact sums (units 2^-22 x 2^-22)
-            const float tsum = ((float)__float_as_int(pi.z) * ss - (float)__float_as_int(pi.w) * sc) *
-                               (1.0f / (kFixNbF * kFixNbF));
-            const float gz = sqrtf(-2.0f * logf(u0)) * cospif(2.0f * u1);
-            thn = thi + S.gamma_dt * h * tsum + S.omega_step + S.noise_amp * gz;
-            float co, so;
-            __sincosf(thi, &so, &co);    // streaming direction theta(t), |theta| <= pi
-            dX = __float2int_rn(S.kx * co);
-            dY = __float2int_rn(S.ky * so);
-            cn = 0.f;
-            sn = 0.f;
-        }
-        // boundary rule (Sec. 2.4) in exact fixed point
-        const int TWs = tw << S.sx, THs = th << S.sy;
-        int Xn = X + dX, Yn = Y + dY;
-        int dtx = O.tx, dty = O.ty, twd = tw, thd = th;
-        bool fx = false, fy = false;
-        if (Xn < 0) {
-            if (S.bx && O.tx == 0) { Xn = -Xn; fx = true; }
-            else { dtx = O.tx > 0 ? O.tx - 1 : S.ntx - 1; twd = O.twL; Xn += O.twL << S.sx; }
-        } else if (Xn >= TWs) {
-            if (S.bx && O.tx == S.ntx - 1) {
-                if (Xn == TWs) Xn = TWs - 1; else { Xn = TWs - (Xn - TWs); fx = true; }
-            } else { dtx = O.tx < S.ntx - 1 ? O.tx + 1 : 0; twd = O.twR; Xn -= TWs; }
-        }
-        if (Yn < 0) {
-            if (S.by && O.ty == 0) { Yn = -Yn; fy = true; }
-            else { dty = O.ty > 0 ? O.ty - 1 : S.nty - 1; thd = O.thD; Yn += O.thD << S.sy; }
-        } else if (Yn >= THs) {
-            if (S.by && O.ty == S.nty - 1) {
-                if (Yn == THs) Yn = THs - 1; else { Yn = THs - (Yn - THs); fy = true; }
-            } else { dty = O.ty < S.nty - 1 ? O.ty + 1 : 0; thd = O.thU; Yn -= THs; }
-        }
-        if (fx) { thn = AAP_PI_F - thn; cn = -cn; }
-        if (fy) { thn = -thn; sn = -sn; }
-        if (thn >= AAP_PI_F || thn < -AAP_PI_F)
-            thn -= AAP_2PI_F * floorf((thn + AAP_PI_F) * (1.0f / AAP_2PI_F));
-        if (MODEL == 1) __sincosf(thn, &sn, &cn);
-        if (!isfinite(thn)) atomicOr(S.err, ERR_NAN);
-        dtile = dty * S.ntx + dtx;
-        region = region_of(Xn >> S.sx, Yn >> S.sy, twd, thd);
-        rec = make_int4(Xn, Yn, __float_as_int(thn), (int)id);
-        acc.c += __float2int_rn(cn * kFixStepF);
-        acc.s += __float2int_rn(sn * kFixStepF);
-        acc.c2 += __float2int_rn(fmaf(cn, cn, -sn * sn) * kFixStepF);
-        acc.s2 += __float2int_rn(2.0f * cn * sn * kFixStepF);
-        acc.n += nb;
-        if (S.nbr_out && id < (unsigned long long)S.n) S.nbr_out[id] = nb;
-    }
-    warp_insert(S, nxt, act, dtile, region, rec);
-}
-
 }  // namespace
 
 // nceh: half cells of the largest extended tile, (2 tw + 4)(th + 2).
@@ -723,21 +555,6 @@ __device__ __forceinline__ void flush_hist(PipeShared &sh, const PipeBufs &B, in
                 atomicAdd(S.hist + i, (unsigned long long)mh[i]);
                 mh[i] = 0;
             }
-    }
-}
-
-// A warp's integer sums of one system (exact, so order-free) into that
-// system's step accumulators.
-__device__ __forceinline__ void flush_acc(const Acc &acc, unsigned long long *sys_acc, int cur)
-{
-    const long long a[5] = {acc.c, acc.s, acc.n, acc.c2, acc.s2};
-    const int lane = threadIdx.x & 31;
-    unsigned long long *slot =
-        sys_acc + ((size_t)cur * kAccSlots + ((blockIdx.x * 32 + (threadIdx.x >> 5)) & (kAccSlots - 1))) * kAccWords;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        const long long v = warp_sum_ll(a[k]);
-        if (lane == 0 && v) atomicAdd(slot + k, (unsigned long long)v);
     }
 }
 
@@ -1056,7 +873,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
             const Sys &S = sh.os[b];
             const bool measure = step < S.meas_until;
             if (S.acc != acc_sys) {
-                if (acc_sys) flush_acc(acc, acc_sys, cur);
+                if (acc_sys) flush_acc<false>(acc, acc_sys, cur);
                 acc = {0, 0, 0, 0, 0};
                 acc_sys = S.acc;
             }
@@ -1072,7 +889,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
                 c = __shfl_sync(0xffffffffu, c, 0);
                 const int o0 = c * 32;
                 if (o0 >= O.n_own) break;
-                update_one<MODEL>(S, O, P, cst, RB, OR, OQ, o0 + lane, step, measure, B.mhist(b), acc);
+                update_one<MODEL, false, 1>(S, O, P, cst, RB, OR, OQ, o0 + lane, step, measure, B.mhist(b), acc, ToSystem{});
             }
             __syncwarp();
             if (lane == 0) {
@@ -1084,7 +901,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
             }
             b ^= 1;
         }
-        if (acc_sys) flush_acc(acc, acc_sys, cur);
+        if (acc_sys) flush_acc<false>(acc, acc_sys, cur);
     }
     __syncthreads();
     // --- the last tiles' histograms -> their systems -----------------------

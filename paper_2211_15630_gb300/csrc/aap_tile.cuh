@@ -51,10 +51,12 @@ __device__ __forceinline__ int region_of(int lx, int ly, int tw, int th)
     return ry * 3 + rx;
 }
 
-// Append rec to region `region` of tile `dtile` in buffer b.  Every lane of
-// the warp must call; lanes with act == false take part in the vote only.
-// Lanes headed for the same region share one atomicAdd (warp aggregation).
-__device__ __forceinline__ void warp_insert(const Sys &S, int b, bool act, int dtile, int region, int4 rec)
+// Append rec to region `region` of tile `dtile` in buffer b, whose counters
+// are cnt (per tile and region) and *spill_cnt.  Every lane of the warp must
+// call; lanes with act == false take part in the vote only.  Lanes headed for
+// the same region share one atomicAdd (warp aggregation).
+__device__ __forceinline__ void warp_insert(const Sys &S, int b, bool act, int dtile, int region, int4 rec, int *cnt,
+                                            int *spill_cnt)
 {
     const int lane = threadIdx.x & 31;
     const int key = act ? dtile * kCntStride + region : -1 - lane;
@@ -63,14 +65,14 @@ __device__ __forceinline__ void warp_insert(const Sys &S, int b, bool act, int d
     const unsigned peers = same ? 0xffffffffu : __match_any_sync(0xffffffffu, key);
     const int leader = __ffs(peers) - 1;
     int base = 0;
-    if (act && lane == leader) base = atomicAdd(&S.cnt[b][key], __popc(peers));
+    if (act && lane == leader) base = atomicAdd(&cnt[key], __popc(peers));
     base = __shfl_sync(0xffffffffu, base, leader);
     if (act) {
         const int slot = base + __popc(peers & ((1u << lane) - 1u));
         if (slot < S.cap[region]) {
             S.rec[b][(long long)dtile * S.tile_slots + S.off[region] + slot] = rec;
         } else {
-            const int e = atomicAdd(&S.spill_cnt[b], 1);
+            const int e = atomicAdd(spill_cnt, 1);
             if (e < S.spill_cap) {
                 S.spill_rec[b][e] = rec;
                 S.spill_key[b][e] = key;
@@ -83,6 +85,10 @@ __device__ __forceinline__ void warp_insert(const Sys &S, int b, bool act, int d
     }
 }
 
+__device__ __forceinline__ void warp_insert(const Sys &S, int b, bool act, int dtile, int region, int4 rec)
+{
+    warp_insert(S, b, act, dtile, region, rec, S.cnt[b], &S.spill_cnt[b]);
+}
 
 // ---------------------------------------------------------- tile context --
 // Geometry of one tile and its neighbours' sizes.
@@ -618,6 +624,385 @@ __device__ __forceinline__ void tile_body(TileCtx &T, const Stage &A, const Tabl
             if (tb.mhist[i]) atomicAdd(S.hist + i, (unsigned long long)tb.mhist[i]);
     }
     PHASE_MARK(5);
+}
+
+// What the update needs of a tile sorted by half cell.
+struct OutMeta {
+    int tile;                   // -1: no more tiles, -2: skip (the buffer holds part of a wide tile)
+    int rbuf, rwide;            // raw buffer of the tile's staged records, and whether it spans the next one too
+    int n_own, tx, ty, tw, th, W2, twL, twR, thD, thU;   // W2: half cells per extended row, 2 tw + 4
+    int wide;                   // a half cell holds enough particles for 512 candidates
+    int dense;                  // more than 1.5 staged records per half cell on average
+    int small_gamma;            // several species: every |Gamma dt| is below 1
+};
+
+// ------------------------------------ the update of a half-cell-sorted tile --
+// The neighbour sum of one particle over three rows of five half cells,
+// each row contiguous in the half-cell order.  The particle itself is
+// included (it adds e^{i theta_i} to the VM/NVM sum and sin 0 to the
+// Langevin sum; cnt counts it).  The staged (cos, sin) are integers in units
+// of 2^-22, so the sums are exact and order-free; ACC is int below 512
+// candidates and long long beyond.  LPP lanes share a particle: lane `sub` of
+// them takes every LPP-th candidate of a row (the callers add the shares up).
+template <int MODEL, typename ACC, int UNR, int LPP = 1>
+__device__ __forceinline__ void neighbour_sum_h(const float4 *__restrict__ P, const unsigned short *cstart, int ec,
+                                                int W2, float4 pi, float r2, ACC &sc, ACC &ss, int &cnt, int sub = 0)
+{
+    sc = 0;
+    ss = 0;
+    cnt = 0;
+    const float pcf = (float)__float_as_int(pi.z), psf = (float)__float_as_int(pi.w);
+#pragma unroll
+    for (int dy = -1; dy <= 1; ++dy) {
+        const int c0 = ec + dy * W2 - 2;
+        const int a = cstart[c0], b = cstart[c0 + 5];
+#pragma unroll UNR
+        for (int j = LPP > 1 ? a + sub : a; j < b; j += LPP) {
+            const float4 pj = P[j];
+            const float dx = pj.x - pi.x, dyy = pj.y - pi.y;
+            const float d2 = fmaf(dx, dx, dyy * dyy);
+            if (d2 <= r2) {
+                int cj = __float_as_int(pj.z), sj = __float_as_int(pj.w);
+                if (MODEL == 2 && fmaf(pcf, (float)cj, psf * (float)sj) < 0.f) {
+                    cj = -cj;                         // Eq. (collision_NVM): the reversed direction
+                    sj = -sj;
+                }
+                sc += cj;
+                ss += sj;
+                ++cnt;
+            }
+        }
+    }
+}
+
+// The Langevin sums with per-species couplings (neighbour_sum_sp above) over
+// the half cells, out of line for couplings of any size: a neighbour's species
+// rides in the upper bits of its staged cosine (pack_species).
+constexpr int kSpeciesShift = 26;           // |cos| 2^22 needs 24 bits with its sign
+__device__ __forceinline__ int pack_species(int c, int sp) { return (c & 0x03ffffff) | (sp << kSpeciesShift); }
+__device__ __forceinline__ int packed_cos(int z) { return (z << 6) >> 6; }
+
+template <int LPP>
+__device__ __noinline__ void neighbour_sum_sp_h(const float4 *__restrict__ P, const unsigned short *cstart, int ec,
+                                                int W2, float4 pi, float r2, const float *grow, long long *out, int sub)
+{
+    long long sc = 0, ss = 0;
+    int cnt = 0;
+    for (int dy = -1; dy <= 1; ++dy) {
+        const int c0 = ec + dy * W2 - 2;
+        const int a = cstart[c0], b = cstart[c0 + 5];
+        for (int j = LPP > 1 ? a + sub : a; j < b; j += LPP) {
+            const float4 pj = P[j];
+            const float dx = pj.x - pi.x, dyy = pj.y - pi.y;
+            if (fmaf(dx, dx, dyy * dyy) <= r2) {
+                const int z = __float_as_int(pj.z);
+                const float g = grow[(z >> kSpeciesShift) & 7];
+                sc += __float2ll_rn(g * (float)packed_cos(z));
+                ss += __float2ll_rn(g * (float)__float_as_int(pj.w));
+                ++cnt;
+            }
+        }
+    }
+    out[0] = sc;
+    out[1] = ss;
+    out[2] = cnt;
+}
+
+// The same sums when every |Gamma dt| is below 1: W[j] holds the weighted,
+// rounded (cos, sin) of staged record j for the particle's species, made once
+// per record when the tile was sorted instead of once per neighbour.
+template <typename ACC, int UNR, int LPP>
+__device__ __forceinline__ void neighbour_sum_w(const float4 *__restrict__ P, const int2 *__restrict__ W,
+                                                const unsigned short *cstart, int ec, int W2, float4 pi, float r2,
+                                                ACC &sc, ACC &ss, int &cnt, int sub)
+{
+    sc = 0;
+    ss = 0;
+    cnt = 0;
+#pragma unroll
+    for (int dy = -1; dy <= 1; ++dy) {
+        const int c0 = ec + dy * W2 - 2;
+        const int a = cstart[c0], b = cstart[c0 + 5];
+#pragma unroll UNR
+        for (int j = LPP > 1 ? a + sub : a; j < b; j += LPP) {
+            const float2 pj = *reinterpret_cast<const float2 *>(P + j);
+            const int2 w = W[j];
+            const float dx = pj.x - pi.x, dyy = pj.y - pi.y;
+            if (fmaf(dx, dx, dyy * dyy) <= r2) {
+                sc += w.x;
+                ss += w.y;
+                ++cnt;
+            }
+        }
+    }
+}
+
+struct Acc {
+    long long c, s, n, c2, s2;
+};
+
+// The system's own counters of its buffer `nxt`.
+struct ToSystem {
+    __device__ __forceinline__ int *cnt(const Sys &S, int nxt) const { return S.cnt[nxt]; }
+    __device__ __forceinline__ int *spill(const Sys &S, int nxt) const { return &S.spill_cnt[nxt]; }
+    __device__ __forceinline__ const int2 *weighted(int) const { return nullptr; }
+};
+
+// One particle per lane (own index o, inactive when o >= n_own); every lane
+// of the warp must call (the scatter is warp-aggregated).  `to` names the
+// counters of the buffer the new records go to, asked for only where they are
+// used (registers).  SP: several species (each
+// particle's speed, noise and chirality looked up by its id).  LPP: lanes per
+// particle (a power of two; o is the same for each group of LPP lanes).
+template <int MODEL, bool SP, int LPP, class TO>
+__device__ __forceinline__ void update_one(const Sys &S, const OutMeta &O, const float4 *__restrict__ P,
+                                           const unsigned short *cstart, const int4 *RB, const unsigned short *OR,
+                                           const unsigned short *OQ,
+                                           int o, long long step, bool measure, int *mhist, Acc &acc,
+                                           const TO &to)
+{
+    const int nxt = (int)(step & 1) ^ 1;
+    const int sub = LPP > 1 ? (int)(threadIdx.x & (LPP - 1)) : 0;
+    const unsigned group = ((1u << LPP) - 1u) << (threadIdx.x & 31 & ~(LPP - 1));   // the particle's lanes
+    bool act = o < O.n_own;
+    int4 rec = make_int4(0, 0, 0, 0);
+    int dtile = 0, region = 0;
+    int X = 0, Y = 0, cnt = 0, sp = 0;
+    float thi = 0.f, sc = 0.f, ss = 0.f;     // neighbour sums in units of 2^-22
+    unsigned id = 0;
+    float4 pi = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int tw = O.tw, th = O.th;
+    if (act) {
+        const int W2 = O.W2;
+        const int4 rk = RB[OR[o]];                // own regions map to themselves (no shift, no mirror)
+        X = rk.x;
+        Y = rk.y;
+        thi = __int_as_float(rk.z);
+        id = (unsigned)rk.w;
+        const int ec = ((Y >> S.sy) + 1) * W2 + (X >> (S.sx - 1)) + 2;      // extended half cell
+        pi = P[OQ[o]];
+        sp = SP ? species_of(S, id) : 0;
+        bool narrow = !O.wide;
+        if (SP && MODEL == 1) {
+            pi.z = __int_as_float(packed_cos(__float_as_int(pi.z)));
+            long long a, b;
+            if (O.small_gamma) {
+                const int2 *w = to.weighted(sp);
+                if (narrow) {
+                    int a4, b4;
+                    if (O.dense) neighbour_sum_w<int, 4, LPP>(P, w, cstart, ec, W2, pi, S.r2, a4, b4, cnt, sub);
+                    else neighbour_sum_w<int, 2, LPP>(P, w, cstart, ec, W2, pi, S.r2, a4, b4, cnt, sub);
+                    a = a4;
+                    b = b4;
+                } else {
+                    neighbour_sum_w<long long, 4, LPP>(P, w, cstart, ec, W2, pi, S.r2, a, b, cnt, sub);
+                }
+            } else {
+                long long out[3];
+                neighbour_sum_sp_h<LPP>(P, cstart, ec, W2, pi, S.r2, S.sp_gamma_dt + sp * kMaxSpecies, out, sub);
+                a = out[0];
+                b = out[1];
+                cnt = (int)out[2];
+            }
+#pragma unroll
+            for (int d = 1; d < LPP; d <<= 1) {
+                a += __shfl_xor_sync(group, a, d);
+                b += __shfl_xor_sync(group, b, d);
+            }
+            sc = (float)a;
+            ss = (float)b;
+        } else {
+            if (!narrow) {
+                const int ncand = cstart[ec - W2 + 3] - cstart[ec - W2 - 2] + cstart[ec + 3] - cstart[ec - 2] +
+                                  cstart[ec + W2 + 3] - cstart[ec + W2 - 2];
+                narrow = ncand < 512;
+            }
+            if (narrow) {
+                // short candidate rows run faster unrolled twice, long ones
+                // (dense tiles) four times
+                int a, b;
+                if (O.dense) neighbour_sum_h<MODEL, int, 4, LPP>(P, cstart, ec, W2, pi, S.r2, a, b, cnt, sub);
+                else neighbour_sum_h<MODEL, int, 2, LPP>(P, cstart, ec, W2, pi, S.r2, a, b, cnt, sub);
+#pragma unroll
+                for (int d = 1; d < LPP; d <<= 1) {
+                    a += __shfl_xor_sync(group, a, d);
+                    b += __shfl_xor_sync(group, b, d);
+                }
+                sc = (float)a;
+                ss = (float)b;
+            } else {
+                long long a, b;
+                neighbour_sum_h<MODEL, long long, 4, LPP>(P, cstart, ec, W2, pi, S.r2, a, b, cnt, sub);
+#pragma unroll
+                for (int d = 1; d < LPP; d <<= 1) {
+                    a += __shfl_xor_sync(group, a, d);
+                    b += __shfl_xor_sync(group, b, d);
+                }
+                sc = (float)a;
+                ss = (float)b;
+            }
+        }
+#pragma unroll
+        for (int d = 1; d < LPP; d <<= 1) cnt += __shfl_xor_sync(group, cnt, d);
+    }
+    if (LPP > 1) act = act && sub == 0;
+    if (act) {
+        const int nb = cnt - 1;          // the particle itself was counted
+        if (measure) {
+            int bt = (int)floorf((thi + AAP_PI_F) * ((float)S.bins_theta * (1.0f / AAP_2PI_F)));
+            bt = min(max(bt, 0), S.bins_theta - 1);
+            atomicAdd(&mhist[bt], 1);
+            atomicAdd(&mhist[S.bins_theta + min(nb, S.bins_nbr - 1)], 1);
+        }
+        uint32_t c4[4] = {id, (uint32_t)step, (uint32_t)((unsigned long long)step >> 32), 0u};
+        philox4x32_10(c4, S.seed_lo, S.seed_hi);
+        const float u0 = u01f(c4[0]);
+        float thn, cn, sn;
+        int dX, dY;
+        if (MODEL != 1) {
+            // Eq. (collision_VM) / (collision_NVM) + noise; Eq. (streaming)
+            thn = arg2(ss, sc) + (SP ? S.sp_omega_step[sp] : S.omega_step) +
+                  (SP ? S.sp_eta_pi[sp] : S.eta_pi) * (2.0f * u0 - 1.0f);
+            __sincosf(thn, &sn, &cn);
+            dX = __float2int_rn((SP ? S.sp_kx[sp] : S.kx) * cn);
+            dY = __float2int_rn((SP ? S.sp_ky[sp] : S.ky) * sn);
+        } else {
+            // Eq. (Langevin_dynamics), one Euler-Maruyama step
+            const float u1 = u01f(c4[1]);
+            const float h = S.wlen > 0 ? S.wtab[min(nb, S.wlen - 1)]
+                                       : (S.weight ? 1.0f : 1.0f / (1.0f + (float)nb));
+            // sum_j sin(o (theta_j - theta_i)) from the exact sums (units 2^-22 x 2^-22);
+            // Gamma dt inside with several species
+            const float tsum = ((float)__float_as_int(pi.z) * ss - (float)__float_as_int(pi.w) * sc) *
+                               (1.0f / (kFixNbF * kFixNbF));
+            const float gz = sqrtf(-2.0f * logf(u0)) * cospif(2.0f * u1);
+            const float drift = SP ? h * tsum : S.gamma_dt * h * tsum;
+            thn = thi + drift + (SP ? S.sp_omega_step[sp] : S.omega_step) + (SP ? S.sp_noise_amp[sp] : S.noise_amp) * gz;
+            float co, so;
+            __sincosf(thi, &so, &co);    // streaming direction theta(t), |theta| <= pi
+            dX = __float2int_rn((SP ? S.sp_kx[sp] : S.kx) * co);
+            dY = __float2int_rn((SP ? S.sp_ky[sp] : S.ky) * so);
+            cn = 0.f;
+            sn = 0.f;
+        }
+        // boundary rule (Sec. 2.4) in exact fixed point
+        const int TWs = tw << S.sx, THs = th << S.sy;
+        int Xn = X + dX, Yn = Y + dY;
+        int dtx = O.tx, dty = O.ty, twd = tw, thd = th;
+        bool fx = false, fy = false;
+        if (Xn < 0) {
+            if (S.bx && O.tx == 0) { Xn = -Xn; fx = true; }
+            else { dtx = O.tx > 0 ? O.tx - 1 : S.ntx - 1; twd = O.twL; Xn += O.twL << S.sx; }
+        } else if (Xn >= TWs) {
+            if (S.bx && O.tx == S.ntx - 1) {
+                if (Xn == TWs) Xn = TWs - 1; else { Xn = TWs - (Xn - TWs); fx = true; }
+            } else { dtx = O.tx < S.ntx - 1 ? O.tx + 1 : 0; twd = O.twR; Xn -= TWs; }
+        }
+        if (Yn < 0) {
+            if (S.by && O.ty == 0) { Yn = -Yn; fy = true; }
+            else { dty = O.ty > 0 ? O.ty - 1 : S.nty - 1; thd = O.thD; Yn += O.thD << S.sy; }
+        } else if (Yn >= THs) {
+            if (S.by && O.ty == S.nty - 1) {
+                if (Yn == THs) Yn = THs - 1; else { Yn = THs - (Yn - THs); fy = true; }
+            } else { dty = O.ty < S.nty - 1 ? O.ty + 1 : 0; thd = O.thU; Yn -= THs; }
+        }
+        if (fx) { thn = AAP_PI_F - thn; cn = -cn; }
+        if (fy) { thn = -thn; sn = -sn; }
+        if (thn >= AAP_PI_F || thn < -AAP_PI_F)
+            thn -= AAP_2PI_F * floorf((thn + AAP_PI_F) * (1.0f / AAP_2PI_F));
+        if (MODEL == 1) __sincosf(thn, &sn, &cn);
+        if (!isfinite(thn)) atomicOr(S.err, ERR_NAN);
+        dtile = dty * S.ntx + dtx;
+        region = region_of(Xn >> S.sx, Yn >> S.sy, twd, thd);
+        rec = make_int4(Xn, Yn, __float_as_int(thn), (int)id);
+        acc.c += __float2int_rn(cn * kFixStepF);
+        acc.s += __float2int_rn(sn * kFixStepF);
+        acc.c2 += __float2int_rn(fmaf(cn, cn, -sn * sn) * kFixStepF);
+        acc.s2 += __float2int_rn(2.0f * cn * sn * kFixStepF);
+        acc.n += nb;
+        if (S.nbr_out && id < (unsigned long long)S.n) S.nbr_out[id] = nb;
+    }
+    warp_insert(S, nxt, act, dtile, region, rec, to.cnt(S, nxt), to.spill(S, nxt));
+}
+
+// Warp sum of v, exact for |v| < 2^43: two 32-bit warp reductions of its low
+// 16 and its high bits instead of five rounds of 64-bit shuffles.
+__device__ __forceinline__ long long warp_redux_ll(long long v)
+{
+    const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)v & 0xffffu);
+    const int hi = __reduce_add_sync(0xffffffffu, (int)(v >> 16));
+    return (long long)hi * 65536 + (long long)lo;
+}
+
+// A warp's integer sums of one system (exact, so order-free) into that
+// system's step accumulators.
+template <bool REDUX>
+__device__ __forceinline__ void flush_acc(const Acc &acc, unsigned long long *sys_acc, int cur)
+{
+    const long long a[5] = {acc.c, acc.s, acc.n, acc.c2, acc.s2};
+    const int lane = threadIdx.x & 31;
+    unsigned long long *slot =
+        sys_acc + ((size_t)cur * kAccSlots + ((blockIdx.x * 32 + (threadIdx.x >> 5)) & (kAccSlots - 1))) * kAccWords;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const long long v = REDUX ? warp_redux_ll(a[k]) : warp_sum_ll(a[k]);
+        if (lane == 0 && v) atomicAdd(slot + k, (unsigned long long)v);
+    }
+}
+
+// Close step `step` of one system (one warp): p(t + 1) and q(t + 1) from the
+// step's integer sums (its 64 accumulator slots loaded at once past the L1,
+// then cleared), the trace and the on-the-fly measurement (Sec. 3.4).
+__device__ __forceinline__ void close_sums(const Sys &S, long long step, int lane)
+{
+    static_assert(kAccSlots == 64, "two accumulator slots per lane");
+    const int cur = (int)(step & 1);
+    unsigned long long *a = S.acc + (size_t)cur * kAccSlots * kAccWords;
+    unsigned long long x0[5], x1[5];
+#pragma unroll
+    for (int w = 0; w < 5; ++w) {
+        x0[w] = __ldcg(a + lane * kAccWords + w);
+        x1[w] = __ldcg(a + (lane + 32) * kAccWords + w);
+    }
+#pragma unroll
+    for (int w = 0; w < 5; ++w) {
+        a[lane * kAccWords + w] = 0;
+        a[(lane + 32) * kAccWords + w] = 0;
+    }
+    long long v[5];
+#pragma unroll
+    for (int w = 0; w < 5; ++w) v[w] = warp_sum_ll((long long)(x0[w] + x1[w]));   // exact, lane 0 holds it
+    if (lane != 0) return;
+    const double n = (double)S.n;
+    const double dc = (double)v[0] / kFixStep, ds = (double)v[1] / kFixStep;
+    const double dc2 = (double)v[3] / kFixStep, ds2 = (double)v[4] / kFixStep;
+    const double phi = n > 0 ? sqrt(dc * dc + ds * ds) / n : 0.0;
+    const double q = n > 0 ? sqrt(dc2 * dc2 + ds2 * ds2) / n : 0.0;
+    const double nbar = n > 0 ? (double)v[2] / n : 0.0;
+    if (S.trace) {
+        const long long i1 = step + 1 - S.trace_base, i0 = step - S.trace_base;
+        if (i1 >= 0 && i1 < S.trace_cap) S.trace[i1] = phi;
+        if (i0 >= 0 && i0 < S.trace_cap) S.trace_nbar[i0] = nbar;
+    }
+    if (step < S.meas_until) {
+        // on-the-fly measurement (Sec. 3.4): state t contributes p(t),
+        // q(t) and the mean neighbour number measured on it
+        const double p0 = S.last[0], q0 = S.last[1];
+        double pk = 1.0, qk = 1.0, nk = 1.0;
+        for (int k = 0; k < 4; ++k) {
+            pk *= p0;
+            qk *= q0;
+            nk *= nbar;
+            S.stats[k] += pk;
+            S.stats[4 + k] += qk;
+            S.stats[8 + k] += nk;
+        }
+        S.stats[12] += 1.0;
+    }
+    S.last[0] = phi;
+    S.last[1] = q;
+    S.last[2] = nbar;
+    S.last[3] = (double)(step + 1);
 }
 
 }  // namespace aapk
