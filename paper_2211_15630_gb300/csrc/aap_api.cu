@@ -105,8 +105,11 @@ struct aap_handle {
     long long since_copy = 0;       // steps queued since the last copy
     bool err_pending = false;
     int relayouts = 0;
-    // ensemble membership: steps are launched by the ensemble for all members
+    // ensemble membership: steps are launched by the ensemble for all members,
+    // whose error words and measurement sums lie side by side in its arrays
     bool member = false;
+    int *ens_err = nullptr;
+    double *ens_stats = nullptr;
     int nom_tw = 0, nom_th = 0;     // nominal tile shape actually used
     // coarse-graining accumulator (3 * bins 64-bit sums)
     unsigned long long *d_cg = nullptr;
@@ -639,11 +642,13 @@ int alloc_all(aap_handle *h)
         if ((rc = dev_alloc(h, &S.spill_bits[b], spill_bits_bytes(S)))) return rc;
     if ((rc = dev_alloc(h, &S.acc, 2 * aapk::kAccSlots * aapk::kAccWords * sizeof(unsigned long long)))) return rc;
     if ((rc = dev_alloc(h, &S.last, 4 * sizeof(double)))) return rc;
-    if ((rc = dev_alloc(h, &S.stats, 16 * sizeof(double)))) return rc;
+    if (h->member) S.stats = h->ens_stats;
+    else if ((rc = dev_alloc(h, &S.stats, 16 * sizeof(double)))) return rc;
     S.bins_theta = h->p.binnum_theta ? h->p.binnum_theta : 100;     // theta + |Omega| bins = L.hist_words
     S.bins_nbr = h->p.binnum_neighbors ? h->p.binnum_neighbors : 100;
     if ((rc = dev_alloc(h, &S.hist, (size_t)(S.bins_theta + S.bins_nbr) * sizeof(unsigned long long)))) return rc;
-    if ((rc = dev_alloc(h, &S.err, sizeof(int)))) return rc;
+    if (h->member) S.err = h->ens_err;
+    else if ((rc = dev_alloc(h, &S.err, sizeof(int)))) return rc;
     if (S.knn > 0) {
         const long long ncell = (long long)S.ncx * S.ncy;
         const long long nchunk = (ncell + 1 + aapk::kScanChunk - 1) / aapk::kScanChunk;
@@ -702,12 +707,9 @@ int alloc_all(aap_handle *h)
     return push_sys(h);
 }
 
-// Read and clear nothing: map the sticky device error word to a status.
-int read_errors(aap_handle *h)
+// Map a copy of the sticky device error word to a status.
+int error_status(aap_handle *h, int err)
 {
-    int err = 0;
-    AAP_CK(cudaMemcpyAsync(&err, h->hs.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    AAP_CK(cudaStreamSynchronize(h->stream));
     if (err & aapk::ERR_SPILL) h->flags |= AAP_FLAG_SPILLED;
     if (err & (aapk::ERR_LOST | aapk::ERR_STAGE)) {
         h->broken = true;
@@ -724,6 +726,15 @@ int read_errors(aap_handle *h)
     }
     if (err & aapk::ERR_NAN) return fail(AAP_ENAN, "a non-finite orientation was produced");
     return AAP_OK;
+}
+
+// Read and clear nothing: the status of the device error word.
+int read_errors(aap_handle *h)
+{
+    int err = 0;
+    AAP_CK(cudaMemcpyAsync(&err, h->hs.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    AAP_CK(cudaStreamSynchronize(h->stream));
+    return error_status(h, err);
 }
 
 // Fold the durations of recorded timing events into h->ms.
@@ -988,32 +999,18 @@ int poll_capacity(aap_handle *h)
 
 
 // Start a measurement window of nsteps steps at the current step: the
-// current state's p and q seed last[0..1] (state t0 is the first sample).
+// current state's p and q seed last[0..1] (state t0 is the first sample), all
+// on the device (nothing waits).
 int begin_measure(aap_handle *h, long long nsteps)
 {
-    aap_obs ob;
-    const Sys &S = h->hs;
-    AAP_CK(cudaMemsetAsync(h->d_obs, 0, 8 * sizeof(unsigned long long), h->stream));
-    AAP_CK(aapk::launch_observe(S, (int)(h->step & 1), h->d_obs, h->stream));
-    unsigned long long o[8];
-    AAP_CK(cudaMemcpyAsync(o, h->d_obs, sizeof(o), cudaMemcpyDeviceToHost, h->stream));
-    AAP_CK(cudaStreamSynchronize(h->stream));
-    const double n = (double)h->p.n;
-    const double c1 = (double)(long long)o[0] / aapk::kFix, s1 = (double)(long long)o[1] / aapk::kFix;
-    const double c2 = (double)(long long)o[2] / aapk::kFix, s2 = (double)(long long)o[3] / aapk::kFix;
-    double last[2] = {n > 0 ? std::sqrt(c1 * c1 + s1 * s1) / n : 0.0, n > 0 ? std::sqrt(c2 * c2 + s2 * s2) / n : 0.0};
-    (void)ob;
-    AAP_CK(cudaMemcpyAsync(h->hs.last, last, sizeof(last), cudaMemcpyHostToDevice, h->stream));
     h->hs.meas_until = h->step + nsteps;
-    AAP_CK(cudaStreamSynchronize(h->stream));
-    return push_sys(h);
+    AAP_CK(aapk::launch_begin_measure(h->d_sys, 1, h->p.n, (int)(h->step & 1), h->d_obs, h->hs.meas_until, h->stream));
+    return AAP_OK;
 }
 
-int read_results(aap_handle *h, aap_results *out)
+// The same sums as results (Sec. 3.4); st: the 16 words of Sys::stats.
+void fill_results(const double *st, aap_results *out)
 {
-    double st[16];
-    AAP_CK(cudaMemcpyAsync(st, h->hs.stats, sizeof(st), cudaMemcpyDeviceToHost, h->stream));
-    AAP_CK(cudaStreamSynchronize(h->stream));
     const double c = st[12];
     out->samples = (int64_t)c;
     for (int k = 0; k < 4; ++k) {
@@ -1022,6 +1019,14 @@ int read_results(aap_handle *h, aap_results *out)
         out->nbar[k] = c > 0 ? st[8 + k] / c : NAN;
     }
     out->binder = (c > 0 && out->p[1] > 0) ? 1.0 - out->p[3] / (3.0 * out->p[1] * out->p[1]) : NAN;
+}
+
+int read_results(aap_handle *h, aap_results *out)
+{
+    double st[16];
+    AAP_CK(cudaMemcpyAsync(st, h->hs.stats, sizeof(st), cudaMemcpyDeviceToHost, h->stream));
+    AAP_CK(cudaStreamSynchronize(h->stream));
+    fill_results(st, out);
     return AAP_OK;
 }
 
@@ -1064,6 +1069,10 @@ struct aap_ens {
     size_t scratch_bytes = 0;
     int *d_dense = nullptr;             // pipelined step: tiles left to the whole-block routine
     size_t dense_tiles = 0;
+    std::vector<int> order;             // replicas in the order of their descriptors (densest first)
+    int *d_err = nullptr;               // [count] the replicas' error words
+    double *d_stats = nullptr;          // [count][16] their measurement sums
+    unsigned long long *d_obs = nullptr;    // [count][8] observed sums of a window's first state
     LaunchCfg L{};
     long long step = 0;
     cudaStream_t cap = nullptr;
@@ -1094,6 +1103,12 @@ void ens_free(aap_ens *e)
     if (e->d_ctl) cudaFree(e->d_ctl);
     if (e->d_scratch) cudaFree(e->d_scratch);
     if (e->d_dense) cudaFree(e->d_dense);
+    if (e->d_err) cudaFree(e->d_err);
+    if (e->d_stats) cudaFree(e->d_stats);
+    if (e->d_obs) cudaFree(e->d_obs);
+    e->d_err = nullptr;
+    e->d_stats = nullptr;
+    e->d_obs = nullptr;
     e->d_sys = nullptr;
     e->d_tile_base = nullptr;
     e->d_ctl = nullptr;
@@ -1130,7 +1145,7 @@ int ens_combine(aap_ens *e)
         L.hist_words = std::max(L.hist_words, h->L.hist_words);
         L.scratch_cap = std::max(L.scratch_cap, h->L.scratch_cap);
         L.spill_list_cap = std::max(L.spill_list_cap, h->L.spill_list_cap);
-        total += h->hs.ntiles;
+        total += e->m[e->order[r]]->hs.ntiles;
         tb[r + 1] = (int)total;
     }
     if (total >= (1ll << 30)) return fail(AAP_EINVAL, "too many tiles in the ensemble");
@@ -1216,11 +1231,24 @@ int ens_build(aap_ens *e, int pol)
     const int count = (int)e->params.size();
     if (cudaMalloc(&e->d_sys, (size_t)count * sizeof(Sys)) != cudaSuccess ||
         cudaMalloc(&e->d_tile_base, (size_t)(count + 1) * sizeof(int)) != cudaSuccess ||
-        cudaMalloc(&e->d_ctl, sizeof(Ctl)) != cudaSuccess) {
+        cudaMalloc(&e->d_ctl, sizeof(Ctl)) != cudaSuccess ||
+        cudaMalloc(&e->d_err, (size_t)count * sizeof(int)) != cudaSuccess ||
+        cudaMalloc(&e->d_stats, (size_t)count * 16 * sizeof(double)) != cudaSuccess ||
+        cudaMalloc(&e->d_obs, (size_t)count * 8 * sizeof(unsigned long long)) != cudaSuccess) {
         cudaGetLastError();
         return fail(AAP_ENOMEM, "ensemble descriptor allocation failed");
     }
     AAP_CK(cudaMemset(e->d_ctl, 0, sizeof(Ctl)));
+    // the tiles of the densest replicas are claimed first (the longest jobs
+    // first, so that the step does not end on one): replica r has the
+    // descriptor slot[r]
+    std::vector<int> order(count), slot(count);
+    for (int r = 0; r < count; ++r) order[r] = r;
+    const auto density = [&](int r) { return (double)e->params[r].n * e->params[r].r * e->params[r].r /
+                                             (e->params[r].lx * e->params[r].ly); };
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return density(a) > density(b); });
+    for (int k = 0; k < count; ++k) slot[order[k]] = k;
+    e->order = order;
     for (int r = 0; r < count; ++r) {
         aap_handle *h = new aap_handle();
         e->m.push_back(h);
@@ -1231,8 +1259,10 @@ int ens_build(aap_ens *e, int pol)
         h->nom_th = kPolicies[pol].th;
         if (h->nom_tw == 0) density_tile(h->p, &h->nom_tw, &h->nom_th);
         if (!h->p.threads) h->p.threads = kPolicies[pol].threads;
-        h->d_sys = e->d_sys + r;
+        h->d_sys = e->d_sys + slot[r];
         h->d_ctl = e->d_ctl;
+        h->ens_err = e->d_err + r;
+        h->ens_stats = e->d_stats + 16 * (size_t)r;
         int rc;
         if ((rc = build_layout(h)) || (rc = alloc_all(h)) || (rc = reinsert(h, h->factor, 1)) ||
             (rc = read_errors(h))) {
@@ -1711,9 +1741,12 @@ int aap_coarse_grain(aap_handle *h, int32_t nbx, int32_t nby, float *dev_out)
     const long long bins = (long long)nbx * nby;
     if (h->cg_bins < bins) {
         int rc;
-        if (h->d_cg && (rc = dev_free(h, h->d_cg, (size_t)h->cg_bins * 3 * sizeof(unsigned long long)))) return rc;
+        const auto words = [](long long nb) { return (size_t)(3 * nb + 1) * sizeof(unsigned long long); };
+        if (h->d_cg && (rc = dev_free(h, h->d_cg, words(h->cg_bins)))) return rc;
         h->d_cg = nullptr;
-        if ((rc = dev_alloc(h, &h->d_cg, (size_t)bins * 3 * sizeof(unsigned long long)))) return rc;
+        h->cg_bins = 0;
+        if ((rc = dev_alloc(h, &h->d_cg, words(bins)))) return rc;
+        AAP_CK(cudaMemsetAsync(h->d_cg, 0, words(bins), h->stream));
         h->cg_bins = bins;
     }
     AAP_CK(aapk::launch_coarse(h->hs, (int)(h->step & 1), nbx, nby, h->d_cg, dev_out, h->stream));
@@ -1801,9 +1834,8 @@ int aap_ens_step(aap_ens *e, int64_t nsteps)
         if (e->since_copy < kAdaptSteps) continue;
         e->since_copy = 0;
         const int slot = e->batch_slot;
-        for (size_t r = 0; r < count; ++r)
-            AAP_CK(cudaMemcpyAsync(e->pinned_err + (1 + slot) * count + r, e->m[r]->hs.err, sizeof(int),
-                                   cudaMemcpyDeviceToHost, e->stream));
+        AAP_CK(cudaMemcpyAsync(e->pinned_err + (1 + slot) * count, e->d_err, count * sizeof(int),
+                               cudaMemcpyDeviceToHost, e->stream));
         AAP_CK(cudaEventRecord(e->batch_ev[slot], e->stream));
         e->batch_slot ^= 1;
         const int prev = e->batch_prev;
@@ -1813,8 +1845,7 @@ int aap_ens_step(aap_ens *e, int64_t nsteps)
             if ((rc = ens_act(e, e->pinned_err + (1 + prev) * count))) return rc;
         }
     }
-    for (size_t r = 0; r < e->m.size(); ++r)
-        AAP_CK(cudaMemcpyAsync(e->pinned_err + r, e->m[r]->hs.err, sizeof(int), cudaMemcpyDeviceToHost, e->stream));
+    AAP_CK(cudaMemcpyAsync(e->pinned_err, e->d_err, count * sizeof(int), cudaMemcpyDeviceToHost, e->stream));
     AAP_CK(cudaEventRecord(e->err_event, e->stream));
     e->err_pending = true;
     return AAP_OK;
@@ -1827,20 +1858,30 @@ int aap_ens_measure(aap_ens *e, int64_t nsteps)
     if (nsteps < 0) return fail(AAP_EINVAL, "nsteps < 0");
     int rc = ens_poll(e);
     if (rc) return rc;
-    for (aap_handle *h : e->m)
-        if ((rc = begin_measure(h, nsteps))) return rc;
+    long long max_n = 0;
+    for (aap_handle *h : e->m) {
+        max_n = std::max<long long>(max_n, h->p.n);
+        h->hs.meas_until = e->step + nsteps;
+    }
+    AAP_CK(aapk::launch_begin_measure(e->d_sys, (int)e->m.size(), max_n, (int)(e->step & 1), e->d_obs,
+                                      e->step + nsteps, e->stream));
     return aap_ens_step(e, nsteps);
 }
 
 int aap_ens_phi_mean(aap_ens *e, double *out)
 {
     if (!e || !out) return fail(AAP_EINVAL, "NULL argument");
+    const size_t count = e->m.size();
+    std::vector<int> err(count);
+    std::vector<double> st(16 * count);
+    AAP_CK(cudaMemcpyAsync(err.data(), e->d_err, count * sizeof(int), cudaMemcpyDeviceToHost, e->stream));
+    AAP_CK(cudaMemcpyAsync(st.data(), e->d_stats, st.size() * sizeof(double), cudaMemcpyDeviceToHost, e->stream));
     AAP_CK(cudaStreamSynchronize(e->stream));
-    for (size_t r = 0; r < e->m.size(); ++r) {
+    for (size_t r = 0; r < count; ++r) {
         aap_results res;
-        int rc = read_errors(e->m[r]);
+        int rc = error_status(e->m[r], err[r]);
         if (rc) return rc;
-        if ((rc = read_results(e->m[r], &res))) return rc;
+        fill_results(&st[16 * r], &res);
         out[r] = res.p[0];
     }
     return AAP_OK;

@@ -6,6 +6,7 @@
 
 #include <cuda_runtime.h>
 
+#include "aap_device.cuh"
 #include "aap_internal.cuh"
 #include "aap_kernels.cuh"
 
@@ -68,9 +69,26 @@ __device__ __forceinline__ void coarse_add(unsigned long long *acc, long long nb
     atomicAdd(acc + 2 * nb + bin, (unsigned long long)fix32_ll(sn));
 }
 
+// Fields per unit area from the integer sums: density, polarisation x,
+// polarisation y (planes of nb floats, row-major with x fastest); the sums
+// are cleared for the next call.
+__device__ __forceinline__ void coarse_fields(unsigned long long *acc, long long nb, double inv_area, float *out,
+                                              long long i0, long long stride)
+{
+    for (long long i = i0; i < nb; i += stride) {
+        const unsigned long long a0 = __ldcg(acc + i), a1 = __ldcg(acc + nb + i), a2 = __ldcg(acc + 2 * nb + i);
+        acc[i] = 0ull;
+        acc[nb + i] = 0ull;
+        acc[2 * nb + i] = 0ull;
+        out[i] = (float)((double)a0 * inv_area);
+        out[nb + i] = (float)((double)(long long)a1 / kFix * inv_area);
+        out[2 * nb + i] = (float)((double)(long long)a2 / kFix * inv_area);
+    }
+}
+
 // Counts and sums of cos theta, sin theta per bin of the state in buffer b,
 // in exact 64-bit integers (cos scaled by 2^32), so that the fields are
-// reproducible bit for bit.  acc: [3][nbx*nby], zeroed by the caller.  Blocks
+// reproducible bit for bit.  acc: [3][nbx*nby], zero between calls.  Blocks
 // take whole tiles and read only the stored records (the valid slots of the
 // nine regions, taken as one index range so that a tile costs one read of
 // its counts and the block's threads stay busy across the small edge
@@ -78,11 +96,17 @@ __device__ __forceinline__ void coarse_add(unsigned long long *acc, long long nb
 // go straight to acc, one atomic per record and field: merging a warp's
 // lanes of one bin first (by match and reductions, or by runs of records per
 // thread) was slower, as was a shared-memory window of the tile's bins
-// (same-address shared atomics serialise).
+// (same-address shared atomics serialise).  ticket != null (few bins): the
+// block that ends last turns the sums into fields, which saves a launch (a
+// replica's frame of 32 x 32 bins is three launches of 2 to 8 us otherwise).
 template <int NT>
-__global__ void __launch_bounds__(NT) k_coarse_tiles(Sys S, int b, BinAxis ax, BinAxis ay, unsigned long long *acc)
+__global__ void __launch_bounds__(NT) k_coarse_tiles(Sys S, int b, BinAxis ax, BinAxis ay, unsigned long long *acc,
+                                                     unsigned *ticket, double inv_area, float *out)
 {
+    __shared__ int s_last;
     const long long nb = (long long)ax.nb * ay.nb;
+    pdl_next();
+    pdl_wait();
     __shared__ int s_pre[kRegions + 1];
     for (int tile = blockIdx.x; tile < S.ntiles; tile += gridDim.x) {
         const int tx = tile % S.ntx, ty = tile / S.ntx;
@@ -121,19 +145,24 @@ __global__ void __launch_bounds__(NT) k_coarse_tiles(Sys S, int b, BinAxis ax, B
         const int ix = coarse_bin(S.x0tab[tx], rec.x, ax), iy = coarse_bin(S.y0tab[ty], rec.y, ay);
         coarse_add(acc, nb, (long long)iy * ax.nb + ix, __int_as_float(rec.z));
     }
+    if (!ticket) return;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        if (s_last) *ticket = 0u;
+        __threadfence();
+    }
+    __syncthreads();
+    if (s_last) coarse_fields(acc, nb, inv_area, out, threadIdx.x, NT);
 }
 
-// Fields per unit area: density, polarisation x, polarisation y (planes of
-// nbx*nby floats, row-major with x fastest).
-__global__ void k_coarse_finish(const unsigned long long *acc, int nbx, int nby, double inv_area, float *out)
+__global__ void k_coarse_finish(unsigned long long *acc, int nbx, int nby, double inv_area, float *out)
 {
-    const long long nb = (long long)nbx * nby;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nb;
-         i += (long long)gridDim.x * blockDim.x) {
-        out[i] = (float)((double)acc[i] * inv_area);
-        out[nb + i] = (float)((double)(long long)acc[nb + i] / kFix * inv_area);
-        out[2 * nb + i] = (float)((double)(long long)acc[2 * nb + i] / kFix * inv_area);
-    }
+    pdl_next();
+    pdl_wait();
+    coarse_fields(acc, (long long)nbx * nby, inv_area, out, blockIdx.x * (long long)blockDim.x + threadIdx.x,
+                  (long long)gridDim.x * blockDim.x);
 }
 
 }  // namespace
@@ -142,8 +171,6 @@ cudaError_t launch_coarse(const Sys &S, int b, int nbx, int nby, unsigned long l
                           cudaStream_t st)
 {
     const long long nb = (long long)nbx * nby;
-    cudaError_t e = cudaMemsetAsync(acc, 0, (size_t)nb * 3 * sizeof(unsigned long long), st);
-    if (e != cudaSuccess) return e;
     BinAxis ax, ay;
     ax.cs_unit = S.csx_d / (double)(1ll << S.sx);
     ax.f = (double)nbx / S.lx;
@@ -160,11 +187,15 @@ cudaError_t launch_coarse(const Sys &S, int b, int nbx, int nby, unsigned long l
     int dev = 0, nsm = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const int grid = std::max(1, std::min(S.ntiles, 8 * nsm));
-    k_coarse_tiles<256><<<grid, 256, 0, st>>>(S, b, ax, ay, acc);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const double inv_area = (double)nbx * nby / (S.lx * S.ly);
-    k_coarse_finish<<<(unsigned)std::min<long long>((nb + 255) / 256, 4096), 256, 0, st>>>(acc, nbx, nby, inv_area, out);
-    return cudaGetLastError();
+    // up to 2048 bins one block converts them in a few rounds; beyond, a
+    // second launch spreads them over the chip
+    const bool one = nb <= 2048;
+    cudaError_t e = launch_after(k_coarse_tiles<256>, grid, 256, 0, st, S, b, ax, ay, acc,
+                                 one ? reinterpret_cast<unsigned *>(acc + 3 * nb) : nullptr, inv_area, out);
+    if (e != cudaSuccess || one) return e;
+    return launch_after(k_coarse_finish, (unsigned)std::min<long long>((nb + 255) / 256, 4096), 256, 0, st, acc, nbx, nby,
+                        inv_area, out);
 }
 
 }  // namespace aapk

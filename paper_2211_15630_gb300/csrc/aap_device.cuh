@@ -11,6 +11,31 @@ namespace aapk {
 #define AAP_PI_F 3.14159265358979f
 #define AAP_2PI_F 6.28318530717959f
 
+// Programmatic dependent launch: a kernel launched with launch_after() may
+// start while the one before it in the stream drains; pdl_wait() returns once
+// that one is complete and its writes are visible (at once for an ordinary
+// launch), and pdl_next() lets the kernel after this one start.  Nothing but
+// the block's own shared memory is touched before pdl_wait().
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Launch k so that it may start while the kernel before it drains.
+template <class... P, class... A>
+inline cudaError_t launch_after(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute a[1];
+    a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = a;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, k, static_cast<P>(args)...);
+}
+
 // ---------------------------------------------------------------- Philox --
 // Philox4x32-10 (Salmon et al., SC'11): counter c, key (k0, k1).
 __device__ __forceinline__ void philox4x32_10(uint32_t c[4], uint32_t k0, uint32_t k1)

@@ -42,6 +42,8 @@ k_step(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_base,
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ TileCtx T;
+    pdl_next();
+    pdl_wait();
     const long long step = ctl->step;
     const int cur = (int)(step & 1);
     const int total = tile_base[nsys];
@@ -124,6 +126,8 @@ k_step(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_base,
 __global__ void k_finish(Sys *sys, int nsys, const int *__restrict__ tile_base, Ctl *ctl)
 {
     __shared__ int s_last;
+    pdl_next();
+    pdl_wait();
     const long long step = ctl->step;
     const int cur = (int)(step & 1);
     const long long gt = blockIdx.x * (long long)blockDim.x + threadIdx.x, gs = (long long)gridDim.x * blockDim.x;
@@ -137,12 +141,12 @@ __global__ void k_finish(Sys *sys, int nsys, const int *__restrict__ tile_base, 
         for (long long i = gt; i < n4; i += gs) c4[i] = make_int4(0, 0, 0, 0);
         for (long long i = gt; i < (nt + 31) / 32; i += gs) sb[i] = 0u;    // the tiles' spill marks
     } else {
-        const long long nw = (long long)tile_base[nsys] * kCntStride;
+        const long long nw = (long long)tile_base[nsys] * (kCntStride / 4);     // 16-byte words
         for (long long i = gt; i < nw; i += gs) {
-            const int g = (int)(i / kCntStride);
+            const int g = (int)(i / (kCntStride / 4)), w = (int)(i % (kCntStride / 4));
             const int si = sys_of_tile(tile_base, nsys, g);
-            const int t = g - tile_base[si], w = (int)(i % kCntStride);
-            sys[si].cnt[cur][(long long)t * kCntStride + w] = 0;
+            const int t = g - tile_base[si];
+            reinterpret_cast<int4 *>(sys[si].cnt[cur])[(long long)t * (kCntStride / 4) + w] = make_int4(0, 0, 0, 0);
             if (w == 0 && (t & 31) == 0) sys[si].spill_bits[cur][t >> 5] = 0u;    // the tiles' spill marks
         }
     }
@@ -169,10 +173,26 @@ __global__ void k_finish(Sys *sys, int nsys, const int *__restrict__ tile_base, 
 }
 
 // ------------------------------------------------- state in and out --------
+// llrint(p / cs * scale), scale a power of two, without the FP64 division (the
+// FP64 pipe is narrow on this GPU; two divisions a particle took most of the
+// insert: N = 2^24, 854 us).  p r, r = 1 / cs rounded, is within 2^-51 relative
+// of the rounded quotient, so the two round to the same integer unless p r
+// scale lies that close to a half-integer: then the division decides (for
+// fewer than one particle in a thousand, out of line).
+__device__ __noinline__ long long grid_round_div(double p, double cs, double scale) { return llrint(p / cs * scale); }
+
+__device__ __forceinline__ long long grid_round(double p, double cs, double r, double scale)
+{
+    const double v = p * r * scale;
+    const double i = rint(v);
+    if (!(fabs(v - i) < 0.5 - fabs(v) * 1e-15)) return grid_round_div(p, cs, scale);
+    return (long long)i;
+}
+
 // Place one particle given in box coordinates into buffer b (exact rounding
 // of the position to the fixed-point grid).  mode 0: from arrays; mode 1: draw
 // the uniform isotropic initial state from Philox, tag 1.
-__global__ void k_insert(Sys S, int b, const double *x, const double *y, const float *th, int mode)
+__global__ void k_insert(Sys S, int b, const double *x, const double *y, const float *th, int mode, double rx, double ry)
 {
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const bool act = i < S.n;
@@ -192,8 +212,8 @@ __global__ void k_insert(Sys S, int b, const double *x, const double *y, const f
             py = y[i];
             pt = th[i];
         }
-        long long gx = llrint(px / S.csx_d * (double)(1ll << S.sx));
-        long long gy = llrint(py / S.csy_d * (double)(1ll << S.sy));
+        long long gx = grid_round(px, S.csx_d, rx, (double)(1ll << S.sx));
+        long long gy = grid_round(py, S.csy_d, ry, (double)(1ll << S.sy));
         const long long wx = (long long)S.ncx << S.sx, wy = (long long)S.ncy << S.sy;
         if (gx >= wx) gx = S.bx ? wx - 1 : gx - wx;
         if (gx < 0) gx = S.bx ? 0 : gx + wx;
@@ -212,8 +232,6 @@ __global__ void k_insert(Sys S, int b, const double *x, const double *y, const f
     warp_insert(S, b, act, dtile, region, rec);
 }
 
-// Visit every stored record of buffer b: slots [0, tiles * tile_slots) then
-// the spill list.  Returns false for empty slots.
 // The lowest index whose position lies outside [0, lx] x [0, ly] (bad[0])
 // and whose orientation is not finite (bad[1]); both start at all ones.
 __global__ void k_validate_state(const double *x, const double *y, const float *th, long long n, double lx,
@@ -225,87 +243,160 @@ __global__ void k_validate_state(const double *x, const double *y, const float *
     }
 }
 
-__device__ __forceinline__ bool fetch_record(const Sys &S, int b, long long g, int4 &r, int &tile)
+// Warp `w` of `nw` visits its share of the stored records of buffer b (a warp
+// or several a tile, only the valid slots of its nine regions taken as one index
+// range; a flat system's single region in runs of 32 records), and of the
+// spill list: f(record, tile column, tile row), some lanes idle.  (A thread per
+// slot, empty ones included, with two divisions each to find its region, took
+// 1671 us to gather N = 2^24 at the start's four-fold capacity.)
+template <class F>
+__device__ __forceinline__ void warp_records(const Sys &S, int b, long long w, long long nw, F &&f)
 {
-    const long long nslot = (long long)S.ntiles * S.tile_slots;
-    if (g < nslot) {
-        tile = (int)(g / S.tile_slots);
-        const int o = (int)(g - (long long)tile * S.tile_slots);
-        int reg = 0;
+    const int lane = threadIdx.x & 31;
+    if (S.flat) {
+        const int n = min(S.cnt[b][0], S.cap[0]);
+        for (long long k = w * 32 + lane; k < n; k += nw * 32) f(S.rec[b][S.off[0] + k], 0, 0);
+    } else {
+        // several warps a tile while there are more warps than tiles
+        const int parts = (int)min(max(nw / max(S.ntiles, 1), 1ll), 32ll);
+        for (long long t = w; t < (long long)S.ntiles * parts; t += nw) {
+            const int tile = (int)(t / parts), part = (int)(t - (long long)tile * parts), ty = tile / S.ntx, tx = tile - ty * S.ntx;
+            const int c = lane < kRegions ? min(S.cnt[b][tile * kCntStride + lane], S.cap[lane]) : 0;
+            const int incl = warp_incl_scan(c);
+            const int total = __shfl_sync(0xffffffffu, incl, kRegions - 1);
+            int end[kRegions - 1];              // one past the last record of each region but the last
 #pragma unroll
-        for (int k = 1; k < kRegions; ++k)
-            if (o >= S.off[k]) reg = k;
-        const int slot = o - S.off[reg];
-        if (slot >= S.cap[reg]) return false;
-        if (slot >= S.cnt[b][tile * kCntStride + reg]) return false;
-        r = S.rec[b][g];
-        return true;
-    }
-    const long long e = g - nslot;
-    if (e >= min(S.spill_cnt[b], S.spill_cap)) return false;
-    r = S.spill_rec[b][e];
-    tile = S.spill_key[b][e] / kCntStride;
-    return true;
-}
-
-__global__ void k_gather(Sys S, int b, double *x, double *y, float *th, int *seen)
-{
-    const long long total = (long long)S.ntiles * S.tile_slots + S.spill_cap;
-    for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < total;
-         g += (long long)gridDim.x * blockDim.x) {
-        int4 r;
-        int tile;
-        if (!fetch_record(S, b, g, r, tile)) continue;
-        const int tx = tile % S.ntx, ty = tile / S.ntx;
-        const unsigned id = (unsigned)r.w;
-        if (id >= (unsigned long long)S.n) {
-            atomicOr(S.err, ERR_BOUNDS);
-            continue;
+            for (int r = 0; r < kRegions - 1; ++r) end[r] = __shfl_sync(0xffffffffu, incl, r);
+            // slot of record k: k plus the offset of its region past the records before it
+            const int shift = lane < kRegions ? S.off[lane] - (incl - c) : 0;
+            const int4 *base = S.rec[b] + (long long)tile * S.tile_slots;
+            for (int k0 = 32 * part; k0 < total; k0 += 32 * parts) {
+                const int k = k0 + lane;
+                int r = 0;
+#pragma unroll
+                for (int q = 0; q < kRegions - 1; ++q) r += k >= end[q];
+                const int at = k + __shfl_sync(0xffffffffu, shift, r);
+                if (k < total) f(base[at], tx, ty);
+            }
         }
-        const double gx = (double)((long long)tile_x0(S, tx) << S.sx) + (double)r.x;
-        const double gy = (double)((long long)tile_y0(S, ty) << S.sy) + (double)r.y;
-        x[id] = gx * (S.csx_d / (double)(1ll << S.sx));
-        y[id] = gy * (S.csy_d / (double)(1ll << S.sy));
-        th[id] = __int_as_float(r.z);
-        atomicAdd(seen, 1);
+    }
+    const int nsp = min(S.spill_cnt[b], S.spill_cap);
+    for (long long e = w * 32 + lane; e < nsp; e += nw * 32) {
+        const int tile = S.spill_key[b][e] / kCntStride;
+        f(S.spill_rec[b][e], tile % S.ntx, tile / S.ntx);
     }
 }
 
-// p and q of buffer b (Sec. 3.4), in exact 64-bit integer sums (order-free,
-// so the result is reproducible bit for bit), plus the number of records.
-__global__ void k_observe(Sys S, int b, unsigned long long *out)
-{
-    __shared__ long long red[5][32];
-    const long long total = (long long)S.ntiles * S.tile_slots + S.spill_cap;
-    long long a[5] = {0, 0, 0, 0, 0};
-    for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < total;
-         g += (long long)gridDim.x * blockDim.x) {
-        int4 r;
-        int tile;
-        if (!fetch_record(S, b, g, r, tile)) continue;
-        const float t = __int_as_float(r.z);
-        if (!isfinite(t)) atomicOr(S.err, ERR_NAN);
-        float s1, c1, s2, c2;
-        sincosf(t, &s1, &c1);
-        sincosf(2.0f * t, &s2, &c2);
-        a[0] += __float2ll_rn(c1 * 4294967296.0f);
-        a[1] += __float2ll_rn(s1 * 4294967296.0f);
-        a[2] += __float2ll_rn(c2 * 4294967296.0f);
-        a[3] += __float2ll_rn(s2 * 4294967296.0f);
-        a[4] += 1;
+// Position (FP64, exact) of a record in box coordinates.
+struct BoxMap {
+    double fx, fy, ux, uy;
+    __device__ __forceinline__ explicit BoxMap(const Sys &S)
+        : fx((double)(1ll << S.sx)), fy((double)(1ll << S.sy)), ux(S.csx_d / fx), uy(S.csy_d / fy)
+    {
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __device__ __forceinline__ double x(const Sys &S, int tx, int X) const
+    {
+        return ((double)tile_x0(S, tx) * fx + (double)X) * ux;          // the sum is exact
+    }
+    __device__ __forceinline__ double y(const Sys &S, int ty, int Y) const
+    {
+        return ((double)tile_y0(S, ty) * fy + (double)Y) * uy;
+    }
+};
+
+// The state by particle id.  BUCKET false: straight into x, y, th.  true: into
+// `mix`, one aligned 32-byte entry per particle, which k_split then spreads
+// over the arrays: scattered writes of whole sectors instead of three partial
+// ones per particle, for states that outgrow the L2.
+template <bool BUCKET>
+__global__ void k_gather(Sys S, int b, double *x, double *y, float *th, int4 *mix, int *seen)
+{
+    const BoxMap m(S);
+    int n = 0;
+    warp_records(S, b, (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5, (long long)gridDim.x * blockDim.x >> 5,
+                 [&](const int4 &r, int tx, int ty) {
+                     const unsigned id = (unsigned)r.w;
+                     if (id >= (unsigned long long)S.n) {
+                         atomicOr(S.err, ERR_BOUNDS);
+                         return;
+                     }
+                     const double px = m.x(S, tx, r.x), py = m.y(S, ty, r.y);
+                     if (BUCKET) {
+                         const long long u = __double_as_longlong(px), v = __double_as_longlong(py);
+                         int4 *o = mix + 2 * (size_t)id;
+                         o[0] = make_int4((int)u, (int)(u >> 32), (int)v, (int)(v >> 32));
+                         o[1] = make_int4(r.z, 0, 0, 0);
+                     } else {
+                         x[id] = px;
+                         y[id] = py;
+                         th[id] = __int_as_float(r.z);
+                     }
+                     ++n;
+                 });
+    n = __reduce_add_sync(0xffffffffu, n);
+    if ((threadIdx.x & 31) == 0 && n) atomicAdd(seen, n);
+}
+
+__global__ void k_split(const int4 *__restrict__ mix, long long n, double *x, double *y, float *th)
+{
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const int4 u = mix[2 * i];
+        const int t = mix[2 * i + 1].x;
+        x[i] = __hiloint2double(u.y, u.x);
+        y[i] = __hiloint2double(u.w, u.z);
+        th[i] = __int_as_float(t);
+    }
+}
+
+// p and q of buffer b (Sec. 3.4) of one or more systems, in exact 64-bit
+// integer sums (order-free, so the result is reproducible bit for bit), plus
+// the number of records: out[8 s + 0..4] of system s, which the blocks of grid
+// row s sum up.
+__device__ __forceinline__ void observe_system(const Sys &S, int b, unsigned long long *out)
+{
+    long long a[5] = {0, 0, 0, 0, 0};
+    warp_records(S, b, (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5, (long long)gridDim.x * blockDim.x >> 5,
+                 [&](const int4 &r, int, int) {
+                     const float t = __int_as_float(r.z);
+                     if (!isfinite(t)) atomicOr(S.err, ERR_NAN);
+                     float s1, c1, s2, c2;
+                     sincosf(t, &s1, &c1);
+                     sincosf(2.0f * t, &s2, &c2);
+                     a[0] += __float2ll_rn(c1 * 4294967296.0f);
+                     a[1] += __float2ll_rn(s1 * 4294967296.0f);
+                     a[2] += __float2ll_rn(c2 * 4294967296.0f);
+                     a[3] += __float2ll_rn(s2 * 4294967296.0f);
+                     a[4] += 1;
+                 });
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
         const long long v = warp_sum_ll(a[k]);
-        if (lane == 0) red[k][warp] = v;
+        if ((threadIdx.x & 31) == 0 && v) atomicAdd(out + k, (unsigned long long)v);
     }
-    __syncthreads();
-    if (threadIdx.x < 5) {
-        long long v = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[threadIdx.x][w];
-        atomicAdd(out + threadIdx.x, (unsigned long long)v);
-    }
+}
+
+__global__ void k_observe(Sys S, int b, unsigned long long *out) { observe_system(S, b, out); }
+
+__global__ void k_observe_all(const Sys *__restrict__ sys, int b, unsigned long long *out)
+{
+    observe_system(sys[blockIdx.y], b, out + 8 * (size_t)blockIdx.y);
+}
+
+// Start a measurement window at the current state of every system: its p and
+// q (from the observed sums) seed last[0..1], and the steps before `until` are
+// measured.
+__global__ void k_begin_measure(Sys *sys, int nsys, const unsigned long long *sums, long long until)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nsys) return;
+    const unsigned long long *o = sums + 8 * (size_t)i;
+    Sys &S = sys[i];
+    const double n = (double)S.n;
+    const double c1 = (double)(long long)o[0] / kFix, s1 = (double)(long long)o[1] / kFix;
+    const double c2 = (double)(long long)o[2] / kFix, s2 = (double)(long long)o[3] / kFix;
+    S.last[0] = n > 0 ? sqrt(c1 * c1 + s1 * s1) / n : 0.0;
+    S.last[1] = n > 0 ? sqrt(c2 * c2 + s2 * s2) / n : 0.0;
+    S.meas_until = until;
 }
 
 // --------------------------------------------------------------- launchers --
@@ -323,15 +414,12 @@ static cudaError_t launch_step_t(const LaunchCfg &L, cudaStream_t st, cudaEvent_
     if (L.pipe) {
         e = launch_step_pipe(L, st);
     } else {
-        k_step<NT, MODEL><<<L.grid_step, NT, smem, st>>>(L.sys, L.nsys, L.tile_base, L.ctl, L.stage_cap,
-                                                          L.nce_max, L.scratch, L.scratch_per_block,
-                                                          L.scratch_cap, L.spill_list_cap);
-        e = cudaGetLastError();
+        e = launch_after(k_step<NT, MODEL>, L.grid_step, NT, smem, st, L.sys, L.nsys, L.tile_base, L.ctl, L.stage_cap,
+                         L.nce_max, L.scratch, L.scratch_per_block, L.scratch_cap, L.spill_list_cap);
     }
     if (e != cudaSuccess) return e;
     if (ev && (e = cudaEventRecord(ev[1], st)) != cudaSuccess) return e;
-    k_finish<<<L.grid_finish, 256, 0, st>>>(L.sys, L.nsys, L.tile_base, L.ctl);
-    e = cudaGetLastError();
+    e = launch_after(k_finish, L.grid_finish, 256, 0, st, L.sys, L.nsys, L.tile_base, L.ctl);
     if (e != cudaSuccess) return e;
     if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
     return cudaSuccess;
@@ -353,8 +441,7 @@ cudaError_t launch_step(const LaunchCfg &L, cudaStream_t st, cudaEvent_t *ev)
     if (L.knn > 0) {
         cudaError_t e = launch_mf_step(L, st, ev);
         if (e != cudaSuccess) return e;
-        k_finish<<<L.grid_finish, 256, 0, st>>>(L.sys, L.nsys, L.tile_base, L.ctl);
-        e = cudaGetLastError();
+        e = launch_after(k_finish, L.grid_finish, 256, 0, st, L.sys, L.nsys, L.tile_base, L.ctl);
         if (e != cudaSuccess) return e;
         if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
         return cudaSuccess;
@@ -404,7 +491,7 @@ cudaError_t launch_insert(const Sys &S, int b, const double *x, const double *y,
     if (n == 0) return cudaSuccess;
     const int bs = 256;
     const long long grid = (n + bs - 1) / bs;
-    k_insert<<<(unsigned)grid, bs, 0, st>>>(S, b, x, y, th, mode);
+    k_insert<<<(unsigned)grid, bs, 0, st>>>(S, b, x, y, th, mode, 1.0 / S.csx_d, 1.0 / S.csy_d);
     return cudaGetLastError();
 }
 
@@ -417,16 +504,44 @@ cudaError_t launch_validate(const double *x, const double *y, const float *th, l
     return cudaGetLastError();
 }
 
+// Blocks of 256 threads that walk the records of n particles (at most eight per SM).
+static unsigned record_blocks(long long n) { return (unsigned)std::max<long long>(1, std::min<long long>((n + 1023) / 1024, 1216)); }
+
 cudaError_t launch_gather(const Sys &S, int b, double *x, double *y, float *th, int *seen,
                           cudaStream_t st)
 {
-    k_gather<<<1024, 256, 0, st>>>(S, b, x, y, th, seen);
+    // the region buffer of the other parity holds nothing between steps: room
+    // for the 32-byte entries when the regions have at least two slots a
+    // particle.  Below 2^21 particles (40 MB of arrays) the L2 collects the
+    // partial writes itself.  N = 2^24, one pass: 1313 us of a get_state.
+    const size_t room = (size_t)S.ntiles * S.tile_slots * sizeof(int4);
+    if (S.n >= (1ll << 21) && room >= (size_t)S.n * 32) {
+        int4 *mix = S.rec[b ^ 1];
+        k_gather<true><<<record_blocks(S.n), 256, 0, st>>>(S, b, nullptr, nullptr, nullptr, mix, seen);
+        k_split<<<1216, 256, 0, st>>>(mix, S.n, x, y, th);
+    } else {
+        k_gather<false><<<record_blocks(S.n), 256, 0, st>>>(S, b, x, y, th, nullptr, seen);
+    }
     return cudaGetLastError();
 }
 
 cudaError_t launch_observe(const Sys &S, int b, unsigned long long *out, cudaStream_t st)
 {
-    k_observe<<<1024, 256, 0, st>>>(S, b, out);
+    k_observe<<<record_blocks(S.n), 256, 0, st>>>(S, b, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_begin_measure(Sys *sys, int nsys, long long max_n, int b, unsigned long long *sums, long long until,
+                                 cudaStream_t st)
+{
+    cudaError_t e = cudaMemsetAsync(sums, 0, 8 * sizeof(unsigned long long) * (size_t)nsys, st);
+    if (e != cudaSuccess) return e;
+    for (int s0 = 0; s0 < nsys; s0 += 65535) {
+        const int n = std::min(nsys - s0, 65535);
+        const dim3 grid(std::min(record_blocks(max_n), 256u), (unsigned)n);
+        k_observe_all<<<grid, 256, 0, st>>>(sys + s0, b, sums + 8 * (size_t)s0);
+    }
+    k_begin_measure<<<(unsigned)((nsys + 63) / 64), 64, 0, st>>>(sys, nsys, sums, until);
     return cudaGetLastError();
 }
 

@@ -84,8 +84,11 @@ cudaError_t launch_validate(const double *x, const double *y, const float *th, l
 cudaError_t launch_gather(const Sys &S, int b, double *x, double *y, float *th, int *seen,
                           cudaStream_t st);
 cudaError_t launch_observe(const Sys &S, int b, unsigned long long *out, cudaStream_t st);
+// Start a measurement window of `nsys` systems (device array) at their current states in buffer b.
+cudaError_t launch_begin_measure(Sys *sys, int nsys, long long max_n, int b, unsigned long long *sums, long long until,
+                                 cudaStream_t st);
 // Coarse-grained fields of buffer b into out[3][nby][nbx] (device), using
-// acc[3 * nbx * nby] (device scratch) for the integer sums.
+// acc[3 * nbx * nby + 1] (device scratch, zero before and after) for the integer sums and a block count.
 cudaError_t launch_coarse(const Sys &S, int b, int nbx, int nby, unsigned long long *acc, float *out,
                           cudaStream_t st);
 

@@ -590,6 +590,8 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
     }
     for (int i = tid; i < nceh_max; i += kPipeThreads) B.hist[i] = 0;
     for (int i = tid; i < 2 * B.mh_stride; i += kPipeThreads) B.mhist0[i] = 0;
+    pdl_next();
+    pdl_wait();         // the step before is closed
     // pipeline waits that run out are reported in the first system's error word
     int *const err0 = sys[0].err;
     if (tid == 0) sh.flag = *((volatile int *)err0) & ERR_TIMEOUT;
@@ -809,11 +811,11 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
                 break;
             }
             t0 = PT_NOW();
-            // the buffer's histograms go to the system of its previous tile (when
-            // measuring); the buffer takes this tile's system
+            // the buffer takes this tile's system; the counts of the one before
+            // go to it (when measuring; tiles of one system share the counts)
             const int si = sh.raw[r].si;
             const int oi = sh.osys[b];
-            if (oi >= 0 && step < sh.os[b].meas_until) {
+            if (oi >= 0 && oi != si && step < sh.os[b].meas_until) {
                 flush_hist(sh, B, b, step, st, NS);
                 sort_sync(NS);
             }
@@ -1050,10 +1052,9 @@ template <int MODEL>
 static cudaError_t launch_pipe_t(const LaunchCfg &L, cudaStream_t st)
 {
     const size_t smem = pipe_smem_bytes(L.pipe_cap, L.pipe_cap_own, L.pipe_nceh, L.hist_words);
-    k_step_pipe<MODEL, AAP_PIPE_SORT_WARPS><<<L.pipe_grid, kPipeThreads, smem, st>>>(
-        L.sys, L.nsys, L.tile_base, L.ctl, L.pipe_cap, L.pipe_cap_own, L.pipe_nceh, L.nce_max, L.hist_words,
-        L.dense_list, L.scratch, L.scratch_per_block, L.scratch_cap, L.spill_list_cap);
-    return cudaGetLastError();
+    return launch_after(k_step_pipe<MODEL, AAP_PIPE_SORT_WARPS>, L.pipe_grid, kPipeThreads, smem, st, L.sys, L.nsys,
+                        L.tile_base, L.ctl, L.pipe_cap, L.pipe_cap_own, L.pipe_nceh, L.nce_max, L.hist_words,
+                        L.dense_list, L.scratch, L.scratch_per_block, L.scratch_cap, L.spill_list_cap);
 }
 
 cudaError_t launch_step_pipe(const LaunchCfg &L, cudaStream_t st)

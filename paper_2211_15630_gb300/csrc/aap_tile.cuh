@@ -38,10 +38,12 @@ __device__ __forceinline__ int tile_x0(const Sys &S, int tx) { return S.x0tab[tx
 __device__ __forceinline__ int tile_y0(const Sys &S, int ty) { return S.y0tab[ty]; }
 __device__ __forceinline__ int tile_of_x(const Sys &S, int cx)
 {
+    if (S.ncx < 32768) return (int)(((unsigned)(cx + 1) * (unsigned)S.ntx - 1u) / (unsigned)S.ncx);   // ntx <= ncx
     return (int)((((long long)cx + 1) * S.ntx - 1) / S.ncx);
 }
 __device__ __forceinline__ int tile_of_y(const Sys &S, int cy)
 {
+    if (S.ncy < 32768) return (int)(((unsigned)(cy + 1) * (unsigned)S.nty - 1u) / (unsigned)S.ncy);
     return (int)((((long long)cy + 1) * S.nty - 1) / S.ncy);
 }
 __device__ __forceinline__ int region_of(int lx, int ly, int tw, int th)
@@ -958,12 +960,21 @@ __device__ __forceinline__ void close_sums(const Sys &S, long long step, int lan
     static_assert(kAccSlots == 64, "two accumulator slots per lane");
     const int cur = (int)(step & 1);
     unsigned long long *a = S.acc + (size_t)cur * kAccSlots * kAccWords;
+    // everything read up front: loads that stand behind a store wait for it in
+    // turn (the 13 measurement sums one after another took most of this)
+    double *const last = S.last, *const stats = S.stats, *const trace = S.trace, *const trace_nbar = S.trace_nbar;
+    const bool measure = step < S.meas_until;
+    const long long i1 = step + 1 - S.trace_base, cap = trace ? S.trace_cap : 0;
+    const double n = (double)S.n;
+    const double p0 = last[0], q0 = last[1];
+    double st = measure && lane < 13 ? stats[lane] : 0.0;      // lane k: sum k
     unsigned long long x0[5], x1[5];
 #pragma unroll
     for (int w = 0; w < 5; ++w) {
         x0[w] = __ldcg(a + lane * kAccWords + w);
         x1[w] = __ldcg(a + (lane + 32) * kAccWords + w);
     }
+    __syncwarp();
 #pragma unroll
     for (int w = 0; w < 5; ++w) {
         a[lane * kAccWords + w] = 0;
@@ -971,38 +982,30 @@ __device__ __forceinline__ void close_sums(const Sys &S, long long step, int lan
     }
     long long v[5];
 #pragma unroll
-    for (int w = 0; w < 5; ++w) v[w] = warp_sum_ll((long long)(x0[w] + x1[w]));   // exact, lane 0 holds it
-    if (lane != 0) return;
-    const double n = (double)S.n;
+    for (int w = 0; w < 5; ++w) v[w] = __shfl_sync(0xffffffffu, warp_sum_ll((long long)(x0[w] + x1[w])), 0);   // exact
     const double dc = (double)v[0] / kFixStep, ds = (double)v[1] / kFixStep;
     const double dc2 = (double)v[3] / kFixStep, ds2 = (double)v[4] / kFixStep;
     const double phi = n > 0 ? sqrt(dc * dc + ds * ds) / n : 0.0;
     const double q = n > 0 ? sqrt(dc2 * dc2 + ds2 * ds2) / n : 0.0;
     const double nbar = n > 0 ? (double)v[2] / n : 0.0;
-    if (S.trace) {
-        const long long i1 = step + 1 - S.trace_base, i0 = step - S.trace_base;
-        if (i1 >= 0 && i1 < S.trace_cap) S.trace[i1] = phi;
-        if (i0 >= 0 && i0 < S.trace_cap) S.trace_nbar[i0] = nbar;
+    if (measure) {
+        // on-the-fly measurement (Sec. 3.4): state t contributes the powers of
+        // p(t), q(t) and of the mean neighbour number measured on it
+        const double b = lane < 4 ? p0 : (lane < 8 ? q0 : nbar);
+        double pk = b;
+        for (int k = 0; k < (lane & 3); ++k) pk *= b;
+        st += lane == 12 ? 1.0 : pk;
+        if (lane < 13) stats[lane] = st;
     }
-    if (step < S.meas_until) {
-        // on-the-fly measurement (Sec. 3.4): state t contributes p(t),
-        // q(t) and the mean neighbour number measured on it
-        const double p0 = S.last[0], q0 = S.last[1];
-        double pk = 1.0, qk = 1.0, nk = 1.0;
-        for (int k = 0; k < 4; ++k) {
-            pk *= p0;
-            qk *= q0;
-            nk *= nbar;
-            S.stats[k] += pk;
-            S.stats[4 + k] += qk;
-            S.stats[8 + k] += nk;
-        }
-        S.stats[12] += 1.0;
+    __syncwarp();
+    if (lane == 0) {
+        if (i1 >= 0 && i1 < cap) trace[i1] = phi;
+        if (i1 >= 1 && i1 <= cap) trace_nbar[i1 - 1] = nbar;
+        last[0] = phi;
+        last[1] = q;
+        last[2] = nbar;
+        last[3] = (double)(step + 1);
     }
-    S.last[0] = phi;
-    S.last[1] = q;
-    S.last[2] = nbar;
-    S.last[3] = (double)(step + 1);
 }
 
 }  // namespace aapk
