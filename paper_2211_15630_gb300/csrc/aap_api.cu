@@ -314,13 +314,13 @@ int set_capacity_mf(aap_handle *h)
 // Shared buffers of the pipelined step: the largest staging capacity (a
 // multiple of 64, at most kPipeMaxStage) whose two raw and two sorted buffers,
 // with own lists sized for 7/8 of it, fit the block's shared memory.
-int set_pipe_launch(LaunchCfg &L, int twmax, int thmax, int total_tiles)
+int set_pipe_launch(LaunchCfg &L, bool species, int twmax, int thmax, int total_tiles)
 {
     int dev = 0, optin = 0;
     AAP_CK(cudaGetDevice(&dev));
     AAP_CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     size_t stat = 0;
-    AAP_CK(aapk::pipe_static_smem(L.model, &stat));
+    AAP_CK(species ? aapk::pipe_static_smem_species(L.model, &stat) : aapk::pipe_static_smem(L.model, &stat));
     int cap = aapk::kPipeMaxStage;
     auto own_of = [](int c) { return aapk::round_up(c * 7 / 8, 64); };
     L.pipe_nceh = (2 * twmax + 4) * (thmax + 2);
@@ -334,14 +334,15 @@ int set_pipe_launch(LaunchCfg &L, int twmax, int thmax, int total_tiles)
     L.pipe_cap = cap;
     L.pipe_cap_own = own_of(cap);
     L.pipe_grid = std::max(1, std::min(total_tiles, sm_count()));
-    AAP_CK(aapk::configure_pipe_kernel(L.model, aapk::pipe_smem_bytes(L.pipe_cap, L.pipe_cap_own, L.pipe_nceh,
-                                                                      L.hist_words)));
+    const size_t smem = aapk::pipe_smem_bytes(L.pipe_cap, L.pipe_cap_own, L.pipe_nceh, L.hist_words);
+    AAP_CK(species ? aapk::configure_pipe_kernel_species(L.model, smem) : aapk::configure_pipe_kernel(L.model, smem));
+    L.pipe_species = species ? 1 : 0;
     L.pipe = 1;
     L.threads = 1024;
     return AAP_OK;
 }
 
-int set_pipe(aap_handle *h) { return set_pipe_launch(h->L, h->hs.twmax, h->hs.thmax, h->hs.ntiles); }
+int set_pipe(aap_handle *h) { return set_pipe_launch(h->L, h->p.nspecies > 1, h->hs.twmax, h->hs.thmax, h->hs.ntiles); }
 
 int set_capacity(aap_handle *h, double factor)
 {
@@ -380,10 +381,9 @@ int set_capacity(aap_handle *h, double factor)
     L.scratch_per_block = aapk::stage_bytes(L.scratch_cap) + aapk::spill_list_bytes(L.spill_list_cap);
     L.scratch_per_block = (L.scratch_per_block + 255) / 256 * 256;
     L.nsys = 1;
-    // the pipelined step: one system, one species (ensemble members use the
-    // whole-block kernel, which batches systems)
+    // the pipelined step (an ensemble sets up one launch for its members)
     L.pipe = 0;
-    if (!h->member && p.nspecies <= 1 && (p.threads == 0 || p.threads == 1024)) {
+    if (!h->member && (p.threads == 0 || p.threads == 1024)) {
         int rc = set_pipe(h);
         if (rc) return rc;
         if (!L.pipe && p.threads == 1024) return fail(AAP_EINVAL, "the pipelined step kernel does not fit this tiling");
@@ -392,13 +392,8 @@ int set_capacity(aap_handle *h, double factor)
     L.multi = 0;
     if (!h->member && p.threads == 0) {
         L.pipe_nceh = (2 * S.twmax + 4) * (S.thmax + 2);
-        AAP_CK(aapk::configure_multi(L, p.nspecies, S.ntiles, nsm, scap));
-        if (L.multi) {
-            // a scratch slice for every block, with room for the weighted records
-            L.grid_step = std::max(L.grid_step, S.ntiles);
-            L.scratch_per_block += (size_t)L.multi_wsp * 8 * L.scratch_cap;
-            L.scratch_per_block = (L.scratch_per_block + 255) / 256 * 256;
-        }
+        AAP_CK(aapk::configure_multi(L, p.nspecies > 1, S.ntiles, nsm, scap));
+        if (L.multi) L.grid_step = std::max(L.grid_step, S.ntiles);     // a scratch slice for every block
     }
     return AAP_OK;
 }
@@ -434,6 +429,10 @@ void set_model(Sys &S, const aap_params &p)
         for (int b = 0; b < aapk::kMaxSpecies; ++b)
             S.sp_gamma_dt[a * aapk::kMaxSpecies + b] = (float)((multi ? p.species_gamma[8 * a + b] : p.gamma) * p.dt);
     }
+    float gmax = 0.f;
+    for (int a = 0; a < S.nsp; ++a)
+        for (int b = 0; b < S.nsp; ++b) gmax = std::max(gmax, std::fabs(S.sp_gamma_dt[a * aapk::kMaxSpecies + b]));
+    S.small_gamma = gmax < 1.0f;
     if (!multi) {
         S.sp_eta_pi[0] = S.eta_pi;
         S.sp_omega_step[0] = S.omega_step;
@@ -1211,7 +1210,7 @@ int ens_combine(aap_ens *e)
         }
         AAP_CK(cudaMemset(e->d_dense, 0, (size_t)total * sizeof(int)));
         L.dense_list = e->d_dense;
-        int rc = set_pipe_launch(L, twmax, thmax, (int)total);
+        int rc = set_pipe_launch(L, false, twmax, thmax, (int)total);
         if (rc) return rc;
         if (!L.pipe && e->params[0].threads == 1024)
             return fail(AAP_EINVAL, "the pipelined step kernel does not fit this ensemble's tiling");
@@ -1359,6 +1358,7 @@ int aap_test_pipe_wait(int64_t wait_cycles, int32_t stall)
 {
     if (stall != 0 && stall != 1) return fail(AAP_EINVAL, "stall must be 0 or 1");
     AAP_CK(aapk::set_pipe_test(wait_cycles, stall));
+    AAP_CK(aapk::set_pipe_test_species(wait_cycles, stall));
     AAP_CK(aapk::set_multi_test(wait_cycles, stall));
     return AAP_OK;
 }

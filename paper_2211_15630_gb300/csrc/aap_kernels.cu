@@ -412,7 +412,7 @@ static cudaError_t launch_step_t(const LaunchCfg &L, cudaStream_t st, cudaEvent_
     cudaError_t e;
     if (ev && (e = cudaEventRecord(ev[0], st)) != cudaSuccess) return e;
     if (L.pipe) {
-        e = launch_step_pipe(L, st);
+        e = L.pipe_species ? launch_step_pipe_species(L, st) : launch_step_pipe(L, st);
     } else {
         e = launch_after(k_step<NT, MODEL>, L.grid_step, NT, smem, st, L.sys, L.nsys, L.tile_base, L.ctl, L.stage_cap,
                          L.nce_max, L.scratch, L.scratch_per_block, L.scratch_cap, L.spill_list_cap);

@@ -24,15 +24,15 @@ struct LaunchCfg {
     int nce_max;                 // cells of the largest tile plus its ring
     int hist_words;              // histogram bins (theta + |Omega|) of the widest system
     int grid_step, grid_finish;
-    // pipelined step (one system, one species): shared buffers of pipe_cap
+    // pipelined step (pipe_species: systems of several species): shared buffers of pipe_cap
     // staged / pipe_cap_own own particles per tile, one block per SM; tiles
     // that do not fit go to dense_list (device [ntiles], zero between steps)
-    int pipe;
+    int pipe, pipe_species;
     int pipe_cap, pipe_cap_own, pipe_grid;
     int pipe_nceh;               // half cells (split along x) of the largest extended tile, (2 tw + 4)(th + 2)
     int *dense_list;
     // many steps per launch (a small system, one block per tile, all resident)
-    int multi, multi_species, multi_cap, multi_tiles, multi_threads, multi_wsp;
+    int multi, multi_species, multi_cap, multi_tiles, multi_threads;
     int *multi_cnt;              // device: three private counter sets and two barrier words, zero between launches
     // metric-free step (knn > 0): cell count, scan, scatter, k-nearest update
     int knn;
@@ -45,14 +45,33 @@ size_t step_smem_bytes(int stage_cap, int nce_max, int hist_words);
 // of its blocks fit on one SM.
 cudaError_t configure_step_kernel(int model, int threads, size_t smem_bytes, int *blocks_per_sm);
 
-// Dynamic shared memory of the pipelined step kernel.
-__host__ __device__ size_t pipe_smem_bytes(int cap, int cap_own, int nceh, int hist_words);
-// Static shared memory of the pipelined step kernel of a model.
+// Raw buffers of the pipelined step kernel: a tile's holds its staged records
+// from the copy until its update is done (the update reads its own particles'
+// records there).
+#ifndef AAP_PIPE_RAW_BUFFERS
+#define AAP_PIPE_RAW_BUFFERS 3
+#endif
+constexpr int kPipeRawBuffers = AAP_PIPE_RAW_BUFFERS;
+
+// Dynamic shared memory of the pipelined step kernel; nceh: half cells of the
+// largest extended tile, (2 tw + 4)(th + 2).
+__host__ __device__ inline size_t pipe_smem_bytes(int cap, int cap_own, int nceh, int hist_words)
+{
+    return (size_t)(kPipeRawBuffers + 2) * cap * 16 + 2 * (size_t)round_up(nceh + 1, 8) * 2 +
+           4 * (size_t)round_up(cap_own, 8) * 2 + 2 * (size_t)round_up(2 * cap, 8) * 2 +
+           (size_t)round_up(nceh, 4) * 4 + (size_t)(kMaxTile + 4) * 4 + 2 * (size_t)round_up(hist_words, 4) * 4;
+}
+// Static shared memory of the pipelined step kernel of a model; its dynamic
+// limit; the test hook of its waits (the wait bound, <= 0: default, and the
+// stall injection).  The _species functions are those of the kernel for
+// several species.
 cudaError_t pipe_static_smem(int model, size_t *bytes);
-// Set the dynamic shared-memory limit of the pipelined step kernel.
 cudaError_t configure_pipe_kernel(int model, size_t smem);
-// test hook: the wait bound of the pipelined kernel (<= 0: default) and the stall injection
 cudaError_t set_pipe_test(long long wait_cycles, int stall);
+cudaError_t pipe_static_smem_species(int model, size_t *bytes);
+cudaError_t configure_pipe_kernel_species(int model, size_t smem);
+cudaError_t set_pipe_test_species(long long wait_cycles, int stall);
+cudaError_t launch_step_pipe_species(const LaunchCfg &L, cudaStream_t st);
 // The pipelined step kernel alone (launch_step adds k_finish).
 cudaError_t launch_step_pipe(const LaunchCfg &L, cudaStream_t st);
 
@@ -61,7 +80,7 @@ inline int multi_stride(int ntiles) { return (ntiles + 1) * kCntStride; }
 inline size_t multi_bytes(int ntiles) { return (3 * (size_t)multi_stride(ntiles) + 4) * sizeof(int); }
 // Decide whether a system of ntiles tiles can run many steps per launch (L.multi): all its blocks resident with at
 // least min_cap staged records each.
-cudaError_t configure_multi(LaunchCfg &L, int nspecies, int ntiles, int sm_count, int min_cap);
+cudaError_t configure_multi(LaunchCfg &L, bool species, int ntiles, int sm_count, int min_cap);
 cudaError_t launch_multi(const LaunchCfg &L, int nsteps, cudaStream_t st);
 cudaError_t set_multi_test(long long wait_cycles, int stall);
 

@@ -69,25 +69,18 @@ struct MultiStage {
     float4 *P;                  // records in half-cell order
     int4 *R;                    // staged records, mapped into the extended frame
     unsigned short *cellw, *slotw, *oq, *orr;
-    int2 *W;                    // [species][cap] weighted (cos, sin) of the staged records (Langevin couplings)
-    int cap;
 };
 
-// Where a step's new records and neighbour weights are found.
+// The counters of a step's new records.
 struct ToStep {
     int *c, *s;
-    const int2 *W;
-    int cap;
     __device__ __forceinline__ int *cnt(const Sys &, int) const { return c; }
     __device__ __forceinline__ int *spill(const Sys &, int) const { return s; }
-    __device__ __forceinline__ const int2 *weighted(int sp) const { return W + sp * cap; }
 };
 
-__device__ __forceinline__ MultiStage carve_multi(unsigned char *p, unsigned char *w, int cap)
+__device__ __forceinline__ MultiStage carve_multi(unsigned char *p, int cap)
 {
     MultiStage A;
-    A.cap = cap;
-    A.W = (int2 *)w;
     A.P = (float4 *)p;
     p += (size_t)cap * 16;
     A.R = (int4 *)p;
@@ -242,22 +235,9 @@ __device__ __forceinline__ bool multi_tile(MultiShared &sh, const MultiStage &A,
             if (MODEL != 1 || (S.order & 1)) cs = -cs; else sn = -sn;
         }
         if (flip & 2) sn = -sn;
-        int ci = __float2int_rn(cs * kFixNbF);
-        const int si = __float2int_rn(sn * kFixNbF);
-        if (SP && MODEL == 1) {
-            // the couplings: weighted and rounded once per record and species
-            // pair, or (couplings of any size) the species packed in the cosine
-            const int sp = species_of(S, (unsigned)rk.w);
-            if (sh.O.small_gamma) {
-                for (int a = 0; a < S.nsp; ++a) {
-                    const float g = S.sp_gamma_dt[a * kMaxSpecies + sp];
-                    A.W[a * A.cap + q] = make_int2(__float2int_rn(g * (float)ci), __float2int_rn(g * (float)si));
-                }
-            } else {
-                ci = pack_species(ci, sp);
-            }
-        }
-        A.P[q] = make_float4((float)(rk.x - xc) * S.ux, (float)(rk.y - yc) * S.uy, __int_as_float(ci), __int_as_float(si));
+        float zc, zs;
+        stage_angle<MODEL, SP>(S, rk.w, __float2int_rn(cs * kFixNbF), __float2int_rn(sn * kFixNbF), zc, zs);
+        A.P[q] = make_float4((float)(rk.x - xc) * S.ux, (float)(rk.y - yc) * S.uy, zc, zs);
         if (ex >= 2 && ex < 2 * tw + 2 && ey >= 1 && ey <= th) {
             const int o = q + tb.rowoff[ey];
             A.oq[o] = (unsigned short)q;
@@ -269,7 +249,7 @@ __device__ __forceinline__ bool multi_tile(MultiShared &sh, const MultiStage &A,
     // a tile of few particles gives each of them two or four lanes: its warps
     // are otherwise idle, and the candidate rows are the longest chain
     const bool measure = step < S.meas_until;
-    const ToStep to = {wc, ws, A.W, A.cap};
+    const ToStep to = {wc, ws};
     const auto run = [&](auto lpp) {
         constexpr int LPP = decltype(lpp)::value;
         for (int o0 = warp * (32 / LPP); o0 < n_own; o0 += NT / LPP)
@@ -304,7 +284,6 @@ k_multi(Sys *__restrict__ sys, Ctl *ctl, int nsteps, int cap, int nceh, int hist
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tile = blockIdx.x, nblk = gridDim.x;
     MultiTables tb;
-    unsigned char *w0;
     {
         unsigned char *p = smem + (size_t)cap * 40;
         tb.hist = (int *)p;
@@ -314,9 +293,8 @@ k_multi(Sys *__restrict__ sys, Ctl *ctl, int nsteps, int cap, int nceh, int hist
         tb.mhist = (int *)p;
         p += (size_t)round_up(hist_words, 4) * 4;
         tb.cst = (unsigned short *)p;
-        w0 = p + (size_t)round_up(nceh + 1, 8) * 2;
     }
-    const MultiStage As = carve_multi(smem, w0, cap);
+    const MultiStage As = carve_multi(smem, cap);
     {
         const int words = (int)(sizeof(Sys) / 4);
         const int *src = reinterpret_cast<const int *>(sys);
@@ -351,10 +329,6 @@ k_multi(Sys *__restrict__ sys, Ctl *ctl, int nsteps, int cap, int nceh, int hist
             O.rbuf = O.rwide = 0;
             O.tx = G.tx; O.ty = G.ty; O.tw = G.tw; O.th = G.th; O.W2 = 2 * G.tw + 4;
             O.twL = G.twL; O.twR = G.twR; O.thD = G.thD; O.thU = G.thU;
-            float g = 0.f;
-            for (int a = 0; a < S.nsp; ++a)
-                for (int b = 0; b < S.nsp; ++b) g = fmaxf(g, fabsf(S.sp_gamma_dt[a * kMaxSpecies + b]));
-            O.small_gamma = SP && g < 1.0f;
         }
     }
     __syncthreads();
@@ -406,7 +380,6 @@ k_multi(Sys *__restrict__ sys, Ctl *ctl, int nsteps, int cap, int nceh, int hist
             unsigned char *const mine = scratch + scratch_per_block * blockIdx.x;
             int *const spill_e = (int *)(mine + stage_bytes(scratch_cap));
             unsigned char *const spill_s = (unsigned char *)(spill_e + spill_list_cap);
-            unsigned char *const spill_s_end = mine + stage_bytes(scratch_cap) + spill_list_bytes(spill_list_cap);
             if (nsp > 0) {
                 // records parked in the spill list for one of the segments
                 __syncthreads();
@@ -430,7 +403,7 @@ k_multi(Sys *__restrict__ sys, Ctl *ctl, int nsteps, int cap, int nceh, int hist
             if (m <= cap)
                 any = multi_tile<NT, MODEL, SP>(sh, As, tb, m, m_seg, step, spill_e, spill_s, wc, ws, acc);
             else if (m <= scratch_cap)
-                any = multi_tile<NT, MODEL, SP>(sh, carve_multi(mine, spill_s_end, scratch_cap), tb, m, m_seg, step, spill_e, spill_s, wc, ws, acc);
+                any = multi_tile<NT, MODEL, SP>(sh, carve_multi(mine, scratch_cap), tb, m, m_seg, step, spill_e, spill_s, wc, ws, acc);
             else if (tid == 0)
                 atomicOr(S.err, ERR_STAGE | ERR_LOST);
             if (any) flush_acc<true>(acc, S.acc, cur);
@@ -463,9 +436,9 @@ k_multi(Sys *__restrict__ sys, Ctl *ctl, int nsteps, int cap, int nceh, int hist
     }
 }
 
-size_t multi_smem(int cap, int nceh, int hist_words, int wsp)
+size_t multi_smem(int cap, int nceh, int hist_words)
 {
-    return (size_t)cap * (40 + 8 * wsp) + (size_t)round_up(nceh, 4) * 4 + (size_t)(kMaxTile + 4) * 4 +
+    return (size_t)cap * 40 + (size_t)round_up(nceh, 4) * 4 + (size_t)(kMaxTile + 4) * 4 +
            (size_t)round_up(hist_words, 4) * 4 + (size_t)round_up(nceh + 1, 8) * 2;
 }
 
@@ -496,10 +469,8 @@ cudaError_t set_multi_test(long long wait_cycles, int stall)
     return cudaMemcpyToSymbol(c_multi_stall, &stall, sizeof(stall));
 }
 
-cudaError_t configure_multi(LaunchCfg &L, int nspecies, int ntiles, int sm_count, int min_cap)
+cudaError_t configure_multi(LaunchCfg &L, bool species, int ntiles, int sm_count, int min_cap)
 {
-    const bool species = nspecies > 1;
-    const int wsp = species && L.model == 1 ? nspecies : 0;     // weighted copies of the staged records
     L.multi = 0;
     // One block of 512 threads (128 registers each) per SM.  Beyond that, with
     // up to four blocks of 256 threads per SM, light tiles still gain (N =
@@ -524,9 +495,9 @@ cudaError_t configure_multi(LaunchCfg &L, int nspecies, int ntiles, int sm_count
     const int bps = (blocks + sm_count - 1) / sm_count;
     const long long room = std::min<long long>(optin, per_sm / bps - 1024) - (long long)a.sharedSizeBytes;
     int cap = 4096;
-    while (cap >= min_cap && (long long)multi_smem(cap, L.pipe_nceh, L.hist_words, wsp) > room) cap -= 32;
+    while (cap >= min_cap && (long long)multi_smem(cap, L.pipe_nceh, L.hist_words) > room) cap -= 32;
     if (cap < min_cap) return cudaSuccess;
-    const int smem = (int)multi_smem(cap, L.pipe_nceh, L.hist_words, wsp);
+    const int smem = (int)multi_smem(cap, L.pipe_nceh, L.hist_words);
     // the limit belongs to the kernel, not to a handle: keep the largest any
     // handle of this process asked for
     static std::atomic<int> limit{0};
@@ -541,7 +512,6 @@ cudaError_t configure_multi(LaunchCfg &L, int nspecies, int ntiles, int sm_count
     L.multi = 1;
     L.multi_species = species ? 1 : 0;
     L.multi_cap = cap;
-    L.multi_wsp = wsp;
     L.multi_threads = threads;
     L.multi_tiles = ntiles;
     return cudaSuccess;
@@ -560,7 +530,7 @@ cudaError_t launch_multi(const LaunchCfg &L, int nsteps, cudaStream_t st)
     int scap = L.scratch_cap, slc = L.spill_list_cap;
     void *args[] = {&sys, &ctl, &nsteps, &cap, &nceh, &hw, &cnt3, &stride, &bar, &scratch, &spb, &scap, &slc};
     return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k), dim3(L.multi_tiles + 1), dim3(L.multi_threads), args,
-                                       multi_smem(cap, nceh, hw, L.multi_wsp), st);
+                                       multi_smem(cap, nceh, hw), st);
 }
 
 }  // namespace aapk

@@ -52,19 +52,29 @@
 #include "aap_kernels.cuh"
 #include "aap_tile.cuh"
 
+// The kernel is compiled twice, in two translation units: here for systems of
+// one species and, with AAP_PIPE_SPECIES set, in aap_pipe_species.cu for
+// several (per-particle speed, noise and chirality, coupled Langevin sums).
+#ifndef AAP_PIPE_SPECIES
+#define AAP_PIPE_SPECIES 0
+#endif
+#if AAP_PIPE_SPECIES
+#define PIPE_FN(name) name##_species
+#else
+#define PIPE_FN(name) name
+#endif
+
 namespace aapk {
 
 namespace {
 
+constexpr bool kSpecies = AAP_PIPE_SPECIES != 0;
 constexpr int kPipeThreads = 1024;
 constexpr int kPipeWarps = kPipeThreads / 32;
 constexpr int kPipeMaxChunks = 2 * kPipeMaxStage / 32 + 1;   // a wide tile spans two raw buffers
 // raw buffers: a tile's holds its staged records from the copy until its
 // update is done (the update reads its own particles' records there)
-#ifndef AAP_PIPE_RAW_BUFFERS
-#define AAP_PIPE_RAW_BUFFERS 3
-#endif
-constexpr int kNR = AAP_PIPE_RAW_BUFFERS;
+constexpr int kNR = kPipeRawBuffers;
 constexpr long long kPipeWaitCycles = 4000000000ll;    // about 2 s at 2 GHz
 
 // test hooks (aap_test_pipe_wait): the wait bound (<= 0: kPipeWaitCycles) and
@@ -82,7 +92,7 @@ __constant__ int c_pipe_stall;
 // 10 tiles through the pipeline, 11 whole-block tiles, 12 kernel per block,
 // 13 copy waiting for its next tile index, 14 copy planning, 15 copy spill
 // records and proxy fence.
-#ifdef AAP_PIPE_TIMING
+#if defined(AAP_PIPE_TIMING) && !AAP_PIPE_SPECIES
 __device__ unsigned long long g_pipe_t[16];
 #define PT_NOW() clock64()
 #define PT_ADD(i, v) atomicAdd(&g_pipe_t[i], (unsigned long long)(v))
@@ -421,7 +431,7 @@ __device__ __forceinline__ void sort_map(PipeShared &sh, const PipeBufs &B, int 
 // Scan the histogram into output buffer b's cell starts (clearing the
 // histogram), the own-row offsets and the tile's output meta, then place the
 // records in cell order.  The output buffer must be free.
-template <int MODEL>
+template <int MODEL, bool SP>
 __device__ __forceinline__ void sort_order(PipeShared &sh, const PipeBufs &B, int r, int b, int tid, int NS,
                                            int cap_own)
 {
@@ -520,8 +530,9 @@ __device__ __forceinline__ void sort_order(PipeShared &sh, const PipeBufs &B, in
             if (MODEL != 1 || (M.order & 1)) cs = -cs; else sn = -sn;
         }
         if (flip & 2) sn = -sn;
-        P[q] = make_float4((float)(rk.x - xc) * M.ux, (float)(rk.y - yc) * M.uy,
-                           __int_as_float(__float2int_rn(cs * kFixNbF)), __int_as_float(__float2int_rn(sn * kFixNbF)));
+        float zc, zs;
+        stage_angle<MODEL, SP>(sh.os[b], rk.w, __float2int_rn(cs * kFixNbF), __float2int_rn(sn * kFixNbF), zc, zs);
+        P[q] = make_float4((float)(rk.x - xc) * M.ux, (float)(rk.y - yc) * M.uy, zc, zs);
         if (ex >= 2 && ex < 2 * tw + 2 && ey >= 1 && ey <= th) {
             const int o = q + B.rowoff[ey];
             if (o < cap_own) {
@@ -533,14 +544,6 @@ __device__ __forceinline__ void sort_order(PipeShared &sh, const PipeBufs &B, in
 }
 
 }  // namespace
-
-// nceh: half cells of the largest extended tile, (2 tw + 4)(th + 2).
-__host__ __device__ size_t pipe_smem_bytes(int cap, int cap_own, int nceh, int hist_words)
-{
-    return (size_t)(kNR + 2) * cap * 16 + 2 * (size_t)round_up(nceh + 1, 8) * 2 +
-           4 * (size_t)round_up(cap_own, 8) * 2 + 2 * (size_t)round_up(2 * cap, 8) * 2 +
-           (size_t)round_up(nceh, 4) * 4 + (size_t)(kMaxTile + 4) * 4 + 2 * (size_t)round_up(hist_words, 4) * 4;
-}
 
 // Flush output buffer b's measured histograms into the system of the tile it
 // held, and clear them.  tid, nt: the calling threads.
@@ -561,7 +564,7 @@ __device__ __forceinline__ void flush_hist(PipeShared &sh, const PipeBufs &B, in
 // The pipelined step of one or more systems with one species each (any
 // model; the systems of one launch share it): one block of kPipeThreads
 // threads per SM.  tile_base[nsys + 1] is the prefix of the systems' tiles.
-template <int MODEL, int NSORT>
+template <int MODEL, bool SP, int NSORT>
 __global__ void __launch_bounds__(kPipeThreads, 1)
 k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_base, Ctl *ctl, int cap, int cap_own,
             int nceh_max, int nce_max, int hist_words, int *dense_list, unsigned char *scratch,
@@ -826,7 +829,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
                 for (int i = st; i < words; i += NS) dst[i] = src[i];
                 if (st == 0) sh.osys[b] = si;
             }
-            sort_order<MODEL>(sh, B, r, b, st, NS, wide ? 2 * cap_own : cap_own);
+            sort_order<MODEL, SP>(sh, B, r, b, st, NS, wide ? 2 * cap_own : cap_own);
             sort_sync(NS);
             if (st == 0) {
                 PT_ADD(6, PT_NOW() - t0);
@@ -891,7 +894,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
                 c = __shfl_sync(0xffffffffu, c, 0);
                 const int o0 = c * 32;
                 if (o0 >= O.n_own) break;
-                update_one<MODEL, false, 1>(S, O, P, cst, RB, OR, OQ, o0 + lane, step, measure, B.mhist(b), acc, ToSystem{});
+                update_one<MODEL, SP, 1>(S, O, P, cst, RB, OR, OQ, o0 + lane, step, measure, B.mhist(b), acc, ToSystem{});
             }
             __syncwarp();
             if (lane == 0) {
@@ -1002,12 +1005,12 @@ template <int MODEL>
 static cudaError_t static_pipe_t(size_t *bytes)
 {
     cudaFuncAttributes a;
-    const cudaError_t e = cudaFuncGetAttributes(&a, k_step_pipe<MODEL, AAP_PIPE_SORT_WARPS>);
+    const cudaError_t e = cudaFuncGetAttributes(&a, k_step_pipe<MODEL, kSpecies, AAP_PIPE_SORT_WARPS>);
     if (e == cudaSuccess) *bytes = a.sharedSizeBytes;
     return e;
 }
 
-cudaError_t pipe_static_smem(int model, size_t *bytes)
+cudaError_t PIPE_FN(pipe_static_smem)(int model, size_t *bytes)
 {
     switch (model) {
     case 0: return static_pipe_t<0>(bytes);
@@ -1027,18 +1030,18 @@ static cudaError_t config_pipe_t(size_t smem)
     int want = (int)smem, prev = limit.load();
     while (want > prev && !limit.compare_exchange_weak(prev, want)) {
     }
-    return cudaFuncSetAttribute(k_step_pipe<MODEL, AAP_PIPE_SORT_WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(k_step_pipe<MODEL, kSpecies, AAP_PIPE_SORT_WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 std::max(want, limit.load()));
 }
 
-cudaError_t set_pipe_test(long long wait_cycles, int stall)
+cudaError_t PIPE_FN(set_pipe_test)(long long wait_cycles, int stall)
 {
     cudaError_t e = cudaMemcpyToSymbol(c_pipe_wait_cycles, &wait_cycles, sizeof(wait_cycles));
     if (e != cudaSuccess) return e;
     return cudaMemcpyToSymbol(c_pipe_stall, &stall, sizeof(stall));
 }
 
-cudaError_t configure_pipe_kernel(int model, size_t smem)
+cudaError_t PIPE_FN(configure_pipe_kernel)(int model, size_t smem)
 {
     switch (model) {
     case 0: return config_pipe_t<0>(smem);
@@ -1052,12 +1055,12 @@ template <int MODEL>
 static cudaError_t launch_pipe_t(const LaunchCfg &L, cudaStream_t st)
 {
     const size_t smem = pipe_smem_bytes(L.pipe_cap, L.pipe_cap_own, L.pipe_nceh, L.hist_words);
-    return launch_after(k_step_pipe<MODEL, AAP_PIPE_SORT_WARPS>, L.pipe_grid, kPipeThreads, smem, st, L.sys, L.nsys,
+    return launch_after(k_step_pipe<MODEL, kSpecies, AAP_PIPE_SORT_WARPS>, L.pipe_grid, kPipeThreads, smem, st, L.sys, L.nsys,
                         L.tile_base, L.ctl, L.pipe_cap, L.pipe_cap_own, L.pipe_nceh, L.nce_max, L.hist_words,
                         L.dense_list, L.scratch, L.scratch_per_block, L.scratch_cap, L.spill_list_cap);
 }
 
-cudaError_t launch_step_pipe(const LaunchCfg &L, cudaStream_t st)
+cudaError_t PIPE_FN(launch_step_pipe)(const LaunchCfg &L, cudaStream_t st)
 {
     switch (L.model) {
     case 0: return launch_pipe_t<0>(L, st);

@@ -635,7 +635,6 @@ struct OutMeta {
     int n_own, tx, ty, tw, th, W2, twL, twR, thD, thU;   // W2: half cells per extended row, 2 tw + 4
     int wide;                   // a half cell holds enough particles for 512 candidates
     int dense;                  // more than 1.5 staged records per half cell on average
-    int small_gamma;            // several species: every |Gamma dt| is below 1
 };
 
 // ------------------------------------ the update of a half-cell-sorted tile --
@@ -677,13 +676,34 @@ __device__ __forceinline__ void neighbour_sum_h(const float4 *__restrict__ P, co
     }
 }
 
-// The Langevin sums with per-species couplings (neighbour_sum_sp above) over
-// the half cells, out of line for couplings of any size: a neighbour's species
-// rides in the upper bits of its staged cosine (pack_species).
-constexpr int kSpeciesShift = 26;           // |cos| 2^22 needs 24 bits with its sign
-__device__ __forceinline__ int pack_species(int c, int sp) { return (c & 0x03ffffff) | (sp << kSpeciesShift); }
-__device__ __forceinline__ int packed_cos(int z) { return (z << 6) >> 6; }
+constexpr float kMagicF = 12582912.0f;              // 1.5 2^23
+constexpr unsigned kMagicBits = 0x4B400000u;
+__device__ __forceinline__ float stage_cos_species(int c, int sp)
+{
+    return __uint_as_float(((kMagicBits + (unsigned)c) & 0x00ffffffu) | ((unsigned)sp << 24));
+}
+__device__ __forceinline__ float staged_cos(float z)
+{
+    return __uint_as_float((__float_as_uint(z) & 0x00ffffffu) | 0x4B000000u) - kMagicF;
+}
 
+// (cos, sin) of a sorted record as the update reads it.
+template <int MODEL, bool SP>
+__device__ __forceinline__ void stage_angle(const Sys &S, int id, int c, int s, float &zc, float &zs)
+{
+    if (SP && MODEL == 1) {
+        zc = stage_cos_species(c, species_of(S, (unsigned)id));
+        zs = (float)s;
+    } else {
+        zc = __int_as_float(c);
+        zs = __int_as_float(s);
+    }
+}
+
+// The Langevin sums with per-species couplings (neighbour_sum_sp above) over
+// the half cells, for couplings and candidate numbers of any size (out of
+// line: its 64-bit conversions run on the narrow FP64 pipe, and inlined the
+// compiler predicates them into every neighbour's path).
 template <int LPP>
 __device__ __noinline__ void neighbour_sum_sp_h(const float4 *__restrict__ P, const unsigned short *cstart, int ec,
                                                 int W2, float4 pi, float r2, const float *grow, long long *out, int sub)
@@ -697,10 +717,9 @@ __device__ __noinline__ void neighbour_sum_sp_h(const float4 *__restrict__ P, co
             const float4 pj = P[j];
             const float dx = pj.x - pi.x, dyy = pj.y - pi.y;
             if (fmaf(dx, dx, dyy * dyy) <= r2) {
-                const int z = __float_as_int(pj.z);
-                const float g = grow[(z >> kSpeciesShift) & 7];
-                sc += __float2ll_rn(g * (float)packed_cos(z));
-                ss += __float2ll_rn(g * (float)__float_as_int(pj.w));
+                const float g = grow[__float_as_uint(pj.z) >> 24];
+                sc += __float2ll_rn(g * staged_cos(pj.z));
+                ss += __float2ll_rn(g * pj.w);
                 ++cnt;
             }
         }
@@ -710,16 +729,20 @@ __device__ __noinline__ void neighbour_sum_sp_h(const float4 *__restrict__ P, co
     out[2] = cnt;
 }
 
-// The same sums when every |Gamma dt| is below 1: W[j] holds the weighted,
-// rounded (cos, sin) of staged record j for the particle's species, made once
-// per record when the tile was sorted instead of once per neighbour.
-template <typename ACC, int UNR, int LPP>
-__device__ __forceinline__ void neighbour_sum_w(const float4 *__restrict__ P, const int2 *__restrict__ W,
-                                                const unsigned short *cstart, int ec, int W2, float4 pi, float r2,
-                                                ACC &sc, ACC &ss, int &cnt, int sub)
+// The same sums when every |Gamma dt| is below 1 and there are fewer than 512
+// candidates.  A staged record then holds its cosine c (an integer, |c| <=
+// 2^22) as the low 24 bits of the float 1.5 2^23 + c with its species above
+// them, and its sine as a float.  Gamma c is rounded to an integer as the bits
+// of fl(Gamma c) + 1.5 2^23 (one addition whose rounding lands on an integer,
+// ties to even: what __float2ll_rn(fl(Gamma c)) gives for |Gamma c| <= 2^22),
+// so that no conversion runs per neighbour; the sum of n such words minus n
+// biases is the exact integer sum (below 2^31).
+template <int UNR, int LPP>
+__device__ __forceinline__ void neighbour_sum_spm(const float4 *__restrict__ P, const unsigned short *cstart, int ec,
+                                                  int W2, float4 pi, float r2, const float *grow, int &sc, int &ss,
+                                                  int &cnt, int sub)
 {
-    sc = 0;
-    ss = 0;
+    unsigned wc = 0, ws = 0;
     cnt = 0;
 #pragma unroll
     for (int dy = -1; dy <= 1; ++dy) {
@@ -727,16 +750,18 @@ __device__ __forceinline__ void neighbour_sum_w(const float4 *__restrict__ P, co
         const int a = cstart[c0], b = cstart[c0 + 5];
 #pragma unroll UNR
         for (int j = LPP > 1 ? a + sub : a; j < b; j += LPP) {
-            const float2 pj = *reinterpret_cast<const float2 *>(P + j);
-            const int2 w = W[j];
+            const float4 pj = P[j];
             const float dx = pj.x - pi.x, dyy = pj.y - pi.y;
             if (fmaf(dx, dx, dyy * dyy) <= r2) {
-                sc += w.x;
-                ss += w.y;
+                const float g = grow[__float_as_uint(pj.z) >> 24];
+                wc += __float_as_uint(__fadd_rn(__fmul_rn(g, staged_cos(pj.z)), kMagicF));
+                ws += __float_as_uint(__fadd_rn(__fmul_rn(g, pj.w), kMagicF));
                 ++cnt;
             }
         }
     }
+    sc = (int)(wc - kMagicBits * (unsigned)cnt);
+    ss = (int)(ws - kMagicBits * (unsigned)cnt);
 }
 
 struct Acc {
@@ -747,7 +772,6 @@ struct Acc {
 struct ToSystem {
     __device__ __forceinline__ int *cnt(const Sys &S, int nxt) const { return S.cnt[nxt]; }
     __device__ __forceinline__ int *spill(const Sys &S, int nxt) const { return &S.spill_cnt[nxt]; }
-    __device__ __forceinline__ const int2 *weighted(int) const { return nullptr; }
 };
 
 // One particle per lane (own index o, inactive when o >= n_own); every lane
@@ -786,33 +810,31 @@ __device__ __forceinline__ void update_one(const Sys &S, const OutMeta &O, const
         sp = SP ? species_of(S, id) : 0;
         bool narrow = !O.wide;
         if (SP && MODEL == 1) {
-            pi.z = __int_as_float(packed_cos(__float_as_int(pi.z)));
-            long long a, b;
-            if (O.small_gamma) {
-                const int2 *w = to.weighted(sp);
-                if (narrow) {
-                    int a4, b4;
-                    if (O.dense) neighbour_sum_w<int, 4, LPP>(P, w, cstart, ec, W2, pi, S.r2, a4, b4, cnt, sub);
-                    else neighbour_sum_w<int, 2, LPP>(P, w, cstart, ec, W2, pi, S.r2, a4, b4, cnt, sub);
-                    a = a4;
-                    b = b4;
-                } else {
-                    neighbour_sum_w<long long, 4, LPP>(P, w, cstart, ec, W2, pi, S.r2, a, b, cnt, sub);
+            const float *grow = S.sp_gamma_dt + sp * kMaxSpecies;
+            if (S.small_gamma && narrow) {
+                int a, b;
+                neighbour_sum_spm<2, LPP>(P, cstart, ec, W2, pi, S.r2, grow, a, b, cnt, sub);
+#pragma unroll
+                for (int d = 1; d < LPP; d <<= 1) {
+                    a += __shfl_xor_sync(group, a, d);
+                    b += __shfl_xor_sync(group, b, d);
                 }
+                sc = (float)a;
+                ss = (float)b;
             } else {
                 long long out[3];
-                neighbour_sum_sp_h<LPP>(P, cstart, ec, W2, pi, S.r2, S.sp_gamma_dt + sp * kMaxSpecies, out, sub);
-                a = out[0];
-                b = out[1];
+                neighbour_sum_sp_h<LPP>(P, cstart, ec, W2, pi, S.r2, grow, out, sub);
                 cnt = (int)out[2];
-            }
 #pragma unroll
-            for (int d = 1; d < LPP; d <<= 1) {
-                a += __shfl_xor_sync(group, a, d);
-                b += __shfl_xor_sync(group, b, d);
+                for (int d = 1; d < LPP; d <<= 1) {
+                    out[0] += __shfl_xor_sync(group, out[0], d);
+                    out[1] += __shfl_xor_sync(group, out[1], d);
+                }
+                sc = (float)out[0];
+                ss = (float)out[1];
             }
-            sc = (float)a;
-            ss = (float)b;
+            pi.z = __int_as_float((int)staged_cos(pi.z));       // as the other models stage them
+            pi.w = __int_as_float((int)pi.w);
         } else {
             if (!narrow) {
                 const int ncand = cstart[ec - W2 + 3] - cstart[ec - W2 - 2] + cstart[ec + 3] - cstart[ec - 2] +

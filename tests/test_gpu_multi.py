@@ -1,5 +1,5 @@
-"""Many steps per launch (small systems with the automatic choice of kernel)
-against the whole-block step kernel (threads = 512), which runs one step per
+"""The automatic choice of kernel -- many steps per launch for small systems,
+the pipelined step beyond, with one species or several -- against the whole-block step kernel (threads = 512), which runs one step per
 launch: states, traces, measurements and histograms bit for bit, over every
 split of the steps the buffer rotation distinguishes (1, 2, 3, even, odd, more
 than one launch), every model and boundary, species, tiles at the edge of the
@@ -52,6 +52,10 @@ CASES = [
     (dict(n=120000, lx=260.0, ly=231.0, eta=0.3, seed=10, model=A.AAP_LANGEVIN, v=1.0), None),
     (dict(n=60000, lx=160.0, ly=171.0, eta=0.3, seed=10, model=A.AAP_LANGEVIN, v=1.0),
      ([20000, 20000, 20000],) + WEAK[1:]),
+    (dict(n=60000, lx=160.0, ly=171.0, seed=11, model=A.AAP_LANGEVIN, order=2, weight=A.AAP_H_ONE, bx=1),
+     ([30000, 0, 30000],) + SPECIES[1:]),
+    (dict(n=60001, lx=160.0, ly=171.0, seed=12, by=1), ([1, 30000, 30000],) + WEAK[1:]),
+    (dict(n=60001, lx=160.0, ly=171.0, seed=13, model=A.AAP_NVM), ([20001, 30000, 10000],) + WEAK[1:]),
     (dict(n=7, lx=3.0, ly=3.2, eta=0.3, seed=11), None),
     (dict(n=0, lx=9.0, ly=9.0, eta=0.3, seed=12), None),
 ]
