@@ -96,8 +96,8 @@ typedef struct aap_params {
                             pipelined kernel: one block per SM with copy, sort
                             and update warps; one species per system).
                             Automatic picks 1024 where it applies, else 512,
-                            and runs a system of at most one tile per SM
-                            many steps per launch (the same trajectory bit
+                            and runs a system of at most four tiles per SM
+                            many steps per launch while none is dense (the same trajectory bit
                             for bit; aap_get_layout reports the kernel of
                             the single steps); an ensemble follows its
                             first replica's value                           */

@@ -97,7 +97,7 @@ struct aap_handle {
     long long launches[3] = {0, 0, 0};
     // capacity management
     double factor = 4.0;            // region slots over the mean occupancy
-    int *pinned_err = nullptr;      // [3]: error word copied after each aap_step; two batch slots
+    int *pinned_err = nullptr;      // [3][4]: error and load words copied after each aap_step; two batch slots
     cudaEvent_t err_event = nullptr;
     cudaEvent_t batch_ev[2] = {nullptr, nullptr};   // error words taken every kAdaptSteps steps
     int batch_prev = -1;            // slot of the newest copy not yet read (-1: none)
@@ -105,6 +105,7 @@ struct aap_handle {
     long long since_copy = 0;       // steps queued since the last copy
     bool err_pending = false;
     int relayouts = 0;
+    bool multi_on = true;           // the tiles are light enough for many steps per launch
     // ensemble membership: steps are launched by the ensemble for all members,
     // whose error words and measurement sums lie side by side in its arrays
     bool member = false;
@@ -624,7 +625,7 @@ int clear_buffers(aap_handle *h)
     for (int b = 0; b < 2; ++b)
         AAP_CK(cudaMemsetAsync(S.spill_bits[b], 0, spill_bits_bytes(S), h->stream));
     AAP_CK(cudaMemsetAsync(S.acc, 0, 2 * aapk::kAccSlots * aapk::kAccWords * sizeof(unsigned long long), h->stream));
-    AAP_CK(cudaMemsetAsync(S.err, 0, sizeof(int), h->stream));
+    AAP_CK(cudaMemsetAsync(S.err, 0, (h->member ? 1 : 4) * sizeof(int), h->stream));
     if (h->d_multi) AAP_CK(cudaMemsetAsync(h->d_multi, 0, aapk::multi_bytes(S.ntiles), h->stream));
     return AAP_OK;
 }
@@ -647,7 +648,7 @@ int alloc_all(aap_handle *h)
     S.bins_nbr = h->p.binnum_neighbors ? h->p.binnum_neighbors : 100;
     if ((rc = dev_alloc(h, &S.hist, (size_t)(S.bins_theta + S.bins_nbr) * sizeof(unsigned long long)))) return rc;
     if (h->member) S.err = h->ens_err;
-    else if ((rc = dev_alloc(h, &S.err, sizeof(int)))) return rc;
+    else if ((rc = dev_alloc(h, &S.err, 4 * sizeof(int)))) return rc;
     if (S.knn > 0) {
         const long long ncell = (long long)S.ncx * S.ncy;
         const long long nchunk = (ncell + 1 + aapk::kScanChunk - 1) / aapk::kScanChunk;
@@ -683,7 +684,7 @@ int alloc_all(aap_handle *h)
     }
     if ((rc = dev_alloc(h, &h->d_obs, 8 * sizeof(unsigned long long)))) return rc;
     if ((rc = dev_alloc(h, &h->d_seen, sizeof(int)))) return rc;
-    AAP_CK(cudaMallocHost(&h->pinned_err, 3 * sizeof(int)));
+    AAP_CK(cudaMallocHost(&h->pinned_err, 12 * sizeof(int)));
     AAP_CK(cudaEventCreateWithFlags(&h->err_event, cudaEventDisableTiming));
     for (cudaEvent_t &e : h->batch_ev) AAP_CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     if ((rc = clear_buffers(h))) return rc;
@@ -793,6 +794,36 @@ int launch_steps(const LaunchCfg &L, cudaStream_t st, long long nsteps, cudaStre
     return AAP_OK;
 }
 
+// Many steps per launch, or one: a launch of many steps gives each tile one
+// block, so that a step lasts as long as its densest tile (and a tile that
+// outgrows the block's shared memory is staged in global memory), while the
+// pipelined step spreads the tiles over warps.  The step kernels report the
+// largest tile load and staged set; past a load of 4096 (twice that in blocks
+// of 512 threads, half of it for coupled species, whose sums cost twice as
+// much) or a staged set beyond the block's, single steps take over until both
+// have fallen by a quarter.  Per step, N = 60,000 to 100,000, many steps
+// against one: load 307: 13.3 / 31.0 us, 2138: 22.9 / 35.6, 4307: 19.5 / 30.8,
+// 7232: 38.5 / 36.4; staged beyond the block's: 84 / 38 and 611 / 131.
+bool use_multi(const aap_handle *h) { return h->L.multi && !h->timing && h->multi_on; }
+
+// words: {error bits, load, staged set}
+void act_on_load(aap_handle *h, const int *words)
+{
+    if (!h->L.multi || words[2] == 0) return;       // nothing was reported
+    const int lim = 16 * h->L.multi_threads / (h->L.multi_species && h->p.model == AAP_LANGEVIN ? 2 : 1);
+    if (h->multi_on) h->multi_on = words[1] <= lim && words[2] <= h->L.multi_cap;
+    else h->multi_on = words[1] <= lim / 4 * 3 && words[2] <= h->L.multi_cap / 4 * 3;
+}
+
+// Copy the error and load words to page-locked `dst`; the load of single
+// steps starts anew (a launch of many steps starts its own).
+int copy_words(aap_handle *h, int *dst)
+{
+    AAP_CK(cudaMemcpyAsync(dst, h->hs.err, 4 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    if (h->L.multi && !h->multi_on) AAP_CK(cudaMemsetAsync(h->hs.err + 1, 0, 2 * sizeof(int), h->stream));
+    return AAP_OK;
+}
+
 int run_steps(aap_handle *h, long long nsteps);
 int act_on_error(aap_handle *h, int err, bool *relaid);
 
@@ -813,14 +844,14 @@ int run_steps_adaptive(aap_handle *h, long long nsteps)
     while (left > 0) {
         long long k = std::min(left, kAdaptSteps - h->since_copy);
         // many steps per launch: no launch of fewer than four steps unless the call itself is that short
-        if (h->L.multi && (k < 4 || left - k < 4)) k = std::min(left, kAdaptSteps + 3);
+        if (use_multi(h) && (k < 4 || left - k < 4)) k = std::min(left, kAdaptSteps + 3);
         if ((rc = run_steps(h, k))) return rc;
         left -= k;
         h->since_copy += k;
         if (h->since_copy < kAdaptSteps) continue;
         h->since_copy = 0;
         const int slot = h->batch_slot;
-        AAP_CK(cudaMemcpyAsync(h->pinned_err + 1 + slot, h->hs.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+        if ((rc = copy_words(h, h->pinned_err + 4 * (1 + slot)))) return rc;
         AAP_CK(cudaEventRecord(h->batch_ev[slot], h->stream));
         h->batch_slot ^= 1;
         const int prev = h->batch_prev;
@@ -828,7 +859,8 @@ int run_steps_adaptive(aap_handle *h, long long nsteps)
         if (prev >= 0) {
             AAP_CK(cudaEventSynchronize(h->batch_ev[prev]));
             // a re-layout resets the copies (the newer one predates it)
-            if ((rc = act_on_error(h, h->pinned_err[1 + prev], nullptr))) return rc;
+            act_on_load(h, h->pinned_err + 4 * (1 + prev));
+            if ((rc = act_on_error(h, h->pinned_err[4 * (1 + prev)], nullptr))) return rc;
         }
     }
     return AAP_OK;
@@ -836,7 +868,7 @@ int run_steps_adaptive(aap_handle *h, long long nsteps)
 
 int run_steps(aap_handle *h, long long nsteps)
 {
-    if (!h->timing && h->L.multi) {
+    if (use_multi(h)) {
         if (nsteps > 0) AAP_CK(aapk::launch_multi(h->L, (int)nsteps, h->stream));
         h->step += nsteps;
         return AAP_OK;
@@ -921,9 +953,16 @@ int reinsert(aap_handle *h, double factor, int mode)
         if ((rc = clear_buffers(h))) return rc;
         if ((rc = push_sys(h))) return rc;
         AAP_CK(aapk::launch_insert(h->hs, (int)(h->step & 1), h->d_x, h->d_y, h->d_th, mode, h->stream));
-        int err = 0;
-        AAP_CK(cudaMemcpyAsync(&err, h->hs.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+        int err = 0, words[4] = {0, 0, 0, 0};
+        if (h->L.multi) {
+            AAP_CK(aapk::launch_tile_load(h->hs, (int)(h->step & 1), h->stream));
+            AAP_CK(cudaMemcpyAsync(words, h->hs.err, sizeof(words), cudaMemcpyDeviceToHost, h->stream));
+        } else {
+            AAP_CK(cudaMemcpyAsync(words, h->hs.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+        }
         AAP_CK(cudaStreamSynchronize(h->stream));
+        err = words[0];
+        act_on_load(h, words);
         const bool spilled = err & (aapk::ERR_SPILL | aapk::ERR_LOST);
         // spilled particles are kept exactly: accepted with an explicit
         // capacity, or when doubling the regions would exceed the staged indices
@@ -993,6 +1032,7 @@ int poll_capacity(aap_handle *h)
     if (q == cudaErrorNotReady) return AAP_OK;
     if (q != cudaSuccess) return fail(AAP_ECUDA, std::string("error event: ") + cudaGetErrorString(q));
     h->err_pending = false;
+    act_on_load(h, h->pinned_err);
     return act_on_error(h, *h->pinned_err, nullptr);
 }
 
@@ -1069,7 +1109,7 @@ struct aap_ens {
     int *d_dense = nullptr;             // pipelined step: tiles left to the whole-block routine
     size_t dense_tiles = 0;
     std::vector<int> order;             // replicas in the order of their descriptors (densest first)
-    int *d_err = nullptr;               // [count] the replicas' error words
+    int *d_err = nullptr;               // [count + 4] the replicas' error words
     double *d_stats = nullptr;          // [count][16] their measurement sums
     unsigned long long *d_obs = nullptr;    // [count][8] observed sums of a window's first state
     LaunchCfg L{};
@@ -1231,7 +1271,7 @@ int ens_build(aap_ens *e, int pol)
     if (cudaMalloc(&e->d_sys, (size_t)count * sizeof(Sys)) != cudaSuccess ||
         cudaMalloc(&e->d_tile_base, (size_t)(count + 1) * sizeof(int)) != cudaSuccess ||
         cudaMalloc(&e->d_ctl, sizeof(Ctl)) != cudaSuccess ||
-        cudaMalloc(&e->d_err, (size_t)count * sizeof(int)) != cudaSuccess ||
+        cudaMalloc(&e->d_err, ((size_t)count + 4) * sizeof(int)) != cudaSuccess ||
         cudaMalloc(&e->d_stats, (size_t)count * 16 * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&e->d_obs, (size_t)count * 8 * sizeof(unsigned long long)) != cudaSuccess) {
         cudaGetLastError();
@@ -1426,7 +1466,7 @@ int aap_step(aap_handle *h, int64_t nsteps)
     int rc = poll_capacity(h);
     if (rc) return rc;
     if ((rc = run_steps_adaptive(h, nsteps))) return rc;
-    AAP_CK(cudaMemcpyAsync(h->pinned_err, h->hs.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    if ((rc = copy_words(h, h->pinned_err))) return rc;
     AAP_CK(cudaEventRecord(h->err_event, h->stream));
     h->err_pending = true;
     return AAP_OK;

@@ -105,8 +105,8 @@ __global__ void __launch_bounds__(NT) k_coarse_tiles(Sys S, int b, BinAxis ax, B
 {
     __shared__ int s_last;
     const long long nb = (long long)ax.nb * ay.nb;
-    pdl_next();
     pdl_wait();
+    pdl_next();
     __shared__ int s_pre[kRegions + 1];
     for (int tile = blockIdx.x; tile < S.ntiles; tile += gridDim.x) {
         const int tx = tile % S.ntx, ty = tile / S.ntx;
@@ -159,8 +159,8 @@ __global__ void __launch_bounds__(NT) k_coarse_tiles(Sys S, int b, BinAxis ax, B
 
 __global__ void k_coarse_finish(unsigned long long *acc, int nbx, int nby, double inv_area, float *out)
 {
-    pdl_next();
     pdl_wait();
+    pdl_next();
     coarse_fields(acc, (long long)nbx * nby, inv_area, out, blockIdx.x * (long long)blockDim.x + threadIdx.x,
                   (long long)gridDim.x * blockDim.x);
 }

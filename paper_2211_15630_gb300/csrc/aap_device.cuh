@@ -14,8 +14,9 @@ namespace aapk {
 // Programmatic dependent launch: a kernel launched with launch_after() may
 // start while the one before it in the stream drains; pdl_wait() returns once
 // that one is complete and its writes are visible (at once for an ordinary
-// launch), and pdl_next() lets the kernel after this one start.  Nothing but
-// the block's own shared memory is touched before pdl_wait().
+// launch), and pdl_next() lets the kernel after this one start: called after
+// pdl_wait(), so that at most one kernel waits on the SMs beside the running
+// one.  Nothing but the block's own shared memory is touched before pdl_wait().
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

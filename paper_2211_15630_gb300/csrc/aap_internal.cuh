@@ -92,7 +92,7 @@ struct Sys {
     unsigned long long *hist;   // [bins_theta + bins_nbr] measured histograms
     int bins_theta, bins_nbr;
     int *nbr_out;               // optional |Omega_i| by particle id
-    int *err;
+    int *err;                   // [4]: error bits; the largest tile load and staged set since the host looked; unused
     // metric-free neighbourhoods (Sec. 2.3): one tile over the whole box whose
     // records all sit in region 0 (flat), re-sorted by cell every step
     int flat;                   // 1: every record goes to region 0 of tile 0
@@ -122,6 +122,13 @@ __host__ __device__ inline int species_of(const Sys &S, unsigned id)
     int s = 0;
     for (int k = 0; k < S.nsp - 1; ++k) s += (long long)id >= S.sp_end[k];
     return s;
+}
+
+// What the neighbour sums of a tile cost, up to a constant: its own particles
+// times the staged records per half cell.
+__host__ __device__ inline int tile_load(int n_own, int m, int nceh)
+{
+    return (int)((float)n_own * (float)m / (float)nceh);
 }
 
 constexpr int kScanChunk = 4096;    // cells per block of the metric-free cell scan

@@ -42,8 +42,8 @@ k_step(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_base,
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ TileCtx T;
-    pdl_next();
     pdl_wait();
+    pdl_next();
     const long long step = ctl->step;
     const int cur = (int)(step & 1);
     const int total = tile_base[nsys];
@@ -126,8 +126,8 @@ k_step(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_base,
 __global__ void k_finish(Sys *sys, int nsys, const int *__restrict__ tile_base, Ctl *ctl)
 {
     __shared__ int s_last;
-    pdl_next();
     pdl_wait();
+    pdl_next();
     const long long step = ctl->step;
     const int cur = (int)(step & 1);
     const long long gt = blockIdx.x * (long long)blockDim.x + threadIdx.x, gs = (long long)gridDim.x * blockDim.x;
@@ -285,6 +285,22 @@ __device__ __forceinline__ void warp_records(const Sys &S, int b, long long w, l
         const int tile = S.spill_key[b][e] / kCntStride;
         f(S.spill_rec[b][e], tile % S.ntx, tile / S.ntx);
     }
+}
+
+// The largest tile load and staged set of the state in buffer b into err[1]
+// and err[2] (a thread per tile; what the step kernels report of later states).
+__global__ void k_tile_load(Sys S, int b)
+{
+    const int tile = blockIdx.x * blockDim.x + threadIdx.x;
+    if (tile >= S.ntiles) return;
+    const TileGeo G = tile_geo(S, tile);
+    int own = 0, m = 0;
+    for (int s = 0; s < kSegs; ++s) {
+        m += make_seg(S, G, s, b).count;
+        if (s == 8) own = m;
+    }
+    atomicMax(S.err + 1, tile_load(own, m, (2 * G.tw + 4) * (G.th + 2)));
+    atomicMax(S.err + 2, m);
 }
 
 // Position (FP64, exact) of a record in box coordinates.
@@ -492,6 +508,12 @@ cudaError_t launch_insert(const Sys &S, int b, const double *x, const double *y,
     const int bs = 256;
     const long long grid = (n + bs - 1) / bs;
     k_insert<<<(unsigned)grid, bs, 0, st>>>(S, b, x, y, th, mode, 1.0 / S.csx_d, 1.0 / S.csy_d);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_tile_load(const Sys &S, int b, cudaStream_t st)
+{
+    k_tile_load<<<(unsigned)((S.ntiles + 63) / 64), 64, 0, st>>>(S, b);
     return cudaGetLastError();
 }
 

@@ -61,6 +61,7 @@ struct MultiShared {
     int warp_tot[kMultiWarps];
     int maxc;
     int ok;
+    int load, staged;           // the tile's largest load and staged set over the launch's steps
 };
 
 // Staging arrays of one tile: shared memory, or the block's global scratch
@@ -266,6 +267,10 @@ __device__ __forceinline__ bool multi_tile(MultiShared &sh, const MultiStage &A,
     } else {
         run(std::integral_constant<int, 1>{});
     }
+    if (tid == NT - 1) {
+        sh.load = max(sh.load, tile_load(n_own, m, nce));
+        sh.staged = max(sh.staged, m);
+    }
     return warp * (32 / lpp) < n_own;
 }
 
@@ -310,6 +315,7 @@ k_multi(Sys *__restrict__ sys, Ctl *ctl, int nsteps, int cap, int nceh, int hist
     if (tid == 0) {
         sh.ok = (*((volatile int *)S.err) & ERR_TIMEOUT) == 0;
         sh.maxc = 0;
+        sh.load = sh.staged = 0;
     }
     const bool closer = tile == nblk - 1;
     if (warp == 0 && !closer) {
@@ -344,6 +350,7 @@ k_multi(Sys *__restrict__ sys, Ctl *ctl, int nsteps, int cap, int nceh, int hist
         int *wc = i == nsteps - 1 ? S.cnt[cur ^ 1] : cnt3 + (size_t)(i % 3) * stride;
         int *ws = i == nsteps - 1 ? &S.spill_cnt[cur ^ 1] : wc + spw;
         if (closer) {
+            if (i == 0 && tid < 2) S.err[1 + tid] = 0;
             // the sums of the step before (complete since the last barrier),
             // and the spill count it consumed
             if (i >= 1 && warp == 0) {
@@ -425,6 +432,10 @@ k_multi(Sys *__restrict__ sys, Ctl *ctl, int nsteps, int cap, int nceh, int hist
     } else {
         if (warp == 0 && lane < kCntStride)
             (nsteps == 1 ? S.cnt[step0 & 1] : cnt3 + (size_t)((nsteps + 1) % 3) * stride)[tile * kCntStride + lane] = 0;
+        if (tid == NT - 1) {
+            atomicMax(S.err + 1, sh.load);      // the closing block cleared them before the first barrier
+            atomicMax(S.err + 2, sh.staged);
+        }
         if ((tile & 31) == 0 && tid == 32) S.spill_bits[last & 1][tile >> 5] = 0u;
         if (step0 < S.meas_until)
             for (int i = tid; i < S.bins_theta + S.bins_nbr; i += NT)
@@ -455,9 +466,9 @@ MultiKernel multi_kernel_t(int model, bool species)
     }
 }
 
-MultiKernel multi_kernel(int model, bool species)
+MultiKernel multi_kernel(int model, bool species, int threads)
 {
-    return multi_kernel_t<512, 1>(model, species);
+    return threads == 512 ? multi_kernel_t<512, 1>(model, species) : multi_kernel_t<256, 4>(model, species);
 }
 
 }  // namespace
@@ -472,14 +483,13 @@ cudaError_t set_multi_test(long long wait_cycles, int stall)
 cudaError_t configure_multi(LaunchCfg &L, bool species, int ntiles, int sm_count, int min_cap)
 {
     L.multi = 0;
-    // One block of 512 threads (128 registers each) per SM.  Beyond that, with
-    // up to four blocks of 256 threads per SM, light tiles still gain (N =
-    // 50,021 in 400 tiles, uniform: 46 -> 13 us per step) but a step lasts as
-    // long as its densest tile: the same system clustered, 800 particles in
-    // one tile, 57 -> 64 us.
+    // One block of 512 threads (128 registers each) per SM while that holds every
+    // tile, else up to four blocks of 256 threads (N = 50,021 in 400 tiles,
+    // uniform: 46 us per step in single launches, 13 us so; the caller goes back
+    // to single steps while some tile is dense).
     const int blocks = ntiles + 1;
-    const int threads = 512;
-    if (ntiles < 1 || blocks > sm_count) return cudaSuccess;
+    const int threads = blocks <= sm_count ? 512 : 256;
+    if (ntiles < 1 || blocks > 4 * sm_count) return cudaSuccess;
     int dev = 0, coop = 0, optin = 0, per_sm = 0;
     cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -487,7 +497,7 @@ cudaError_t configure_multi(LaunchCfg &L, bool species, int ntiles, int sm_count
     if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess) return e;
     if (!coop) return cudaSuccess;
-    const MultiKernel k = multi_kernel(L.model, species);
+    const MultiKernel k = multi_kernel(L.model, species, threads);
     if (!k) return cudaErrorInvalidValue;
     cudaFuncAttributes a;
     if ((e = cudaFuncGetAttributes(&a, k)) != cudaSuccess) return e;
@@ -519,7 +529,7 @@ cudaError_t configure_multi(LaunchCfg &L, bool species, int ntiles, int sm_count
 
 cudaError_t launch_multi(const LaunchCfg &L, int nsteps, cudaStream_t st)
 {
-    const MultiKernel k = multi_kernel(L.model, L.multi_species != 0);
+    const MultiKernel k = multi_kernel(L.model, L.multi_species != 0, L.multi_threads);
     Sys *sys = L.sys;
     Ctl *ctl = L.ctl;
     int cap = L.multi_cap, nceh = L.pipe_nceh, hw = L.hist_words, stride = multi_stride(L.multi_tiles);

@@ -137,6 +137,7 @@ struct PipeShared {
     int chunk[2];               // next chunk of 32 own particles, per output buffer
     int flag;                   // a previous step's wait ran out
     int dense_tile;
+    int load, staged;           // largest tile load and staged set of the block's tiles
     int warp_tot[kPipeWarps];
     long long red[5][kPipeWarps];
     __align__(8) unsigned long long bar_raw_full[kNR], bar_raw_empty[kNR], bar_full[2], bar_empty[2];
@@ -500,6 +501,8 @@ __device__ __forceinline__ void sort_order(PipeShared &sh, const PipeBufs &B, in
             O.wide = 15 * mx >= 512;
             O.dense = 2 * m > 3 * nce;
             sh.chunk[b] = 0;
+            sh.load = max(sh.load, tile_load(carry, m, nce));
+            sh.staged = max(sh.staged, m);
             if (carry != M.n_own) atomicOr(M.err, ERR_BOUNDS);
         }
     }
@@ -593,11 +596,14 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
     }
     for (int i = tid; i < nceh_max; i += kPipeThreads) B.hist[i] = 0;
     for (int i = tid; i < 2 * B.mh_stride; i += kPipeThreads) B.mhist0[i] = 0;
-    pdl_next();
     pdl_wait();         // the step before is closed
+    pdl_next();
     // pipeline waits that run out are reported in the first system's error word
     int *const err0 = sys[0].err;
-    if (tid == 0) sh.flag = *((volatile int *)err0) & ERR_TIMEOUT;
+    if (tid == 0) {
+        sh.flag = *((volatile int *)err0) & ERR_TIMEOUT;
+        sh.load = sh.staged = 0;
+    }
     __syncthreads();
     // after a wait has run out the handle is unusable: later steps do nothing
     // (so that a queue of steps cannot each wait out their bounds)
@@ -959,6 +965,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
         __syncthreads();
         const int g = sh.dense_tile;
         if (g < 0) break;
+        if (tid == 0) sh.load = sh.staged = 0x7fffffff;
         const int si = nsys > 1 ? sys_of_tile(tile_base, nsys, g) : 0;
         if (first || si != T.sysi) {
             __syncthreads();                // every thread is done with the previous system
@@ -991,6 +998,12 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
         }
         if (tid == 0) PT_ADD(11, 1);
         __syncthreads();
+    }
+    // what the host goes by when it chooses between this kernel and many steps
+    // per launch (a single system)
+    if (nsys == 1 && tid == 0 && sh.staged > 0) {
+        atomicMax(err0 + 1, sh.load);
+        atomicMax(err0 + 2, sh.staged);
     }
     if (tid == 0) PT_ADD(12, PT_NOW() - tk0);
     (void)td0;
