@@ -18,6 +18,9 @@
 //                             forward with the residual update, or the data
 //                             gradient (flipped, transposed weights) masked by
 //                             the ReLU of the layer input
+//   k_net                     one application of the whole network to a tile,
+//                             the four layers in shared memory (calls too small
+//                             to fill the chip layer by layer)
 //   k_conv_dw_tc<CIN, COUT>   weight and bias gradients on the tcgen05
 //                             tensor cores (shifted input rows and the
 //                             transposed dy as K-major operands, pixels along
@@ -25,7 +28,8 @@
 //                             accumulator per column shift for all of a block's
 //                             tiles), one partial per block, reduced in a fixed
 //                             order (deterministic)
-//   k_adam                    Adam step on the FP32 master weights
+//   k_grad_adam_pack          gradients from the partials, the Adam step on the
+//                             FP32 master weights and their BF16 copies
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -38,10 +42,16 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include "aap_device.cuh"
+
 #include "../../include/aap.h"
 #include "../../include/aap_surrogate.h"
 
 namespace aaps {
+
+using aapk::launch_after;
+using aapk::pdl_next;
+using aapk::pdl_wait;
 
 typedef __nv_bfloat16 bf16;
 
@@ -382,6 +392,334 @@ __global__ void __launch_bounds__(kConvThreads) k_conv_ws(const bf16 *__restrict
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(32 * NA));
 }
 
+// Channels whose per-sample grid mean one application keeps (conserve bits:
+// 1 the density, 2 both polarisation channels).
+__host__ __device__ inline bool conserved(int conserve, int c) { return c == 0 ? (conserve & 1) : (conserve & 2); }
+
+// Conservation projection in two passes over chunks of kCenterChunk pixels
+// of a sample (NHWC 8 FP32, channels 0..2 read as one float4 per pixel):
+// k_center_part writes each chunk's sums of a - b per channel (fixed order,
+// so the result is deterministic); the means follow from a sample's chunk
+// sums in chunk order.
+constexpr int kCenterChunk = 2048;
+
+// The sums of one chunk by the first 256 threads of a block (every thread of
+// it calls): each thread its pixels in order, then a tree.
+__device__ __forceinline__ void center_chunk(const float4 *__restrict__ a, const float4 *__restrict__ b, int stride,
+                                             long long base, int p0, int p1, float (*red)[256], float *part)
+{
+    const int tid = threadIdx.x;
+    if (tid < 256) {
+        float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+        for (int p = p0 + tid; p < p1; p += 256) {
+            const float4 u = __ldcg(a + (base + p) * stride), v = __ldcg(b + (base + p) * stride);
+            s0 += u.x - v.x;
+            s1 += u.y - v.y;
+            s2 += u.z - v.z;
+        }
+        red[0][tid] = s0;
+        red[1][tid] = s1;
+        red[2][tid] = s2;
+    }
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if (tid < o)
+            for (int c = 0; c < 3; ++c) red[c][tid] += red[c][tid + o];
+        __syncthreads();
+    }
+    if (tid < 3) part[tid] = red[tid][0];
+}
+
+__global__ void __launch_bounds__(256) k_center_part(const float *__restrict__ a, const float *__restrict__ b,
+                                                     int npix, int nchunk, float *__restrict__ part)
+{
+    __shared__ float red[3][256];
+    pdl_wait();
+    pdl_next();
+    const int smp = blockIdx.x / nchunk, ch = blockIdx.x % nchunk;
+    const int p0 = ch * kCenterChunk, p1 = min(npix, p0 + kCenterChunk);
+    center_chunk(reinterpret_cast<const float4 *>(a), reinterpret_cast<const float4 *>(b), 2, (long long)smp * npix, p0, p1,
+                 red, part + (long long)blockIdx.x * 4);
+}
+
+// Grid mean of channel c of sample smp from its chunk sums.
+__device__ __forceinline__ float chunk_mean(const float *__restrict__ part, int smp, int nchunk, int c, int npix)
+{
+    float t = 0.f;
+    for (int k = 0; k < nchunk; ++k) t += part[((long long)smp * nchunk + k) * 4 + c];
+    return t / (float)npix;
+}
+
+// ------------------------------------------------- the whole network, fused --
+// One application of the network to a 16 x 8 tile of one sample per block, all
+// four layers in shared memory, for calls too small to fill the chip layer by
+// layer (there a layer is mostly its launch, its weights and its latency).
+// The tile's region of 24 x 16 pixels (four rings) is flattened with a row
+// pitch of 16 pixels, so that every tap of a layer is the same planes of
+// 16-byte pixels (8 channels each) read from a shifted start, and 128
+// consecutive pixels are one MMA: layer l is computed on rows l .. 23 - l as
+// two or three such runs (the last ones overlap, writing the same values
+// twice).  Rings are recomputed by neighbouring tiles: 171 MMAs a tile against
+// 63, which is why large batches go layer by layer.
+// The conservation projection needs the whole grid: the block that completes a
+// chunk of 2048 pixels sums (out - in) over it, in the order of k_center_part
+// (so that the results are those of the other path bit for bit), and the next
+// application (or the output) subtracts the mean as it reads this one's raw
+// result.  10 applications with the projection, fused against layer by layer
+// (70 kernels): 128 tiles (one sample of 128 x 128) 137 / 285 us, 256 tiles 168
+// / 316, 512 tiles 324 / 379.
+constexpr int kNetRows = kTH + 8, kNetPitch = kTW + 8, kNetPix = kNetRows * kNetPitch;
+constexpr int kNetGuard = 16;                                   // pixels before the first (a tap reaches back 17)
+constexpr int kNetPlane = (kNetGuard + kNetPix + 8) * 16;       // bytes of a plane of 8 channels
+constexpr int kNetThreads = 416;                                // 12 epilogue warps, one that issues
+constexpr int kNetW0 = 9 * 1 * 1024, kNetW1 = 9 * 2 * 1024, kNetW3 = 9 * 2 * 512;   // staged weights of a layer
+constexpr int kNetWeights = kNetW0 + 2 * kNetW1 + kNetW3;
+constexpr size_t kNetSmem = 8 * (size_t)kNetPlane + kNetWeights + kTH * kTW * 16 + 1024;
+static_assert(kNetPix == 384 && kNetThreads >= kNetPix, "a thread per input pixel");
+
+struct NetArgs {
+    const bf16 *wf[4];
+    const float *bias[4];
+    const float *fields;        // first application: FP32 planes [B][3][H][W]
+    const float4 *raw_in;       // later ones: the previous result before the projection
+    float4 *raw_out;
+    float4 *in_out;             // the projected input, for the sums
+    const float *part_in;       // [B][chunks][4] sums of the previous application
+    float *part_out;
+    int *count;                 // [B][chunks] tiles done (zero between launches)
+    const float *eta;
+    int H, W, conserve;
+    float rho0, eta_c, eta_s;
+};
+
+// The weights of a layer as N x 16 core matrices per (tap, K step).
+template <int CIN, int COUT, int NP>
+__device__ __forceinline__ void net_stage_weights(unsigned char *s_w, const bf16 *__restrict__ wt)
+{
+    constexpr int G = CIN / 8, KC = CIN / 16, WBLK = (NP / 8) * 2 * 128;
+    for (int i = threadIdx.x; i < 9 * NP * G; i += kNetThreads) {
+        const int tap = i / (NP * G), rem = i - tap * (NP * G), co = rem / G, g = rem - co * G;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (co < COUT) v = *(reinterpret_cast<const uint4 *>(wt + ((size_t)tap * COUT + co) * CIN) + g);
+        *reinterpret_cast<uint4 *>(s_w + (tap * KC + (g >> 1)) * WBLK + ((co >> 3) * 2 + (g & 1)) * 128 + (co & 7) * 16) =
+            v;
+    }
+}
+
+// First pixel of run t of layer l (1 .. 4): consecutive runs of 128 from row l
+// on, the last one pulled back to end with row 23 - l.
+__device__ __forceinline__ int net_run(int l, int t)
+{
+    return min(kNetPitch * l + 128 * t, kNetPitch * (kNetRows - l) - 128);
+}
+
+// Issue the MMAs of a layer (one thread): runs 0 .. NT - 1 into the
+// accumulators at 32 t, each committed to its barrier.
+template <int KC, int NP, int NT>
+__device__ __forceinline__ void net_issue(uint32_t tmem, uint32_t in, uint32_t w, int l, uint64_t *bar)
+{
+    constexpr uint32_t idesc = umma_idesc_bf16(128, NP);
+    constexpr int WBLK = (NP / 8) * 2 * 128;
+    for (int t = 0; t < NT; ++t) {
+        const uint32_t a0 = in + (kNetGuard + net_run(l, t)) * 16;
+        uint32_t acc = 0;
+#pragma unroll
+        for (int tap = 0; tap < 9; ++tap) {
+            const int off = ((tap / 3 - 1) * kNetPitch + tap % 3 - 1) * 16;
+#pragma unroll
+            for (int kc = 0; kc < KC; ++kc) {
+                umma_bf16(tmem + 32 * t, umma_desc(a0 + off + 2 * kc * kNetPlane, kNetPlane, 128),
+                          umma_desc(w + (tap * KC + kc) * WBLK, 128, 256), idesc, acc);
+                acc = 1;
+            }
+        }
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                     ::"r"(smem_addr(&bar[t])));
+    }
+}
+
+__global__ void __launch_bounds__(kNetThreads, 2) k_net(const NetArgs a)
+{
+    extern __shared__ unsigned char s_dyn[];
+    unsigned char *base = (unsigned char *)(((uintptr_t)s_dyn + 1023) & ~(uintptr_t)1023);
+    unsigned char *buf0 = base, *buf1 = base + 4 * kNetPlane;       // four planes each; the input starts in buf1
+    unsigned char *s_w = base + 8 * kNetPlane;
+    float4 *s_u = reinterpret_cast<float4 *>(s_w + kNetWeights);    // [128] the tile's own input
+    __shared__ uint32_t s_tmem;
+    __shared__ __align__(8) uint64_t bar[3];
+    __shared__ float s_mean[3], s_bias[3][32], s_bias3[8];
+    __shared__ int s_done;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+        for (int k = 0; k < 3; ++k) bar_init(&bar[k], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+    if (warp == 12) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&s_tmem)),
+                     "r"(128));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    // the weights (written before the kernel that may still run) while the
+    // previous application drains
+    net_stage_weights<16, 32, 32>(s_w, a.wf[0]);
+    net_stage_weights<32, 32, 32>(s_w + kNetW0, a.wf[1]);
+    net_stage_weights<32, 32, 32>(s_w + kNetW0 + kNetW1, a.wf[2]);
+    net_stage_weights<32, 8, 16>(s_w + kNetW0 + 2 * kNetW1, a.wf[3]);
+    if (tid < 96) s_bias[tid >> 5][lane] = a.bias[tid >> 5][lane];
+    else if (tid < 104) s_bias3[tid - 96] = a.bias[3][tid - 96];
+    pdl_wait();
+    const int tx = a.W / kTW, ntile = tx * (a.H / kTH);
+    const int smp = blockIdx.x / ntile, tile = blockIdx.x - smp * ntile;
+    const int y0 = (tile / tx) * kTH, x0 = (tile % tx) * kTW;
+    const size_t plane = (size_t)a.H * a.W;
+    const int nchunk = ((int)plane + kCenterChunk - 1) / kCenterChunk;
+    if (tid < 3)
+        s_mean[tid] = a.part_in && conserved(a.conserve, tid) ? chunk_mean(a.part_in, smp, nchunk, tid, (int)plane) : 0.f;
+    __syncthreads();
+    // --- the region's input: 3 fields and the noise strength, BF16 ----------
+    if (tid < kNetPix) {
+        const int ry = tid / kNetPitch, rx = tid - ry * kNetPitch;
+        int gy = y0 + ry - 4, gx = x0 + rx - 4;
+        gy += gy < 0 ? a.H : 0;
+        gy -= gy >= a.H ? a.H : 0;
+        gx += gx < 0 ? a.W : 0;
+        gx -= gx >= a.W ? a.W : 0;
+        const size_t p = (size_t)gy * a.W + gx;
+        float4 u;
+        if (a.fields) {
+            const float *f = a.fields + smp * 3 * plane + p;
+            u = make_float4(f[0] / a.rho0 - 1.f, f[plane] / a.rho0, f[2 * plane] / a.rho0, 0.f);
+        } else {
+            u = a.raw_in[smp * plane + p];
+            u.x -= s_mean[0];
+            u.y -= s_mean[1];
+            u.z -= s_mean[2];
+        }
+        const float e = (a.eta[smp] - a.eta_c) / a.eta_s;
+        const __nv_bfloat162 h0 = __floats2bfloat162_rn(u.x, u.y), h1 = __floats2bfloat162_rn(u.z, e);
+        uint4 *o = reinterpret_cast<uint4 *>(buf1 + (kNetGuard + tid) * 16);
+        *o = make_uint4(*reinterpret_cast<const uint32_t *>(&h0), *reinterpret_cast<const uint32_t *>(&h1), 0u, 0u);
+        *reinterpret_cast<uint4 *>(buf1 + kNetPlane + (kNetGuard + tid) * 16) = make_uint4(0u, 0u, 0u, 0u);
+        if (ry >= 4 && ry < 4 + kTH && rx >= 4 && rx < 4 + kTW) s_u[(ry - 4) * kTW + rx - 4] = u;
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t tmem = s_tmem;
+    const int run = warp >> 2, q = warp & 3;            // epilogue warps: their run, TMEM lane quarter
+    bool ok = true;
+    for (int l = 1; l <= 3; ++l) {
+        unsigned char *src = (l & 1) ? buf1 : buf0, *dst = (l & 1) ? buf0 : buf1;
+        if (warp == 12) {
+            if (lane == 0) {
+                if (l == 1) net_issue<1, 32, 3>(tmem, smem_addr(src), smem_addr(s_w), l, bar);
+                else net_issue<2, 32, 3>(tmem, smem_addr(src), smem_addr(s_w + kNetW0 + (l - 2) * kNetW1), l, bar);
+            }
+            __syncwarp();
+        } else {
+            ok = __all_sync(0xffffffffu, bar_wait(&bar[run], (uint32_t)(l - 1) & 1u));
+            if (ok) {
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                uint32_t r[32];
+                tmem_load<32>(tmem + 32 * run + ((uint32_t)(q * 32) << 16), r);
+                unsigned char *o = dst + (kNetGuard + net_run(l, run) + q * 32 + lane) * 16;
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                    uint32_t pk[4];
+#pragma unroll
+                    for (int j = 0; j < 8; j += 2) {
+                        const int co = 8 * g + j;
+                        const float v0 = fmaxf(__uint_as_float(r[co]) + s_bias[l - 1][co], 0.f);
+                        const float v1 = fmaxf(__uint_as_float(r[co + 1]) + s_bias[l - 1][co + 1], 0.f);
+                        const __nv_bfloat162 h2 = __floats2bfloat162_rn(v0, v1);
+                        pk[j / 2] = *reinterpret_cast<const uint32_t *>(&h2);
+                    }
+                    *reinterpret_cast<uint4 *>(o + g * kNetPlane) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                }
+            }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;");
+        ok = __syncthreads_and(ok) != 0;
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        if (!ok) break;
+    }
+    if (ok) {
+        if (warp == 12) {
+            if (lane == 0) net_issue<2, 16, 2>(tmem, smem_addr(buf0), smem_addr(s_w + kNetW0 + 2 * kNetW1), 4, bar);
+            __syncwarp();
+        } else if (warp < 8) {
+            ok = __all_sync(0xffffffffu, bar_wait(&bar[run], 1u));
+            if (ok) {
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                uint32_t r[16];
+                tmem_load<16>(tmem + 32 * run + ((uint32_t)(q * 32) << 16), r);
+                const int p = net_run(4, run) + q * 32 + lane, ry = p / kNetPitch - 4, rx = p % kNetPitch - 4;
+                if (rx >= 0 && rx < kTW) {
+                    const float4 u = s_u[ry * kTW + rx];
+                    const float4 o = make_float4(u.x + (__uint_as_float(r[0]) + s_bias3[0]),
+                                                 u.y + (__uint_as_float(r[1]) + s_bias3[1]),
+                                                 u.z + (__uint_as_float(r[2]) + s_bias3[2]), 0.f);
+                    const size_t at = smp * plane + (size_t)(y0 + ry) * a.W + x0 + rx;
+                    a.raw_out[at] = o;
+                    if (a.conserve) a.in_out[at] = u;
+                }
+            }
+        }
+    }
+    // MMAs still running (only when a wait ran out): the last commit of each
+    // barrier is waited for once more before TMEM is freed
+    if (!ok && tid == 0)
+        for (int k = 0; k < 3; ++k) bar_wait(&bar[k], 0u);
+    pdl_next();
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    if (warp == 12) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(128));
+    if (!a.conserve) return;
+    // the chunks of the tile's sixteen rows, each counted by every tile of the
+    // rows it touches: the last one to come sums it
+    const int first = y0 * a.W / kCenterChunk, last = ((y0 + kTH) * a.W - 1) / kCenterChunk;
+    float(*red)[256] = reinterpret_cast<float(*)[256]>(buf0);
+    for (int c = first; c <= last; ++c) {
+        const int p0 = c * kCenterChunk, p1 = min((int)plane, p0 + kCenterChunk);
+        if (tid == 0) {
+            const int all = ((p1 - 1) / a.W / kTH - p0 / a.W / kTH + 1) * tx;
+            __threadfence();
+            s_done = atomicAdd(a.count + smp * nchunk + c, 1) == all - 1;
+            if (s_done) a.count[smp * nchunk + c] = 0;
+            __threadfence();
+        }
+        __syncthreads();
+        if (s_done)
+            center_chunk(a.raw_out, a.in_out, 1, (long long)(smp * plane), p0, p1, red,
+                         a.part_out + (smp * (long long)nchunk + c) * 4);
+        __syncthreads();
+    }
+}
+
+// The last application's raw result, projected, as fields (FP32 planes); one
+// block takes pixels of one sample.
+__global__ void __launch_bounds__(256) k_net_out(const float4 *__restrict__ raw, const float *__restrict__ part, int H,
+                                                 int W, int conserve, float rho0, float *__restrict__ f)
+{
+    __shared__ float s_mean[3];
+    pdl_wait();
+    pdl_next();
+    const int npix = H * W, nchunk = (npix + kCenterChunk - 1) / kCenterChunk, per = (npix + 255) / 256;
+    const int smp = blockIdx.x / per, p = (blockIdx.x - smp * per) * 256 + threadIdx.x;
+    if (threadIdx.x < 3)
+        s_mean[threadIdx.x] = conserved(conserve, threadIdx.x) ? chunk_mean(part, smp, nchunk, threadIdx.x, npix) : 0.f;
+    __syncthreads();
+    if (p >= npix) return;
+    const float4 u = raw[(size_t)smp * npix + p];
+    float *o = f + (size_t)smp * 3 * npix + p;
+    o[0] = rho0 * ((u.x - s_mean[0]) + 1.f);
+    o[npix] = rho0 * (u.y - s_mean[1]);
+    o[2 * (size_t)npix] = rho0 * (u.z - s_mean[2]);
+}
+
 // Weight / bias gradient on the tensor cores.  For every column shift dx the
 // block accumulates D_dx[(dy, ci)][co] = sum_p x[p + (dy, dx) - 1][ci] dy[p][co]
 // over all its tiles in TMEM (accumulator dx at columns 32 dx): one MMA per dx
@@ -625,25 +963,36 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_conv_dw_tc(const bf16 *__rest
     (void)ok;
 }
 
-// out[i] = sum_k part[k][i] in a fixed order (deterministic): a block takes
-// 32 consecutive i; its eight warps sum eight consecutive ranges of k, and
-// the eight partial sums are added in warp order.
-__global__ void __launch_bounds__(256) k_reduce_parts(const float *__restrict__ part, int nparts, int len,
-                                                      float *__restrict__ w_out, int wlen, float *__restrict__ b_out)
+// sum_k part[k][i] in a fixed order (deterministic): a block of 256 threads
+// takes 32 consecutive i; its eight warps sum eight consecutive ranges of k,
+// and warp 0 adds the eight partial sums in warp order and returns the total
+// for i = i0 + lane (the other warps return 0).
+__device__ __forceinline__ float reduce_parts(const float *__restrict__ part, int nparts, int len, int i)
 {
     __shared__ float s_sum[8][33];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int i = blockIdx.x * 32 + lane;
     const int per = (nparts + 7) / 8, k0 = min(w * per, nparts), k1 = min(k0 + per, nparts);
     float acc = 0.f;
     if (i < len)
         for (int k = k0; k < k1; ++k) acc += part[(size_t)k * len + i];
     s_sum[w][lane] = acc;
     __syncthreads();
-    if (w == 0 && i < len) {
-        float t = 0.f;
+    float t = 0.f;
+    if (w == 0) {
 #pragma unroll
         for (int v = 0; v < 8; ++v) t += s_sum[v][lane];
+    }
+    return t;
+}
+
+__global__ void __launch_bounds__(256) k_reduce_parts(const float *__restrict__ part, int nparts, int len,
+                                                      float *__restrict__ w_out, int wlen, float *__restrict__ b_out)
+{
+    pdl_wait();
+    pdl_next();
+    const int i = blockIdx.x * 32 + (threadIdx.x & 31);
+    const float t = reduce_parts(part, nparts, len, i);
+    if ((threadIdx.x >> 5) == 0 && i < len) {
         if (i < wlen) w_out[i] = t; else b_out[i - wlen] = t;
     }
 }
@@ -663,6 +1012,8 @@ __device__ __forceinline__ void store_input_pixel(bf16 *px, float a, float b, fl
 __global__ void k_fields_in(const float *__restrict__ f, const float *__restrict__ eta, int B, int H, int W,
                             float rho0, float eta_c, float eta_s, float *__restrict__ state, bf16 *__restrict__ x0)
 {
+    pdl_wait();
+    pdl_next();
     const long long n = (long long)B * H * W;
     const long long plane = (long long)H * W;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -682,6 +1033,8 @@ __global__ void k_fields_in(const float *__restrict__ f, const float *__restrict
 __global__ void k_state_to_input(const float *__restrict__ state, const float *__restrict__ eta, int B, int H,
                                  int W, float eta_c, float eta_s, bf16 *__restrict__ x0)
 {
+    pdl_wait();
+    pdl_next();
     const long long n = (long long)B * H * W;
     const long long plane = (long long)H * W;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -695,6 +1048,8 @@ __global__ void k_state_to_input(const float *__restrict__ state, const float *_
 // Normalised state -> fields (FP32 planes).
 __global__ void k_fields_out(const float *__restrict__ state, int B, int H, int W, float rho0, float *__restrict__ f)
 {
+    pdl_wait();
+    pdl_next();
     const long long n = (long long)B * H * W;
     const long long plane = (long long)H * W;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -715,6 +1070,8 @@ __global__ void k_mse(const float *__restrict__ pred, const float *__restrict__ 
                       int plane)
 {
     __shared__ float red[256];
+    pdl_wait();
+    pdl_next();
     float s = 0.f;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < npix; i += (long long)gridDim.x * blockDim.x) {
         const float4 u = *reinterpret_cast<const float4 *>(pred + i * 8);
@@ -736,61 +1093,20 @@ __global__ void k_mse(const float *__restrict__ pred, const float *__restrict__ 
     if (threadIdx.x == 0) part[blockIdx.x] = red[0];
 }
 
-// Channels whose per-sample grid mean one application keeps (conserve bits:
-// 1 the density, 2 both polarisation channels).
-__host__ __device__ inline bool conserved(int conserve, int c) { return c == 0 ? (conserve & 1) : (conserve & 2); }
-
-// Conservation projection in two passes over chunks of kCenterChunk pixels
-// of a sample (NHWC 8 FP32, channels 0..2 read as one float4 per pixel):
-// k_center_part writes each chunk's sums of a - b per channel (fixed order,
-// so the result is deterministic); the means follow from a sample's chunk
-// sums in chunk order.
-constexpr int kCenterChunk = 2048;
-
-__global__ void __launch_bounds__(256) k_center_part(const float *__restrict__ a, const float *__restrict__ b,
-                                                     int npix, int nchunk, float *__restrict__ part)
-{
-    __shared__ float red[3][256];
-    const int smp = blockIdx.x / nchunk, ch = blockIdx.x % nchunk;
-    const long long base = (long long)smp * npix;
-    const int p0 = ch * kCenterChunk, p1 = min(npix, p0 + kCenterChunk);
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-    for (int p = p0 + threadIdx.x; p < p1; p += 256) {
-        const float4 u = *reinterpret_cast<const float4 *>(a + (base + p) * 8);
-        const float4 v = *reinterpret_cast<const float4 *>(b + (base + p) * 8);
-        s0 += u.x - v.x;
-        s1 += u.y - v.y;
-        s2 += u.z - v.z;
-    }
-    red[0][threadIdx.x] = s0;
-    red[1][threadIdx.x] = s1;
-    red[2][threadIdx.x] = s2;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o)
-            for (int c = 0; c < 3; ++c) red[c][threadIdx.x] += red[c][threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x < 3) part[(long long)blockIdx.x * 4 + threadIdx.x] = red[threadIdx.x][0];
-}
-
-// Grid mean of channel c of sample smp from its chunk sums.
-__device__ __forceinline__ float chunk_mean(const float *__restrict__ part, int smp, int nchunk, int c, int npix)
-{
-    float t = 0.f;
-    for (int k = 0; k < nchunk; ++k) t += part[((long long)smp * nchunk + k) * 4 + c];
-    return t / (float)npix;
-}
-
 // Remove the mean of out - in from the conserved channels of out (one block
-// per chunk of a sample).
+// per chunk of a sample); x0 != null: write the result as the next network
+// input too (NHWC 16).
 __global__ void __launch_bounds__(256) k_center_apply(float *__restrict__ out, const float *__restrict__ part,
-                                                      int npix, int nchunk, int conserve)
+                                                      int npix, int nchunk, int conserve, const float *__restrict__ eta,
+                                                      float eta_c, float eta_s, bf16 *__restrict__ x0)
 {
     __shared__ float mean[3];
+    pdl_wait();
+    pdl_next();
     const int smp = blockIdx.x / nchunk, ch = blockIdx.x % nchunk;
     if (threadIdx.x < 3)
         mean[threadIdx.x] = conserved(conserve, threadIdx.x) ? chunk_mean(part, smp, nchunk, threadIdx.x, npix) : 0.f;
+    const float e = x0 ? (eta[smp] - eta_c) / eta_s : 0.f;
     __syncthreads();
     const long long base = (long long)smp * npix;
     const int p0 = ch * kCenterChunk, p1 = min(npix, p0 + kCenterChunk);
@@ -801,6 +1117,7 @@ __global__ void __launch_bounds__(256) k_center_apply(float *__restrict__ out, c
         u.y -= mean[1];
         u.z -= mean[2];
         *o = u;
+        if (x0) store_input_pixel(x0 + (base + p) * 16, u.x, u.y, u.z, e);
     }
 }
 
@@ -810,39 +1127,78 @@ __global__ void __launch_bounds__(256) k_center_apply(float *__restrict__ out, c
 __global__ void k_dmean(const float *__restrict__ part, int B, int npix, int nchunk, int conserve,
                         float *__restrict__ dmean)
 {
+    pdl_wait();
+    pdl_next();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= B * 3) return;
     const int smp = i / 3, c = i % 3;
     dmean[i] = conserved(conserve, c) ? chunk_mean(part, smp, nchunk, c, npix) : 0.f;
 }
 
-// Adam (Kingma & Ba) on the FP32 master parameters.
-__global__ void k_adam(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m,
-                       float *__restrict__ v, int n, float lr, float b1, float b2, float eps, float c1, float c2)
+// One layer's packed BF16 weights: master [co][tap][ci] -> forward layout
+// [tap][co][ci] and (wb) the data-gradient layout [tap'][ci][cob] with tap' =
+// 8 - tap the flipped tap and cob >= cout output channels (zero beyond cout:
+// cleared once, never written).
+struct Layer {
+    int cin, cout, cob;
+    int woff, boff;             // in the parameter vector
+    const float *part;          // the weight gradient's block partials
+    int nparts;
+    bf16 *wf, *wb;
+};
+struct Layers {
+    Layer l[4];
+    int first[5];               // first block of each layer's parameters, 32 to a block
+};
+
+__device__ __forceinline__ void pack_weight(const Layer &L, int i, float w)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.f - b1) * gi;
-        const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    }
+    const int co = i / (9 * L.cin), r = i - co * 9 * L.cin, tap = r / L.cin, ci = r - tap * L.cin;
+    const bf16 v = __float2bfloat16_rn(w);
+    L.wf[((size_t)tap * L.cout + co) * L.cin + ci] = v;
+    if (L.wb) L.wb[((size_t)(8 - tap) * L.cin + ci) * L.cob + co] = v;
 }
 
-// Master weights [co][tap][ci] -> BF16 forward layout [tap][co][ci] and the
-// data-gradient layout [tap'][ci][cob] with tap' = 8 - tap the flipped tap and
-// cob >= cout output channels (zero beyond cout; the buffer is cleared first).
-__global__ void k_pack(const float *__restrict__ w, int cout, int cin, bf16 *__restrict__ wf, bf16 *__restrict__ wb,
-                       int cob)
+// The layer of this block and the thread's index among its weights and biases.
+__device__ __forceinline__ int layer_of(const Layers &Ls, int &i)
 {
-    const int n = cout * 9 * cin;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int co = i / (9 * cin), r = i - co * 9 * cin, tap = r / cin, ci = r - tap * cin;
-        const bf16 v = __float2bfloat16_rn(w[i]);
-        wf[((size_t)tap * cout + co) * cin + ci] = v;
-        if (wb) wb[((size_t)(8 - tap) * cin + ci) * cob + co] = v;
-    }
+    int l = 0;
+    while ((int)blockIdx.x >= Ls.first[l + 1]) ++l;
+    i = ((int)blockIdx.x - Ls.first[l]) * 32 + (threadIdx.x & 31);
+    return l;
+}
+
+// All of a training step that follows the weight-gradient kernels, in one
+// launch over the parameters of the four layers (before: four reductions,
+// Adam, three clears and four packings): the gradient from the block partials,
+// Adam (Kingma & Ba) on the FP32 master parameters, the BF16 copies.
+__global__ void __launch_bounds__(256) k_grad_adam_pack(const Layers Ls, float *__restrict__ w, float *__restrict__ g,
+                                                        float *__restrict__ m, float *__restrict__ v, float lr, float b1,
+                                                        float b2, float eps, float c1, float c2)
+{
+    pdl_wait();
+    pdl_next();
+    int i;
+    const Layer &L = Ls.l[layer_of(Ls, i)];
+    const int wlen = L.cout * 9 * L.cin, len = wlen + L.cout;
+    const float gi = reduce_parts(L.part, L.nparts, len, i);
+    if ((threadIdx.x >> 5) != 0 || i >= len) return;
+    const int k = i < wlen ? L.woff + i : L.boff + i - wlen;
+    g[k] = gi;
+    const float mi = b1 * m[k] + (1.f - b1) * gi;
+    const float vi = b2 * v[k] + (1.f - b2) * gi * gi;
+    m[k] = mi;
+    v[k] = vi;
+    const float wk = w[k] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    w[k] = wk;
+    if (i < wlen) pack_weight(L, i, wk);
+}
+
+__global__ void __launch_bounds__(32) k_pack(const Layers Ls, const float *__restrict__ w)
+{
+    int i;
+    const Layer &L = Ls.l[layer_of(Ls, i)];
+    if (i < L.cout * 9 * L.cin) pack_weight(L, i, w[L.woff + i]);
 }
 
 }  // namespace aaps
@@ -916,9 +1272,12 @@ cudaError_t conv_configure_all()
                               conv_configure<16, 8, MODE_LINEAR>()};
     for (cudaError_t e : es)
         if (e != cudaSuccess) return e;
-    return cudaSuccess;
+    return cudaFuncSetAttribute(k_net, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kNetSmem);
 }
 
+// An ordinary launch: as dependents of one another the persistent blocks start
+// on the first SMs with room and crowd there (10 applications at batch 32:
+// 1058 -> 1344 us).
 template <int CIN, int COUT, int MODE>
 cudaError_t conv(const bf16 *in, int B, int H, int W, const bf16 *w, const float *bias, bf16 *out, const bf16 *mask,
                  const float *rin, float *rout, cudaStream_t st)
@@ -927,16 +1286,23 @@ cudaError_t conv(const bf16 *in, int B, int H, int W, const bf16 *w, const float
     constexpr size_t smem = conv_ws_smem<CIN, COUT>();
     const cudaError_t ce = conv_configure<CIN, COUT, MODE>();
     if (ce != cudaSuccess) return ce;
-    k_conv_ws<CIN, COUT, MODE><<<std::min(ntiles, 2 * sm_count()), kConvThreads, smem, st>>>(in, H, W, ntiles, w, bias,
-                                                                                            out, mask, rin, rout);
+    const int grid = std::min(ntiles, 2 * sm_count());
+    k_conv_ws<CIN, COUT, MODE><<<grid, kConvThreads, smem, st>>>(in, H, W, ntiles, w, bias, out, mask, rin, rout);
     return cudaGetLastError();
+}
+
+// Blocks of the kernels that run over a batch's pixels.
+int pixel_blocks(int B, int H, int W)
+{
+    return (int)std::min<long long>(((long long)B * H * W + 255) / 256, 8 * sm_count());
 }
 
 int dw_rows(int H) { return H % 4 == 0 ? 4 : (H % 2 == 0 ? 2 : 1); }
 
+// The weight gradient's block partials; nblk: their number.
 template <int CIN, int COUT>
-cudaError_t conv_dw(const bf16 *x, const bf16 *dy, int dy_stride, int B, int H, int W, float *part, float *dw,
-                    float *db, cudaStream_t st)
+cudaError_t conv_dw_parts(const bf16 *x, const bf16 *dy, int dy_stride, int B, int H, int W, float *part, int &nblk,
+                          cudaStream_t st)
 {
     constexpr size_t smem = dw_tc_smem<CIN, COUT>();
     static std::atomic<int> configured{0};
@@ -949,13 +1315,20 @@ cudaError_t conv_dw(const bf16 *x, const bf16 *dy, int dy_stride, int B, int H, 
     const int ntiles = (W / kTW) * (H / kTH) * B;
     // one persistent block per SM (about 117 KB of shared memory each), no
     // more partials than the documented scratch holds
-    const int nblk = std::max(1, std::min(std::min(ntiles, sm_count()), (H / dw_rows(H)) * B));
+    nblk = std::max(1, std::min(std::min(ntiles, sm_count()), (H / dw_rows(H)) * B));
     k_conv_dw_tc<CIN, COUT><<<nblk, kDwThreads, smem, st>>>(x, dy, dy_stride, H, W, ntiles, part);
-    cudaError_t e = cudaGetLastError();
+    return cudaGetLastError();
+}
+
+template <int CIN, int COUT>
+cudaError_t conv_dw(const bf16 *x, const bf16 *dy, int dy_stride, int B, int H, int W, float *part, float *dw,
+                    float *db, cudaStream_t st)
+{
+    int nblk = 0;
+    const cudaError_t e = conv_dw_parts<CIN, COUT>(x, dy, dy_stride, B, H, W, part, nblk, st);
     if (e != cudaSuccess) return e;
     const int len = COUT * 9 * CIN + COUT;
-    k_reduce_parts<<<std::max(1, (len + 31) / 32), 256, 0, st>>>(part, nblk, len, dw, COUT * 9 * CIN, db);
-    return cudaGetLastError();
+    return launch_after(k_reduce_parts, std::max(1, (len + 31) / 32), 256, 0, st, part, nblk, len, dw, COUT * 9 * CIN, db);
 }
 
 bool valid_shape(int H, int W) { return H >= 16 && W >= 16 && H % 16 == 0 && W % 16 == 0 && H <= 4096 && W <= 4096; }
@@ -976,16 +1349,18 @@ struct aap_sur {
     bf16 *wf[4] = {}, *wb[4] = {};                                     // packed BF16 weights
     bf16 *x0 = nullptr, *a[3] = {}, *d[3] = {}, *dout = nullptr;       // activations and gradients
     float *state = nullptr, *state2 = nullptr, *target = nullptr, *eta = nullptr;
-    float *part = nullptr, *loss_part = nullptr;
+    float *part[4] = {}, *loss_part = nullptr;                         // weight-gradient partials of each layer
+    int nparts[4] = {};
+    float *h_loss = nullptr;                                           // page-locked: loss partials, wait flag
     float *dmean = nullptr;                                            // [max_batch * 3] projected gradient means
     float *cpart = nullptr;                                            // chunk sums of the projection
+    int *ncount = nullptr;                                             // tiles done per chunk (fused network)
     // the last predict call, captured as a CUDA graph (replayed while the
     // buffers, batch and number of applications stay the same)
     cudaGraphExec_t pexec = nullptr;
     cudaStream_t pstream = nullptr;
     const void *pkey[3] = {nullptr, nullptr, nullptr};
     int pbatch = -1, papps = -1;
-    size_t part_floats = 0;
     int loss_blocks = 0;
     long long t = 0;                                                   // Adam step
     std::vector<void *> allocs;
@@ -1012,6 +1387,8 @@ void sfree(aap_sur *s)
     s->pexec = nullptr;
     if (s->pstream) cudaStreamDestroy(s->pstream);
     s->pstream = nullptr;
+    if (s->h_loss) cudaFreeHost(s->h_loss);
+    s->h_loss = nullptr;
     for (void *q : s->allocs) cudaFree(q);
     s->allocs.clear();
 }
@@ -1020,21 +1397,38 @@ void sfree(aap_sur *s)
 // layer's 8 are padded to 16, the smallest input width of k_conv_ws).
 int cob_of(int l) { return std::max(kLayerCout[l], 16); }
 
+// The layers as the parameter kernels see them.
+Layers layers_of(const aap_sur *s)
+{
+    Layers Ls{};
+    for (int l = 0; l < 4; ++l) {
+        Layer &L = Ls.l[l];
+        L.cin = kLayerCin[l];
+        L.cout = kLayerCout[l];
+        L.cob = cob_of(l);
+        L.woff = (int)s->woff[l];
+        L.boff = (int)s->boff[l];
+        L.part = s->part[l];
+        L.nparts = s->nparts[l];
+        L.wf = s->wf[l];
+        L.wb = l > 0 ? s->wb[l] : nullptr;
+        Ls.first[l + 1] = Ls.first[l] + (L.cout * 9 * L.cin + L.cout + 31) / 32;
+    }
+    return Ls;
+}
+
 int pack_all(aap_sur *s)
 {
-    for (int l = 0; l < 4; ++l) {
-        const int n = kLayerCout[l] * 9 * kLayerCin[l];
-        if (l > 0) SCK(cudaMemsetAsync(s->wb[l], 0, (size_t)cob_of(l) * 9 * kLayerCin[l] * 2, s->stream));
-        k_pack<<<(n + 255) / 256, 256, 0, s->stream>>>(s->w + s->woff[l], kLayerCout[l], kLayerCin[l], s->wf[l],
-                                                       l > 0 ? s->wb[l] : nullptr, cob_of(l));
-        SCK(cudaGetLastError());
-    }
+    const Layers Ls = layers_of(s);
+    k_pack<<<Ls.first[4], 32, 0, s->stream>>>(Ls, s->w);
+    SCK(cudaGetLastError());
     return AAP_OK;
 }
 
 // Forward of `batch` samples from s->x0; the result (normalised state after
-// one application) goes to s->state2 from s->state.
-int forward(aap_sur *s, int batch)
+// one application) goes to s->state2 from s->state.  next: s->x0 becomes the
+// input of another application.
+int forward(aap_sur *s, int batch, bool next)
 {
     const int H = s->H, W = s->W;
     cudaStream_t st = s->stream;
@@ -1044,35 +1438,67 @@ int forward(aap_sur *s, int batch)
     SCK((conv<32, 8, MODE_RESID>(s->a[2], batch, H, W, s->wf[3], s->w + s->boff[3], nullptr, nullptr, s->state, s->state2, st)));
     if (s->p.conserve) {
         const int nchunk = (H * W + kCenterChunk - 1) / kCenterChunk;
-        k_center_part<<<batch * nchunk, 256, 0, st>>>(s->state2, s->state, H * W, nchunk, s->cpart);
-        k_center_apply<<<batch * nchunk, 256, 0, st>>>(s->state2, s->cpart, H * W, nchunk, s->p.conserve);
-        SCK(cudaGetLastError());
+        SCK(launch_after(k_center_part, batch * nchunk, 256, 0, st, s->state2, s->state, H * W, nchunk, s->cpart));
+        SCK(launch_after(k_center_apply, batch * nchunk, 256, 0, st, s->state2, s->cpart, H * W, nchunk, s->p.conserve,
+                         s->eta, (float)s->p.eta_center, (float)s->p.eta_scale, next ? s->x0 : nullptr));
+    } else if (next) {
+        SCK(launch_after(k_state_to_input, pixel_blocks(batch, H, W), 256, 0, st, s->state2, s->eta, batch, H, W,
+                         (float)s->p.eta_center, (float)s->p.eta_scale, s->x0));
     }
     return AAP_OK;
 }
+
+// A predict call of at most this many tiles per SM applies the network fused:
+// two waves of two blocks per SM; at 640 tiles layer by layer takes 391 us for
+// 10 applications where a third wave would take some 480.
+constexpr int kNetWaves = 4;
 
 // The kernels of one predict call on s->stream: normalise, `applications`
 // forward passes, denormalise into dev_out.
 int enqueue_predict(aap_sur *s, const float *dev_in, const float *dev_eta, int batch, int applications, float *dev_out)
 {
     const int H = s->H, W = s->W;
-    const int grid = 1024;
+    const int grid = pixel_blocks(batch, H, W);
     SCK(cudaMemcpyAsync(s->eta, dev_eta, (size_t)batch * 4, cudaMemcpyDeviceToDevice, s->stream));
-    k_fields_in<<<grid, 256, 0, s->stream>>>(dev_in, s->eta, batch, H, W, (float)s->p.rho0, (float)s->p.eta_center,
-                                             (float)s->p.eta_scale, s->state, s->x0);
-    SCK(cudaGetLastError());
-    for (int k = 0; k < applications; ++k) {
-        if (k > 0) {
-            k_state_to_input<<<grid, 256, 0, s->stream>>>(s->state, s->eta, batch, H, W, (float)s->p.eta_center,
-                                                          (float)s->p.eta_scale, s->x0);
-            SCK(cudaGetLastError());
+    const int tiles = batch * (W / kTW) * (H / kTH);
+    if (applications > 0 && tiles <= kNetWaves * sm_count()) {
+        NetArgs a{};
+        for (int l = 0; l < 4; ++l) {
+            a.wf[l] = s->wf[l];
+            a.bias[l] = s->w + s->boff[l];
         }
-        int rc = forward(s, batch);
+        a.eta = s->eta;
+        a.H = H;
+        a.W = W;
+        a.conserve = s->p.conserve;
+        a.rho0 = (float)s->p.rho0;
+        a.eta_c = (float)s->p.eta_center;
+        a.eta_s = (float)s->p.eta_scale;
+        const size_t chunks = (size_t)s->maxb * ((H * W + kCenterChunk - 1) / kCenterChunk);
+        float *raw[2] = {s->state, s->state2}, *part[2] = {s->cpart, s->cpart + 4 * chunks};
+        a.in_out = reinterpret_cast<float4 *>(s->target);
+        a.count = s->ncount;
+        for (int k = 0; k < applications; ++k) {
+            a.fields = k == 0 ? dev_in : nullptr;
+            a.raw_in = reinterpret_cast<const float4 *>(raw[k & 1]);
+            a.raw_out = reinterpret_cast<float4 *>(raw[(k & 1) ^ 1]);
+            a.part_in = k == 0 ? nullptr : part[k & 1];
+            a.part_out = part[(k & 1) ^ 1];
+            SCK(launch_after(k_net, tiles, kNetThreads, kNetSmem, s->stream, a));
+        }
+        const int o = applications & 1;
+        SCK(launch_after(k_net_out, batch * ((H * W + 255) / 256), 256, 0, s->stream,
+                         reinterpret_cast<const float4 *>(raw[o]), part[o], H, W, s->p.conserve, (float)s->p.rho0, dev_out));
+        return AAP_OK;
+    }
+    SCK(launch_after(k_fields_in, grid, 256, 0, s->stream, dev_in, s->eta, batch, H, W, (float)s->p.rho0,
+                     (float)s->p.eta_center, (float)s->p.eta_scale, s->state, s->x0));
+    for (int k = 0; k < applications; ++k) {
+        int rc = forward(s, batch, k + 1 < applications);
         if (rc) return rc;
         std::swap(s->state, s->state2);
     }
-    k_fields_out<<<grid, 256, 0, s->stream>>>(s->state, batch, H, W, (float)s->p.rho0, dev_out);
-    SCK(cudaGetLastError());
+    SCK(launch_after(k_fields_out, grid, 256, 0, s->stream, s->state, batch, H, W, (float)s->p.rho0, dev_out));
     return AAP_OK;
 }
 
@@ -1156,14 +1582,25 @@ int aap_sur_create(const aap_sur_params *p, void *stream, aap_sur **out)
     A(&s->target, pix * 8 * 4);
     A(&s->eta, (size_t)s->maxb * 4);
     // weight-gradient partials: one per block of the gradient kernel (at most
-    // one per row band and sample)
-    const size_t nblk = (size_t)(s->H / dw_rows(s->H)) * s->maxb;
-    s->part_floats = nblk * (32 * 9 * 32 + 32);
-    A(&s->part, s->part_floats * 4);
+    // one per SM, and one per row band and sample)
+    const size_t nblk = std::min<size_t>((size_t)sm_count(), (size_t)(s->H / dw_rows(s->H)) * s->maxb);
+    for (int l = 0; l < 4; ++l) A(&s->part[l], nblk * (kLayerCout[l] * 9 * kLayerCin[l] + kLayerCout[l]) * 4);
     s->loss_blocks = 256;
     A(&s->loss_part, (size_t)s->loss_blocks * 4);
     A(&s->dmean, (size_t)s->maxb * 3 * 4);
-    A(&s->cpart, (size_t)s->maxb * ((s->H * s->W + kCenterChunk - 1) / kCenterChunk) * 4 * 4);
+    const size_t chunks = (size_t)s->maxb * ((s->H * s->W + kCenterChunk - 1) / kCenterChunk);
+    A(&s->cpart, 2 * chunks * 4 * 4);       // two sets: the fused network reads one and writes the other
+    A(&s->ncount, chunks * 4);
+    if (!rc && cudaMallocHost(&s->h_loss, (s->loss_blocks + 1) * 4) != cudaSuccess) {
+        cudaGetLastError();
+        rc = sfail(AAP_ENOMEM, "page-locked loss buffer");
+    }
+    if (!rc && cudaMemsetAsync(s->ncount, 0, chunks * 4, s->stream) != cudaSuccess)
+        rc = sfail(AAP_ECUDA, "surrogate initialisation");
+    // the padded columns of the data-gradient weights stay zero
+    for (int l = 1; l < 4 && !rc; ++l)
+        if (cudaMemsetAsync(s->wb[l], 0, (size_t)cob_of(l) * 9 * kLayerCin[l] * 2, s->stream) != cudaSuccess)
+            rc = sfail(AAP_ECUDA, "surrogate initialisation");
     if (rc) {
         sfree(s);
         delete s;
@@ -1293,55 +1730,51 @@ int aap_sur_train_step(aap_sur *s, const float *dev_in, const float *dev_target,
     if (batch < 1 || batch > s->maxb) return sfail(AAP_EINVAL, "bad batch");
     const int H = s->H, W = s->W;
     cudaStream_t st = s->stream;
-    const int grid = 1024;
+    const int grid = pixel_blocks(batch, H, W);
     SCK(cudaMemcpyAsync(s->eta, dev_eta, (size_t)batch * 4, cudaMemcpyDeviceToDevice, st));
     // targets: normalised through the same path (x0 is overwritten below)
-    k_fields_in<<<grid, 256, 0, st>>>(dev_target, s->eta, batch, H, W, (float)s->p.rho0, (float)s->p.eta_center,
-                                      (float)s->p.eta_scale, s->target, s->x0);
-    k_fields_in<<<grid, 256, 0, st>>>(dev_in, s->eta, batch, H, W, (float)s->p.rho0, (float)s->p.eta_center,
-                                      (float)s->p.eta_scale, s->state, s->x0);
-    SCK(cudaGetLastError());
-    int rc = forward(s, batch);
+    SCK(launch_after(k_fields_in, grid, 256, 0, st, dev_target, s->eta, batch, H, W, (float)s->p.rho0,
+                     (float)s->p.eta_center, (float)s->p.eta_scale, s->target, s->x0));
+    SCK(launch_after(k_fields_in, grid, 256, 0, st, dev_in, s->eta, batch, H, W, (float)s->p.rho0,
+                     (float)s->p.eta_center, (float)s->p.eta_scale, s->state, s->x0));
+    int rc = forward(s, batch, false);
     if (rc) return rc;
     const long long npix = (long long)batch * H * W;
     if (s->p.conserve) {
         const int nchunk = (H * W + kCenterChunk - 1) / kCenterChunk;
-        k_center_part<<<batch * nchunk, 256, 0, st>>>(s->state2, s->target, H * W, nchunk, s->cpart);
-        k_dmean<<<(batch * 3 + 127) / 128, 128, 0, st>>>(s->cpart, batch, H * W, nchunk, s->p.conserve, s->dmean);
-        SCK(cudaGetLastError());
+        SCK(launch_after(k_center_part, batch * nchunk, 256, 0, st, s->state2, s->target, H * W, nchunk, s->cpart));
+        SCK(launch_after(k_dmean, (batch * 3 + 127) / 128, 128, 0, st, s->cpart, batch, H * W, nchunk, s->p.conserve,
+                         s->dmean));
     }
-    k_mse<<<s->loss_blocks, 256, 0, st>>>(s->state2, s->target, npix, (float)(1.0 / (3.0 * (double)npix)),
-                                          s->loss_part, s->dout, s->p.conserve ? s->dmean : nullptr, H * W);
-    SCK(cudaGetLastError());
-    float *g = s->g;
+    SCK(launch_after(k_mse, s->loss_blocks, 256, 0, st, s->state2, s->target, npix, (float)(1.0 / (3.0 * (double)npix)),
+                     s->loss_part, s->dout, s->p.conserve ? s->dmean : nullptr, H * W));
     // layer 4: weight gradient from a[2] and dout (16-channel pixels, 8 used);
     // data gradient through the flipped weights, masked by ReLU(a[2]) > 0
-    SCK((conv_dw<32, 8>(s->a[2], s->dout, 16, batch, H, W, s->part, g + s->woff[3], g + s->boff[3], st)));
+    SCK((conv_dw_parts<32, 8>(s->a[2], s->dout, 16, batch, H, W, s->part[3], s->nparts[3], st)));
     SCK((conv<16, 32, MODE_MASK>(s->dout, batch, H, W, s->wb[3], nullptr, s->d[2], s->a[2], nullptr, nullptr, st)));
     // layer 3
-    SCK((conv_dw<32, 32>(s->a[1], s->d[2], 32, batch, H, W, s->part, g + s->woff[2], g + s->boff[2], st)));
+    SCK((conv_dw_parts<32, 32>(s->a[1], s->d[2], 32, batch, H, W, s->part[2], s->nparts[2], st)));
     SCK((conv<32, 32, MODE_MASK>(s->d[2], batch, H, W, s->wb[2], nullptr, s->d[1], s->a[1], nullptr, nullptr, st)));
     // layer 2
-    SCK((conv_dw<32, 32>(s->a[0], s->d[1], 32, batch, H, W, s->part, g + s->woff[1], g + s->boff[1], st)));
+    SCK((conv_dw_parts<32, 32>(s->a[0], s->d[1], 32, batch, H, W, s->part[1], s->nparts[1], st)));
     SCK((conv<32, 32, MODE_MASK>(s->d[1], batch, H, W, s->wb[1], nullptr, s->d[0], s->a[0], nullptr, nullptr, st)));
     // layer 1 (its input needs no gradient)
-    SCK((conv_dw<16, 32>(s->x0, s->d[0], 32, batch, H, W, s->part, g + s->woff[0], g + s->boff[0], st)));
-    // Adam step and the BF16 copies
+    SCK((conv_dw_parts<16, 32>(s->x0, s->d[0], 32, batch, H, W, s->part[0], s->nparts[0], st)));
+    // gradients, Adam step and the BF16 copies
     s->t += 1;
     const double c1 = 1.0 - std::pow(s->p.beta1, (double)s->t), c2 = 1.0 - std::pow(s->p.beta2, (double)s->t);
-    k_adam<<<(int)std::min<long long>(1024, (s->nparam + 255) / 256), 256, 0, st>>>(
-        s->w, s->g, s->m, s->v, (int)s->nparam, (float)s->p.lr, (float)s->p.beta1, (float)s->p.beta2,
-        (float)s->p.eps, (float)c1, (float)c2);
-    SCK(cudaGetLastError());
-    if ((rc = pack_all(s))) return rc;
+    const Layers Ls = layers_of(s);
+    SCK(launch_after(k_grad_adam_pack, Ls.first[4], 256, 0, st, Ls, s->w, s->g, s->m, s->v, (float)s->p.lr,
+                     (float)s->p.beta1, (float)s->p.beta2, (float)s->p.eps, (float)c1, (float)c2));
     if (loss_out) {
-        std::vector<float> lp(s->loss_blocks);
-        SCK(cudaMemcpyAsync(lp.data(), s->loss_part, lp.size() * 4, cudaMemcpyDeviceToHost, st));
+        int *flag = reinterpret_cast<int *>(s->h_loss + s->loss_blocks);
+        SCK(cudaMemcpyAsync(s->h_loss, s->loss_part, s->loss_blocks * 4, cudaMemcpyDeviceToHost, st));
+        SCK(cudaMemcpyFromSymbolAsync(flag, g_sur_err, sizeof(int), 0, cudaMemcpyDeviceToHost, st));
         SCK(cudaStreamSynchronize(st));
         double tot = 0.0;
-        for (float v : lp) tot += v;
+        for (int k = 0; k < s->loss_blocks; ++k) tot += s->h_loss[k];
         *loss_out = tot / (3.0 * (double)npix);
-        return check_tc(st);
+        if (*flag) return sfail(AAP_ETIMEOUT, "a tensor-core completion wait gave up");
     }
     return AAP_OK;
 }

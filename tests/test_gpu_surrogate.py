@@ -388,3 +388,24 @@ def test_predict_replays_its_graph(lib):
         assert np.allclose(x.cpu().numpy(), first.cpu().numpy(), rtol=1e-4, atol=1e-4)
     finally:
         A.aap_sur_destroy(s)
+
+
+@pytest.mark.parametrize("h,w,apps,conserve", [(16, 16, 1, 0), (16, 32, 3, 3), (48, 16, 2, 1), (128, 128, 1, 3), (64, 80, 4, 0),
+                                               (48, 80, 3, 3), (176, 112, 2, 2), (16, 256, 2, 3)])
+def test_fused_network_equals_layer_by_layer(h, w, apps, conserve):
+    """A small call applies the network fused, one of many samples layer by
+    layer: the same samples give the same fields bit for bit (the same BF16
+    operands, the same order of the FP32 sums, the projection's included)."""
+    g = np.random.default_rng(h + w + apps)
+    many = 4 * 160 * 128 // (h * w) + 3                       # more than four tiles of 128 pixels per SM
+    f = torch.tensor(np.abs(g.normal(size=(many, 3, h, w))) + 0.5, dtype=torch.float32, device="cuda")
+    eta = torch.tensor(g.uniform(0.3, 0.5, many), dtype=torch.float32, device="cuda")
+    s = A.aap_sur_create(A.aap_sur_params_default(nbx=w, nby=h, max_batch=many, conserve=conserve))
+    try:
+        big, small = torch.empty_like(f), torch.empty_like(f[:2])
+        A.aap_sur_predict(s, f.data_ptr(), eta.data_ptr(), many, apps, big.data_ptr())
+        A.aap_sur_predict(s, f.data_ptr(), eta.data_ptr(), 2, apps, small.data_ptr())
+        torch.cuda.synchronize()
+        assert torch.equal(big[:2], small)
+    finally:
+        A.aap_sur_destroy(s)
