@@ -138,8 +138,8 @@ struct Ctl {
     long long step;             // steps taken; parity selects the current buffer
     int tile_next;              // dynamic tile fetch of the step kernel
     int finish_ticket;
-    int dense_count;            // pipelined step: tiles listed for the whole-block routine
-    int dense_next;             // ... and taken
+    alignas(8) int dense_count; // pipelined step: tiles listed for the whole-block routine
+    int dense_next;             // ... and taken (read together)
     int pad[2];
 };
 

@@ -123,7 +123,7 @@ k_step(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_base,
 // range over all systems' tiles; the warps of all blocks take one system each
 // for the sums (its 64 accumulator slots loaded at once, then cleared); the
 // last block to arrive advances the step.
-__global__ void k_finish(Sys *sys, int nsys, const int *__restrict__ tile_base, Ctl *ctl)
+__global__ void __launch_bounds__(1024) k_finish(Sys *sys, int nsys, const int *__restrict__ tile_base, Ctl *ctl)
 {
     __shared__ int s_last;
     pdl_wait();
@@ -157,12 +157,17 @@ __global__ void k_finish(Sys *sys, int nsys, const int *__restrict__ tile_base, 
         close_sums(S, step, lane);
         if (lane == 0) S.spill_cnt[cur] = 0;
     }
+    // the step advances when every block is done with it (a single block: at
+    // once, without the fence and the ticket's round trip)
+    if (threadIdx.x == 0) s_last = 1;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_last = (atomicAdd(&ctl->finish_ticket, 1) == (int)gridDim.x - 1);
+    if (gridDim.x > 1) {
+        if (threadIdx.x == 0) {
+            __threadfence();
+            s_last = (atomicAdd(&ctl->finish_ticket, 1) == (int)gridDim.x - 1);
+        }
+        __syncthreads();
     }
-    __syncthreads();
     if (s_last && threadIdx.x == 0) {
         ctl->tile_next = 0;
         ctl->finish_ticket = 0;
@@ -435,7 +440,7 @@ static cudaError_t launch_step_t(const LaunchCfg &L, cudaStream_t st, cudaEvent_
     }
     if (e != cudaSuccess) return e;
     if (ev && (e = cudaEventRecord(ev[1], st)) != cudaSuccess) return e;
-    e = launch_after(k_finish, L.grid_finish, 256, 0, st, L.sys, L.nsys, L.tile_base, L.ctl);
+    e = launch_after(k_finish, L.grid_finish, L.grid_finish == 1 ? 1024 : 256, 0, st, L.sys, L.nsys, L.tile_base, L.ctl);
     if (e != cudaSuccess) return e;
     if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
     return cudaSuccess;
@@ -457,7 +462,7 @@ cudaError_t launch_step(const LaunchCfg &L, cudaStream_t st, cudaEvent_t *ev)
     if (L.knn > 0) {
         cudaError_t e = launch_mf_step(L, st, ev);
         if (e != cudaSuccess) return e;
-        e = launch_after(k_finish, L.grid_finish, 256, 0, st, L.sys, L.nsys, L.tile_base, L.ctl);
+        e = launch_after(k_finish, L.grid_finish, L.grid_finish == 1 ? 1024 : 256, 0, st, L.sys, L.nsys, L.tile_base, L.ctl);
         if (e != cudaSuccess) return e;
         if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
         return cudaSuccess;

@@ -136,6 +136,9 @@ struct PipeShared {
     OutMeta out[2];
     int chunk[2];               // next chunk of 32 own particles, per output buffer
     int flag;                   // a previous step's wait ran out
+    int total;                  // tiles of the launch
+    long long step;
+    int dense_any;              // tiles were listed for the whole-block routine
     int dense_tile;
     int load, staged;           // largest tile load and staged set of the block's tiles
     int warp_tot[kPipeWarps];
@@ -590,7 +593,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
         for (int b = 0; b < 2; ++b) {
             mbar_init(&sh.bar_full[b], 1);
             mbar_init(&sh.bar_empty[b], NU);
-            sh.osys[b] = -1;
+            if (nsys > 1) sh.osys[b] = -1;
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -598,19 +601,37 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
     for (int i = tid; i < 2 * B.mh_stride; i += kPipeThreads) B.mhist0[i] = 0;
     pdl_wait();         // the step before is closed
     pdl_next();
+    // everything the roles start with is read side by side (a step of a few
+    // tiles per SM waits for these loads): the first tile's claim, the system
+    // (one system: its copy and both output buffers' copies), the step, the
+    // tile count and the error word
     // pipeline waits that run out are reported in the first system's error word
     int *const err0 = sys[0].err;
-    if (tid == 0) {
+    int g0 = 0;
+    if (warp == 0) {
+        if (lane == 0) g0 = atomicAdd(&ctl->tile_next, 1);
+        g0 = __shfl_sync(0xffffffffu, g0, 0);
+    } else if (tid == kPipeThreads - 1) {
         sh.flag = *((volatile int *)err0) & ERR_TIMEOUT;
         sh.load = sh.staged = 0;
+    } else if (tid == kPipeThreads - 33) {
+        sh.step = ctl->step;
+    } else if (tid == kPipeThreads - 65) {
+        sh.total = tile_base[nsys];
+    } else if (nsys == 1 && warp <= 24) {
+        const int words = (int)(sizeof(Sys) / 4), k = (warp - 1) / 8;       // eight warps a copy
+        const int *src = reinterpret_cast<const int *>(sys);
+        int *dst = reinterpret_cast<int *>(k == 0 ? &sh.cs : &sh.os[k - 1]);
+        for (int i = tid - 32 - 256 * k; i < words; i += 256) dst[i] = src[i];
+        if (lane == 0 && k > 0 && (warp & 7) == 1) sh.osys[k - 1] = 0;
     }
     __syncthreads();
     // after a wait has run out the handle is unusable: later steps do nothing
     // (so that a queue of steps cannot each wait out their bounds)
     if (sh.flag) return;
-    const long long step = ctl->step;
+    const long long step = sh.step;
     const int cur = (int)(step & 1);
-    const int total = tile_base[nsys];
+    const int total = sh.total;
     unsigned char *mine = scratch + scratch_per_block * blockIdx.x;
 
     if (warp == 0) {
@@ -626,12 +647,14 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
         unsigned char *spill_s = reinterpret_cast<unsigned char *>(spill_e + kPipeMaxSpill);
         unsigned kpar = 0, used = 0;       // per raw buffer: parity of its fills, filled before
         int r = 0;
-        int g = 0;
-        if (lane == 0) g = atomicAdd(&ctl->tile_next, 1);
-        g = __shfl_sync(0xffffffffu, g, 0);
+        int g = g0;
         // the planned tile: its system, local index and the system's spill
         // list length (final during this step), re-read when the system changes
         int si = -1, lt = 0, nsp = 0;
+        if (nsys == 1) {
+            si = 0;
+            nsp = *((volatile int *)&sh.cs.spill_cnt[cur]);
+        }
         CopyPlan pl;
         const Sys &Sc = sh.cs;
         auto plan = [&](int gg) {
@@ -643,7 +666,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
                 int *dst = reinterpret_cast<int *>(&sh.cs);
                 for (int i = lane; i < words; i += 32) dst[i] = src[i];
                 __syncwarp();
-                nsp = min(*((volatile int *)&Sc.spill_cnt[cur]), Sc.spill_cap);
+                nsp = *((volatile int *)&Sc.spill_cnt[cur]);
             }
             lt = gg - (nsys > 1 ? tile_base[si] : 0);
             copy_plan(Sc, lt, cur, pl);
@@ -658,7 +681,8 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
             if (g < total && lane == 0) gn = atomicAdd(&ctl->tile_next, 1);
             int n_spill = 0, n_own = 0, mode = 0;               // 0: whole-block list, 1: normal, 2: wide
             if (g < total) {
-                const bool scanned = copy_spills(Sc, pl, cur, nsp, spill_e, spill_s, n_spill, n_own);
+                const bool scanned = copy_spills(Sc, pl, cur, min(nsp, Sc.spill_cap), spill_e, spill_s, n_spill,
+                                                 n_own);
                 const int m = pl.m_seg + n_spill;
                 if (scanned && n_spill <= kPipeMaxSpill) {
                     if (m <= cap && n_own <= cap_own) mode = 1;
@@ -767,6 +791,12 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
             // latest and the bounded wait returns at once.
             for (int b = 0; b < kNR; ++b)
                 if ((used >> b) & 1u) warp_wait(&sh.bar_raw_full[b], ((kpar >> b) & 1u) ^ 1u, err0);
+        }
+        // whether a listed tile is left, looked up while the last tiles are
+        // updated (a block that lists one later does it itself)
+        if (lane == 0) {
+            const long long d = *((volatile long long *)&ctl->dense_count);     // dense_count, dense_next
+            sh.dense_any = (int)(d >> 32) < (int)d;
         }
         if (lane == 0) PT_ADD(0, PT_NOW() - tc0);
     } else if (warp <= NSORT) {
@@ -922,6 +952,16 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
 
     // --- tiles too large for the pipeline's buffers: the whole block, with
     //     the shared staging area or the block's global scratch ------------
+    if (!sh.dense_any) {
+        // what the host goes by when it chooses between this kernel and many
+        // steps per launch (a single system)
+        if (nsys == 1 && tid == 0 && sh.staged > 0) {
+            atomicMax(err0 + 1, sh.load);
+            atomicMax(err0 + 2, sh.staged);
+        }
+        if (tid == 0) PT_ADD(12, PT_NOW() - tk0);
+        return;
+    }
     __shared__ TileCtx T;
     const size_t tbytes = table_bytes(nce_max, hist_words);
     const size_t dyn = pipe_smem_bytes(cap, cap_own, nceh_max, hist_words);
@@ -999,9 +1039,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
         if (tid == 0) PT_ADD(11, 1);
         __syncthreads();
     }
-    // what the host goes by when it chooses between this kernel and many steps
-    // per launch (a single system)
-    if (nsys == 1 && tid == 0 && sh.staged > 0) {
+    if (nsys == 1 && tid == 0) {
         atomicMax(err0 + 1, sh.load);
         atomicMax(err0 + 2, sh.staged);
     }
