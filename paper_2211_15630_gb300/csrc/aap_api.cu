@@ -69,6 +69,7 @@ struct aap_handle {
     int *d_x0tab = nullptr, *d_y0tab = nullptr;
     unsigned char *d_scratch = nullptr;
     int *d_dense = nullptr;             // pipelined step: tiles left to the whole-block routine
+    int *d_order = nullptr;             // pipelined step: the order in which tiles are claimed
     int *d_multi = nullptr;             // many steps per launch: private counters and barrier
     unsigned long long *d_obs = nullptr;
     int *d_seen = nullptr;
@@ -670,6 +671,7 @@ int alloc_all(aap_handle *h)
         if ((rc = dev_alloc(h, &h->d_ctl, sizeof(Ctl)))) return rc;
         if ((rc = dev_alloc(h, &h->d_dense, (size_t)std::max(S.ntiles, 1) * sizeof(int)))) return rc;
         AAP_CK(cudaMemsetAsync(h->d_dense, 0, (size_t)std::max(S.ntiles, 1) * sizeof(int), h->stream));
+        if (h->L.pipe && (rc = dev_alloc(h, &h->d_order, 2 * (size_t)std::max(S.ntiles, 1) * sizeof(int)))) return rc;
         if (h->L.multi && (rc = dev_alloc(h, &h->d_multi, aapk::multi_bytes(S.ntiles)))) return rc;
     }
     if ((rc = dev_alloc(h, &h->d_x0tab, (size_t)(S.ntx + 1) * sizeof(int)))) return rc;
@@ -704,6 +706,8 @@ int alloc_all(aap_handle *h)
     L.tile_base = h->d_tile_base;
     L.ctl = h->d_ctl;
     L.dense_list = h->d_dense;
+    L.order = h->d_order;
+    L.order_tiles = S.ntiles;
     L.multi_cnt = h->d_multi;
     return push_sys(h);
 }
@@ -851,6 +855,7 @@ int run_steps_adaptive(aap_handle *h, long long nsteps)
         h->since_copy += k;
         if (h->since_copy < kAdaptSteps) continue;
         h->since_copy = 0;
+        if (h->L.pipe && !use_multi(h)) AAP_CK(aapk::launch_tile_order(h->L, h->stream));
         const int slot = h->batch_slot;
         if ((rc = copy_words(h, h->pinned_err + 4 * (1 + slot)))) return rc;
         AAP_CK(cudaEventRecord(h->batch_ev[slot], h->stream));
@@ -969,6 +974,7 @@ int reinsert(aap_handle *h, double factor, int mode)
         // capacity, or when doubling the regions would exceed the staged indices
         if (!spilled || (!(err & aapk::ERR_LOST) && (h->p.capacity > 0 || !capacity_fits(h, factor * 2.0)))) {
             h->factor = factor;
+            if (!h->member && h->L.pipe) AAP_CK(aapk::launch_tile_order(h->L, h->stream));
             return AAP_OK;
         }
         if (h->p.capacity > 0) return fail(AAP_EOVERFLOW, "the particles do not fit the explicit capacity");
@@ -1107,7 +1113,7 @@ struct aap_ens {
     Ctl *d_ctl = nullptr;
     unsigned char *d_scratch = nullptr;
     size_t scratch_bytes = 0;
-    int *d_dense = nullptr;             // pipelined step: tiles left to the whole-block routine
+    int *d_dense = nullptr;             // pipelined step: tiles left to the whole-block routine; their order
     size_t dense_tiles = 0;
     std::vector<int> order;             // replicas in the order of their descriptors (densest first)
     int *d_err = nullptr;               // [count + 4] the replicas' error words
@@ -1243,7 +1249,7 @@ int ens_combine(aap_ens *e)
             if (e->d_dense) cudaFree(e->d_dense);
             e->d_dense = nullptr;
             e->dense_tiles = 0;
-            if (cudaMalloc(&e->d_dense, (size_t)total * sizeof(int)) != cudaSuccess) {
+            if (cudaMalloc(&e->d_dense, 3 * (size_t)total * sizeof(int)) != cudaSuccess) {
                 cudaGetLastError();
                 return fail(AAP_ENOMEM, "ensemble tile list allocation failed");
             }
@@ -1251,10 +1257,14 @@ int ens_combine(aap_ens *e)
         }
         AAP_CK(cudaMemset(e->d_dense, 0, (size_t)total * sizeof(int)));
         L.dense_list = e->d_dense;
+        L.order = e->d_dense + total;
+        L.order_tiles = (int)total;
+        AAP_CK(cudaStreamSynchronize(e->stream));
         int rc = set_pipe_launch(L, false, twmax, thmax, (int)total);
         if (rc) return rc;
         if (!L.pipe && e->params[0].threads == 1024)
             return fail(AAP_EINVAL, "the pipelined step kernel does not fit this ensemble's tiling");
+        if (L.pipe) AAP_CK(aapk::launch_tile_order(L, e->stream));
     }
     if (e->exec) cudaGraphExecDestroy(e->exec);
     e->exec = nullptr;
@@ -1874,6 +1884,7 @@ int aap_ens_step(aap_ens *e, int64_t nsteps)
         e->since_copy += k;
         if (e->since_copy < kAdaptSteps) continue;
         e->since_copy = 0;
+        if (e->L.pipe) AAP_CK(aapk::launch_tile_order(e->L, e->stream));
         const int slot = e->batch_slot;
         AAP_CK(cudaMemcpyAsync(e->pinned_err + (1 + slot) * count, e->d_err, count * sizeof(int),
                                cudaMemcpyDeviceToHost, e->stream));

@@ -177,6 +177,82 @@ __global__ void __launch_bounds__(1024) k_finish(Sys *sys, int nsys, const int *
     }
 }
 
+// ------------------------------------------------------- order of the tiles --
+// The order in which the pipelined step claims tiles: a step ends when its
+// longest tile does, so the longest start first.  One block sorts the tiles of
+// all systems by the class of their cost (two classes per factor of two),
+// stable inside a class, so that neighbours stay together: states that outgrow
+// the L2 keep the raster order but for tiles of more than about twice the mean
+// cost (their halo regions are read while they are there).  Run every few
+// dozen steps: loads change slowly.  order: [total], cost: [total] scratch.
+__global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys, int nsys,
+                                                     const int *__restrict__ tile_base, const Ctl *__restrict__ ctl,
+                                                     int *order, float *cost)
+{
+    constexpr int kClasses = 16;
+    __shared__ float s_sum[32];
+    __shared__ int s_cnt[kClasses], s_warp[32][kClasses];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int b = (int)(ctl->step & 1), total = tile_base[nsys];
+    float sum = 0.f;
+    for (int g = tid; g < total; g += 1024) {
+        const int si = nsys > 1 ? sys_of_tile(tile_base, nsys, g) : 0;
+        const Sys &S = sys[si];
+        const int *c = S.cnt[b] + (size_t)(g - tile_base[si]) * kCntStride;
+        int own = 0;
+#pragma unroll
+        for (int r = 0; r < kRegions; ++r) own += c[r];
+        // staging and update per particle, and the candidates of 15 half cells
+        const float f = (float)own * (24.0f + 7.5f * (float)own / (float)(S.twmax * S.thmax));
+        cost[g] = f;
+        sum += f;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) s_sum[warp] = sum;
+    if (tid < kClasses) s_cnt[tid] = 0;
+    __syncthreads();
+    float mean = 0.f;
+    for (int w = 0; w < 32; ++w) mean += s_sum[w];
+    mean = fmaxf(mean / (float)max(total, 1), 1e-20f);
+    const int kmax = total <= 4096 ? kClasses - 1 : 6;
+    const auto cls = [&](float f) {
+        return min(max((int)floorf(8.0f - 2.0f * __log2f(fmaxf(f, 1e-20f) / mean)), 0), kmax);
+    };
+    for (int g = tid; g < total; g += 1024) atomicAdd(&s_cnt[cls(cost[g])], 1);
+    __syncthreads();
+    if (tid == 0) {
+        int run = 0;
+        for (int k = 0; k < kClasses; ++k) {
+            const int n = s_cnt[k];
+            s_cnt[k] = run;
+            run += n;
+        }
+    }
+    __syncthreads();
+    for (int g0 = 0; g0 < total; g0 += 1024) {
+        const int g = g0 + tid;
+        const int k = g < total ? cls(cost[g]) : -1;
+        const unsigned peers = __match_any_sync(0xffffffffu, k);
+        if (lane < kClasses) s_warp[warp][lane] = 0;
+        __syncwarp();
+        if (k >= 0 && lane == __ffs(peers) - 1) s_warp[warp][k] = __popc(peers);
+        __syncthreads();
+        if (tid < kClasses) {
+            int run = s_cnt[tid];
+            for (int w = 0; w < 32; ++w) {
+                const int n = s_warp[w][tid];
+                s_warp[w][tid] = run;
+                run += n;
+            }
+            s_cnt[tid] = run;
+        }
+        __syncthreads();
+        if (k >= 0) order[s_warp[warp][k] + __popc(peers & ((1u << lane) - 1u))] = g;
+        __syncthreads();
+    }
+}
+
 // ------------------------------------------------- state in and out --------
 // llrint(p / cs * scale), scale a power of two, without the FP64 division (the
 // FP64 pipe is narrow on this GPU; two divisions a particle took most of the
@@ -513,6 +589,12 @@ cudaError_t launch_insert(const Sys &S, int b, const double *x, const double *y,
     const int bs = 256;
     const long long grid = (n + bs - 1) / bs;
     k_insert<<<(unsigned)grid, bs, 0, st>>>(S, b, x, y, th, mode, 1.0 / S.csx_d, 1.0 / S.csy_d);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_tile_order(const LaunchCfg &L, cudaStream_t st)
+{
+    k_tile_order<<<1, 1024, 0, st>>>(L.sys, L.nsys, L.tile_base, L.ctl, L.order, reinterpret_cast<float *>(L.order + L.order_tiles));
     return cudaGetLastError();
 }
 

@@ -31,6 +31,8 @@ struct LaunchCfg {
     int pipe_cap, pipe_cap_own, pipe_grid;
     int pipe_nceh;               // half cells (split along x) of the largest extended tile, (2 tw + 4)(th + 2)
     int *dense_list;
+    int *order;                  // device [2 * order_tiles]: the order in which tiles are claimed; scratch
+    int order_tiles;
     // many steps per launch (a small system, one block per tile, all resident)
     int multi, multi_species, multi_cap, multi_tiles, multi_threads;
     int *multi_cnt;              // device: three private counter sets and two barrier words, zero between launches
@@ -96,6 +98,8 @@ cudaError_t launch_mf_step(const LaunchCfg &L, cudaStream_t st, cudaEvent_t *ev)
 
 cudaError_t launch_insert(const Sys &S, int b, const double *x, const double *y, const float *th,
                           int mode, cudaStream_t st);
+// The order in which the pipelined step claims the tiles of its systems, from their current loads.
+cudaError_t launch_tile_order(const LaunchCfg &L, cudaStream_t st);
 // The largest tile load and staged set of buffer b into S.err[1] and [2].
 cudaError_t launch_tile_load(const Sys &S, int b, cudaStream_t st);
 // bad[0]: the lowest index with a position outside [0, lx] x [0, ly]; bad[1]:

@@ -573,7 +573,7 @@ __device__ __forceinline__ void flush_hist(PipeShared &sh, const PipeBufs &B, in
 template <int MODEL, bool SP, int NSORT>
 __global__ void __launch_bounds__(kPipeThreads, 1)
 k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_base, Ctl *ctl, int cap, int cap_own,
-            int nceh_max, int nce_max, int hist_words, int *dense_list, unsigned char *scratch,
+            int nceh_max, int nce_max, int hist_words, const int *__restrict__ order, int *dense_list, unsigned char *scratch,
             size_t scratch_per_block, int scratch_cap, int spill_list_cap)
 {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -607,10 +607,15 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
     // tile count and the error word
     // pipeline waits that run out are reported in the first system's error word
     int *const err0 = sys[0].err;
-    int g0 = 0;
+    int g0 = 0, t0 = 0;
     if (warp == 0) {
-        if (lane == 0) g0 = atomicAdd(&ctl->tile_next, 1);
+        // tiles are claimed in `order`, the longest first (k_tile_order)
+        if (lane == 0) {
+            g0 = atomicAdd(&ctl->tile_next, 1);
+            t0 = g0 < tile_base[nsys] ? order[g0] : 0;
+        }
         g0 = __shfl_sync(0xffffffffu, g0, 0);
+        t0 = __shfl_sync(0xffffffffu, t0, 0);
     } else if (tid == kPipeThreads - 1) {
         sh.flag = *((volatile int *)err0) & ERR_TIMEOUT;
         sh.load = sh.staged = 0;
@@ -647,7 +652,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
         unsigned char *spill_s = reinterpret_cast<unsigned char *>(spill_e + kPipeMaxSpill);
         unsigned kpar = 0, used = 0;       // per raw buffer: parity of its fills, filled before
         int r = 0;
-        int g = g0;
+        int g = g0, gt = t0;               // the claim, and the tile it stands for
         // the planned tile: its system, local index and the system's spill
         // list length (final during this step), re-read when the system changes
         int si = -1, lt = 0, nsp = 0;
@@ -672,7 +677,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
             copy_plan(Sc, lt, cur, pl);
         };
         const long long tc0 = PT_NOW();
-        if (g < total) plan(g);
+        if (g < total) plan(gt);
         bool ok = true;
         bool withhold = c_pipe_stall != 0;
         for (;;) {
@@ -692,10 +697,13 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
                     // done by the whole block after the pipeline
                     if (lane == 0) {
                         const int j = atomicAdd(&ctl->dense_count, 1);
-                        dense_list[j] = g + 1;
+                        dense_list[j] = gt + 1;
                     }
+                    int tn = 0;
+                    if (lane == 0 && gn < total) tn = order[gn];
                     g = __shfl_sync(0xffffffffu, gn, 0);
-                    if (g < total) plan(g);
+                    gt = __shfl_sync(0xffffffffu, tn, 0);
+                    if (g < total) plan(gt);
                     continue;
                 }
                 if (mode == 2 && r == kNR - 1) {
@@ -737,6 +745,8 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
             const Sys &Sg = Sc;
             const long long ts0 = PT_NOW();
             copy_commit(pl, Sg, si, lt, M, n_spill, n_own, mode == 2, spill_s);
+            int tn = 0;
+            if (lane == 0 && gn < total) tn = order[gn];        // in flight beside the copies
             if (lane == 0) PT_ADD(2, PT_NOW() - ts0);
             const long long ti0 = PT_NOW();
             int4 *R = B.raw(r);
@@ -777,7 +787,8 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
             const long long tq0 = PT_NOW();
             g = __shfl_sync(0xffffffffu, gn, 0);
             const long long tq1 = PT_NOW();
-            if (g < total) plan(g);
+            gt = __shfl_sync(0xffffffffu, tn, 0);
+            if (g < total) plan(gt);
             if (lane == 0) {
                 PT_ADD(13, tq1 - tq0);
                 PT_ADD(14, PT_NOW() - tq1);
@@ -1108,7 +1119,7 @@ static cudaError_t launch_pipe_t(const LaunchCfg &L, cudaStream_t st)
     const size_t smem = pipe_smem_bytes(L.pipe_cap, L.pipe_cap_own, L.pipe_nceh, L.hist_words);
     return launch_after(k_step_pipe<MODEL, kSpecies, AAP_PIPE_SORT_WARPS>, L.pipe_grid, kPipeThreads, smem, st, L.sys, L.nsys,
                         L.tile_base, L.ctl, L.pipe_cap, L.pipe_cap_own, L.pipe_nceh, L.nce_max, L.hist_words,
-                        L.dense_list, L.scratch, L.scratch_per_block, L.scratch_cap, L.spill_list_cap);
+                        L.order, L.dense_list, L.scratch, L.scratch_per_block, L.scratch_cap, L.spill_list_cap);
 }
 
 cudaError_t PIPE_FN(launch_step_pipe)(const LaunchCfg &L, cudaStream_t st)
