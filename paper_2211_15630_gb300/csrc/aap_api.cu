@@ -106,6 +106,7 @@ struct aap_handle {
     long long since_copy = 0;       // steps queued since the last copy
     bool err_pending = false;
     int relayouts = 0;
+    int order_age = 0;
     bool multi_on = true;           // the tiles are light enough for many steps per launch
     // ensemble membership: steps are launched by the ensemble for all members,
     // whose error words and measurement sums lie side by side in its arrays
@@ -671,7 +672,7 @@ int alloc_all(aap_handle *h)
         if ((rc = dev_alloc(h, &h->d_ctl, sizeof(Ctl)))) return rc;
         if ((rc = dev_alloc(h, &h->d_dense, (size_t)std::max(S.ntiles, 1) * sizeof(int)))) return rc;
         AAP_CK(cudaMemsetAsync(h->d_dense, 0, (size_t)std::max(S.ntiles, 1) * sizeof(int), h->stream));
-        if (h->L.pipe && (rc = dev_alloc(h, &h->d_order, 2 * (size_t)std::max(S.ntiles, 1) * sizeof(int)))) return rc;
+        if (h->L.pipe && (rc = dev_alloc(h, &h->d_order, (2 * (size_t)std::max(S.ntiles, 1) + 1) * sizeof(int)))) return rc;
         if (h->L.multi && (rc = dev_alloc(h, &h->d_multi, aapk::multi_bytes(S.ntiles)))) return rc;
     }
     if ((rc = dev_alloc(h, &h->d_x0tab, (size_t)(S.ntx + 1) * sizeof(int)))) return rc;
@@ -855,7 +856,9 @@ int run_steps_adaptive(aap_handle *h, long long nsteps)
         h->since_copy += k;
         if (h->since_copy < kAdaptSteps) continue;
         h->since_copy = 0;
-        if (h->L.pipe && !use_multi(h)) AAP_CK(aapk::launch_tile_order(h->L, h->stream));
+        // (an order of more than 4096 tiles takes 55 us and matters less: a quarter as often)
+        if (h->L.pipe && !use_multi(h) && (h->hs.ntiles <= 4096 || (++h->order_age & 3) == 0))
+            AAP_CK(aapk::launch_tile_order(h->L, h->stream));
         const int slot = h->batch_slot;
         if ((rc = copy_words(h, h->pinned_err + 4 * (1 + slot)))) return rc;
         AAP_CK(cudaEventRecord(h->batch_ev[slot], h->stream));
@@ -1249,7 +1252,7 @@ int ens_combine(aap_ens *e)
             if (e->d_dense) cudaFree(e->d_dense);
             e->d_dense = nullptr;
             e->dense_tiles = 0;
-            if (cudaMalloc(&e->d_dense, 3 * (size_t)total * sizeof(int)) != cudaSuccess) {
+            if (cudaMalloc(&e->d_dense, (3 * (size_t)total + 1) * sizeof(int)) != cudaSuccess) {
                 cudaGetLastError();
                 return fail(AAP_ENOMEM, "ensemble tile list allocation failed");
             }

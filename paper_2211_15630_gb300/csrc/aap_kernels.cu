@@ -184,17 +184,22 @@ __global__ void __launch_bounds__(1024) k_finish(Sys *sys, int nsys, const int *
 // stable inside a class, so that neighbours stay together: states that outgrow
 // the L2 keep the raster order but for tiles of more than about twice the mean
 // cost (their halo regions are read while they are there).  Run every few
-// dozen steps: loads change slowly.  order: [total], cost: [total] scratch.
+// dozen steps: loads change slowly.  order: [total], cost: [total] scratch;
+// nfront: the leading tiles that hold more own particles than two buffers of
+// the pipeline (own_max), which whole blocks do first.
 __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys, int nsys,
                                                      const int *__restrict__ tile_base, const Ctl *__restrict__ ctl,
-                                                     int *order, float *cost)
+                                                     int own_max, int *order, float *cost, int *nfront)
 {
     constexpr int kClasses = 16;
     __shared__ float s_sum[32];
-    __shared__ int s_cnt[kClasses], s_warp[32][kClasses];
+    __shared__ int s_cnt[kClasses], s_warp[32][kClasses], s_front;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = (int)(ctl->step & 1), total = tile_base[nsys];
     float sum = 0.f;
+    if (tid == 0) s_front = 0;
+    __syncthreads();
+    int front = 0;
     for (int g = tid; g < total; g += 1024) {
         const int si = nsys > 1 ? sys_of_tile(tile_base, nsys, g) : 0;
         const Sys &S = sys[si];
@@ -206,7 +211,9 @@ __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys
         const float f = (float)own * (24.0f + 7.5f * (float)own / (float)(S.twmax * S.thmax));
         cost[g] = f;
         sum += f;
+        front += own > own_max;
     }
+    if (front) atomicAdd(&s_front, front);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     if (lane == 0) s_sum[warp] = sum;
@@ -230,6 +237,7 @@ __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys
         }
     }
     __syncthreads();
+    if (tid == 0) *nfront = min(s_front, total);
     for (int g0 = 0; g0 < total; g0 += 1024) {
         const int g = g0 + tid;
         const int k = g < total ? cls(cost[g]) : -1;
@@ -594,7 +602,9 @@ cudaError_t launch_insert(const Sys &S, int b, const double *x, const double *y,
 
 cudaError_t launch_tile_order(const LaunchCfg &L, cudaStream_t st)
 {
-    k_tile_order<<<1, 1024, 0, st>>>(L.sys, L.nsys, L.tile_base, L.ctl, L.order, reinterpret_cast<float *>(L.order + L.order_tiles));
+    k_tile_order<<<1, 1024, 0, st>>>(L.sys, L.nsys, L.tile_base, L.ctl, 2 * L.pipe_cap_own, L.order,
+                                     reinterpret_cast<float *>(L.order + L.order_tiles),
+                                     L.order + 2 * (size_t)L.order_tiles);
     return cudaGetLastError();
 }
 

@@ -31,7 +31,8 @@ struct LaunchCfg {
     int pipe_cap, pipe_cap_own, pipe_grid;
     int pipe_nceh;               // half cells (split along x) of the largest extended tile, (2 tw + 4)(th + 2)
     int *dense_list;
-    int *order;                  // device [2 * order_tiles]: the order in which tiles are claimed; scratch
+    int *order;                  // device [2 * order_tiles + 1]: the order in which tiles are claimed; scratch; how many
+                                 // of the first whole blocks do before the pipeline
     int order_tiles;
     // many steps per launch (a small system, one block per tile, all resident)
     int multi, multi_species, multi_cap, multi_tiles, multi_threads;

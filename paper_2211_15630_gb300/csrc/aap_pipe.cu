@@ -137,6 +137,7 @@ struct PipeShared {
     int chunk[2];               // next chunk of 32 own particles, per output buffer
     int flag;                   // a previous step's wait ran out
     int total;                  // tiles of the launch
+    int nfront;                 // tiles done by whole blocks before the pipeline
     long long step;
     int dense_any;              // tiles were listed for the whole-block routine
     int dense_tile;
@@ -567,13 +568,70 @@ __device__ __forceinline__ void flush_hist(PipeShared &sh, const PipeBufs &B, in
     }
 }
 
+// A tile too large for the pipeline's buffers, by the whole block (every thread
+// calls) with the shared staging area or the block's global scratch.  Out of
+// line: it is called before and after the pipeline.
+template <int MODEL>
+__device__ __noinline__ void whole_block_tile(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_base,
+                                              int g, int cap, int cap_own, int nceh_max, int nce_max, int hist_words,
+                                              unsigned char *mine, int scratch_cap, int spill_list_cap, long long step,
+                                              int total)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int tid = threadIdx.x, cur = (int)(step & 1);
+    __shared__ TileCtx T;
+    const size_t tbytes = table_bytes(nce_max, hist_words);
+    const size_t dyn = pipe_smem_bytes(cap, cap_own, nceh_max, hist_words);
+    // stage_bytes(a) <= 41 a + 18: the staging area and the tables fit in dyn
+    const int as_cap = (int)(((dyn - tbytes - 256) / 41) & ~63);
+    Stage As;
+    carve_stage(As, smem, as_cap);
+    Tables tb;
+    carve_tables(tb, smem + stage_bytes(as_cap), nce_max);
+    Stage Ag;
+    carve_stage(Ag, mine, scratch_cap);
+    int *spill_e = (int *)(mine + stage_bytes(scratch_cap));
+    unsigned char *spill_s = (unsigned char *)(spill_e + spill_list_cap);
+    const int si = nsys > 1 ? sys_of_tile(tile_base, nsys, g) : 0;
+    __syncthreads();                    // every thread is done with the previous tile
+    {
+        const int words = (int)(sizeof(Sys) / 4);
+        const int *src = reinterpret_cast<const int *>(sys + si);
+        int *dst = reinterpret_cast<int *>(&T.S);
+        for (int i = tid; i < words; i += kPipeThreads) dst[i] = src[i];
+    }
+    __syncthreads();
+    if (tid == 0) {
+        T.sysi = si;
+        T.tile = g - tile_base[si];
+        T.pf_tile = -1;
+        T.total = total;
+        T.nsys = nsys;
+        T.tile_base = tile_base;
+        T.next = total;
+    }
+    __syncthreads();
+    tile_setup<kPipeThreads>(T, tb, cur, nce_max, spill_e, spill_s, spill_list_cap);
+    if (T.m <= as_cap) {
+        tile_body<kPipeThreads, MODEL>(T, As, tb, step, spill_e, spill_s, total);
+    } else if (T.m <= scratch_cap) {
+        Stage Ah = Ag;
+        if ((size_t)T.m * sizeof(float4) <= stage_bytes(as_cap)) Ah.P = reinterpret_cast<float4 *>(smem);
+        tile_body<kPipeThreads, MODEL>(T, Ah, tb, step, spill_e, spill_s, total);
+    } else if (tid == 0) {
+        atomicOr(T.S.err, ERR_STAGE | ERR_LOST);
+    }
+    __syncthreads();
+}
+
 // The pipelined step of one or more systems with one species each (any
 // model; the systems of one launch share it): one block of kPipeThreads
 // threads per SM.  tile_base[nsys + 1] is the prefix of the systems' tiles.
 template <int MODEL, bool SP, int NSORT>
 __global__ void __launch_bounds__(kPipeThreads, 1)
 k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_base, Ctl *ctl, int cap, int cap_own,
-            int nceh_max, int nce_max, int hist_words, const int *__restrict__ order, int *dense_list, unsigned char *scratch,
+            int nceh_max, int nce_max, int hist_words, const int *__restrict__ order, const int *__restrict__ nfront,
+            int *dense_list, unsigned char *scratch,
             size_t scratch_per_block, int scratch_cap, int spill_list_cap)
 {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -597,8 +655,11 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int i = tid; i < nceh_max; i += kPipeThreads) B.hist[i] = 0;
-    for (int i = tid; i < 2 * B.mh_stride; i += kPipeThreads) B.mhist0[i] = 0;
+    const auto clear_tables = [&]() {
+        for (int i = tid; i < nceh_max; i += kPipeThreads) B.hist[i] = 0;
+        for (int i = tid; i < 2 * B.mh_stride; i += kPipeThreads) B.mhist0[i] = 0;
+    };
+    clear_tables();
     pdl_wait();         // the step before is closed
     pdl_next();
     // everything the roles start with is read side by side (a step of a few
@@ -609,9 +670,10 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
     int *const err0 = sys[0].err;
     int g0 = 0, t0 = 0;
     if (warp == 0) {
-        // tiles are claimed in `order`, the longest first (k_tile_order)
+        // tiles are claimed in `order`, the longest first (k_tile_order), after
+        // the `nfront` that whole blocks do before
         if (lane == 0) {
-            g0 = atomicAdd(&ctl->tile_next, 1);
+            g0 = atomicAdd(&ctl->tile_next, 1) + *nfront;
             t0 = g0 < tile_base[nsys] ? order[g0] : 0;
         }
         g0 = __shfl_sync(0xffffffffu, g0, 0);
@@ -623,6 +685,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
         sh.step = ctl->step;
     } else if (tid == kPipeThreads - 65) {
         sh.total = tile_base[nsys];
+        sh.nfront = *nfront;
     } else if (nsys == 1 && warp <= 24) {
         const int words = (int)(sizeof(Sys) / 4), k = (warp - 1) / 8;       // eight warps a copy
         const int *src = reinterpret_cast<const int *>(sys);
@@ -638,6 +701,17 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
     const int cur = (int)(step & 1);
     const int total = sh.total;
     unsigned char *mine = scratch + scratch_per_block * blockIdx.x;
+
+    // tiles that were far too large for the buffers when they were ordered: now,
+    // not after the pipeline, where they would be what the step waits for
+    if ((int)blockIdx.x < sh.nfront) {
+        for (int d = blockIdx.x; d < min(sh.nfront, total); d += gridDim.x)
+            whole_block_tile<MODEL>(sys, nsys, tile_base, order[d], cap, cap_own, nceh_max, nce_max, hist_words, mine,
+                                    scratch_cap, spill_list_cap, step, total);
+        if (tid == 0) sh.load = sh.staged = 0x7fffffff;
+        clear_tables();
+        __syncthreads();
+    }
 
     if (warp == 0) {
         // ---------------------------------------------------- copy warp --
@@ -683,7 +757,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
         for (;;) {
             // the following tile, claimed now so that its round trip overlaps this one's copies
             int gn = 0;
-            if (g < total && lane == 0) gn = atomicAdd(&ctl->tile_next, 1);
+            if (g < total && lane == 0) gn = atomicAdd(&ctl->tile_next, 1) + sh.nfront;
             int n_spill = 0, n_own = 0, mode = 0;               // 0: whole-block list, 1: normal, 2: wide
             if (g < total) {
                 const bool scanned = copy_spills(Sc, pl, cur, min(nsp, Sc.spill_cap), spill_e, spill_s, n_spill,
@@ -973,21 +1047,6 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
         if (tid == 0) PT_ADD(12, PT_NOW() - tk0);
         return;
     }
-    __shared__ TileCtx T;
-    const size_t tbytes = table_bytes(nce_max, hist_words);
-    const size_t dyn = pipe_smem_bytes(cap, cap_own, nceh_max, hist_words);
-    // stage_bytes(a) <= 41 a + 18: the staging area and the tables fit in dyn
-    const int as_cap = (int)(((dyn - tbytes - 256) / 41) & ~63);
-    Stage As;
-    carve_stage(As, smem, as_cap);
-    Tables tb;
-    carve_tables(tb, smem + stage_bytes(as_cap), nce_max);
-    Stage Ag;
-    carve_stage(Ag, mine, scratch_cap);
-    int *spill_e = (int *)(mine + stage_bytes(scratch_cap));
-    unsigned char *spill_s = (unsigned char *)(spill_e + spill_list_cap);
-    bool first = true;
-    const long long td0 = PT_NOW();
     for (;;) {
         if (tid == 0) {
             int got = -1;
@@ -1017,45 +1076,15 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
         const int g = sh.dense_tile;
         if (g < 0) break;
         if (tid == 0) sh.load = sh.staged = 0x7fffffff;
-        const int si = nsys > 1 ? sys_of_tile(tile_base, nsys, g) : 0;
-        if (first || si != T.sysi) {
-            __syncthreads();                // every thread is done with the previous system
-            const int words = (int)(sizeof(Sys) / 4);
-            const int *src = reinterpret_cast<const int *>(sys + si);
-            int *dst = reinterpret_cast<int *>(&T.S);
-            for (int i = tid; i < words; i += kPipeThreads) dst[i] = src[i];
-            first = false;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            T.sysi = si;
-            T.tile = g - tile_base[si];
-            T.pf_tile = -1;
-            T.total = total;
-            T.nsys = nsys;
-            T.tile_base = tile_base;
-            T.next = total;
-        }
-        __syncthreads();
-        tile_setup<kPipeThreads>(T, tb, cur, nce_max, spill_e, spill_s, spill_list_cap);
-        if (T.m <= as_cap) {
-            tile_body<kPipeThreads, MODEL>(T, As, tb, step, spill_e, spill_s, total);
-        } else if (T.m <= scratch_cap) {
-            Stage Ah = Ag;
-            if ((size_t)T.m * sizeof(float4) <= stage_bytes(as_cap)) Ah.P = reinterpret_cast<float4 *>(smem);
-            tile_body<kPipeThreads, MODEL>(T, Ah, tb, step, spill_e, spill_s, total);
-        } else if (tid == 0) {
-            atomicOr(T.S.err, ERR_STAGE | ERR_LOST);
-        }
+        whole_block_tile<MODEL>(sys, nsys, tile_base, g, cap, cap_own, nceh_max, nce_max, hist_words, mine, scratch_cap,
+                                spill_list_cap, step, total);
         if (tid == 0) PT_ADD(11, 1);
-        __syncthreads();
     }
     if (nsys == 1 && tid == 0) {
         atomicMax(err0 + 1, sh.load);
         atomicMax(err0 + 2, sh.staged);
     }
     if (tid == 0) PT_ADD(12, PT_NOW() - tk0);
-    (void)td0;
 }
 
 #ifndef AAP_PIPE_SORT_WARPS
@@ -1119,7 +1148,7 @@ static cudaError_t launch_pipe_t(const LaunchCfg &L, cudaStream_t st)
     const size_t smem = pipe_smem_bytes(L.pipe_cap, L.pipe_cap_own, L.pipe_nceh, L.hist_words);
     return launch_after(k_step_pipe<MODEL, kSpecies, AAP_PIPE_SORT_WARPS>, L.pipe_grid, kPipeThreads, smem, st, L.sys, L.nsys,
                         L.tile_base, L.ctl, L.pipe_cap, L.pipe_cap_own, L.pipe_nceh, L.nce_max, L.hist_words,
-                        L.order, L.dense_list, L.scratch, L.scratch_per_block, L.scratch_cap, L.spill_list_cap);
+                        L.order, L.order + 2 * (size_t)L.order_tiles, L.dense_list, L.scratch, L.scratch_per_block, L.scratch_cap, L.spill_list_cap);
 }
 
 cudaError_t PIPE_FN(launch_step_pipe)(const LaunchCfg &L, cudaStream_t st)
