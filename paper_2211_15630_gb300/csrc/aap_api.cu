@@ -69,7 +69,7 @@ struct aap_handle {
     int *d_x0tab = nullptr, *d_y0tab = nullptr;
     unsigned char *d_scratch = nullptr;
     int *d_dense = nullptr;             // pipelined step: tiles left to the whole-block routine
-    int *d_order = nullptr;             // pipelined step: the order in which tiles are claimed
+    int2 *d_jobs = nullptr;             // pipelined step: what is claimed, in order
     int *d_multi = nullptr;             // many steps per launch: private counters and barrier
     unsigned long long *d_obs = nullptr;
     int *d_seen = nullptr;
@@ -670,9 +670,10 @@ int alloc_all(aap_handle *h)
         if ((rc = dev_alloc(h, &h->d_sys, sizeof(Sys)))) return rc;
         if ((rc = dev_alloc(h, &h->d_tile_base, 2 * sizeof(int)))) return rc;
         if ((rc = dev_alloc(h, &h->d_ctl, sizeof(Ctl)))) return rc;
-        if ((rc = dev_alloc(h, &h->d_dense, (size_t)std::max(S.ntiles, 1) * sizeof(int)))) return rc;
-        AAP_CK(cudaMemsetAsync(h->d_dense, 0, (size_t)std::max(S.ntiles, 1) * sizeof(int), h->stream));
-        if (h->L.pipe && (rc = dev_alloc(h, &h->d_order, (2 * (size_t)std::max(S.ntiles, 1) + 1) * sizeof(int)))) return rc;
+        const size_t dense = aapk::job_count(S.ntiles) * sizeof(int);
+        if ((rc = dev_alloc(h, &h->d_dense, dense))) return rc;
+        AAP_CK(cudaMemsetAsync(h->d_dense, 0, dense, h->stream));
+        if (h->L.pipe && (rc = dev_alloc(h, &h->d_jobs, aapk::job_bytes(S.ntiles)))) return rc;
         if (h->L.multi && (rc = dev_alloc(h, &h->d_multi, aapk::multi_bytes(S.ntiles)))) return rc;
     }
     if ((rc = dev_alloc(h, &h->d_x0tab, (size_t)(S.ntx + 1) * sizeof(int)))) return rc;
@@ -707,8 +708,8 @@ int alloc_all(aap_handle *h)
     L.tile_base = h->d_tile_base;
     L.ctl = h->d_ctl;
     L.dense_list = h->d_dense;
-    L.order = h->d_order;
-    L.order_tiles = S.ntiles;
+    L.jobs = h->d_jobs;
+    L.job_tiles = S.ntiles;
     L.multi_cnt = h->d_multi;
     return push_sys(h);
 }
@@ -1116,7 +1117,7 @@ struct aap_ens {
     Ctl *d_ctl = nullptr;
     unsigned char *d_scratch = nullptr;
     size_t scratch_bytes = 0;
-    int *d_dense = nullptr;             // pipelined step: tiles left to the whole-block routine; their order
+    int *d_dense = nullptr;             // pipelined step: its jobs, and those left to the whole-block routine
     size_t dense_tiles = 0;
     std::vector<int> order;             // replicas in the order of their descriptors (densest first)
     int *d_err = nullptr;               // [count + 4] the replicas' error words
@@ -1252,16 +1253,17 @@ int ens_combine(aap_ens *e)
             if (e->d_dense) cudaFree(e->d_dense);
             e->d_dense = nullptr;
             e->dense_tiles = 0;
-            if (cudaMalloc(&e->d_dense, (3 * (size_t)total + 1) * sizeof(int)) != cudaSuccess) {
+            if (cudaMalloc(&e->d_dense, aapk::job_bytes((int)total) + aapk::job_count((int)total) * sizeof(int)) !=
+                cudaSuccess) {
                 cudaGetLastError();
                 return fail(AAP_ENOMEM, "ensemble tile list allocation failed");
             }
             e->dense_tiles = (size_t)total;
         }
-        AAP_CK(cudaMemset(e->d_dense, 0, (size_t)total * sizeof(int)));
-        L.dense_list = e->d_dense;
-        L.order = e->d_dense + total;
-        L.order_tiles = (int)total;
+        L.jobs = reinterpret_cast<int2 *>(e->d_dense);
+        L.job_tiles = (int)total;
+        L.dense_list = e->d_dense + aapk::job_bytes((int)total) / sizeof(int);
+        AAP_CK(cudaMemset(L.dense_list, 0, aapk::job_count((int)total) * sizeof(int)));
         AAP_CK(cudaStreamSynchronize(e->stream));
         int rc = set_pipe_launch(L, false, twmax, thmax, (int)total);
         if (rc) return rc;

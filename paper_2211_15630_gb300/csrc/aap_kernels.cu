@@ -59,6 +59,8 @@ k_step(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_base,
     if (threadIdx.x == 0) {
         T.sysi = -1;
         T.pf_tile = -1;
+        T.part = 0;
+        T.parts = 1;
         T.total = total;
         T.nsys = nsys;
         T.tile_base = tile_base;
@@ -178,28 +180,31 @@ __global__ void __launch_bounds__(1024) k_finish(Sys *sys, int nsys, const int *
 }
 
 // ------------------------------------------------------- order of the tiles --
-// The order in which the pipelined step claims tiles: a step ends when its
-// longest tile does, so the longest start first.  One block sorts the tiles of
+// The order in which the pipelined step claims its work: a step ends when its
+// longest job does, so the longest start first, and a tile that would keep its
+// SM longer than half of what an SM has to do on average is split into up to
+// eight parts, each of which stages and sorts the whole tile and updates its
+// share of the particles (a clustered state of N = 524,288: its densest tile
+// has three times the pairs of an average SM).  One block sorts the jobs of
 // all systems by the class of their cost (two classes per factor of two),
 // stable inside a class, so that neighbours stay together: states that outgrow
-// the L2 keep the raster order but for tiles of more than about twice the mean
-// cost (their halo regions are read while they are there).  Run every few
-// dozen steps: loads change slowly.  order: [total], cost: [total] scratch;
-// nfront: the leading tiles that hold more own particles than two buffers of
-// the pipeline (own_max), which whole blocks do first.
+// the L2 keep the raster order but for jobs of more than about twice the mean
+// tile's cost (their halo regions are read while they are there).  Run every
+// few dozen steps: loads change slowly.
+// jobs: [total + kMaxParts] {tile, part | parts << 8}; cost: [total] scratch;
+// meta: the number of leading jobs that whole blocks do first (tiles of more
+// own particles than own_max, two buffers of the pipeline), and of all jobs.
+constexpr float kSplitAbove = 0.75f, kSplitTo = 2.0f;      // of an SM's average: split tiles above, into parts of 1 / kSplitTo
 __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys, int nsys,
                                                      const int *__restrict__ tile_base, const Ctl *__restrict__ ctl,
-                                                     int own_max, int *order, float *cost, int *nfront)
+                                                     int own_max, int blocks, int2 *jobs, float *cost, int *meta)
 {
-    constexpr int kClasses = 16;
+    constexpr int kClasses = 17;                // 0: whole blocks first
     __shared__ float s_sum[32];
-    __shared__ int s_cnt[kClasses], s_warp[32][kClasses], s_front;
+    __shared__ int s_cnt[kClasses], s_warp[32][kClasses], s_extra, s_kmax;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = (int)(ctl->step & 1), total = tile_base[nsys];
     float sum = 0.f;
-    if (tid == 0) s_front = 0;
-    __syncthreads();
-    int front = 0;
     for (int g = tid; g < total; g += 1024) {
         const int si = nsys > 1 ? sys_of_tile(tile_base, nsys, g) : 0;
         const Sys &S = sys[si];
@@ -207,57 +212,82 @@ __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys
         int own = 0;
 #pragma unroll
         for (int r = 0; r < kRegions; ++r) own += c[r];
-        // staging and update per particle, and the candidates of 15 half cells
+        // staging and update per particle, and the candidates of 15 half
+        // cells; negative: a tile for whole blocks
         const float f = (float)own * (24.0f + 7.5f * (float)own / (float)(S.twmax * S.thmax));
-        cost[g] = f;
+        cost[g] = own > own_max ? -f : f;
         sum += f;
-        front += own > own_max;
     }
-    if (front) atomicAdd(&s_front, front);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     if (lane == 0) s_sum[warp] = sum;
     if (tid < kClasses) s_cnt[tid] = 0;
+    if (tid == 0) {
+        s_extra = 0;
+        s_kmax = 1;
+    }
     __syncthreads();
-    float mean = 0.f;
-    for (int w = 0; w < 32; ++w) mean += s_sum[w];
-    mean = fmaxf(mean / (float)max(total, 1), 1e-20f);
-    const int kmax = total <= 4096 ? kClasses - 1 : 6;
-    const auto cls = [&](float f) {
-        return min(max((int)floorf(8.0f - 2.0f * __log2f(fmaxf(f, 1e-20f) / mean)), 0), kmax);
+    float all = 0.f;
+    for (int w = 0; w < 32; ++w) all += s_sum[w];
+    const float mean = fmaxf(all / (float)max(total, 1), 1e-20f), share = fmaxf(all / (float)blocks, 1e-20f);
+    const int cmax = total <= 4096 ? kClasses - 2 : 6;
+    const auto cls = [&](float f, int K) {
+        if (f < 0.f) return 0;
+        return 1 + min(max((int)floorf(8.0f - 2.0f * __log2f(fmaxf(f, 1e-20f) / ((float)K * mean))), 0), cmax);
     };
-    for (int g = tid; g < total; g += 1024) atomicAdd(&s_cnt[cls(cost[g])], 1);
+    const auto parts = [&](float f) {
+        return fabsf(f) > kSplitAbove * share && fabsf(f) > 1.5f * mean ? min((int)ceilf(kSplitTo * fabsf(f) / share), 8) : 1;
+    };
+    for (int g = tid; g < total; g += 1024) {
+        const int K = parts(cost[g]);
+        if (K > 1) {
+            atomicAdd(&s_extra, K - 1);
+            atomicMax(&s_kmax, K);
+        }
+    }
+    __syncthreads();
+    const bool split = s_extra <= kMaxParts;
+    const int kmax = split ? s_kmax : 1;
+    for (int g = tid; g < total; g += 1024) {
+        const int K = split ? parts(cost[g]) : 1;
+        atomicAdd(&s_cnt[cls(cost[g], K)], K);
+    }
     __syncthreads();
     if (tid == 0) {
         int run = 0;
+        meta[0] = s_cnt[0];
         for (int k = 0; k < kClasses; ++k) {
             const int n = s_cnt[k];
             s_cnt[k] = run;
             run += n;
         }
+        meta[1] = run;
     }
     __syncthreads();
-    if (tid == 0) *nfront = min(s_front, total);
     for (int g0 = 0; g0 < total; g0 += 1024) {
         const int g = g0 + tid;
-        const int k = g < total ? cls(cost[g]) : -1;
-        const unsigned peers = __match_any_sync(0xffffffffu, k);
-        if (lane < kClasses) s_warp[warp][lane] = 0;
-        __syncwarp();
-        if (k >= 0 && lane == __ffs(peers) - 1) s_warp[warp][k] = __popc(peers);
-        __syncthreads();
-        if (tid < kClasses) {
-            int run = s_cnt[tid];
-            for (int w = 0; w < 32; ++w) {
-                const int n = s_warp[w][tid];
-                s_warp[w][tid] = run;
-                run += n;
+        const float f = g < total ? cost[g] : 0.f;
+        const int K = g < total ? (split ? parts(f) : 1) : 0;
+        for (int p = 0; p < kmax; ++p) {
+            const int k = p < K ? cls(f, K) : -1;
+            const unsigned peers = __match_any_sync(0xffffffffu, k);
+            if (lane < kClasses) s_warp[warp][lane] = 0;
+            __syncwarp();
+            if (k >= 0 && lane == __ffs(peers) - 1) s_warp[warp][k] = __popc(peers);
+            __syncthreads();
+            if (tid < kClasses) {
+                int run = s_cnt[tid];
+                for (int w = 0; w < 32; ++w) {
+                    const int n = s_warp[w][tid];
+                    s_warp[w][tid] = run;
+                    run += n;
+                }
+                s_cnt[tid] = run;
             }
-            s_cnt[tid] = run;
+            __syncthreads();
+            if (k >= 0) jobs[s_warp[warp][k] + __popc(peers & ((1u << lane) - 1u))] = make_int2(g, p | (K << 8));
+            __syncthreads();
         }
-        __syncthreads();
-        if (k >= 0) order[s_warp[warp][k] + __popc(peers & ((1u << lane) - 1u))] = g;
-        __syncthreads();
     }
 }
 
@@ -602,9 +632,8 @@ cudaError_t launch_insert(const Sys &S, int b, const double *x, const double *y,
 
 cudaError_t launch_tile_order(const LaunchCfg &L, cudaStream_t st)
 {
-    k_tile_order<<<1, 1024, 0, st>>>(L.sys, L.nsys, L.tile_base, L.ctl, 2 * L.pipe_cap_own, L.order,
-                                     reinterpret_cast<float *>(L.order + L.order_tiles),
-                                     L.order + 2 * (size_t)L.order_tiles);
+    k_tile_order<<<1, 1024, 0, st>>>(L.sys, L.nsys, L.tile_base, L.ctl, 2 * L.pipe_cap_own, L.pipe_grid, L.jobs,
+                                     job_cost(L), job_meta(L));
     return cudaGetLastError();
 }
 

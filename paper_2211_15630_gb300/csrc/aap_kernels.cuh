@@ -26,14 +26,13 @@ struct LaunchCfg {
     int grid_step, grid_finish;
     // pipelined step (pipe_species: systems of several species): shared buffers of pipe_cap
     // staged / pipe_cap_own own particles per tile, one block per SM; tiles
-    // that do not fit go to dense_list (device [ntiles], zero between steps)
+    // that do not fit go to dense_list (device [job_count], zero between steps)
     int pipe, pipe_species;
     int pipe_cap, pipe_cap_own, pipe_grid;
     int pipe_nceh;               // half cells (split along x) of the largest extended tile, (2 tw + 4)(th + 2)
     int *dense_list;
-    int *order;                  // device [2 * order_tiles + 1]: the order in which tiles are claimed; scratch; how many
-                                 // of the first whole blocks do before the pipeline
-    int order_tiles;
+    int2 *jobs;                  // device [job_bytes(job_tiles)]: what is claimed, in order (k_tile_order)
+    int job_tiles;
     // many steps per launch (a small system, one block per tile, all resident)
     int multi, multi_species, multi_cap, multi_tiles, multi_threads;
     int *multi_cnt;              // device: three private counter sets and two barrier words, zero between launches
@@ -42,6 +41,14 @@ struct LaunchCfg {
     long long mf_n, mf_ncell;
     int mf_grid;                 // persistent blocks of the k-nearest update
 };
+
+// The pipelined step's jobs: up to one per tile and kMaxParts more, the tiles'
+// costs (scratch), and {leading jobs for whole blocks, jobs}.
+constexpr int kMaxParts = 1024;
+inline size_t job_count(int tiles) { return (size_t)tiles + kMaxParts; }
+inline size_t job_bytes(int tiles) { return job_count(tiles) * sizeof(int2) + (size_t)round_up(tiles, 4) * 4 + 16; }
+inline float *job_cost(const LaunchCfg &L) { return reinterpret_cast<float *>(L.jobs + job_count(L.job_tiles)); }
+inline int *job_meta(const LaunchCfg &L) { return reinterpret_cast<int *>(job_cost(L) + round_up(L.job_tiles, 4)); }
 
 size_t step_smem_bytes(int stage_cap, int nce_max, int hist_words);
 // Set the dynamic shared-memory limit of the step kernel and report how many
@@ -99,7 +106,7 @@ cudaError_t launch_mf_step(const LaunchCfg &L, cudaStream_t st, cudaEvent_t *ev)
 
 cudaError_t launch_insert(const Sys &S, int b, const double *x, const double *y, const float *th,
                           int mode, cudaStream_t st);
-// The order in which the pipelined step claims the tiles of its systems, from their current loads.
+// The jobs of the pipelined step, in the order they are claimed, from the tiles' current loads.
 cudaError_t launch_tile_order(const LaunchCfg &L, cudaStream_t st);
 // The largest tile load and staged set of buffer b into S.err[1] and [2].
 cudaError_t launch_tile_load(const Sys &S, int b, cudaStream_t st);

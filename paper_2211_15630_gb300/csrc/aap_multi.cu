@@ -211,6 +211,7 @@ __device__ __forceinline__ bool multi_tile(MultiShared &sh, const MultiStage &A,
         n_own += __shfl_sync(0xffffffffu, incl, 31);
     }
     if (lane == 0) {
+        sh.O.o_first = 0;
         sh.O.n_own = n_own;
         sh.O.wide = 15 * sh.maxc >= 512;
         sh.O.dense = 2 * m > 3 * nce;

@@ -112,6 +112,7 @@ struct RawMeta {
     int tile;                   // tile index, -1: no more tiles, -2: the second half of the wide tile in the
                                 // buffer before (released with it), -3: empty (released at once)
     int m, m_seg, n_spill, n_own;
+    int part;                   // part | parts << 8 of the tile that is updated
     int wide;                   // 1: the tile spans both raw buffers (staged from buffer 0's start)
     int si;                     // system of the tile (ensembles: its replica)
     int sx, sy, order;          // of that system: fixed-point bits per cell side, interaction order
@@ -136,8 +137,8 @@ struct PipeShared {
     OutMeta out[2];
     int chunk[2];               // next chunk of 32 own particles, per output buffer
     int flag;                   // a previous step's wait ran out
-    int total;                  // tiles of the launch
-    int nfront;                 // tiles done by whole blocks before the pipeline
+    int total;                  // jobs of the launch
+    int nfront;                 // those that whole blocks do before the pipeline
     long long step;
     int dense_any;              // tiles were listed for the whole-block routine
     int dense_tile;
@@ -346,7 +347,7 @@ __device__ __forceinline__ bool copy_spills(const Sys &S, const CopyPlan &pl, in
 // The planned tile's meta into raw buffer meta M (the raw buffer, or both for
 // a wide tile, must be free).
 __device__ __forceinline__ void copy_commit(const CopyPlan &pl, const Sys &S, int si, int g, RawMeta &M, int n_spill,
-                                            int n_own, int wide, const unsigned char *spill_s)
+                                            int n_own, int wide, int part, const unsigned char *spill_s)
 {
     const int lane = threadIdx.x & 31;
     const Seg &sg = pl.sg;
@@ -369,6 +370,7 @@ __device__ __forceinline__ void copy_commit(const CopyPlan &pl, const Sys &S, in
         M.n_spill = n_spill;
         M.n_own = n_own;
         M.wide = wide;
+        M.part = part;
         M.si = si;
         M.sx = S.sx;
         M.sy = S.sy;
@@ -494,12 +496,21 @@ __device__ __forceinline__ void sort_order(PipeShared &sh, const PipeBufs &B, in
         int mx = lane < nw ? sh.warp_tot[lane] : 0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        int first = 0, last = carry;
+        if ((M.part >> 8) > 1) {
+            __syncwarp();
+            const auto row_start = [&](int rw) { return cst[(rw + 1) * W2 + 2] + B.rowoff[rw + 1]; };
+            const auto cell_start = [&](int rw, int c) { return cst[(rw + 1) * W2 + 2 + 2 * c] + B.rowoff[rw + 1]; };
+            first = part_start(M.part & 255, M.part >> 8, carry, tw, th, row_start, cell_start);
+            last = part_start((M.part & 255) + 1, M.part >> 8, carry, tw, th, row_start, cell_start);
+        }
         if (lane == 0) {
             OutMeta &O = sh.out[b];
             O.tile = M.tile;
             O.rbuf = r;
             O.rwide = M.wide;
-            O.n_own = min(carry, cap_own);
+            O.o_first = first;
+            O.n_own = min(last, cap_own);
             O.tx = M.tx; O.ty = M.ty; O.tw = tw; O.th = th; O.W2 = W2;
             O.twL = M.twL; O.twR = M.twR; O.thD = M.thD; O.thU = M.thU;
             O.wide = 15 * mx >= 512;
@@ -573,7 +584,7 @@ __device__ __forceinline__ void flush_hist(PipeShared &sh, const PipeBufs &B, in
 // line: it is called before and after the pipeline.
 template <int MODEL>
 __device__ __noinline__ void whole_block_tile(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_base,
-                                              int g, int cap, int cap_own, int nceh_max, int nce_max, int hist_words,
+                                              int2 job, int cap, int cap_own, int nceh_max, int nce_max, int hist_words,
                                               unsigned char *mine, int scratch_cap, int spill_list_cap, long long step,
                                               int total)
 {
@@ -592,6 +603,7 @@ __device__ __noinline__ void whole_block_tile(const Sys *__restrict__ sys, int n
     carve_stage(Ag, mine, scratch_cap);
     int *spill_e = (int *)(mine + stage_bytes(scratch_cap));
     unsigned char *spill_s = (unsigned char *)(spill_e + spill_list_cap);
+    const int g = job.x;
     const int si = nsys > 1 ? sys_of_tile(tile_base, nsys, g) : 0;
     __syncthreads();                    // every thread is done with the previous tile
     {
@@ -605,6 +617,8 @@ __device__ __noinline__ void whole_block_tile(const Sys *__restrict__ sys, int n
         T.sysi = si;
         T.tile = g - tile_base[si];
         T.pf_tile = -1;
+        T.part = job.y & 255;
+        T.parts = job.y >> 8;
         T.total = total;
         T.nsys = nsys;
         T.tile_base = tile_base;
@@ -630,7 +644,7 @@ __device__ __noinline__ void whole_block_tile(const Sys *__restrict__ sys, int n
 template <int MODEL, bool SP, int NSORT>
 __global__ void __launch_bounds__(kPipeThreads, 1)
 k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_base, Ctl *ctl, int cap, int cap_own,
-            int nceh_max, int nce_max, int hist_words, const int *__restrict__ order, const int *__restrict__ nfront,
+            int nceh_max, int nce_max, int hist_words, const int2 *__restrict__ jobs, const int *__restrict__ meta,
             int *dense_list, unsigned char *scratch,
             size_t scratch_per_block, int scratch_cap, int spill_list_cap)
 {
@@ -668,24 +682,27 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
     // tile count and the error word
     // pipeline waits that run out are reported in the first system's error word
     int *const err0 = sys[0].err;
-    int g0 = 0, t0 = 0;
+    int g0 = 0;
+    int2 job0 = make_int2(0, 0);
     if (warp == 0) {
-        // tiles are claimed in `order`, the longest first (k_tile_order), after
-        // the `nfront` that whole blocks do before
+        // jobs (tiles, or parts of dense ones) are claimed in the order of
+        // k_tile_order, after the leading ones that whole blocks do before
         if (lane == 0) {
-            g0 = atomicAdd(&ctl->tile_next, 1) + *nfront;
-            t0 = g0 < tile_base[nsys] ? order[g0] : 0;
+            const int front = meta[0], njobs = meta[1];
+            g0 = atomicAdd(&ctl->tile_next, 1) + front;
+            if (g0 < njobs) job0 = jobs[g0];
         }
         g0 = __shfl_sync(0xffffffffu, g0, 0);
-        t0 = __shfl_sync(0xffffffffu, t0, 0);
+        job0.x = __shfl_sync(0xffffffffu, job0.x, 0);
+        job0.y = __shfl_sync(0xffffffffu, job0.y, 0);
     } else if (tid == kPipeThreads - 1) {
         sh.flag = *((volatile int *)err0) & ERR_TIMEOUT;
         sh.load = sh.staged = 0;
     } else if (tid == kPipeThreads - 33) {
         sh.step = ctl->step;
     } else if (tid == kPipeThreads - 65) {
-        sh.total = tile_base[nsys];
-        sh.nfront = *nfront;
+        sh.nfront = meta[0];
+        sh.total = meta[1];
     } else if (nsys == 1 && warp <= 24) {
         const int words = (int)(sizeof(Sys) / 4), k = (warp - 1) / 8;       // eight warps a copy
         const int *src = reinterpret_cast<const int *>(sys);
@@ -706,7 +723,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
     // not after the pipeline, where they would be what the step waits for
     if ((int)blockIdx.x < sh.nfront) {
         for (int d = blockIdx.x; d < min(sh.nfront, total); d += gridDim.x)
-            whole_block_tile<MODEL>(sys, nsys, tile_base, order[d], cap, cap_own, nceh_max, nce_max, hist_words, mine,
+            whole_block_tile<MODEL>(sys, nsys, tile_base, jobs[d], cap, cap_own, nceh_max, nce_max, hist_words, mine,
                                     scratch_cap, spill_list_cap, step, total);
         if (tid == 0) sh.load = sh.staged = 0x7fffffff;
         clear_tables();
@@ -726,7 +743,8 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
         unsigned char *spill_s = reinterpret_cast<unsigned char *>(spill_e + kPipeMaxSpill);
         unsigned kpar = 0, used = 0;       // per raw buffer: parity of its fills, filled before
         int r = 0;
-        int g = g0, gt = t0;               // the claim, and the tile it stands for
+        int g = g0;
+        int2 job = job0;                   // the claimed job: a tile, part | parts << 8
         // the planned tile: its system, local index and the system's spill
         // list length (final during this step), re-read when the system changes
         int si = -1, lt = 0, nsp = 0;
@@ -751,7 +769,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
             copy_plan(Sc, lt, cur, pl);
         };
         const long long tc0 = PT_NOW();
-        if (g < total) plan(gt);
+        if (g < total) plan(job.x);
         bool ok = true;
         bool withhold = c_pipe_stall != 0;
         for (;;) {
@@ -771,13 +789,14 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
                     // done by the whole block after the pipeline
                     if (lane == 0) {
                         const int j = atomicAdd(&ctl->dense_count, 1);
-                        dense_list[j] = gt + 1;
+                        dense_list[j] = g + 1;
                     }
-                    int tn = 0;
-                    if (lane == 0 && gn < total) tn = order[gn];
+                    int2 jn = make_int2(0, 0);
+                    if (lane == 0 && gn < total) jn = jobs[gn];
                     g = __shfl_sync(0xffffffffu, gn, 0);
-                    gt = __shfl_sync(0xffffffffu, tn, 0);
-                    if (g < total) plan(gt);
+                    job.x = __shfl_sync(0xffffffffu, jn.x, 0);
+                    job.y = __shfl_sync(0xffffffffu, jn.y, 0);
+                    if (g < total) plan(job.x);
                     continue;
                 }
                 if (mode == 2 && r == kNR - 1) {
@@ -818,9 +837,9 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
             }
             const Sys &Sg = Sc;
             const long long ts0 = PT_NOW();
-            copy_commit(pl, Sg, si, lt, M, n_spill, n_own, mode == 2, spill_s);
-            int tn = 0;
-            if (lane == 0 && gn < total) tn = order[gn];        // in flight beside the copies
+            copy_commit(pl, Sg, si, lt, M, n_spill, n_own, mode == 2, job.y, spill_s);
+            int2 jn = make_int2(0, 0);
+            if (lane == 0 && gn < total) jn = jobs[gn];         // in flight beside the copies
             if (lane == 0) PT_ADD(2, PT_NOW() - ts0);
             const long long ti0 = PT_NOW();
             int4 *R = B.raw(r);
@@ -861,8 +880,9 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
             const long long tq0 = PT_NOW();
             g = __shfl_sync(0xffffffffu, gn, 0);
             const long long tq1 = PT_NOW();
-            gt = __shfl_sync(0xffffffffu, tn, 0);
-            if (g < total) plan(gt);
+            job.x = __shfl_sync(0xffffffffu, jn.x, 0);
+            job.y = __shfl_sync(0xffffffffu, jn.y, 0);
+            if (g < total) plan(job.x);
             if (lane == 0) {
                 PT_ADD(13, tq1 - tq0);
                 PT_ADD(14, PT_NOW() - tq1);
@@ -1013,7 +1033,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
                 int c = 0;
                 if (lane == 0) c = atomicAdd(&sh.chunk[b], 1);
                 c = __shfl_sync(0xffffffffu, c, 0);
-                const int o0 = c * 32;
+                const int o0 = O.o_first + c * 32;
                 if (o0 >= O.n_own) break;
                 update_one<MODEL, SP, 1>(S, O, P, cst, RB, OR, OQ, o0 + lane, step, measure, B.mhist(b), acc, ToSystem{});
             }
@@ -1076,7 +1096,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
         const int g = sh.dense_tile;
         if (g < 0) break;
         if (tid == 0) sh.load = sh.staged = 0x7fffffff;
-        whole_block_tile<MODEL>(sys, nsys, tile_base, g, cap, cap_own, nceh_max, nce_max, hist_words, mine, scratch_cap,
+        whole_block_tile<MODEL>(sys, nsys, tile_base, jobs[g], cap, cap_own, nceh_max, nce_max, hist_words, mine, scratch_cap,
                                 spill_list_cap, step, total);
         if (tid == 0) PT_ADD(11, 1);
     }
@@ -1148,7 +1168,7 @@ static cudaError_t launch_pipe_t(const LaunchCfg &L, cudaStream_t st)
     const size_t smem = pipe_smem_bytes(L.pipe_cap, L.pipe_cap_own, L.pipe_nceh, L.hist_words);
     return launch_after(k_step_pipe<MODEL, kSpecies, AAP_PIPE_SORT_WARPS>, L.pipe_grid, kPipeThreads, smem, st, L.sys, L.nsys,
                         L.tile_base, L.ctl, L.pipe_cap, L.pipe_cap_own, L.pipe_nceh, L.nce_max, L.hist_words,
-                        L.order, L.order + 2 * (size_t)L.order_tiles, L.dense_list, L.scratch, L.scratch_per_block, L.scratch_cap, L.spill_list_cap);
+                        L.jobs, job_meta(L), L.dense_list, L.scratch, L.scratch_per_block, L.scratch_cap, L.spill_list_cap);
 }
 
 cudaError_t PIPE_FN(launch_step_pipe)(const LaunchCfg &L, cudaStream_t st)

@@ -104,6 +104,8 @@ struct TileCtx {
     int sysi, tile, tx, ty, tw, th, W2, H2, nce;
     int twL, twR, thD, thU;     // widths / heights of the neighbour tiles
     int m_seg, n_spill, m, n_own;
+    int part, parts;            // the update takes part `part` of `parts` of the tile's own particles
+    int o_first, o_last;        // those: own indices (in cell order)
     int next;                   // index of the next tile this block takes
     int total, nsys;            // tiles and systems of the launch
     const int *tile_base;
@@ -330,6 +332,32 @@ __device__ __forceinline__ void neighbour_sum_sp(const float4 *__restrict__ P, c
     }
 }
 
+// First own index (own particles in row, cell order) of part k of K of a
+// tile: the first start of a cell at or after the share n_own k / K, so that
+// the parts do not depend on the arrival order inside a cell and are the same
+// for every block that sorts the tile.  row_start(r), cell_start(r, c): own
+// index of the first particle of own row r / of its own cell c or a later one.
+// Every lane of the warp calls.
+template <class R, class C>
+__device__ __forceinline__ int part_start(int k, int K, int n_own, int tw, int th, R &&row_start, C &&cell_start)
+{
+    if (k <= 0) return 0;
+    if (k >= K) return n_own;
+    const int lane = threadIdx.x & 31;
+    const int target = (int)((long long)n_own * k / K);
+    int row = 0;                                        // the last row that starts at or before the share
+    for (int r0 = 0; r0 < th; r0 += 32) {
+        const unsigned b = __ballot_sync(0xffffffffu, r0 + lane < th && row_start(r0 + lane) <= target);
+        if (b) row = r0 + 31 - __clz(b);
+    }
+    for (int c0 = 0; c0 < tw; c0 += 32) {
+        const int s = c0 + lane < tw ? cell_start(row, c0 + lane) : -1;
+        const unsigned b = __ballot_sync(0xffffffffu, s >= target);
+        if (b) return __shfl_sync(0xffffffffu, s, __ffs(b) - 1);
+    }
+    return row + 1 < th ? row_start(row + 1) : n_own;
+}
+
 // Phase 2 of a tile, staged in A (shared memory or the block's scratch).
 template <int NT, int MODEL>
 __device__ __forceinline__ void tile_body(TileCtx &T, const Stage &A, const Tables &tb, long long step,
@@ -453,20 +481,34 @@ __device__ __forceinline__ void tile_body(TileCtx &T, const Stage &A, const Tabl
             tb.rowpre[th] = carry;
             T.n_own = carry;
         }
+        int first = 0, last = carry;
+        if (T.parts > 1) {
+            __syncwarp();
+            const auto row_start = [&](int r) { return tb.rowpre[r]; };
+            const auto cell_start = [&](int r, int c) {
+                return tb.rowpre[r] + tb.cstart[(r + 1) * W2 + 1 + c] - tb.cstart[(r + 1) * W2 + 1];
+            };
+            first = part_start(T.part, T.parts, carry, tw, th, row_start, cell_start);
+            last = part_start(T.part + 1, T.parts, carry, tw, th, row_start, cell_start);
+        }
+        if (lane == 0) {
+            T.o_first = first;
+            T.o_last = last;
+        }
     }
     __syncthreads();
     PHASE_MARK(2);
     PHASE_MARK(3);
 
     // --- interact, update, scatter ---------------------------------------
-    const int n_own = T.n_own;
+    const int o_last = T.o_last;
     const float r2 = S.r2;
     const int TWs = tw << S.sx, THs = th << S.sy;
     const bool measure = step < S.meas_until;   // on-the-fly histograms (Sec. 3.4)
     long long acc_c = 0, acc_s = 0, acc_n = 0, acc_c2 = 0, acc_s2 = 0;
-    for (int base = 0; base < n_own; base += NT) {
+    for (int base = T.o_first; base < o_last; base += NT) {
         const int o = base + tid;
-        const bool act = o < n_own;
+        const bool act = o < o_last;
         int4 rec = make_int4(0, 0, 0, 0);
         int dtile = 0, region = 0;
         if (act) {
@@ -632,7 +674,8 @@ __device__ __forceinline__ void tile_body(TileCtx &T, const Stage &A, const Tabl
 struct OutMeta {
     int tile;                   // -1: no more tiles, -2: skip (the buffer holds part of a wide tile)
     int rbuf, rwide;            // raw buffer of the tile's staged records, and whether it spans the next one too
-    int n_own, tx, ty, tw, th, W2, twL, twR, thD, thU;   // W2: half cells per extended row, 2 tw + 4
+    int o_first, n_own;         // the own particles to update: o_first .. n_own - 1
+    int tx, ty, tw, th, W2, twL, twR, thD, thU;   // W2: half cells per extended row, 2 tw + 4
     int wide;                   // a half cell holds enough particles for 512 candidates
     int dense;                  // more than 1.5 staged records per half cell on average
 };
