@@ -106,6 +106,7 @@ struct aap_handle {
     long long since_copy = 0;       // steps queued since the last copy
     bool err_pending = false;
     int relayouts = 0;
+    bool multi_refused = false;     // the cooperative launch did not fit the context
     int order_age = 0;
     bool multi_on = true;           // the tiles are light enough for many steps per launch
     // ensemble membership: steps are launched by the ensemble for all members,
@@ -811,7 +812,7 @@ int launch_steps(const LaunchCfg &L, cudaStream_t st, long long nsteps, cudaStre
 // have fallen by a quarter.  Per step, N = 60,000 to 100,000, many steps
 // against one: load 307: 13.3 / 31.0 us, 2138: 22.9 / 35.6, 4307: 19.5 / 30.8,
 // 7232: 38.5 / 36.4; staged beyond the block's: 84 / 38 and 611 / 131.
-bool use_multi(const aap_handle *h) { return h->L.multi && !h->timing && h->multi_on; }
+bool use_multi(const aap_handle *h) { return h->L.multi && !h->timing && h->multi_on && !h->multi_refused; }
 
 // words: {error bits, load, staged set}
 void act_on_load(aap_handle *h, const int *words)
@@ -879,9 +880,16 @@ int run_steps_adaptive(aap_handle *h, long long nsteps)
 int run_steps(aap_handle *h, long long nsteps)
 {
     if (use_multi(h)) {
-        if (nsteps > 0) AAP_CK(aapk::launch_multi(h->L, (int)nsteps, h->stream));
-        h->step += nsteps;
-        return AAP_OK;
+        cudaError_t e = nsteps > 0 ? aapk::launch_multi(h->L, (int)nsteps, h->stream) : cudaSuccess;
+        if (e == cudaSuccess) {
+            h->step += nsteps;
+            return AAP_OK;
+        }
+        // fewer SMs than the device has (a partitioned context): single steps from now on
+        if (e != cudaErrorCooperativeLaunchTooLarge) AAP_CK(e);
+        cudaGetLastError();
+        h->multi_on = false;
+        h->multi_refused = true;
     }
     if (!h->timing) {
         int rc = launch_steps(h->L, h->stream, nsteps, h->cap_stream, h->gexec);

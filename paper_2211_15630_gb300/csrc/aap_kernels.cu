@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(1024) k_finish(Sys *sys, int nsys, const int *
 // ------------------------------------------------------- order of the tiles --
 // The order in which the pipelined step claims its work: a step ends when its
 // longest job does, so the longest start first, and a tile that would keep its
-// SM longer than half of what an SM has to do on average is split into up to
+// SM longer than some 60% of what an SM has to do on average is split into up to
 // eight parts, each of which stages and sorts the whole tile and updates its
 // share of the particles (a clustered state of N = 524,288: its densest tile
 // has three times the pairs of an average SM).  One block sorts the jobs of
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(1024) k_finish(Sys *sys, int nsys, const int *
 // jobs: [total + kMaxParts] {tile, part | parts << 8}; cost: [total] scratch;
 // meta: the number of leading jobs that whole blocks do first (tiles of more
 // own particles than own_max, two buffers of the pipeline), and of all jobs.
-constexpr float kSplitAbove = 0.75f, kSplitTo = 2.0f;      // of an SM's average: split tiles above, into parts of 1 / kSplitTo
+constexpr float kSplitAbove = 0.6f, kSplitTo = 2.0f;       // of an SM's average: split tiles above, into parts of 1 / kSplitTo
 __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys, int nsys,
                                                      const int *__restrict__ tile_base, const Ctl *__restrict__ ctl,
                                                      int own_max, int blocks, int2 *jobs, float *cost, int *meta)

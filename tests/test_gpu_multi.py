@@ -10,8 +10,8 @@ import numpy as np
 import pytest
 
 import paper_2211_15630_gb300 as A
-from gpu_helpers import params
-from inputs import clustered_state, uniform_state
+from tests.gpu_helpers import params
+from tests.inputs import clustered_state, uniform_state
 
 pytestmark = pytest.mark.gpu
 

@@ -194,3 +194,35 @@ def test_pipelined_ensemble_equals_block_kernel(lib):
     finally:
         A.aap_ens_destroy(e1)
         A.aap_ens_destroy(e2)
+
+
+@pytest.mark.parametrize("kw,w", [
+    (dict(n=60000, lx=170.0, ly=160.0, eta=0.3, seed=31), 9.0),
+    (dict(n=60000, lx=170.0, ly=160.0, eta=0.2, seed=32, model=A.AAP_NVM, by=1), 3.0),
+    (dict(n=50000, lx=400.0, ly=380.0, eta=0.4, v=1.0, seed=33, model=A.AAP_LANGEVIN, bx=1, by=1), 14.0),
+    (dict(n=9000, lx=60.0, ly=60.0, eta=0.3, seed=34, tile_w=64, tile_h=6), 20.0)])
+def test_split_tiles_match_whole_block_kernel(kw, w):
+    """Tiles far denser than the rest are split into parts that several blocks
+    update (and the densest go to whole blocks before the pipeline): states,
+    counts and measured histograms equal to the whole-block kernel's, bit for
+    bit, over the steps that reorder the tiles."""
+    n, lx, ly = kw["n"], kw["lx"], kw["ly"]
+    c = inputs.clustered_state(n // 4, lx, ly, 5, 0.3 * lx, 0.6 * ly, w)
+    d = inputs.clustered_state(n // 8, lx, ly, 6, 0.9 * lx, 0.1 * ly, 2.0 * w)
+    u = inputs.uniform_state(n - n // 4 - n // 8, lx, ly, 7)
+    x, y, th = (np.concatenate(v) for v in zip(c, d, u))
+    hs = [A.aap_create(params(threads=t, **kw)) for t in (1024, 512)]
+    try:
+        for h in hs:
+            A.aap_set_state(h, np.clip(x, 0.0, lx), np.clip(y, 0.0, ly), th.astype(np.float32), 0)
+        for steps in (1, 7, 60):
+            for h in hs:
+                A.aap_measure(h, steps)
+            for a, b in zip(*(A.aap_get_state(h, n) for h in hs)):
+                assert np.array_equal(a, b)
+        for a, b in zip(*(A.aap_get_histograms(h, 100, 100) for h in hs)):
+            assert np.array_equal(a, b)
+        assert np.array_equal(*(A.aap_step_neighbours(h, n) for h in hs))
+    finally:
+        for h in hs:
+            A.aap_destroy(h)
