@@ -671,11 +671,16 @@ int alloc_all(aap_handle *h)
         if ((rc = dev_alloc(h, &h->d_sys, sizeof(Sys)))) return rc;
         if ((rc = dev_alloc(h, &h->d_tile_base, 2 * sizeof(int)))) return rc;
         if ((rc = dev_alloc(h, &h->d_ctl, sizeof(Ctl)))) return rc;
-        const size_t dense = aapk::job_count(S.ntiles) * sizeof(int);
-        if ((rc = dev_alloc(h, &h->d_dense, dense))) return rc;
+        // one allocation: the pipelined step's jobs, its list of dense tiles, and
+        // the counters of the many-steps kernel
+        const size_t jobs = (aapk::job_bytes(S.ntiles) + 15) / 16 * 16;
+        const size_t dense = (aapk::job_count(S.ntiles) * sizeof(int) + 15) / 16 * 16;
+        unsigned char *buf = nullptr;
+        if ((rc = dev_alloc(h, &buf, jobs + dense + (h->L.multi ? aapk::multi_bytes(S.ntiles) : 0)))) return rc;
+        h->d_jobs = reinterpret_cast<int2 *>(buf);
+        h->d_dense = reinterpret_cast<int *>(buf + jobs);
+        if (h->L.multi) h->d_multi = reinterpret_cast<int *>(buf + jobs + dense);
         AAP_CK(cudaMemsetAsync(h->d_dense, 0, dense, h->stream));
-        if (h->L.pipe && (rc = dev_alloc(h, &h->d_jobs, aapk::job_bytes(S.ntiles)))) return rc;
-        if (h->L.multi && (rc = dev_alloc(h, &h->d_multi, aapk::multi_bytes(S.ntiles)))) return rc;
     }
     if ((rc = dev_alloc(h, &h->d_x0tab, (size_t)(S.ntx + 1) * sizeof(int)))) return rc;
     if ((rc = dev_alloc(h, &h->d_y0tab, (size_t)(S.nty + 1) * sizeof(int)))) return rc;
@@ -1127,7 +1132,6 @@ struct aap_ens {
     size_t scratch_bytes = 0;
     int *d_dense = nullptr;             // pipelined step: its jobs, and those left to the whole-block routine
     size_t dense_tiles = 0;
-    std::vector<int> order;             // replicas in the order of their descriptors (densest first)
     int *d_err = nullptr;               // [count + 4] the replicas' error words
     double *d_stats = nullptr;          // [count][16] their measurement sums
     unsigned long long *d_obs = nullptr;    // [count][8] observed sums of a window's first state
@@ -1203,7 +1207,7 @@ int ens_combine(aap_ens *e)
         L.hist_words = std::max(L.hist_words, h->L.hist_words);
         L.scratch_cap = std::max(L.scratch_cap, h->L.scratch_cap);
         L.spill_list_cap = std::max(L.spill_list_cap, h->L.spill_list_cap);
-        total += e->m[e->order[r]]->hs.ntiles;
+        total += h->hs.ntiles;
         tb[r + 1] = (int)total;
     }
     if (total >= (1ll << 30)) return fail(AAP_EINVAL, "too many tiles in the ensemble");
@@ -1302,16 +1306,6 @@ int ens_build(aap_ens *e, int pol)
         return fail(AAP_ENOMEM, "ensemble descriptor allocation failed");
     }
     AAP_CK(cudaMemset(e->d_ctl, 0, sizeof(Ctl)));
-    // the tiles of the densest replicas are claimed first (the longest jobs
-    // first, so that the step does not end on one): replica r has the
-    // descriptor slot[r]
-    std::vector<int> order(count), slot(count);
-    for (int r = 0; r < count; ++r) order[r] = r;
-    const auto density = [&](int r) { return (double)e->params[r].n * e->params[r].r * e->params[r].r /
-                                             (e->params[r].lx * e->params[r].ly); };
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return density(a) > density(b); });
-    for (int k = 0; k < count; ++k) slot[order[k]] = k;
-    e->order = order;
     for (int r = 0; r < count; ++r) {
         aap_handle *h = new aap_handle();
         e->m.push_back(h);
@@ -1322,7 +1316,7 @@ int ens_build(aap_ens *e, int pol)
         h->nom_th = kPolicies[pol].th;
         if (h->nom_tw == 0) density_tile(h->p, &h->nom_tw, &h->nom_th);
         if (!h->p.threads) h->p.threads = kPolicies[pol].threads;
-        h->d_sys = e->d_sys + slot[r];
+        h->d_sys = e->d_sys + r;
         h->d_ctl = e->d_ctl;
         h->ens_err = e->d_err + r;
         h->ens_stats = e->d_stats + 16 * (size_t)r;

@@ -500,11 +500,18 @@ cudaError_t configure_multi(LaunchCfg &L, bool species, int ntiles, int sm_count
     if (!coop) return cudaSuccess;
     const MultiKernel k = multi_kernel(L.model, species, threads);
     if (!k) return cudaErrorInvalidValue;
-    cudaFuncAttributes a;
-    if ((e = cudaFuncGetAttributes(&a, k)) != cudaSuccess) return e;
+    // the kernel's static shared memory, looked up once per kernel (a handle is
+    // laid out several times while it is made)
+    static std::atomic<int> stat[2][3][2];
+    std::atomic<int> &st = stat[threads == 512][L.model][species];
+    if (st.load() == 0) {
+        cudaFuncAttributes a;
+        if ((e = cudaFuncGetAttributes(&a, k)) != cudaSuccess) return e;
+        st.store((int)a.sharedSizeBytes + 1);
+    }
     // every block resident at once: as much staging as that leaves each
     const int bps = (blocks + sm_count - 1) / sm_count;
-    const long long room = std::min<long long>(optin, per_sm / bps - 1024) - (long long)a.sharedSizeBytes;
+    const long long room = std::min<long long>(optin, per_sm / bps - 1024) - (st.load() - 1);
     int cap = 4096;
     while (cap >= min_cap && (long long)multi_smem(cap, L.pipe_nceh, L.hist_words) > room) cap -= 32;
     if (cap < min_cap) return cudaSuccess;
@@ -517,9 +524,8 @@ cudaError_t configure_multi(LaunchCfg &L, bool species, int ntiles, int sm_count
     }
     e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, std::max(smem, limit.load()));
     if (e != cudaSuccess) return e;
-    int fit = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, k, threads, smem)) != cudaSuccess) return e;
-    if ((long long)fit * sm_count < blocks) return cudaSuccess;
+    // bps blocks fit an SM: their registers by the launch bounds, their shared
+    // memory by `room` (the cooperative launch itself checks)
     L.multi = 1;
     L.multi_species = species ? 1 : 0;
     L.multi_cap = cap;

@@ -1,4 +1,4 @@
-// aap_pipe.cu -- the pipelined tile step of one system or an ensemble of
+// aap_pipe.cu -- the pipelined tile step of one system, or of an ensemble of
 // systems with one species each (sm_103a).
 //
 // One time step (Sec. 2 of Kuersten, "Aligning Active Particles Py
@@ -36,9 +36,13 @@
 //
 // Tile i+1 is copied and sorted while the update warps work on tile i, and an
 // update warp that is done with tile i starts on tile i+1 without waiting for
-// the slowest warp.  Tiles whose staged set does not fit the shared buffers
-// go to a list and are done at the end by the whole block with the tile
-// routine of aap_tile.cuh (shared staging area or global scratch).  Every
+// the slowest warp.  What is claimed are jobs, the longest first: a tile, or a
+// part of a dense one (the whole tile staged and sorted, a share of its own
+// particles updated; k_tile_order in aap_kernels.cu).  Tiles whose staged set
+// does not fit the shared buffers are done by the whole block with the tile
+// routine of aap_tile.cuh (shared staging area or global scratch): those known
+// when the jobs were ordered before the pipeline starts, others, which go to a
+// list, at the end.  Every
 // mbarrier wait is bounded (about two seconds of SM clock); a wait that runs
 // out sets ERR_TIMEOUT in the error word and the block winds down.
 #include <algorithm>
