@@ -107,7 +107,6 @@ struct aap_handle {
     bool err_pending = false;
     int relayouts = 0;
     bool multi_refused = false;     // the cooperative launch did not fit the context
-    int order_age = 0;
     bool multi_on = true;           // the tiles are light enough for many steps per launch
     // ensemble membership: steps are launched by the ensemble for all members,
     // whose error words and measurement sums lie side by side in its arrays
@@ -341,6 +340,7 @@ int set_pipe_launch(LaunchCfg &L, bool species, int twmax, int thmax, int total_
     const size_t smem = aapk::pipe_smem_bytes(L.pipe_cap, L.pipe_cap_own, L.pipe_nceh, L.hist_words);
     AAP_CK(species ? aapk::configure_pipe_kernel_species(L.model, smem) : aapk::configure_pipe_kernel(L.model, smem));
     L.pipe_species = species ? 1 : 0;
+    L.pipe_few = total_tiles <= aapk::kFewPerBlock * L.pipe_grid;
     L.pipe = 1;
     L.threads = 1024;
     return AAP_OK;
@@ -863,9 +863,7 @@ int run_steps_adaptive(aap_handle *h, long long nsteps)
         h->since_copy += k;
         if (h->since_copy < kAdaptSteps) continue;
         h->since_copy = 0;
-        // (an order of more than 4096 tiles takes 55 us and matters less: a quarter as often)
-        if (h->L.pipe && !use_multi(h) && (h->hs.ntiles <= 4096 || (++h->order_age & 3) == 0))
-            AAP_CK(aapk::launch_tile_order(h->L, h->stream));
+        if (h->L.pipe && !use_multi(h)) AAP_CK(aapk::launch_tile_order(h->L, h->stream));
         const int slot = h->batch_slot;
         if ((rc = copy_words(h, h->pinned_err + 4 * (1 + slot)))) return rc;
         AAP_CK(cudaEventRecord(h->batch_ev[slot], h->stream));

@@ -187,17 +187,14 @@ __global__ void __launch_bounds__(1024) k_finish(Sys *sys, int nsys, const int *
 // share of the particles (a clustered state of N = 524,288: its densest tile
 // has three times the pairs of an average SM).  One block sorts the jobs of
 // all systems by the class of their cost (two classes per factor of two),
-// stable inside a class, so that neighbours stay together.  With many tiles per
-// SM only the few that alone would take half of an SM's time go first and the
-// rest keeps the raster order: dense tiles one after another leave the
-// pipeline's roles waiting for each other, where light ones between them fill
-// the gaps (N = 2^24, clustered, all dense tiles first: 0.83 -> 0.86 ms per
-// step; 256 replicas: 1.04 -> 1.15 ms).  Run every few dozen steps: loads change
-// slowly.
+// stable inside a class, so that neighbours stay together.  Only for systems of
+// few tiles per SM (pipe_few): with many, dense tiles one after another leave
+// the pipeline's roles waiting for each other where light ones between them
+// fill the gaps (N = 2^24, clustered: 0.83 -> 0.86 ms per step).  Run every few
+// dozen steps: loads change slowly.
 // jobs: [total + kMaxParts] {tile, part | parts << 8}; cost: [total] scratch;
 // meta: the number of leading jobs that whole blocks do first (tiles of more
 // own particles than own_max, two buffers of the pipeline), and of all jobs.
-constexpr int kFewPerBlock = 12;
 constexpr float kSplitAbove = 0.6f, kSplitTo = 2.0f;       // of an SM's average: split tiles above, into parts of 1 / kSplitTo
 __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys, int nsys,
                                                      const int *__restrict__ tile_base, const Ctl *__restrict__ ctl,
@@ -234,11 +231,8 @@ __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys
     float all = 0.f;
     for (int w = 0; w < 32; ++w) all += s_sum[w];
     const float mean = fmaxf(all / (float)max(total, 1), 1e-20f), share = fmaxf(all / (float)blocks, 1e-20f);
-    const bool few = total <= kFewPerBlock * blocks;
     const auto cls = [&](float f, int K) {
-        if (!few && fabsf(f) <= 0.5f * share) return 2;
         if (f < 0.f) return 0;
-        if (!few) return 1;
         return 1 + min(max((int)floorf(8.0f - 2.0f * __log2f(fmaxf(f, 1e-20f) / ((float)K * mean))), 0), kClasses - 2);
     };
     const auto parts = [&](float f) {
@@ -638,6 +632,7 @@ cudaError_t launch_insert(const Sys &S, int b, const double *x, const double *y,
 
 cudaError_t launch_tile_order(const LaunchCfg &L, cudaStream_t st)
 {
+    if (!L.pipe_few) return cudaSuccess;
     k_tile_order<<<1, 1024, 0, st>>>(L.sys, L.nsys, L.tile_base, L.ctl, 2 * L.pipe_cap_own, L.pipe_grid, L.jobs,
                                      job_cost(L), job_meta(L));
     return cudaGetLastError();

@@ -27,7 +27,7 @@ struct LaunchCfg {
     // pipelined step (pipe_species: systems of several species): shared buffers of pipe_cap
     // staged / pipe_cap_own own particles per tile, one block per SM; tiles
     // that do not fit go to dense_list (device [job_count], zero between steps)
-    int pipe, pipe_species;
+    int pipe, pipe_species, pipe_few;    // pipe_few: at most kFewPerBlock tiles per block
     int pipe_cap, pipe_cap_own, pipe_grid;
     int pipe_nceh;               // half cells (split along x) of the largest extended tile, (2 tw + 4)(th + 2)
     int *dense_list;
@@ -45,6 +45,7 @@ struct LaunchCfg {
 // The pipelined step's jobs: up to one per tile and kMaxParts more, the tiles'
 // costs (scratch), and {leading jobs for whole blocks, jobs}.
 constexpr int kMaxParts = 1024;
+constexpr int kFewPerBlock = 12;
 inline size_t job_count(int tiles) { return (size_t)tiles + kMaxParts; }
 inline size_t job_bytes(int tiles) { return job_count(tiles) * sizeof(int2) + (size_t)round_up(tiles, 4) * 4 + 16; }
 inline float *job_cost(const LaunchCfg &L) { return reinterpret_cast<float *>(L.jobs + job_count(L.job_tiles)); }

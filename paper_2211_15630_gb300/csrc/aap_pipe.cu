@@ -442,7 +442,7 @@ __device__ __forceinline__ void sort_map(PipeShared &sh, const PipeBufs &B, int 
 // Scan the histogram into output buffer b's cell starts (clearing the
 // histogram), the own-row offsets and the tile's output meta, then place the
 // records in cell order.  The output buffer must be free.
-template <int MODEL, bool SP>
+template <int MODEL, bool SP, bool FEW>
 __device__ __forceinline__ void sort_order(PipeShared &sh, const PipeBufs &B, int r, int b, int tid, int NS,
                                            int cap_own)
 {
@@ -501,7 +501,7 @@ __device__ __forceinline__ void sort_order(PipeShared &sh, const PipeBufs &B, in
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         int first = 0, last = carry;
-        if ((M.part >> 8) > 1) {
+        if (FEW && (M.part >> 8) > 1) {
             __syncwarp();
             const auto row_start = [&](int rw) { return cst[(rw + 1) * W2 + 2] + B.rowoff[rw + 1]; };
             const auto cell_start = [&](int rw, int c) { return cst[(rw + 1) * W2 + 2 + 2 * c] + B.rowoff[rw + 1]; };
@@ -584,10 +584,9 @@ __device__ __forceinline__ void flush_hist(PipeShared &sh, const PipeBufs &B, in
 }
 
 // A tile too large for the pipeline's buffers, by the whole block (every thread
-// calls) with the shared staging area or the block's global scratch.  Out of
-// line: it is called before and after the pipeline.
+// calls) with the shared staging area or the block's global scratch.
 template <int MODEL>
-__device__ __noinline__ void whole_block_tile(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_base,
+__device__ __forceinline__ void whole_block_tile(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_base,
                                               int2 job, int cap, int cap_own, int nceh_max, int nce_max, int hist_words,
                                               unsigned char *mine, int scratch_cap, int spill_list_cap, long long step,
                                               int total)
@@ -642,10 +641,26 @@ __device__ __noinline__ void whole_block_tile(const Sys *__restrict__ sys, int n
     __syncthreads();
 }
 
+// The same out of line, for the kernel that calls it before and after the
+// pipeline.
+template <int MODEL>
+__device__ __noinline__ void whole_block_tile_call(const Sys *__restrict__ sys, int nsys,
+                                                   const int *__restrict__ tile_base, int2 job, int cap, int cap_own,
+                                                   int nceh_max, int nce_max, int hist_words, unsigned char *mine,
+                                                   int scratch_cap, int spill_list_cap, long long step, int total)
+{
+    whole_block_tile<MODEL>(sys, nsys, tile_base, job, cap, cap_own, nceh_max, nce_max, hist_words, mine, scratch_cap,
+                            spill_list_cap, step, total);
+}
+
 // The pipelined step of one or more systems with one species each (any
 // model; the systems of one launch share it): one block of kPipeThreads
 // threads per SM.  tile_base[nsys + 1] is the prefix of the systems' tiles.
-template <int MODEL, bool SP, int NSORT>
+// FEW: few tiles per SM -- jobs in the order of k_tile_order, dense tiles split
+// or done before the pipeline.  With many tiles per SM these gain nothing and
+// what they add to the kernel costs 2 to 5% (N = 2^24, clustered: 870 -> 901 us
+// per step), so such systems claim their tiles in raster order without them.
+template <int MODEL, bool SP, int NSORT, bool FEW>
 __global__ void __launch_bounds__(kPipeThreads, 1)
 k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_base, Ctl *ctl, int cap, int cap_own,
             int nceh_max, int nce_max, int hist_words, const int2 *__restrict__ jobs, const int *__restrict__ meta,
@@ -692,9 +707,14 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
         // jobs (tiles, or parts of dense ones) are claimed in the order of
         // k_tile_order, after the leading ones that whole blocks do before
         if (lane == 0) {
-            const int front = meta[0], njobs = meta[1];
-            g0 = atomicAdd(&ctl->tile_next, 1) + front;
-            if (g0 < njobs) job0 = jobs[g0];
+            if (FEW) {
+                const int front = meta[0], njobs = meta[1];
+                g0 = atomicAdd(&ctl->tile_next, 1) + front;
+                if (g0 < njobs) job0 = jobs[g0];
+            } else {
+                g0 = atomicAdd(&ctl->tile_next, 1);
+                job0 = make_int2(g0, 1 << 8);
+            }
         }
         g0 = __shfl_sync(0xffffffffu, g0, 0);
         job0.x = __shfl_sync(0xffffffffu, job0.x, 0);
@@ -705,8 +725,8 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
     } else if (tid == kPipeThreads - 33) {
         sh.step = ctl->step;
     } else if (tid == kPipeThreads - 65) {
-        sh.nfront = meta[0];
-        sh.total = meta[1];
+        sh.nfront = FEW ? meta[0] : 0;
+        sh.total = FEW ? meta[1] : tile_base[nsys];
     } else if (nsys == 1 && warp <= 24) {
         const int words = (int)(sizeof(Sys) / 4), k = (warp - 1) / 8;       // eight warps a copy
         const int *src = reinterpret_cast<const int *>(sys);
@@ -725,10 +745,10 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
 
     // tiles that were far too large for the buffers when they were ordered: now,
     // not after the pipeline, where they would be what the step waits for
-    if ((int)blockIdx.x < sh.nfront) {
+    if (FEW && (int)blockIdx.x < sh.nfront) {
         for (int d = blockIdx.x; d < min(sh.nfront, total); d += gridDim.x)
-            whole_block_tile<MODEL>(sys, nsys, tile_base, jobs[d], cap, cap_own, nceh_max, nce_max, hist_words, mine,
-                                    scratch_cap, spill_list_cap, step, total);
+            whole_block_tile_call<MODEL>(sys, nsys, tile_base, jobs[d], cap, cap_own, nceh_max, nce_max, hist_words, mine,
+                                         scratch_cap, spill_list_cap, step, total);
         if (tid == 0) sh.load = sh.staged = 0x7fffffff;
         clear_tables();
         __syncthreads();
@@ -779,7 +799,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
         for (;;) {
             // the following tile, claimed now so that its round trip overlaps this one's copies
             int gn = 0;
-            if (g < total && lane == 0) gn = atomicAdd(&ctl->tile_next, 1) + sh.nfront;
+            if (g < total && lane == 0) gn = atomicAdd(&ctl->tile_next, 1) + (FEW ? sh.nfront : 0);
             int n_spill = 0, n_own = 0, mode = 0;               // 0: whole-block list, 1: normal, 2: wide
             if (g < total) {
                 const bool scanned = copy_spills(Sc, pl, cur, min(nsp, Sc.spill_cap), spill_e, spill_s, n_spill,
@@ -796,10 +816,10 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
                         dense_list[j] = g + 1;
                     }
                     int2 jn = make_int2(0, 0);
-                    if (lane == 0 && gn < total) jn = jobs[gn];
+                    if (FEW && lane == 0 && gn < total) jn = jobs[gn];
                     g = __shfl_sync(0xffffffffu, gn, 0);
-                    job.x = __shfl_sync(0xffffffffu, jn.x, 0);
-                    job.y = __shfl_sync(0xffffffffu, jn.y, 0);
+                    job = FEW ? make_int2(__shfl_sync(0xffffffffu, jn.x, 0), __shfl_sync(0xffffffffu, jn.y, 0))
+                              : make_int2(g, 1 << 8);
                     if (g < total) plan(job.x);
                     continue;
                 }
@@ -843,7 +863,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
             const long long ts0 = PT_NOW();
             copy_commit(pl, Sg, si, lt, M, n_spill, n_own, mode == 2, job.y, spill_s);
             int2 jn = make_int2(0, 0);
-            if (lane == 0 && gn < total) jn = jobs[gn];         // in flight beside the copies
+            if (FEW && lane == 0 && gn < total) jn = jobs[gn];         // in flight beside the copies
             if (lane == 0) PT_ADD(2, PT_NOW() - ts0);
             const long long ti0 = PT_NOW();
             int4 *R = B.raw(r);
@@ -884,8 +904,8 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
             const long long tq0 = PT_NOW();
             g = __shfl_sync(0xffffffffu, gn, 0);
             const long long tq1 = PT_NOW();
-            job.x = __shfl_sync(0xffffffffu, jn.x, 0);
-            job.y = __shfl_sync(0xffffffffu, jn.y, 0);
+            job = FEW ? make_int2(__shfl_sync(0xffffffffu, jn.x, 0), __shfl_sync(0xffffffffu, jn.y, 0))
+                      : make_int2(g, 1 << 8);
             if (g < total) plan(job.x);
             if (lane == 0) {
                 PT_ADD(13, tq1 - tq0);
@@ -974,7 +994,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
                 for (int i = st; i < words; i += NS) dst[i] = src[i];
                 if (st == 0) sh.osys[b] = si;
             }
-            sort_order<MODEL, SP>(sh, B, r, b, st, NS, wide ? 2 * cap_own : cap_own);
+            sort_order<MODEL, SP, FEW>(sh, B, r, b, st, NS, wide ? 2 * cap_own : cap_own);
             sort_sync(NS);
             if (st == 0) {
                 PT_ADD(6, PT_NOW() - t0);
@@ -1037,7 +1057,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
                 int c = 0;
                 if (lane == 0) c = atomicAdd(&sh.chunk[b], 1);
                 c = __shfl_sync(0xffffffffu, c, 0);
-                const int o0 = O.o_first + c * 32;
+                const int o0 = (FEW ? O.o_first : 0) + c * 32;
                 if (o0 >= O.n_own) break;
                 update_one<MODEL, SP, 1>(S, O, P, cst, RB, OR, OQ, o0 + lane, step, measure, B.mhist(b), acc, ToSystem{});
             }
@@ -1100,8 +1120,12 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
         const int g = sh.dense_tile;
         if (g < 0) break;
         if (tid == 0) sh.load = sh.staged = 0x7fffffff;
-        whole_block_tile<MODEL>(sys, nsys, tile_base, jobs[g], cap, cap_own, nceh_max, nce_max, hist_words, mine, scratch_cap,
-                                spill_list_cap, step, total);
+        if (FEW)
+            whole_block_tile_call<MODEL>(sys, nsys, tile_base, jobs[g], cap, cap_own, nceh_max, nce_max, hist_words, mine,
+                                         scratch_cap, spill_list_cap, step, total);
+        else
+            whole_block_tile<MODEL>(sys, nsys, tile_base, make_int2(g, 1 << 8), cap, cap_own, nceh_max, nce_max,
+                                    hist_words, mine, scratch_cap, spill_list_cap, step, total);
         if (tid == 0) PT_ADD(11, 1);
     }
     if (nsys == 1 && tid == 0) {
@@ -1120,8 +1144,11 @@ template <int MODEL>
 static cudaError_t static_pipe_t(size_t *bytes)
 {
     cudaFuncAttributes a;
-    const cudaError_t e = cudaFuncGetAttributes(&a, k_step_pipe<MODEL, kSpecies, AAP_PIPE_SORT_WARPS>);
-    if (e == cudaSuccess) *bytes = a.sharedSizeBytes;
+    cudaError_t e = cudaFuncGetAttributes(&a, k_step_pipe<MODEL, kSpecies, AAP_PIPE_SORT_WARPS, true>);
+    if (e != cudaSuccess) return e;
+    *bytes = a.sharedSizeBytes;
+    e = cudaFuncGetAttributes(&a, k_step_pipe<MODEL, kSpecies, AAP_PIPE_SORT_WARPS, false>);
+    *bytes = std::max<size_t>(*bytes, a.sharedSizeBytes);
     return e;
 }
 
@@ -1145,8 +1172,12 @@ static cudaError_t config_pipe_t(size_t smem)
     int want = (int)smem, prev = limit.load();
     while (want > prev && !limit.compare_exchange_weak(prev, want)) {
     }
-    return cudaFuncSetAttribute(k_step_pipe<MODEL, kSpecies, AAP_PIPE_SORT_WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                std::max(want, limit.load()));
+    want = std::max(want, limit.load());
+    const cudaError_t e = cudaFuncSetAttribute(k_step_pipe<MODEL, kSpecies, AAP_PIPE_SORT_WARPS, true>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, want);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_step_pipe<MODEL, kSpecies, AAP_PIPE_SORT_WARPS, false>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, want);
 }
 
 cudaError_t PIPE_FN(set_pipe_test)(long long wait_cycles, int stall)
@@ -1170,7 +1201,9 @@ template <int MODEL>
 static cudaError_t launch_pipe_t(const LaunchCfg &L, cudaStream_t st)
 {
     const size_t smem = pipe_smem_bytes(L.pipe_cap, L.pipe_cap_own, L.pipe_nceh, L.hist_words);
-    return launch_after(k_step_pipe<MODEL, kSpecies, AAP_PIPE_SORT_WARPS>, L.pipe_grid, kPipeThreads, smem, st, L.sys, L.nsys,
+    const auto k = L.pipe_few ? k_step_pipe<MODEL, kSpecies, AAP_PIPE_SORT_WARPS, true>
+                              : k_step_pipe<MODEL, kSpecies, AAP_PIPE_SORT_WARPS, false>;
+    return launch_after(k, L.pipe_grid, kPipeThreads, smem, st, L.sys, L.nsys,
                         L.tile_base, L.ctl, L.pipe_cap, L.pipe_cap_own, L.pipe_nceh, L.nce_max, L.hist_words,
                         L.jobs, job_meta(L), L.dense_list, L.scratch, L.scratch_per_block, L.scratch_cap, L.spill_list_cap);
 }
