@@ -45,7 +45,7 @@ struct LaunchCfg {
 // The pipelined step's jobs: up to one per tile and kMaxParts more, the tiles'
 // costs (scratch), and {leading jobs for whole blocks, jobs}.
 constexpr int kMaxParts = 1024;
-constexpr int kFewPerBlock = 12;
+constexpr int kFewPerBlock = 12;     // (2^24 at 28 tiles per SM loses 4% with the job order, 10^6 flocking at 6 to 7 gains 23%)
 inline size_t job_count(int tiles) { return (size_t)tiles + kMaxParts; }
 inline size_t job_bytes(int tiles) { return job_count(tiles) * sizeof(int2) + (size_t)round_up(tiles, 4) * 4 + 16; }
 inline float *job_cost(const LaunchCfg &L) { return reinterpret_cast<float *>(L.jobs + job_count(L.job_tiles)); }

@@ -226,3 +226,28 @@ def test_split_tiles_match_whole_block_kernel(kw, w):
     finally:
         for h in hs:
             A.aap_destroy(h)
+
+
+@pytest.mark.parametrize("model", [A.AAP_VM, A.AAP_NVM, A.AAP_LANGEVIN])
+@pytest.mark.parametrize("side", [330.0, 420.0])
+def test_raster_and_job_order_match_whole_block_kernel(model, side):
+    """Fewer and more than 12 tiles per SM (tiles of 8 x 8 cells: about 1700
+    and 2700), with tiles that do not fit the pipeline: states equal to the
+    whole-block kernel's, bit for bit."""
+    n = 120000
+    kw = dict(n=n, lx=side, ly=side, eta=0.3, seed=41, model=model, tile_w=8, tile_h=8)
+    c = inputs.clustered_state(n // 4, side, side, 5, 0.3 * side, 0.6 * side, 6.0)
+    u = inputs.uniform_state(n - n // 4, side, side, 7)
+    x, y, th = (np.concatenate(v) for v in zip(c, u))
+    hs = [A.aap_create(params(threads=t, **kw)) for t in (1024, 512)]
+    try:
+        for h in hs:
+            A.aap_set_state(h, np.clip(x, 0.0, side), np.clip(y, 0.0, side), th.astype(np.float32), 0)
+        for steps in (1, 40):
+            for h in hs:
+                A.aap_step(h, steps)
+            for a, b in zip(*(A.aap_get_state(h, n) for h in hs)):
+                assert np.array_equal(a, b)
+    finally:
+        for h in hs:
+            A.aap_destroy(h)
