@@ -57,7 +57,7 @@ struct MultiShared {
     int cap[kSegs];
     int4 map[kSegs];            // as RawMeta::map of the pipelined step
     int segpre[kSegs + 1];
-    int n_spill;
+    int n_spill, own_spill;     // spill matches, and those of the tile's own regions
     int warp_tot[kMultiWarps];
     int maxc;
     int ok;
@@ -132,11 +132,15 @@ __device__ __forceinline__ bool multi_barrier(unsigned *bar, unsigned target, in
 }
 
 // One step of the block's tile, staged in A.  m records in all, of which
-// m_seg from the segments and the rest from the spill matches.  true when
-// the warp updated particles.
+// m_seg from the segments and the rest from the spill matches; own of them
+// are the tile's own by the counters.  true when the warp updated particles.
+// A record's rank in its half cell takes all 16 bits of slotw (the global
+// scratch stages up to 65,472 records, and nothing keeps them out of a single
+// half cell), so the mirror flips are not stored beside it: a record in the
+// halo beyond a reflecting wall is a mirror image, and no other record is.
 template <int NT, int MODEL, bool SP>
 __device__ __forceinline__ bool multi_tile(MultiShared &sh, const MultiStage &A, const MultiTables &tb, int m, int m_seg,
-                                           long long step, const int *spill_e, const unsigned char *spill_s, int *wc,
+                                           int own, long long step, const int *spill_e, const unsigned char *spill_s, int *wc,
                                            int *ws, Acc &acc)
 {
     const Sys &S = sh.S;
@@ -169,7 +173,7 @@ __device__ __forceinline__ bool multi_tile(MultiShared &sh, const MultiStage &A,
         const unsigned Ye = ((unsigned)rr.y ^ (unsigned)my) - (unsigned)my + (unsigned)g.y;
         A.R[k] = make_int4((int)Xe, (int)Ye, rr.z, rr.w);
         A.cellw[k] = (unsigned short)((ey << 8) | ex);
-        A.slotw[k] = (unsigned short)((((g.z & 1) | ((g.w & 1) << 1)) << 14) | atomicAdd(&tb.hist[ey * W2 + ex], 1));
+        A.slotw[k] = (unsigned short)atomicAdd(&tb.hist[ey * W2 + ex], 1);
     }
     __syncthreads();
     // --- prefix scan of the histogram (cleared for the next step) ----------
@@ -215,14 +219,18 @@ __device__ __forceinline__ bool multi_tile(MultiShared &sh, const MultiStage &A,
         sh.O.n_own = n_own;
         sh.O.wide = 15 * sh.maxc >= 512;
         sh.O.dense = 2 * m > 3 * nce;
+        if (n_own != own) atomicOr(S.err, ERR_BOUNDS);
     }
     __syncwarp();
     // --- records into half-cell order, own particles listed ----------------
     const int xc = tw << (S.sx - 1), yc = th << (S.sy - 1);
+    // first and last column (row) that a mirror image cannot lie in
+    const int mxl = S.bx && sh.O.tx == 0 ? 2 : 0, mxr = S.bx && sh.O.tx == S.ntx - 1 ? 2 * tw + 1 : W2;
+    const int myl = S.by && sh.O.ty == 0 ? 1 : 0, myr = S.by && sh.O.ty == S.nty - 1 ? th : H2;
     for (int k = tid; k < m; k += NT) {
-        const unsigned cf = A.cellw[k], sl = A.slotw[k];
+        const unsigned cf = A.cellw[k];
         const int ex = cf & 255, ey = cf >> 8;
-        const int q = tb.cst[ey * W2 + ex] + (sl & 0x3fff);
+        const int q = tb.cst[ey * W2 + ex] + A.slotw[k];
         const int4 rk = A.R[k];
         float thv = __int_as_float(rk.z);
         float sn, cs;
@@ -232,11 +240,10 @@ __device__ __forceinline__ bool multi_tile(MultiShared &sh, const MultiStage &A,
         } else {
             __sincosf(thv, &sn, &cs);       // |theta| <= pi: within 2^-21.4 absolute
         }
-        const int flip = sl >> 14;
-        if (flip & 1) {
+        if (ex < mxl || ex > mxr) {
             if (MODEL != 1 || (S.order & 1)) cs = -cs; else sn = -sn;
         }
-        if (flip & 2) sn = -sn;
+        if (ey < myl || ey > myr) sn = -sn;
         float zc, zs;
         stage_angle<MODEL, SP>(S, rk.w, __float2int_rn(cs * kFixNbF), __float2int_rn(sn * kFixNbF), zc, zs);
         A.P[q] = make_float4((float)(rk.x - xc) * S.ux, (float)(rk.y - yc) * S.uy, zc, zs);
@@ -374,7 +381,7 @@ k_multi(Sys *__restrict__ sys, Ctl *ctl, int nsteps, int cap, int nceh, int hist
             // itself, the same values: no block barrier before the records)
             if (tid == 0) {
                 sh.maxc = 0;
-                sh.n_spill = 0;
+                sh.n_spill = sh.own_spill = 0;
             }
             const int c = lane < kSegs ? min(__ldcg(rc + sh.cidx[lane]), sh.cap[lane])
                                        : (lane == 31 ? min(__ldcg(rs), S.spill_cap) : 0);
@@ -382,7 +389,7 @@ k_multi(Sys *__restrict__ sys, Ctl *ctl, int nsteps, int cap, int nceh, int hist
             if (lane <= kSegs) sh.segpre[lane] = lane < kSegs ? incl - c : incl;
             const int m_seg = __shfl_sync(0xffffffffu, incl, kSegs - 1), nsp = __shfl_sync(0xffffffffu, c, 31);
             __syncwarp();
-            int m = m_seg;
+            int m = m_seg, own = sh.segpre[kRegions];
             // the block's scratch slice: staging of a tile that outgrows the
             // shared memory, then the spill matches
             unsigned char *const mine = scratch + scratch_per_block * blockIdx.x;
@@ -399,19 +406,22 @@ k_multi(Sys *__restrict__ sys, Ctl *ctl, int nsteps, int cap, int nceh, int hist
                             if (j < spill_list_cap) {
                                 spill_e[j] = e;
                                 spill_s[j] = (unsigned char)s;
+                                if (s < kRegions) atomicAdd(&sh.own_spill, 1);
                             }
                         }
                 }
                 __syncthreads();
                 if (tid == 0 && sh.n_spill > spill_list_cap) atomicOr(S.err, ERR_STAGE);
                 m += min(sh.n_spill, spill_list_cap);
+                own += sh.own_spill;
             }
             Acc acc = {0, 0, 0, 0, 0};
             bool any = false;
             if (m <= cap)
-                any = multi_tile<NT, MODEL, SP>(sh, As, tb, m, m_seg, step, spill_e, spill_s, wc, ws, acc);
+                any = multi_tile<NT, MODEL, SP>(sh, As, tb, m, m_seg, own, step, spill_e, spill_s, wc, ws, acc);
             else if (m <= scratch_cap)
-                any = multi_tile<NT, MODEL, SP>(sh, carve_multi(mine, scratch_cap), tb, m, m_seg, step, spill_e, spill_s, wc, ws, acc);
+                any = multi_tile<NT, MODEL, SP>(sh, carve_multi(mine, scratch_cap), tb, m, m_seg, own, step, spill_e, spill_s, wc, ws,
+                                                acc);
             else if (tid == 0)
                 atomicOr(S.err, ERR_STAGE | ERR_LOST);
             if (any) flush_acc<true>(acc, S.acc, cur);

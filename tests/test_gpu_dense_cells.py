@@ -1,0 +1,51 @@
+"""More than 16,384 records in one half cell: a ring of particles that move to
+its centre without noise or coupling (or a weak one) and meet there on one
+step, inside a single call, so that the kernel that runs many steps per launch
+is the one that meets them.  Equal bit for bit to the whole-block kernel
+(threads = 512), whose ranks inside a cell have the full 16 bits."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import paper_2211_15630_gb300 as A
+from tests.gpu_helpers import params
+
+pytestmark = pytest.mark.gpu
+
+N, L, RADIUS = 18000, 128.0, 40         # the ring meets after 40 steps of one cell side each
+
+
+@pytest.fixture(scope="module", autouse=True)
+def lib():
+    return A.load()
+
+
+def ring():
+    """Aimed at the middle of a half cell inside the tile of 32 x 16 cells at (64, 32)."""
+    g = np.random.default_rng(3)
+    th = g.permutation(N) * (2.0 * np.pi / N) - np.pi
+    return np.mod(80.25 - RADIUS * np.cos(th), L), np.mod(40.5 - RADIUS * np.sin(th), L), th.astype(np.float32)
+
+
+@pytest.mark.parametrize("gamma,steps", [(0.0, 41), (0.0, 45), (1e-3, 43)])
+def test_ring_that_meets_in_one_half_cell(gamma, steps):
+    x, y, th = ring()
+    out = []
+    for threads in (0, 512):
+        p = params(n=N, lx=L, ly=L, model=A.AAP_LANGEVIN, v=1.0, dt=1.0, eta=0.0, gamma=gamma, seed=31, threads=threads,
+                   tile_w=32, tile_h=16, capacity=40.0)
+        h = A.aap_create(p)
+        try:
+            A.aap_set_state(h, x, y, th, 0)
+            A.aap_step(h, steps)
+            out.append(A.aap_get_state(h, N) + (A.aap_observe(h).mean_neighbours,))
+        finally:
+            A.aap_destroy(h)
+    if gamma == 0.0:
+        # straight paths: on step RADIUS every particle is at the centre, to the
+        # fixed-point rounding and the FP32 sine of 45 steps
+        d = (steps - RADIUS) * np.array([np.cos(th), np.sin(th)])
+        assert np.abs(out[0][0] - (80.25 + d[0])).max() < 1e-3 and np.abs(out[0][1] - (40.5 + d[1])).max() < 1e-3
+    for u, v in zip(*out):
+        assert np.array_equal(u, v)
