@@ -273,6 +273,13 @@ int aap_test_fail_alloc_after(int32_t n);
  * while no step kernel is running.  The GPU context stays usable. */
 int aap_test_pipe_wait(int64_t wait_cycles, int32_t stall);
 
+/* What ran, for tests of the automatic choice of kernel.  out[0], out[1]:
+ * launches of many steps so far, and the steps in them; out[2], out[3]: of the
+ * pipelined step's last job list, the leading jobs (whole blocks do them before
+ * the pipeline starts) and all jobs (more than there are tiles where dense ones
+ * are split), both 0 where tiles are claimed in raster order.  Synchronises. */
+int aap_test_paths(aap_handle *h, int64_t out[4]);
+
 /* Forget the accumulated measurements (moments and histograms). */
 int aap_clear_results(aap_handle *h);
 
@@ -398,6 +405,9 @@ int aap_ens_info(aap_ens *e, int32_t *count, int64_t *step);
 
 /* Free the ensemble (NULL accepted).  Synchronises its stream. */
 int aap_ens_destroy(aap_ens *e);
+
+/* aap_test_paths of an ensemble's launches (out[0], out[1] are 0). */
+int aap_ens_test_paths(aap_ens *e, int64_t out[4]);
 
 #ifdef __cplusplus
 }

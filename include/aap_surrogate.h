@@ -70,6 +70,10 @@ int aap_sur_param_count(aap_sur *s, int64_t *count);
 int aap_sur_get_params(aap_sur *s, float *host, int64_t count);
 int aap_sur_set_params(aap_sur *s, const float *host, int64_t count);
 
+/* What ran, for tests of the choice between them: applications of the network
+ * by aap_sur_predict in one fused kernel (out[0]) and layer by layer (out[1]). */
+int aap_sur_test_paths(aap_sur *s, int64_t out[2]);
+
 /* FP32 gradient of the loss of the last train step (same layout).  Sync. */
 int aap_sur_get_grads(aap_sur *s, float *host, int64_t count);
 

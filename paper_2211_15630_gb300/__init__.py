@@ -29,6 +29,7 @@ EXPORTS = (
     "aap_step_neighbours", "aap_sync", "aap_get_layout", "aap_set_timing", "aap_get_timing",
     "aap_measure", "aap_get_results", "aap_clear_results", "aap_coarse_grain", "aap_get_histograms",
     "aap_save", "aap_load", "aap_test_fail_alloc_after", "aap_test_pipe_wait",
+    "aap_test_paths", "aap_ens_test_paths", "aap_sur_test_paths",
     "aap_ens_create", "aap_ens_step", "aap_ens_measure", "aap_ens_phi_mean", "aap_ens_results",
     "aap_ens_get_state", "aap_ens_get_layout", "aap_ens_autotune", "aap_ens_info", "aap_ens_destroy",
     "aap_ens_coarse_grain",
@@ -125,6 +126,9 @@ def load(path: str = LIB_PATH):
         "aap_save": (C.c_int, [vp, C.c_char_p]),
         "aap_test_fail_alloc_after": (C.c_int, [i32]),
         "aap_test_pipe_wait": (C.c_int, [i64, i32]),
+        "aap_test_paths": (C.c_int, [vp, vp]),
+        "aap_ens_test_paths": (C.c_int, [vp, vp]),
+        "aap_sur_test_paths": (C.c_int, [vp, vp]),
         "aap_load": (C.c_int, [C.c_char_p, vp, P(vp)]),
         "aap_coarse_grain": (C.c_int, [vp, i32, i32, vp]),
         "aap_ens_create": (C.c_int, [vp, i32, vp, P(vp)]),
@@ -241,6 +245,27 @@ def aap_test_pipe_wait(wait_cycles: int, stall: int) -> None:
     bound in SM cycles (<= 0: default) and whether every block's copy warp
     withholds its first tile (process-wide; call while no step runs)."""
     _check(load().aap_test_pipe_wait(int(wait_cycles), int(stall)))
+
+
+def aap_test_paths(h) -> np.ndarray:
+    """What ran (for tests): launches of many steps, the steps in them, leading jobs, jobs of the last job list."""
+    out = np.zeros(4, np.int64)
+    _check(load().aap_test_paths(h, _p(out)))
+    return out
+
+
+def aap_ens_test_paths(e) -> np.ndarray:
+    """aap_test_paths of an ensemble's launches."""
+    out = np.zeros(4, np.int64)
+    _check(load().aap_ens_test_paths(e, _p(out)))
+    return out
+
+
+def aap_sur_test_paths(s) -> np.ndarray:
+    """What ran (for tests): applications by the fused kernel, and layer by layer."""
+    out = np.zeros(2, np.int64)
+    _scheck(load().aap_sur_test_paths(s, _p(out)))
+    return out
 
 
 def aap_destroy(h) -> None:

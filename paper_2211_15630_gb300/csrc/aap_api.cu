@@ -108,6 +108,7 @@ struct aap_handle {
     int relayouts = 0;
     bool multi_refused = false;     // the cooperative launch did not fit the context
     bool multi_on = true;           // the tiles are light enough for many steps per launch
+    long long multi_launches = 0, multi_steps = 0;
     // ensemble membership: steps are launched by the ensemble for all members,
     // whose error words and measurement sums lie side by side in its arrays
     bool member = false;
@@ -789,6 +790,18 @@ int capture_steps(const LaunchCfg &L, cudaStream_t &cap, cudaGraphExec_t &exec)
     return AAP_OK;
 }
 
+// {leading jobs, jobs} of the job list of L.
+int read_jobs(const LaunchCfg &L, cudaStream_t st, int64_t *out)
+{
+    int meta[2] = {0, 0};
+    if (L.pipe && L.pipe_few)
+        AAP_CK(cudaMemcpyAsync(meta, aapk::job_meta(L), sizeof(meta), cudaMemcpyDeviceToHost, st));
+    AAP_CK(cudaStreamSynchronize(st));
+    out[0] = meta[0];
+    out[1] = meta[1];
+    return AAP_OK;
+}
+
 // nsteps steps of L on stream st: whole chunks replay the captured graph (the
 // step index and buffer parity live on the device, so one graph serves every
 // chunk), the rest launch directly.
@@ -886,6 +899,8 @@ int run_steps(aap_handle *h, long long nsteps)
         cudaError_t e = nsteps > 0 ? aapk::launch_multi(h->L, (int)nsteps, h->stream) : cudaSuccess;
         if (e == cudaSuccess) {
             h->step += nsteps;
+            h->multi_launches += nsteps > 0;
+            h->multi_steps += nsteps;
             return AAP_OK;
         }
         // fewer SMs than the device has (a partitioned context): single steps from now on
@@ -1417,6 +1432,21 @@ int aap_test_pipe_wait(int64_t wait_cycles, int32_t stall)
     AAP_CK(aapk::set_pipe_test_species(wait_cycles, stall));
     AAP_CK(aapk::set_multi_test(wait_cycles, stall));
     return AAP_OK;
+}
+
+int aap_test_paths(aap_handle *h, int64_t out[4])
+{
+    if (!h || !out) return fail(AAP_EINVAL, "NULL argument");
+    out[0] = h->multi_launches;
+    out[1] = h->multi_steps;
+    return read_jobs(h->L, h->stream, out + 2);
+}
+
+int aap_ens_test_paths(aap_ens *e, int64_t out[4])
+{
+    if (!e || !out) return fail(AAP_EINVAL, "NULL argument");
+    out[0] = out[1] = 0;
+    return read_jobs(e->L, e->stream, out + 2);
 }
 
 int32_t aap_abi_version(void) { return 2; }

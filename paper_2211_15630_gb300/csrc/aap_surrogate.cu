@@ -1361,6 +1361,7 @@ struct aap_sur {
     cudaStream_t pstream = nullptr;
     const void *pkey[3] = {nullptr, nullptr, nullptr};
     int pbatch = -1, papps = -1;
+    long long napps[2] = {0, 0};                                       // applications: fused, layer by layer
     int loss_blocks = 0;
     long long t = 0;                                                   // Adam step
     std::vector<void *> allocs;
@@ -1452,6 +1453,10 @@ int forward(aap_sur *s, int batch, bool next)
 // two waves of two blocks per SM; at 640 tiles layer by layer takes 391 us for
 // 10 applications where a third wave would take some 480.
 constexpr int kNetWaves = 4;
+bool fused_predict(const aap_sur *s, int batch, int applications)
+{
+    return applications > 0 && batch * (s->W / kTW) * (s->H / kTH) <= kNetWaves * sm_count();
+}
 
 // The kernels of one predict call on s->stream: normalise, `applications`
 // forward passes, denormalise into dev_out.
@@ -1460,8 +1465,8 @@ int enqueue_predict(aap_sur *s, const float *dev_in, const float *dev_eta, int b
     const int H = s->H, W = s->W;
     const int grid = pixel_blocks(batch, H, W);
     SCK(cudaMemcpyAsync(s->eta, dev_eta, (size_t)batch * 4, cudaMemcpyDeviceToDevice, s->stream));
-    const int tiles = batch * (W / kTW) * (H / kTH);
-    if (applications > 0 && tiles <= kNetWaves * sm_count()) {
+    if (fused_predict(s, batch, applications)) {
+        const int tiles = batch * (W / kTW) * (H / kTH);
         NetArgs a{};
         for (int l = 0; l < 4; ++l) {
             a.wf[l] = s->wf[l];
@@ -1654,6 +1659,14 @@ int aap_sur_param_count(aap_sur *s, int64_t *count)
     return AAP_OK;
 }
 
+int aap_sur_test_paths(aap_sur *s, int64_t out[2])
+{
+    if (!s || !out) return sfail(AAP_EINVAL, "NULL argument");
+    out[0] = s->napps[0];
+    out[1] = s->napps[1];
+    return AAP_OK;
+}
+
 int aap_sur_get_params(aap_sur *s, float *host, int64_t count)
 {
     if (!s || !host || count != s->nparam) return sfail(AAP_EINVAL, "bad arguments");
@@ -1719,6 +1732,7 @@ int aap_sur_predict(aap_sur *s, const float *dev_in, const float *dev_eta, int32
         s->papps = applications;
     }
     SCK(cudaGraphLaunch(s->pexec, s->stream));
+    s->napps[fused_predict(s, batch, applications) ? 0 : 1] += applications;
     return AAP_OK;
 }
 

@@ -39,6 +39,7 @@ def test_ring_that_meets_in_one_half_cell(gamma, steps):
         try:
             A.aap_set_state(h, x, y, th, 0)
             A.aap_step(h, steps)
+            assert A.aap_test_paths(h)[1] == (0 if threads else steps)
             out.append(A.aap_get_state(h, N) + (A.aap_observe(h).mean_neighbours,))
         finally:
             A.aap_destroy(h)

@@ -1,0 +1,118 @@
+"""Which kernel ran: the equalities of the other tests hold whatever the
+automatic choice picks, so the choice itself is pinned here (aap_test_paths,
+aap_sur_test_paths)."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import paper_2211_15630_gb300 as A
+from tests.gpu_helpers import params
+from tests.inputs import clustered_state, uniform_state
+from tests.test_gpu_multi import CASES, pair
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def lib():
+    return A.load()
+
+
+@pytest.mark.parametrize("kw,species", CASES)
+def test_small_systems_run_many_steps_per_launch(kw, species):
+    p, q = pair(species, **kw)
+    for prm, steps in ((p, 71), (q, 0)):
+        h = A.aap_create(prm)
+        try:
+            A.aap_step(h, 1)
+            A.aap_step(h, 70)
+            launches, in_them = A.aap_test_paths(h)[:2]
+            assert in_them == steps and launches == (4 if steps else 0)      # 1, 32, 32, 6 steps
+        finally:
+            A.aap_destroy(h)
+
+
+def test_dense_states_leave_many_steps_and_return():
+    """A dense spot (inside one tile of 30 x 15 cells) goes to single steps at once; when it has spread (straight
+    paths, no coupling) the handle returns to many steps per launch."""
+    n, side = 3500, 60.0
+    g = np.random.default_rng(5)
+    th = g.uniform(-np.pi, np.pi, n).astype(np.float32)
+    r = g.uniform(0.0, 0.4, n)
+    h = A.aap_create(params(n=n, lx=side, ly=side, model=A.AAP_LANGEVIN, v=1.0, dt=0.5, eta=0.0, gamma=0.0, seed=6))
+    try:
+        A.aap_set_state(h, 20.2 + r * np.cos(th), 22.2 + r * np.sin(th), th, 0)
+        A.aap_step(h, 2)
+        assert A.aap_test_paths(h)[0] == 0
+        for _ in range(8):
+            A.aap_step(h, 32)
+            A.aap_sync(h)
+        assert A.aap_test_paths(h)[0] > 0
+        x, y, t = uniform_state(n, side, side, 7)
+        A.aap_set_state(h, x, y, t.astype(np.float32), 0)
+        before = A.aap_test_paths(h)[1]
+        A.aap_step(h, 10)
+        assert A.aap_test_paths(h)[1] == before + 10
+    finally:
+        A.aap_destroy(h)
+
+
+def test_withheld_arrival_is_the_many_steps_kernels():
+    h = A.aap_create(params(n=3000, lx=40.0, ly=40.0, eta=0.3, seed=23))
+    try:
+        A.aap_test_pipe_wait(20_000_000, 1)
+        A.aap_step(h, 20)
+        with pytest.raises(A.AapError) as e:
+            A.aap_sync(h)
+        assert e.value.code == A.AAP_ETIMEOUT
+        assert list(A.aap_test_paths(h)[:2]) == [1, 20]
+    finally:
+        A.aap_test_pipe_wait(0, 0)
+        A.aap_destroy(h)
+
+
+@pytest.mark.parametrize("kw,w,front", [
+    (dict(n=60000, lx=170.0, ly=160.0, eta=0.3, seed=31), 9.0, True),
+    (dict(n=60000, lx=170.0, ly=160.0, eta=0.2, seed=32, model=A.AAP_NVM, by=1), 3.0, True),
+    (dict(n=50000, lx=400.0, ly=380.0, eta=0.4, v=1.0, seed=33, model=A.AAP_LANGEVIN, bx=1, by=1), 14.0, True),
+    (dict(n=9000, lx=60.0, ly=60.0, eta=0.3, seed=34, tile_w=64, tile_h=6), 20.0, False)])
+def test_dense_tiles_are_split_and_lead(kw, w, front):
+    """The states of the split-tile test: jobs beyond the tiles, and (where a
+    tile has more own particles than two buffers hold) leading ones."""
+    n, lx, ly = kw["n"], kw["lx"], kw["ly"]
+    c = clustered_state(n // 4, lx, ly, 5, 0.3 * lx, 0.6 * ly, w)
+    d = clustered_state(n // 8, lx, ly, 6, 0.9 * lx, 0.1 * ly, 2.0 * w)
+    u = uniform_state(n - n // 4 - n // 8, lx, ly, 7)
+    x, y, th = (np.concatenate(v) for v in zip(c, d, u))
+    h = A.aap_create(params(threads=1024, **kw))
+    try:
+        A.aap_set_state(h, np.clip(x, 0.0, lx), np.clip(y, 0.0, ly), th.astype(np.float32), 0)
+        lay = A.aap_get_layout(h)
+        lead, jobs = A.aap_test_paths(h)[2:]
+        assert jobs > lay.ntx * lay.nty and (lead > 0) == front
+    finally:
+        A.aap_destroy(h)
+
+
+def test_raster_order_beyond_twelve_tiles_per_sm():
+    for side, few in ((330.0, True), (420.0, False)):
+        h = A.aap_create(params(n=120000, lx=side, ly=side, eta=0.3, seed=41, tile_w=8, tile_h=8, threads=1024))
+        try:
+            assert (A.aap_test_paths(h)[3] > 0) == few
+        finally:
+            A.aap_destroy(h)
+
+
+@pytest.mark.parametrize("batch,h,w,fused", [(1, 16, 16, True), (2, 128, 128, True), (4, 128, 128, True), (5, 128, 128, False)])
+def test_small_predictions_are_fused(batch, h, w, fused):
+    f = torch.full((batch, 3, h, w), 1.5, device="cuda")
+    eta = torch.full((batch,), 0.4, device="cuda")
+    s = A.aap_sur_create(A.aap_sur_params_default(nbx=w, nby=h, max_batch=batch))
+    try:
+        for _ in range(2):
+            A.aap_sur_predict(s, f.data_ptr(), eta.data_ptr(), batch, 3, f.data_ptr())
+        assert list(A.aap_sur_test_paths(s)) == ([6, 0] if fused else [0, 6])
+    finally:
+        A.aap_sur_destroy(s)
