@@ -407,19 +407,37 @@ __device__ __forceinline__ void warp_records(const Sys &S, int b, long long w, l
 }
 
 // The largest tile load and staged set of the state in buffer b into err[1]
-// and err[2] (a thread per tile; what the step kernels report of later states).
-__global__ void k_tile_load(Sys S, int b)
+// and err[2] (what the step kernels report of later states): a warp per tile, a
+// lane per source segment, and the spilled records of those segments.
+__global__ void __launch_bounds__(128) k_tile_load(Sys S, int b)
 {
-    const int tile = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ int s_key[4][kSegs];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tile = blockIdx.x * 4 + warp;
     if (tile >= S.ntiles) return;
     const TileGeo G = tile_geo(S, tile);
-    int own = 0, m = 0;
-    for (int s = 0; s < kSegs; ++s) {
-        m += make_seg(S, G, s, b).count;
-        if (s == 8) own = m;
+    int m = 0;
+    if (lane < kSegs) {
+        const Seg g = make_seg(S, G, lane, b);
+        m = g.count;
+        s_key[warp][lane] = g.tile * kCntStride + g.region;
     }
-    atomicMax(S.err + 1, tile_load(own, m, (2 * G.tw + 4) * (G.th + 2)));
-    atomicMax(S.err + 2, m);
+    int own = lane < kRegions ? m : 0;
+    __syncwarp();
+    const int nsp = min(S.spill_cnt[b], S.spill_cap);
+    for (int e = lane; e < nsp; e += 32) {
+        const int key = S.spill_key[b][e];
+        for (int s = 0; s < kSegs; ++s)
+            if (s_key[warp][s] == key) {
+                ++m;
+                own += s < kRegions;
+            }
+    }
+    own = __reduce_add_sync(0xffffffffu, own);
+    m = __reduce_add_sync(0xffffffffu, m);
+    if (lane == 0) {
+        atomicMax(S.err + 1, tile_load(own, m, (2 * G.tw + 4) * (G.th + 2)));
+        atomicMax(S.err + 2, m);
+    }
 }
 
 // Position (FP64, exact) of a record in box coordinates.
@@ -640,7 +658,7 @@ cudaError_t launch_tile_order(const LaunchCfg &L, cudaStream_t st)
 
 cudaError_t launch_tile_load(const Sys &S, int b, cudaStream_t st)
 {
-    k_tile_load<<<(unsigned)((S.ntiles + 63) / 64), 64, 0, st>>>(S, b);
+    k_tile_load<<<(unsigned)((S.ntiles + 3) / 4), 128, 0, st>>>(S, b);
     return cudaGetLastError();
 }
 

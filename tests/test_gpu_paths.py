@@ -59,6 +59,29 @@ def test_dense_states_leave_many_steps_and_return():
         A.aap_destroy(h)
 
 
+def test_spilled_records_count_as_load():
+    """An explicit capacity that keeps some 2,000 records of a dense spot in
+    the spill list: the regions alone look light (a load of 3,700), the tile is not
+    (15,000 with the spilled ones)."""
+    n, side = 9000, 60.0
+    c = clustered_state(3000, side, side, 5, 20.2, 22.2, 0.8)
+    u = uniform_state(n - 3000, side, side, 6)
+    x, y, th = (np.concatenate(v) for v in zip(c, u))
+    out = []
+    for threads in (0, 512):
+        h = A.aap_create(params(n=n, lx=side, ly=side, eta=0.3, v=0.1, seed=8, capacity=2.0, threads=threads))
+        try:
+            A.aap_set_state(h, x, y, th.astype(np.float32), 0)
+            A.aap_step(h, 3)
+            assert A.aap_test_paths(h)[0] == 0
+            assert A.aap_observe(h).flags & A.AAP_FLAG_SPILLED
+            out.append(A.aap_get_state(h, n))
+        finally:
+            A.aap_destroy(h)
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+
+
 def test_withheld_arrival_is_the_many_steps_kernels():
     h = A.aap_create(params(n=3000, lx=40.0, ly=40.0, eta=0.3, seed=23))
     try:
