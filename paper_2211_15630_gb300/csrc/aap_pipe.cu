@@ -983,11 +983,9 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
             // go to it (when measuring; tiles of one system share the counts)
             const int si = sh.raw[r].si;
             const int oi = sh.osys[b];
-            if (oi >= 0 && oi != si && step < sh.os[b].meas_until) {
-                flush_hist(sh, B, b, step, st, NS);
-                sort_sync(NS);
-            }
             if (oi != si) {
+                if (oi >= 0 && step < sh.os[b].meas_until) flush_hist(sh, B, b, step, st, NS);
+                sort_sync(NS);          // every sort thread has read the system before and its index
                 const int words = (int)(sizeof(Sys) / 4);
                 const int *src = reinterpret_cast<const int *>(sys + si);
                 int *dst = reinterpret_cast<int *>(&sh.os[b]);

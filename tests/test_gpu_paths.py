@@ -139,3 +139,32 @@ def test_small_predictions_are_fused(batch, h, w, fused):
         assert list(A.aap_sur_test_paths(s)) == ([6, 0] if fused else [0, 6])
     finally:
         A.aap_sur_destroy(s)
+
+
+@pytest.mark.parametrize("sizes", [[(900, 1.0)] * 400, [(30000, 8.0), (30000, 0.5), (20000, 1.0), (300, 2.0), (60000, 4.0)]])
+def test_ensemble_of_changing_systems_and_split_tiles(sizes):
+    """The sort warps change the system of an output buffer with nearly every
+    tile (400 replicas of a tile or two each, measured and not), and dense
+    replicas beside dilute ones split their tiles: equal to the whole-block
+    kernel's ensemble bit for bit."""
+    out = []
+    for threads in (1024, 512):
+        ps = [params(n=n, lx=(n / rho) ** 0.5, ly=(n / rho) ** 0.5, eta=0.2 + 0.001 * r, seed=50 + r, threads=threads)
+              for r, (n, rho) in enumerate(sizes)]
+        e = A.aap_ens_create(ps)
+        try:
+            lays = [A.aap_ens_get_layout(e, r) for r in range(len(ps))]
+            jobs = A.aap_ens_test_paths(e)[3]
+            tiles = sum(v.ntx * v.nty for v in lays)
+            if threads == 1024:
+                assert jobs == tiles if len(ps) > 100 else jobs > tiles
+            for steps in (1, 40):
+                A.aap_ens_step(e, steps)
+                A.aap_ens_measure(e, steps)
+            res = [A.aap_ens_results(e, r) for r in range(len(ps))]
+            out.append([v for r, p in enumerate(ps) for v in A.aap_ens_get_state(e, r, p.n)] +
+                       [np.array(list(v.p) + list(v.q) + list(v.nbar)) for v in res] + [A.aap_ens_phi_mean(e)])
+        finally:
+            A.aap_ens_destroy(e)
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
