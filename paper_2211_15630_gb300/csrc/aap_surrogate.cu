@@ -43,6 +43,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "aap_device.cuh"
+#include "aap_drain.cuh"
 
 #include "../../include/aap.h"
 #include "../../include/aap_surrogate.h"
@@ -609,7 +610,8 @@ __global__ void __launch_bounds__(kNetThreads, 2) k_net(const NetArgs a)
     const uint32_t tmem = s_tmem;
     const int run = warp >> 2, q = warp & 3;            // epilogue warps: their run, TMEM lane quarter
     bool ok = true;
-    for (int l = 1; l <= 3; ++l) {
+    int l = 1;                                          // at the end: the last layer issued
+    for (; l <= 3; ++l) {
         unsigned char *src = (l & 1) ? buf1 : buf0, *dst = (l & 1) ? buf0 : buf1;
         if (warp == 12) {
             if (lane == 0) {
@@ -618,7 +620,7 @@ __global__ void __launch_bounds__(kNetThreads, 2) k_net(const NetArgs a)
             }
             __syncwarp();
         } else {
-            ok = __all_sync(0xffffffffu, bar_wait(&bar[run], (uint32_t)(l - 1) & 1u));
+            ok = __all_sync(0xffffffffu, bar_wait(&bar[run], nth_parity(net_commits(l, run))));
             if (ok) {
                 asm volatile("tcgen05.fence::after_thread_sync;");
                 uint32_t r[32];
@@ -650,7 +652,7 @@ __global__ void __launch_bounds__(kNetThreads, 2) k_net(const NetArgs a)
             if (lane == 0) net_issue<2, 16, 2>(tmem, smem_addr(buf0), smem_addr(s_w + kNetW0 + 2 * kNetW1), 4, bar);
             __syncwarp();
         } else if (warp < 8) {
-            ok = __all_sync(0xffffffffu, bar_wait(&bar[run], 1u));
+            ok = __all_sync(0xffffffffu, bar_wait(&bar[run], nth_parity(net_commits(4, run))));
             if (ok) {
                 asm volatile("tcgen05.fence::after_thread_sync;");
                 uint32_t r[16];
@@ -668,14 +670,18 @@ __global__ void __launch_bounds__(kNetThreads, 2) k_net(const NetArgs a)
             }
         }
     }
-    // MMAs still running (only when a wait ran out): the last commit of each
-    // barrier is waited for once more before TMEM is freed
-    if (!ok && tid == 0)
-        for (int k = 0; k < 3; ++k) bar_wait(&bar[k], 0u);
     pdl_next();
     asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
+    ok = __syncthreads_and(ok) != 0;
     asm volatile("tcgen05.fence::after_thread_sync;");
+    if (!ok) {
+        // a wait ran out, of whichever warps: MMAs may still be running, and the
+        // commits of the last layer issued are waited for (again bounded) before
+        // TMEM is freed
+        if (tid == 0)
+            for (int k = 0; k < 3; ++k) bar_wait(&bar[k], nth_parity(net_commits(l, k)));
+        __syncthreads();
+    }
     if (warp == 12) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(128));
     if (!a.conserve) return;
     // the chunks of the tile's sixteen rows, each counted by every tile of the
