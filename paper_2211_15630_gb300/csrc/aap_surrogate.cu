@@ -302,12 +302,13 @@ __global__ void __launch_bounds__(kConvThreads) k_conv_ws(const bf16 *__restrict
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                              ::"r"(smem_addr(&afull[ac])));
             }
-            // MMAs still running (only when a wait ran out): the last commit
-            // covers every earlier MMA of this thread
-            if (i > 0 && blockIdx.x + (long long)i * gridDim.x < ntiles) {
+            // the last commit covers every MMA of this thread: those still running
+            // when a wait ran out (this thread's, or the epilogue's) end before TMEM
+            // is freed
+            if (i > 0) {
                 const int last = i - 1;
-                if (!bar_wait(&afull[last % NA], (uint32_t)(last / NA) & 1u))
-                    bar_wait(&afull[last % NA], (uint32_t)(last / NA) & 1u);
+                if (!bar_wait(&afull[last % NA], nth_parity(last / NA + 1)))
+                    bar_wait(&afull[last % NA], nth_parity(last / NA + 1));
             }
         }
         __syncwarp();

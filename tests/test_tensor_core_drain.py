@@ -35,6 +35,14 @@ int main()
         }
     for (int n = 1; n <= 9; ++n)
         if (returns(n - 1, nth_parity(n)) || !returns(n, nth_parity(n))) ++bad;
+    // the pipelined convolution: tile k's commit goes to accumulator k % 4; the
+    // last of i tiles is the last completion of its accumulator
+    for (int i = 1; i <= 20; ++i) {
+        const int last = i - 1;
+        int n = 0;
+        for (int k = 0; k < i; ++k) n += k % 4 == last % 4;
+        if (nth_parity(last / 4 + 1) != nth_parity(n)) ++bad;
+    }
     std::printf("bad %d early %d\n", bad, early_zero);
     return 0;
 }
