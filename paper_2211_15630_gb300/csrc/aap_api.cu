@@ -685,12 +685,12 @@ int alloc_all(aap_handle *h)
     }
     if ((rc = dev_alloc(h, &h->d_x0tab, (size_t)(S.ntx + 1) * sizeof(int)))) return rc;
     if ((rc = dev_alloc(h, &h->d_y0tab, (size_t)(S.nty + 1) * sizeof(int)))) return rc;
+    std::vector<int> xt(S.ntx + 1), yt(S.nty + 1);      // (kept until the stream is synchronised)
     {
-        std::vector<int> xt(S.ntx + 1), yt(S.nty + 1);
         for (int t = 0; t <= S.ntx; ++t) xt[t] = (int)((long long)t * S.ncx / S.ntx);
         for (int t = 0; t <= S.nty; ++t) yt[t] = (int)((long long)t * S.ncy / S.nty);
-        AAP_CK(cudaMemcpy(h->d_x0tab, xt.data(), xt.size() * sizeof(int), cudaMemcpyHostToDevice));
-        AAP_CK(cudaMemcpy(h->d_y0tab, yt.data(), yt.size() * sizeof(int), cudaMemcpyHostToDevice));
+        AAP_CK(cudaMemcpyAsync(h->d_x0tab, xt.data(), xt.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
+        AAP_CK(cudaMemcpyAsync(h->d_y0tab, yt.data(), yt.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
         S.x0tab = h->d_x0tab;
         S.y0tab = h->d_y0tab;
     }
@@ -1224,7 +1224,7 @@ int ens_combine(aap_ens *e)
         tb[r + 1] = (int)total;
     }
     if (total >= (1ll << 30)) return fail(AAP_EINVAL, "too many tiles in the ensemble");
-    AAP_CK(cudaMemcpy(e->d_tile_base, tb.data(), tb.size() * sizeof(int), cudaMemcpyHostToDevice));
+    AAP_CK(cudaMemcpyAsync(e->d_tile_base, tb.data(), tb.size() * sizeof(int), cudaMemcpyHostToDevice, e->stream));
     int bps = 0;
     {
         // a second block per SM is worth more than staging the densest
@@ -1288,8 +1288,7 @@ int ens_combine(aap_ens *e)
         L.jobs = reinterpret_cast<int2 *>(e->d_dense);
         L.job_tiles = (int)total;
         L.dense_list = e->d_dense + aapk::job_bytes((int)total) / sizeof(int);
-        AAP_CK(cudaMemset(L.dense_list, 0, aapk::job_count((int)total) * sizeof(int)));
-        AAP_CK(cudaStreamSynchronize(e->stream));
+        AAP_CK(cudaMemsetAsync(L.dense_list, 0, aapk::job_count((int)total) * sizeof(int), e->stream));
         int rc = set_pipe_launch(L, false, twmax, thmax, (int)total);
         if (rc) return rc;
         if (!L.pipe && e->params[0].threads == 1024)
@@ -1298,6 +1297,7 @@ int ens_combine(aap_ens *e)
     }
     if (e->exec) cudaGraphExecDestroy(e->exec);
     e->exec = nullptr;
+    AAP_CK(cudaStreamSynchronize(e->stream));           // the tile prefix is a local
     return AAP_OK;
 }
 
@@ -1318,7 +1318,7 @@ int ens_build(aap_ens *e, int pol)
         cudaGetLastError();
         return fail(AAP_ENOMEM, "ensemble descriptor allocation failed");
     }
-    AAP_CK(cudaMemset(e->d_ctl, 0, sizeof(Ctl)));
+    AAP_CK(cudaMemsetAsync(e->d_ctl, 0, sizeof(Ctl), e->stream));
     for (int r = 0; r < count; ++r) {
         aap_handle *h = new aap_handle();
         e->m.push_back(h);
@@ -1431,6 +1431,7 @@ int aap_test_pipe_wait(int64_t wait_cycles, int32_t stall)
     AAP_CK(aapk::set_pipe_test(wait_cycles, stall));
     AAP_CK(aapk::set_pipe_test_species(wait_cycles, stall));
     AAP_CK(aapk::set_multi_test(wait_cycles, stall));
+    AAP_CK(cudaDeviceSynchronize());                    // the copies, for kernels of any stream
     return AAP_OK;
 }
 

@@ -1634,9 +1634,10 @@ int aap_sur_create(const aap_sur_params *p, void *stream, aap_sur **out)
                         hw[(size_t)s->woff[l] + ((size_t)co * 9 + tap) * kLayerCin[l] + ci] = (float)((2.0 * u - 1.0) * bound);
                 }
     }
-    if (cudaMemcpy(s->w, hw.data(), (size_t)off * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemset(s->m, 0, (size_t)off * 4) != cudaSuccess || cudaMemset(s->v, 0, (size_t)off * 4) != cudaSuccess ||
-        cudaMemset(s->g, 0, (size_t)off * 4) != cudaSuccess) {
+    if (cudaMemcpyAsync(s->w, hw.data(), (size_t)off * 4, cudaMemcpyHostToDevice, s->stream) != cudaSuccess ||
+        cudaMemsetAsync(s->m, 0, (size_t)off * 4, s->stream) != cudaSuccess ||
+        cudaMemsetAsync(s->v, 0, (size_t)off * 4, s->stream) != cudaSuccess ||
+        cudaMemsetAsync(s->g, 0, (size_t)off * 4, s->stream) != cudaSuccess) {
         sfree(s);
         delete s;
         return sfail(AAP_ECUDA, "surrogate initialisation");
