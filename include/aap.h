@@ -200,10 +200,11 @@ int aap_destroy(aap_handle *h);
  * streaming (Sec. 2.1); for the Langevin model one Euler-Maruyama step of
  * length dt (Sec. 2.2); then the boundary rule of Sec. 2.4.  Every step also
  * measures p and the mean neighbour number on the fly.  Enqueues work; every
- * 32 steps (counted across calls) the device error word is copied, and the
- * call waits for the copy taken 32 steps before, so that tile regions
- * overflowed by growing clusters are enlarged in time (the state is kept bit
- * for bit) while the GPU keeps at least 32 steps queued.
+ * 32 steps (up to 35 where several share a launch; counted across calls) the
+ * device error word is copied, and the call waits for the copy taken 32 to 35
+ * steps before, so that tile regions overflowed by growing clusters are
+ * enlarged in time (the state is kept bit for bit) while the GPU keeps at
+ * least 32 steps queued.
  * Mirrors <model>_update_timesteps (Sec. 4). */
 int aap_step(aap_handle *h, int64_t nsteps);
 

@@ -869,8 +869,9 @@ int run_steps_adaptive(aap_handle *h, long long nsteps)
     long long left = nsteps;
     while (left > 0) {
         long long k = std::min(left, kAdaptSteps - h->since_copy);
-        // many steps per launch: no launch of fewer than four steps unless the call itself is that short
-        if (use_multi(h) && (k < 4 || left - k < 4)) k = std::min(left, kAdaptSteps + 3);
+        // many steps per launch: no launch of fewer than four steps unless the call
+        // itself is that short, and a copy after at most three steps more
+        if (use_multi(h) && (k < 4 || left - k < 4)) k = std::min(left, kAdaptSteps + 3 - h->since_copy);
         if ((rc = run_steps(h, k))) return rc;
         left -= k;
         h->since_copy += k;

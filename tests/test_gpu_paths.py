@@ -29,9 +29,22 @@ def test_small_systems_run_many_steps_per_launch(kw, species):
             A.aap_step(h, 1)
             A.aap_step(h, 70)
             launches, in_them = A.aap_test_paths(h)[:2]
-            assert in_them == steps and launches == (4 if steps else 0)      # 1, 32, 32, 6 steps
+            assert in_them == steps and launches == (4 if steps else 0)      # 1, 31, 32, 7 steps
         finally:
             A.aap_destroy(h)
+
+
+@pytest.mark.parametrize("calls,launches", [((31, 66), 4), ((30, 5, 32), 3), ((29, 40), 3), ((1, 2, 3, 4), 4), ((67,), 2)])
+def test_the_load_is_looked_at_every_32_to_35_steps(calls, launches):
+    """Launches end at least every 35 steps counted across calls (31 | 4, 32,
+    30; 30 | 5 | 32; 29 | 6, 34; the calls themselves; 32, 35)."""
+    h = A.aap_create(params(n=1000, lx=32.0, ly=32.0, eta=0.4, seed=3))
+    try:
+        for k in calls:
+            A.aap_step(h, k)
+        assert list(A.aap_test_paths(h)[:2]) == [launches, sum(calls)]
+    finally:
+        A.aap_destroy(h)
 
 
 def test_dense_states_leave_many_steps_and_return():
