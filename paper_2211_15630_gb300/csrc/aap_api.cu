@@ -1829,7 +1829,7 @@ int aap_coarse_grain(aap_handle *h, int32_t nbx, int32_t nby, float *dev_out)
     const long long bins = (long long)nbx * nby;
     if (h->cg_bins < bins) {
         int rc;
-        const auto words = [](long long nb) { return (size_t)(3 * nb + 1) * sizeof(unsigned long long); };
+        const auto words = [](long long nb) { return (size_t)(3 * nb) * sizeof(unsigned long long); };
         if (h->d_cg && (rc = dev_free(h, h->d_cg, words(h->cg_bins)))) return rc;
         h->d_cg = nullptr;
         h->cg_bins = 0;

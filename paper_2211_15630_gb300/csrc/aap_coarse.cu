@@ -96,14 +96,14 @@ __device__ __forceinline__ void coarse_fields(unsigned long long *acc, long long
 // go straight to acc, one atomic per record and field: merging a warp's
 // lanes of one bin first (by match and reductions, or by runs of records per
 // thread) was slower, as was a shared-memory window of the tile's bins
-// (same-address shared atomics serialise).  ticket != null (few bins): the
-// block that ends last turns the sums into fields, which saves a launch (a
-// replica's frame of 32 x 32 bins is three launches of 2 to 8 us otherwise).
+// (same-address shared atomics serialise).  The fields are a second launch,
+// which starts while this one drains: with the block that ends last doing
+// them here instead, the record loop compiled to slower code (N = 4 10^6 into
+// 128 x 128: 104 against 80 us) and a small system paid the last block's round
+// trips (N = 1000 into 32 x 32: 8.3 against 5.1 us).
 template <int NT>
-__global__ void __launch_bounds__(NT) k_coarse_tiles(Sys S, int b, BinAxis ax, BinAxis ay, unsigned long long *acc,
-                                                     unsigned *ticket, double inv_area, float *out)
+__global__ void __launch_bounds__(NT) k_coarse_tiles(Sys S, int b, BinAxis ax, BinAxis ay, unsigned long long *acc)
 {
-    __shared__ int s_last;
     const long long nb = (long long)ax.nb * ay.nb;
     pdl_wait();
     pdl_next();
@@ -145,16 +145,6 @@ __global__ void __launch_bounds__(NT) k_coarse_tiles(Sys S, int b, BinAxis ax, B
         const int ix = coarse_bin(S.x0tab[tx], rec.x, ax), iy = coarse_bin(S.y0tab[ty], rec.y, ay);
         coarse_add(acc, nb, (long long)iy * ax.nb + ix, __int_as_float(rec.z));
     }
-    if (!ticket) return;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-        if (s_last) *ticket = 0u;
-        __threadfence();
-    }
-    __syncthreads();
-    if (s_last) coarse_fields(acc, nb, inv_area, out, threadIdx.x, NT);
 }
 
 __global__ void k_coarse_finish(unsigned long long *acc, int nbx, int nby, double inv_area, float *out)
@@ -188,12 +178,8 @@ cudaError_t launch_coarse(const Sys &S, int b, int nbx, int nby, unsigned long l
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const int grid = std::max(1, std::min(S.ntiles, 8 * nsm));
     const double inv_area = (double)nbx * nby / (S.lx * S.ly);
-    // up to 2048 bins one block converts them in a few rounds; beyond, a
-    // second launch spreads them over the chip
-    const bool one = nb <= 2048;
-    cudaError_t e = launch_after(k_coarse_tiles<256>, grid, 256, 0, st, S, b, ax, ay, acc,
-                                 one ? reinterpret_cast<unsigned *>(acc + 3 * nb) : nullptr, inv_area, out);
-    if (e != cudaSuccess || one) return e;
+    const cudaError_t e = launch_after(k_coarse_tiles<256>, grid, 256, 0, st, S, b, ax, ay, acc);
+    if (e != cudaSuccess) return e;
     return launch_after(k_coarse_finish, (unsigned)std::min<long long>((nb + 255) / 256, 4096), 256, 0, st, acc, nbx, nby,
                         inv_area, out);
 }

@@ -122,7 +122,7 @@ cudaError_t launch_observe(const Sys &S, int b, unsigned long long *out, cudaStr
 cudaError_t launch_begin_measure(Sys *sys, int nsys, long long max_n, int b, unsigned long long *sums, long long until,
                                  cudaStream_t st);
 // Coarse-grained fields of buffer b into out[3][nby][nbx] (device), using
-// acc[3 * nbx * nby + 1] (device scratch, zero before and after) for the integer sums and a block count.
+// acc[3 * nbx * nby] (device scratch, zero before and after) for the integer sums.
 cudaError_t launch_coarse(const Sys &S, int b, int nbx, int nby, unsigned long long *acc, float *out,
                           cudaStream_t st);
 
