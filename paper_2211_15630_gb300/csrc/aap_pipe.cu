@@ -520,8 +520,10 @@ __device__ __forceinline__ void sort_order(PipeShared &sh, const PipeBufs &B, in
             O.wide = 15 * mx >= 512;
             O.dense = 2 * m > 3 * nce;
             sh.chunk[b] = 0;
-            sh.load = max(sh.load, tile_load(carry, m, nce));
-            sh.staged = max(sh.staged, m);
+            if (FEW) {
+                sh.load = max(sh.load, tile_load(carry, m, nce));
+                sh.staged = max(sh.staged, m);
+            }
             if (carry != M.n_own) atomicOr(M.err, ERR_BOUNDS);
         }
     }
@@ -660,6 +662,10 @@ __device__ __noinline__ void whole_block_tile_call(const Sys *__restrict__ sys, 
 // or done before the pipeline.  With many tiles per SM these gain nothing and
 // what they add to the kernel costs 2 to 5% (N = 2^24, clustered: 870 -> 901 us
 // per step), so such systems claim their tiles in raster order without them.
+// The load report of the tiles is FEW's too: only systems of at most four tiles
+// per SM go by it, and one lane's few instructions between the scan and the
+// placing of every tile cost the raster variant 0.7% (N = 2^24, uniform at noise
+// 0.9: 614.5 -> 608.9 us per step with the spill count bounded when it is read).
 template <int MODEL, bool SP, int NSORT, bool FEW>
 __global__ void __launch_bounds__(kPipeThreads, 1)
 k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_base, Ctl *ctl, int cap, int cap_own,
@@ -774,7 +780,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
         int si = -1, lt = 0, nsp = 0;
         if (nsys == 1) {
             si = 0;
-            nsp = *((volatile int *)&sh.cs.spill_cnt[cur]);
+            nsp = min(*((volatile int *)&sh.cs.spill_cnt[cur]), sh.cs.spill_cap);
         }
         CopyPlan pl;
         const Sys &Sc = sh.cs;
@@ -787,7 +793,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
                 int *dst = reinterpret_cast<int *>(&sh.cs);
                 for (int i = lane; i < words; i += 32) dst[i] = src[i];
                 __syncwarp();
-                nsp = *((volatile int *)&Sc.spill_cnt[cur]);
+                nsp = min(*((volatile int *)&Sc.spill_cnt[cur]), Sc.spill_cap);
             }
             lt = gg - (nsys > 1 ? tile_base[si] : 0);
             copy_plan(Sc, lt, cur, pl);
@@ -802,8 +808,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
             if (g < total && lane == 0) gn = atomicAdd(&ctl->tile_next, 1) + (FEW ? sh.nfront : 0);
             int n_spill = 0, n_own = 0, mode = 0;               // 0: whole-block list, 1: normal, 2: wide
             if (g < total) {
-                const bool scanned = copy_spills(Sc, pl, cur, min(nsp, Sc.spill_cap), spill_e, spill_s, n_spill,
-                                                 n_own);
+                const bool scanned = copy_spills(Sc, pl, cur, nsp, spill_e, spill_s, n_spill, n_own);
                 const int m = pl.m_seg + n_spill;
                 if (scanned && n_spill <= kPipeMaxSpill) {
                     if (m <= cap && n_own <= cap_own) mode = 1;
@@ -1081,8 +1086,8 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
     //     the shared staging area or the block's global scratch ------------
     if (!sh.dense_any) {
         // what the host goes by when it chooses between this kernel and many
-        // steps per launch (a single system)
-        if (nsys == 1 && tid == 0 && sh.staged > 0) {
+        // steps per launch (a single system of few tiles)
+        if (FEW && nsys == 1 && tid == 0 && sh.staged > 0) {
             atomicMax(err0 + 1, sh.load);
             atomicMax(err0 + 2, sh.staged);
         }
@@ -1117,7 +1122,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
         __syncthreads();
         const int g = sh.dense_tile;
         if (g < 0) break;
-        if (tid == 0) sh.load = sh.staged = 0x7fffffff;
+        if (FEW && tid == 0) sh.load = sh.staged = 0x7fffffff;
         if (FEW)
             whole_block_tile_call<MODEL>(sys, nsys, tile_base, jobs[g], cap, cap_own, nceh_max, nce_max, hist_words, mine,
                                          scratch_cap, spill_list_cap, step, total);
@@ -1126,7 +1131,7 @@ k_step_pipe(const Sys *__restrict__ sys, int nsys, const int *__restrict__ tile_
                                     hist_words, mine, scratch_cap, spill_list_cap, step, total);
         if (tid == 0) PT_ADD(11, 1);
     }
-    if (nsys == 1 && tid == 0) {
+    if (FEW && nsys == 1 && tid == 0) {
         atomicMax(err0 + 1, sh.load);
         atomicMax(err0 + 2, sh.staged);
     }
