@@ -278,7 +278,8 @@ int aap_test_pipe_wait(int64_t wait_cycles, int32_t stall);
  * launches of many steps so far, and the steps in them; out[2], out[3]: of the
  * pipelined step's last job list, the leading jobs (whole blocks do them before
  * the pipeline starts) and all jobs (more than there are tiles where dense ones
- * are split), both 0 where tiles are claimed in raster order.  Synchronises. */
+ * are split), both 0 where tiles are claimed in raster order (many tiles per SM,
+ * or none of them dense).  Synchronises. */
 int aap_test_paths(aap_handle *h, int64_t out[4]);
 
 /* Forget the accumulated measurements (moments and histograms). */

@@ -57,6 +57,18 @@ int sm_count()
     return n;
 }
 
+// Words copied to the host with the error word: its four (Sys::err), then the
+// verdict on the order of the pipelined step's tiles; three unused.
+constexpr int kWords = 8;
+
+void drop_graphs(cudaGraphExec_t (&g)[2])
+{
+    for (cudaGraphExec_t &e : g) {
+        if (e) cudaGraphExecDestroy(e);
+        e = nullptr;
+    }
+}
+
 }  // namespace
 
 struct aap_handle {
@@ -88,7 +100,7 @@ struct aap_handle {
     int ncx = 0, ncy = 0;
     double csx = 0, csy = 0;
     // captured step graph
-    cudaGraphExec_t gexec = nullptr;
+    cudaGraphExec_t gexec[2] = {nullptr, nullptr};  // of the pipelined step's variants (LaunchCfg::pipe_jobs)
     int gsteps = 0;
     // per-kernel timing (aap_set_timing)
     bool timing = false;
@@ -98,7 +110,7 @@ struct aap_handle {
     long long launches[3] = {0, 0, 0};
     // capacity management
     double factor = 4.0;            // region slots over the mean occupancy
-    int *pinned_err = nullptr;      // [3][4]: error and load words copied after each aap_step; two batch slots
+    int *pinned_err = nullptr;      // [3][kWords]: words copied after each aap_step (copy_words); two batch slots
     cudaEvent_t err_event = nullptr;
     cudaEvent_t batch_ev[2] = {nullptr, nullptr};   // error words taken every kAdaptSteps steps
     int batch_prev = -1;            // slot of the newest copy not yet read (-1: none)
@@ -108,6 +120,7 @@ struct aap_handle {
     int relayouts = 0;
     bool multi_refused = false;     // the cooperative launch did not fit the context
     bool multi_on = true;           // the tiles are light enough for many steps per launch
+    bool order_stale = true;        // the job list predates the state (set by steps that do not use it)
     long long multi_launches = 0, multi_steps = 0;
     // ensemble membership: steps are launched by the ensemble for all members,
     // whose error words and measurement sums lie side by side in its arrays
@@ -145,8 +158,7 @@ int dev_alloc(aap_handle *h, T **ptr, size_t bytes)
 
 void free_all(aap_handle *h)
 {
-    if (h->gexec) cudaGraphExecDestroy(h->gexec);
-    h->gexec = nullptr;
+    drop_graphs(h->gexec);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     h->cap_stream = nullptr;
     for (cudaEvent_t e : h->events) cudaEventDestroy(e);
@@ -342,6 +354,7 @@ int set_pipe_launch(LaunchCfg &L, bool species, int twmax, int thmax, int total_
     AAP_CK(species ? aapk::configure_pipe_kernel_species(L.model, smem) : aapk::configure_pipe_kernel(L.model, smem));
     L.pipe_species = species ? 1 : 0;
     L.pipe_few = total_tiles <= aapk::kFewPerBlock * L.pipe_grid;
+    L.pipe_jobs = L.pipe_few;
     L.pipe = 1;
     L.threads = 1024;
     return AAP_OK;
@@ -610,10 +623,7 @@ int free_regions(aap_handle *h)
     if (h->member) return AAP_OK;
     rc = dev_free(h, h->d_scratch, h->L.scratch_per_block * h->L.grid_step);
     h->d_scratch = nullptr;
-    if (h->gexec) {
-        cudaGraphExecDestroy(h->gexec);
-        h->gexec = nullptr;
-    }
+    drop_graphs(h->gexec);
     return rc;
 }
 
@@ -696,7 +706,7 @@ int alloc_all(aap_handle *h)
     }
     if ((rc = dev_alloc(h, &h->d_obs, 8 * sizeof(unsigned long long)))) return rc;
     if ((rc = dev_alloc(h, &h->d_seen, sizeof(int)))) return rc;
-    AAP_CK(cudaMallocHost(&h->pinned_err, 12 * sizeof(int)));
+    AAP_CK(cudaMallocHost(&h->pinned_err, 3 * kWords * sizeof(int)));
     AAP_CK(cudaEventCreateWithFlags(&h->err_event, cudaEventDisableTiming));
     for (cudaEvent_t &e : h->batch_ev) AAP_CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     if ((rc = clear_buffers(h))) return rc;
@@ -794,7 +804,7 @@ int capture_steps(const LaunchCfg &L, cudaStream_t &cap, cudaGraphExec_t &exec)
 int read_jobs(const LaunchCfg &L, cudaStream_t st, int64_t *out)
 {
     int meta[2] = {0, 0};
-    if (L.pipe && L.pipe_few)
+    if (L.pipe && L.pipe_jobs)
         AAP_CK(cudaMemcpyAsync(meta, aapk::job_meta(L), sizeof(meta), cudaMemcpyDeviceToHost, st));
     AAP_CK(cudaStreamSynchronize(st));
     out[0] = meta[0];
@@ -841,13 +851,27 @@ void act_on_load(aap_handle *h, const int *words)
     else h->multi_on = words[1] <= lim / 4 * 3 && words[2] <= h->L.multi_cap / 4 * 3;
 }
 
-// Copy the error and load words to page-locked `dst`; the load of single
-// steps starts anew (a launch of many steps starts its own).
+// Which variant of the pipelined step: the job list where the last ordering
+// found a dense tile, and always where the tile loads it reports decide when
+// many steps per launch take over again.
+void act_on_order(LaunchCfg &L, int dense) { L.pipe_jobs = L.pipe_few && (L.multi || dense); }
+bool asks_order(const LaunchCfg &L) { return L.pipe && L.pipe_few && !L.multi; }
+
+// Copy the error and load words and the verdict on the tiles' order to
+// page-locked `dst` ([kWords]); the load of single steps starts anew (a launch of
+// many steps starts its own).
 int copy_words(aap_handle *h, int *dst)
 {
     AAP_CK(cudaMemcpyAsync(dst, h->hs.err, 4 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    if (asks_order(h->L)) AAP_CK(aapk::copy_dense(h->L, dst + 4, h->stream));
     if (h->L.multi && !h->multi_on) AAP_CK(cudaMemsetAsync(h->hs.err + 1, 0, 2 * sizeof(int), h->stream));
     return AAP_OK;
+}
+
+void act_on_words(aap_handle *h, const int *words)
+{
+    act_on_load(h, words);
+    if (asks_order(h->L)) act_on_order(h->L, words[4]);
 }
 
 int run_steps(aap_handle *h, long long nsteps);
@@ -879,7 +903,7 @@ int run_steps_adaptive(aap_handle *h, long long nsteps)
         h->since_copy = 0;
         if (h->L.pipe && !use_multi(h)) AAP_CK(aapk::launch_tile_order(h->L, h->stream));
         const int slot = h->batch_slot;
-        if ((rc = copy_words(h, h->pinned_err + 4 * (1 + slot)))) return rc;
+        if ((rc = copy_words(h, h->pinned_err + kWords * (1 + slot)))) return rc;
         AAP_CK(cudaEventRecord(h->batch_ev[slot], h->stream));
         h->batch_slot ^= 1;
         const int prev = h->batch_prev;
@@ -887,8 +911,8 @@ int run_steps_adaptive(aap_handle *h, long long nsteps)
         if (prev >= 0) {
             AAP_CK(cudaEventSynchronize(h->batch_ev[prev]));
             // a re-layout resets the copies (the newer one predates it)
-            act_on_load(h, h->pinned_err + 4 * (1 + prev));
-            if ((rc = act_on_error(h, h->pinned_err[4 * (1 + prev)], nullptr))) return rc;
+            act_on_words(h, h->pinned_err + kWords * (1 + prev));
+            if ((rc = act_on_error(h, h->pinned_err[kWords * (1 + prev)], nullptr))) return rc;
         }
     }
     return AAP_OK;
@@ -900,6 +924,7 @@ int run_steps(aap_handle *h, long long nsteps)
         cudaError_t e = nsteps > 0 ? aapk::launch_multi(h->L, (int)nsteps, h->stream) : cudaSuccess;
         if (e == cudaSuccess) {
             h->step += nsteps;
+            h->order_stale = true;
             h->multi_launches += nsteps > 0;
             h->multi_steps += nsteps;
             return AAP_OK;
@@ -910,8 +935,12 @@ int run_steps(aap_handle *h, long long nsteps)
         h->multi_on = false;
         h->multi_refused = true;
     }
+    if (h->order_stale && h->L.pipe) {
+        AAP_CK(aapk::launch_tile_order(h->L, h->stream));
+        h->order_stale = false;
+    }
     if (!h->timing) {
-        int rc = launch_steps(h->L, h->stream, nsteps, h->cap_stream, h->gexec);
+        int rc = launch_steps(h->L, h->stream, nsteps, h->cap_stream, h->gexec[h->L.pipe_jobs != 0]);
         if (rc) return rc;
         h->step += nsteps;
         return AAP_OK;
@@ -968,10 +997,7 @@ int reinsert(aap_handle *h, double factor, int mode)
                           old_s.spill_cap == h->hs.spill_cap &&
                           (h->member || old_l.scratch_per_block * old_l.grid_step ==
                                             h->L.scratch_per_block * h->L.grid_step);
-        if (h->gexec) {
-            cudaGraphExecDestroy(h->gexec);
-            h->gexec = nullptr;
-        }
+        drop_graphs(h->gexec);
         if (!same) {
             Sys new_s = h->hs;
             LaunchCfg new_l = h->L;
@@ -990,22 +1016,28 @@ int reinsert(aap_handle *h, double factor, int mode)
         if ((rc = clear_buffers(h))) return rc;
         if ((rc = push_sys(h))) return rc;
         AAP_CK(aapk::launch_insert(h->hs, (int)(h->step & 1), h->d_x, h->d_y, h->d_th, mode, h->stream));
-        int err = 0, words[4] = {0, 0, 0, 0};
+        int err = 0, words[4] = {0, 0, 0, 0}, dense = 0;
+        h->order_stale = true;
         if (h->L.multi) {
             AAP_CK(aapk::launch_tile_load(h->hs, (int)(h->step & 1), h->stream));
             AAP_CK(cudaMemcpyAsync(words, h->hs.err, sizeof(words), cudaMemcpyDeviceToHost, h->stream));
         } else {
             AAP_CK(cudaMemcpyAsync(words, h->hs.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+            if (!h->member && asks_order(h->L)) {
+                AAP_CK(aapk::launch_tile_order(h->L, h->stream));
+                AAP_CK(aapk::copy_dense(h->L, &dense, h->stream));
+                h->order_stale = false;
+            }
         }
         AAP_CK(cudaStreamSynchronize(h->stream));
         err = words[0];
         act_on_load(h, words);
+        if (!h->member && asks_order(h->L)) act_on_order(h->L, dense);
         const bool spilled = err & (aapk::ERR_SPILL | aapk::ERR_LOST);
         // spilled particles are kept exactly: accepted with an explicit
         // capacity, or when doubling the regions would exceed the staged indices
         if (!spilled || (!(err & aapk::ERR_LOST) && (h->p.capacity > 0 || !capacity_fits(h, factor * 2.0)))) {
             h->factor = factor;
-            if (!h->member && h->L.pipe) AAP_CK(aapk::launch_tile_order(h->L, h->stream));
             return AAP_OK;
         }
         if (h->p.capacity > 0) return fail(AAP_EOVERFLOW, "the particles do not fit the explicit capacity");
@@ -1070,7 +1102,7 @@ int poll_capacity(aap_handle *h)
     if (q == cudaErrorNotReady) return AAP_OK;
     if (q != cudaSuccess) return fail(AAP_ECUDA, std::string("error event: ") + cudaGetErrorString(q));
     h->err_pending = false;
-    act_on_load(h, h->pinned_err);
+    act_on_words(h, h->pinned_err);
     return act_on_error(h, *h->pinned_err, nullptr);
 }
 
@@ -1152,9 +1184,9 @@ struct aap_ens {
     LaunchCfg L{};
     long long step = 0;
     cudaStream_t cap = nullptr;
-    cudaGraphExec_t exec = nullptr;
+    cudaGraphExec_t exec[2] = {nullptr, nullptr};
     int policy = 0;
-    int *pinned_err = nullptr;      // [3][count]: after each aap_ens_step; two batch slots
+    int *pinned_err = nullptr;      // [3][count + 1]: after each aap_ens_step (copy_ens_words); two batch slots
     cudaEvent_t err_event = nullptr;
     cudaEvent_t batch_ev[2] = {nullptr, nullptr};   // error words taken every kAdaptSteps steps
     int batch_prev = -1;
@@ -1172,8 +1204,7 @@ void ens_free(aap_ens *e)
         delete h;
     }
     e->m.clear();
-    if (e->exec) cudaGraphExecDestroy(e->exec);
-    e->exec = nullptr;
+    drop_graphs(e->exec);
     if (e->d_sys) cudaFree(e->d_sys);
     if (e->d_tile_base) cudaFree(e->d_tile_base);
     if (e->d_ctl) cudaFree(e->d_ctl);
@@ -1296,9 +1327,11 @@ int ens_combine(aap_ens *e)
             return fail(AAP_EINVAL, "the pipelined step kernel does not fit this ensemble's tiling");
         if (L.pipe) AAP_CK(aapk::launch_tile_order(L, e->stream));
     }
-    if (e->exec) cudaGraphExecDestroy(e->exec);
-    e->exec = nullptr;
-    AAP_CK(cudaStreamSynchronize(e->stream));           // the tile prefix is a local
+    drop_graphs(e->exec);
+    int dense = 0;
+    if (asks_order(L)) AAP_CK(aapk::copy_dense(L, &dense, e->stream));
+    AAP_CK(cudaStreamSynchronize(e->stream));           // the tile prefix and the verdict are locals
+    act_on_order(L, dense);
     return AAP_OK;
 }
 
@@ -1351,6 +1384,7 @@ int ens_build(aap_ens *e, int pol)
 int ens_act(aap_ens *e, const int *words)
 {
     bool regrow = false;
+    if (asks_order(e->L)) act_on_order(e->L, words[e->m.size()]);
     for (size_t r = 0; r < e->m.size(); ++r) {
         aap_handle *h = e->m[r];
         const int err = words[r];
@@ -1376,6 +1410,15 @@ int ens_poll(aap_ens *e)
     if (q != cudaSuccess) return fail(AAP_ECUDA, std::string("error event: ") + cudaGetErrorString(q));
     e->err_pending = false;
     return ens_act(e, e->pinned_err);
+}
+
+// The replicas' error words and the verdict on the tiles' order to page-locked `dst` ([count + 1]).
+int copy_ens_words(aap_ens *e, int *dst)
+{
+    const size_t count = e->m.size();
+    AAP_CK(cudaMemcpyAsync(dst, e->d_err, count * sizeof(int), cudaMemcpyDeviceToHost, e->stream));
+    if (asks_order(e->L)) AAP_CK(aapk::copy_dense(e->L, dst + count, e->stream));
+    return AAP_OK;
 }
 
 }  // namespace
@@ -1866,7 +1909,7 @@ int aap_ens_create(const aap_params *params, int32_t count, void *stream, aap_en
     e->stream = static_cast<cudaStream_t>(stream);
     int rc = ens_build(e, 0);
     if (rc == AAP_OK) {
-        if (cudaMallocHost(&e->pinned_err, (size_t)3 * count * sizeof(int)) != cudaSuccess ||
+        if (cudaMallocHost(&e->pinned_err, (size_t)3 * (count + 1) * sizeof(int)) != cudaSuccess ||
             cudaEventCreateWithFlags(&e->err_event, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&e->batch_ev[0], cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&e->batch_ev[1], cudaEventDisableTiming) != cudaSuccess) {
@@ -1914,7 +1957,7 @@ int aap_ens_step(aap_ens *e, int64_t nsteps)
     long long left = nsteps;
     while (left > 0) {
         const long long k = std::min(left, kAdaptSteps - e->since_copy);
-        if ((rc = launch_steps(e->L, e->stream, k, e->cap, e->exec))) return rc;
+        if ((rc = launch_steps(e->L, e->stream, k, e->cap, e->exec[e->L.pipe_jobs != 0]))) return rc;
         e->step += k;
         for (aap_handle *h : e->m) h->step += k;
         left -= k;
@@ -1923,18 +1966,17 @@ int aap_ens_step(aap_ens *e, int64_t nsteps)
         e->since_copy = 0;
         if (e->L.pipe) AAP_CK(aapk::launch_tile_order(e->L, e->stream));
         const int slot = e->batch_slot;
-        AAP_CK(cudaMemcpyAsync(e->pinned_err + (1 + slot) * count, e->d_err, count * sizeof(int),
-                               cudaMemcpyDeviceToHost, e->stream));
+        if ((rc = copy_ens_words(e, e->pinned_err + (1 + slot) * (count + 1)))) return rc;
         AAP_CK(cudaEventRecord(e->batch_ev[slot], e->stream));
         e->batch_slot ^= 1;
         const int prev = e->batch_prev;
         e->batch_prev = slot;
         if (prev >= 0) {
             AAP_CK(cudaEventSynchronize(e->batch_ev[prev]));
-            if ((rc = ens_act(e, e->pinned_err + (1 + prev) * count))) return rc;
+            if ((rc = ens_act(e, e->pinned_err + (1 + prev) * (count + 1)))) return rc;
         }
     }
-    AAP_CK(cudaMemcpyAsync(e->pinned_err, e->d_err, count * sizeof(int), cudaMemcpyDeviceToHost, e->stream));
+    if ((rc = copy_ens_words(e, e->pinned_err))) return rc;
     AAP_CK(cudaEventRecord(e->err_event, e->stream));
     e->err_pending = true;
     return AAP_OK;
@@ -2045,9 +2087,9 @@ int aap_ens_autotune(aap_ens *e, int32_t trial_steps, int32_t *policy_out, doubl
             continue;
         }
         // warm up (captures the graph), then time
-        if ((rc = launch_steps(e->L, e->stream, 2 + 32, e->cap, e->exec))) break;
+        if ((rc = launch_steps(e->L, e->stream, 2 + 32, e->cap, e->exec[e->L.pipe_jobs != 0]))) break;
         AAP_CK(cudaEventRecord(t0, e->stream));
-        if ((rc = launch_steps(e->L, e->stream, trial_steps, e->cap, e->exec))) break;
+        if ((rc = launch_steps(e->L, e->stream, trial_steps, e->cap, e->exec[e->L.pipe_jobs != 0]))) break;
         AAP_CK(cudaEventRecord(t1, e->stream));
         AAP_CK(cudaEventSynchronize(t1));
         float t = 0.f;

@@ -191,10 +191,14 @@ __global__ void __launch_bounds__(1024) k_finish(Sys *sys, int nsys, const int *
 // few tiles per SM (pipe_few): with many, dense tiles one after another leave
 // the pipeline's roles waiting for each other where light ones between them
 // fill the gaps (N = 2^24, clustered: 0.83 -> 0.86 ms per step).  Run every few
-// dozen steps: loads change slowly.
+// dozen steps: loads change slowly.  A state without a dense tile gets a list in
+// raster order, and the verdict that none leads or is split: the host then
+// launches the variant without the list (kernel k_step_pipe), 1 to 7% faster on
+// uniform states.
 // jobs: [total + kMaxParts] {tile, part | parts << 8}; cost: [total] scratch;
 // meta: the number of leading jobs that whole blocks do first (tiles of more
-// own particles than own_max, two buffers of the pipeline), and of all jobs.
+// own particles than own_max, two buffers of the pipeline), of all jobs, and the
+// verdict.
 constexpr float kSplitAbove = 0.6f, kSplitTo = 2.0f;       // of an SM's average: split tiles above, into parts of 1 / kSplitTo
 __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys, int nsys,
                                                      const int *__restrict__ tile_base, const Ctl *__restrict__ ctl,
@@ -202,7 +206,7 @@ __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys
 {
     constexpr int kClasses = 17;                // 0: whole blocks first
     __shared__ float s_sum[32];
-    __shared__ int s_cnt[kClasses], s_warp[32][kClasses], s_extra, s_kmax;
+    __shared__ int s_cnt[kClasses], s_warp[32][kClasses], s_extra, s_kmax, s_lead;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = (int)(ctl->step & 1), total = tile_base[nsys];
     float sum = 0.f;
@@ -224,7 +228,7 @@ __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys
     if (lane == 0) s_sum[warp] = sum;
     if (tid < kClasses) s_cnt[tid] = 0;
     if (tid == 0) {
-        s_extra = 0;
+        s_extra = s_lead = 0;
         s_kmax = 1;
     }
     __syncthreads();
@@ -244,8 +248,15 @@ __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys
             atomicAdd(&s_extra, K - 1);
             atomicMax(&s_kmax, K);
         }
+        if (cost[g] < 0.f) s_lead = 1;
     }
     __syncthreads();
+    const bool dense = s_extra > 0 || s_lead;
+    if (!dense) {
+        for (int g = tid; g < total; g += 1024) jobs[g] = make_int2(g, 1 << 8);
+        if (tid < 3) meta[tid] = tid == 1 ? total : 0;
+        return;
+    }
     const bool split = s_extra <= kMaxParts;
     const int kmax = split ? s_kmax : 1;
     for (int g = tid; g < total; g += 1024) {
@@ -262,6 +273,7 @@ __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys
             run += n;
         }
         meta[1] = run;
+        meta[2] = 1;
     }
     __syncthreads();
     for (int g0 = 0; g0 < total; g0 += 1024) {
@@ -664,6 +676,11 @@ cudaError_t launch_tile_order(const LaunchCfg &L, cudaStream_t st)
     k_tile_order<<<1, 1024, 0, st>>>(L.sys, L.nsys, L.tile_base, L.ctl, 2 * L.pipe_cap_own, L.pipe_grid, L.jobs,
                                      job_cost(L), job_meta(L));
     return cudaGetLastError();
+}
+
+cudaError_t copy_dense(const LaunchCfg &L, int *dst, cudaStream_t st)
+{
+    return cudaMemcpyAsync(dst, job_meta(L) + 2, sizeof(int), cudaMemcpyDeviceToHost, st);
 }
 
 cudaError_t launch_tile_load(const Sys &S, int b, cudaStream_t st)

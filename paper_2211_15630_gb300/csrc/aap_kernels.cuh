@@ -27,7 +27,9 @@ struct LaunchCfg {
     // pipelined step (pipe_species: systems of several species): shared buffers of pipe_cap
     // staged / pipe_cap_own own particles per tile, one block per SM; tiles
     // that do not fit go to dense_list (device [job_count], zero between steps)
-    int pipe, pipe_species, pipe_few;    // pipe_few: at most kFewPerBlock tiles per block
+    int pipe, pipe_species;
+    int pipe_few;                // at most kFewPerBlock tiles per block: a job list is kept (k_tile_order)
+    int pipe_jobs;               // ... and claimed from; else tiles in raster order
     int pipe_cap, pipe_cap_own, pipe_grid;
     int pipe_nceh;               // half cells (split along x) of the largest extended tile, (2 tw + 4)(th + 2)
     int *dense_list;
@@ -43,7 +45,8 @@ struct LaunchCfg {
 };
 
 // The pipelined step's jobs: up to one per tile and kMaxParts more, the tiles'
-// costs (scratch), and {leading jobs for whole blocks, jobs}.
+// costs (scratch), and {leading jobs for whole blocks, jobs, whether a dense
+// tile leads or is split}.
 constexpr int kMaxParts = 1024;
 constexpr int kFewPerBlock = 12;     // (2^24 at 28 tiles per SM loses 4% with the job order, 10^6 flocking at 6 to 7 gains 23%)
 inline size_t job_count(int tiles) { return (size_t)tiles + kMaxParts; }
@@ -109,6 +112,8 @@ cudaError_t launch_insert(const Sys &S, int b, const double *x, const double *y,
                           int mode, cudaStream_t st);
 // The jobs of the pipelined step, in the order they are claimed, from the tiles' current loads.
 cudaError_t launch_tile_order(const LaunchCfg &L, cudaStream_t st);
+// Its verdict (the third word of job_meta) to host memory.
+cudaError_t copy_dense(const LaunchCfg &L, int *dst, cudaStream_t st);
 // The largest tile load and staged set of buffer b into S.err[1] and [2].
 cudaError_t launch_tile_load(const Sys &S, int b, cudaStream_t st);
 // bad[0]: the lowest index with a position outside [0, lx] x [0, ly]; bad[1]:

@@ -132,13 +132,55 @@ def test_dense_tiles_are_split_and_lead(kw, w, front):
         A.aap_destroy(h)
 
 
-def test_raster_order_beyond_twelve_tiles_per_sm():
-    for side, few in ((330.0, True), (420.0, False)):
-        h = A.aap_create(params(n=120000, lx=side, ly=side, eta=0.3, seed=41, tile_w=8, tile_h=8, threads=1024))
-        try:
-            assert (A.aap_test_paths(h)[3] > 0) == few
-        finally:
-            A.aap_destroy(h)
+@pytest.mark.parametrize("side,dense,listed", [(330.0, True, True), (420.0, True, False), (330.0, False, False)])
+def test_job_list_for_dense_states_of_few_tiles_per_sm(side, dense, listed):
+    """Up to 12 tiles per SM (some 1,700 tiles of 8 x 8 cells) a state with a
+    dense spot claims from the job list, beyond (2,700) and without one in
+    raster order."""
+    n = 120000
+    h = A.aap_create(params(n=n, lx=side, ly=side, eta=0.3, seed=41, tile_w=8, tile_h=8, threads=1024))
+    try:
+        assert A.aap_test_paths(h)[3] == 0                  # the uniform start
+        if dense:
+            c = clustered_state(n // 4, side, side, 5, 0.3 * side, 0.6 * side, 6.0)
+            u = uniform_state(n - n // 4, side, side, 7)
+            x, y, th = (np.concatenate(v) for v in zip(c, u))
+            A.aap_set_state(h, x, y, th.astype(np.float32), 0)
+        assert (A.aap_test_paths(h)[3] > 0) == listed
+    finally:
+        A.aap_destroy(h)
+
+
+def test_the_variant_follows_the_state_within_a_call():
+    """A spot that spreads (straight paths) leaves the job list, and a ring
+    that closes in takes it up: the verdicts are read every 32 steps, through
+    both variants' graphs, and the states equal the whole-block kernel's."""
+    n, m, side = 100000, 8000, 330.0
+    g = np.random.default_rng(5)
+    a = g.permutation(m) * (2.0 * np.pi / m) - np.pi
+    u = uniform_state(n - m, side, side, 7)
+    for first, radius, out in ((True, 2.0, 1.0), (False, 100.0, -1.0)):
+        x, y = (np.concatenate([165.3 + radius * f(a), v]) for f, v in ((np.cos, u[0]), (np.sin, u[1])))
+        th = np.concatenate([a if out > 0 else np.mod(a + 2.0 * np.pi, 2.0 * np.pi) - np.pi, u[2]]).astype(np.float32)
+        states = []
+        for threads in (1024, 512):
+            h = A.aap_create(params(n=n, lx=side, ly=side, model=A.AAP_LANGEVIN, v=1.0, dt=1.0, eta=0.0, gamma=0.0, seed=6,
+                                    tile_w=8, tile_h=8, threads=threads))
+            try:
+                A.aap_set_state(h, x, y, th, 0)
+                if threads == 1024:
+                    assert (A.aap_test_paths(h)[3] > 0) == first
+                for _ in range(3):
+                    A.aap_step(h, 32)
+                A.aap_sync(h)
+                A.aap_step(h, 0)
+                if threads == 1024:
+                    assert (A.aap_test_paths(h)[3] > 0) != first
+                states.append(A.aap_get_state(h, n))
+            finally:
+                A.aap_destroy(h)
+        for p, q in zip(*states):
+            assert np.array_equal(p, q)
 
 
 @pytest.mark.parametrize("batch,h,w,fused", [(1, 16, 16, True), (2, 128, 128, True), (4, 128, 128, True), (5, 128, 128, False)])
@@ -170,7 +212,7 @@ def test_ensemble_of_changing_systems_and_split_tiles(sizes):
             jobs = A.aap_ens_test_paths(e)[3]
             tiles = sum(v.ntx * v.nty for v in lays)
             if threads == 1024:
-                assert jobs == tiles if len(ps) > 100 else jobs > tiles
+                assert jobs == 0 if len(ps) > 100 else jobs > tiles
             for steps in (1, 40):
                 A.aap_ens_step(e, steps)
                 A.aap_ens_measure(e, steps)
