@@ -698,10 +698,15 @@ cudaError_t launch_validate(const double *x, const double *y, const float *th, l
     return cudaGetLastError();
 }
 
-// Blocks of 256 threads that walk the records of n particles (at most eight per
-// SM; a thread per particle in small systems: with 1024 particles a block the state
-// of N = 1000 took 59 us to read instead of 50).
-static unsigned record_blocks(long long n) { return (unsigned)std::max<long long>(1, std::min<long long>((n + 255) / 256, 1216)); }
+// Blocks of 256 threads that gather the records of n particles: 1024 particles a
+// block (at most eight blocks per SM), fewer in small systems, which are a chain of
+// latencies (N = 1000: 59 us to read a state with 1024 a block, 50 with 64; N =
+// 200,000: 79 and 91, the counts of so many warps queue up).
+static unsigned record_blocks(long long n)
+{
+    const long long few = std::min<long long>((n + 63) / 64, 128);
+    return (unsigned)std::max<long long>(1, std::min<long long>(std::max((n + 1023) / 1024, few), 1216));
+}
 
 cudaError_t launch_gather(const Sys &S, int b, double *x, double *y, float *th, int *seen,
                           cudaStream_t st)
@@ -723,7 +728,8 @@ cudaError_t launch_gather(const Sys &S, int b, double *x, double *y, float *th, 
 
 cudaError_t launch_observe(const Sys &S, int b, unsigned long long *out, cudaStream_t st)
 {
-    k_observe<<<record_blocks(S.n), 256, 0, st>>>(S, b, out);
+    const long long blocks = std::max<long long>(1, std::min<long long>((S.n + 255) / 256, 1024));
+    k_observe<<<(unsigned)blocks, 256, 0, st>>>(S, b, out);
     return cudaGetLastError();
 }
 
