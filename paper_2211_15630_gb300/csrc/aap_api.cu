@@ -57,9 +57,7 @@ int sm_count()
     return n;
 }
 
-// Words copied to the host with the error word: its four (Sys::err), then the
-// verdict on the order of the pipelined step's tiles; three unused.
-constexpr int kWords = 8;
+constexpr int kWords = 4;           // of Sys::err, copied to the host together
 
 void drop_graphs(cudaGraphExec_t (&g)[2])
 {
@@ -858,12 +856,11 @@ void act_on_order(LaunchCfg &L, int dense) { L.pipe_jobs = L.pipe_few && (L.mult
 bool asks_order(const LaunchCfg &L) { return L.pipe && L.pipe_few && !L.multi; }
 
 // Copy the error and load words and the verdict on the tiles' order to
-// page-locked `dst` ([kWords]); the load of single steps starts anew (a launch of
-// many steps starts its own).
+// page-locked `dst`; the load of single steps starts anew (a launch of many steps
+// starts its own).
 int copy_words(aap_handle *h, int *dst)
 {
-    AAP_CK(cudaMemcpyAsync(dst, h->hs.err, 4 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    if (asks_order(h->L)) AAP_CK(aapk::copy_dense(h->L, dst + 4, h->stream));
+    AAP_CK(cudaMemcpyAsync(dst, h->hs.err, kWords * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     if (h->L.multi && !h->multi_on) AAP_CK(cudaMemsetAsync(h->hs.err + 1, 0, 2 * sizeof(int), h->stream));
     return AAP_OK;
 }
@@ -871,7 +868,7 @@ int copy_words(aap_handle *h, int *dst)
 void act_on_words(aap_handle *h, const int *words)
 {
     act_on_load(h, words);
-    if (asks_order(h->L)) act_on_order(h->L, words[4]);
+    if (asks_order(h->L)) act_on_order(h->L, words[3]);
 }
 
 int run_steps(aap_handle *h, long long nsteps);
@@ -979,8 +976,9 @@ int ensure_xfer(aap_handle *h)
 // Put the particles back into freshly sized regions.  mode 0: from the flat
 // device arrays d_x, d_y, d_th; mode 1: the Philox initial state.  With an
 // automatic capacity the factor doubles until nothing spills; with an explicit
-// one spilled particles are kept (exactly) in the spill list.
-int reinsert(aap_handle *h, double factor, int mode)
+// one spilled particles are kept (exactly) in the spill list.  The device error
+// word of the inserted state goes to *err_out (read with the host's one wait).
+int reinsert(aap_handle *h, double factor, int mode, int *err_out = nullptr)
 {
     int rc;
     for (int attempt = 0; attempt < 12; ++attempt) {
@@ -1016,28 +1014,25 @@ int reinsert(aap_handle *h, double factor, int mode)
         if ((rc = clear_buffers(h))) return rc;
         if ((rc = push_sys(h))) return rc;
         AAP_CK(aapk::launch_insert(h->hs, (int)(h->step & 1), h->d_x, h->d_y, h->d_th, mode, h->stream));
-        int err = 0, words[4] = {0, 0, 0, 0}, dense = 0;
+        int words[kWords] = {0, 0, 0, 0};
         h->order_stale = true;
         if (h->L.multi) {
             AAP_CK(aapk::launch_tile_load(h->hs, (int)(h->step & 1), h->stream));
-            AAP_CK(cudaMemcpyAsync(words, h->hs.err, sizeof(words), cudaMemcpyDeviceToHost, h->stream));
-        } else {
-            AAP_CK(cudaMemcpyAsync(words, h->hs.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-            if (!h->member && asks_order(h->L)) {
-                AAP_CK(aapk::launch_tile_order(h->L, h->stream));
-                AAP_CK(aapk::copy_dense(h->L, &dense, h->stream));
-                h->order_stale = false;
-            }
+        } else if (!h->member && asks_order(h->L)) {
+            AAP_CK(aapk::launch_tile_order(h->L, h->stream));
+            h->order_stale = false;
         }
+        AAP_CK(cudaMemcpyAsync(words, h->hs.err, (h->member ? 1 : kWords) * sizeof(int), cudaMemcpyDeviceToHost,
+                               h->stream));
         AAP_CK(cudaStreamSynchronize(h->stream));
-        err = words[0];
-        act_on_load(h, words);
-        if (!h->member && asks_order(h->L)) act_on_order(h->L, dense);
+        const int err = words[0];
+        if (!h->member) act_on_words(h, words);
         const bool spilled = err & (aapk::ERR_SPILL | aapk::ERR_LOST);
         // spilled particles are kept exactly: accepted with an explicit
         // capacity, or when doubling the regions would exceed the staged indices
         if (!spilled || (!(err & aapk::ERR_LOST) && (h->p.capacity > 0 || !capacity_fits(h, factor * 2.0)))) {
             h->factor = factor;
+            if (err_out) *err_out = err;
             return AAP_OK;
         }
         if (h->p.capacity > 0) return fail(AAP_EOVERFLOW, "the particles do not fit the explicit capacity");
@@ -1367,9 +1362,9 @@ int ens_build(aap_ens *e, int pol)
         h->d_ctl = e->d_ctl;
         h->ens_err = e->d_err + r;
         h->ens_stats = e->d_stats + 16 * (size_t)r;
-        int rc;
-        if ((rc = build_layout(h)) || (rc = alloc_all(h)) || (rc = reinsert(h, h->factor, 1)) ||
-            (rc = read_errors(h))) {
+        int rc, err = 0;
+        if ((rc = build_layout(h)) || (rc = alloc_all(h)) || (rc = reinsert(h, h->factor, 1, &err)) ||
+            (rc = error_status(h, err))) {
             g_err = "replica " + std::to_string(r) + ": " + g_err;
             return rc;
         }
@@ -1530,7 +1525,8 @@ int aap_create(const aap_params *p, void *stream, aap_handle **out)
         delete h;
         return rc;
     }
-    if ((rc = reinsert(h, h->factor, 1)) || (rc = read_errors(h))) {
+    int err = 0;
+    if ((rc = reinsert(h, h->factor, 1, &err)) || (rc = error_status(h, err))) {
         free_all(h);
         delete h;
         return rc;
@@ -1696,8 +1692,9 @@ int aap_set_state(aap_handle *h, const double *x, const double *y, const float *
     h->broken = false;
     // an automatic capacity keeps the size it has grown to (a restored state
     // of the same system needs it again; the re-insert doubles it if not)
-    if ((rc = reinsert(h, h->p.capacity > 0 ? h->p.capacity : h->factor, 0))) return rc;
-    return read_errors(h);
+    int err = 0;
+    if ((rc = reinsert(h, h->p.capacity > 0 ? h->p.capacity : h->factor, 0, &err))) return rc;
+    return error_status(h, err);
 }
 
 int aap_step_neighbours(aap_handle *h, int32_t *nbr_out, int64_t n)

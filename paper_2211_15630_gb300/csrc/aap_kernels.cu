@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(1024) k_finish(Sys *sys, int nsys, const int *
 // jobs: [total + kMaxParts] {tile, part | parts << 8}; cost: [total] scratch;
 // meta: the number of leading jobs that whole blocks do first (tiles of more
 // own particles than own_max, two buffers of the pipeline), of all jobs, and the
-// verdict.
+// verdict (a single system's goes to its fourth error word too).
 constexpr float kSplitAbove = 0.6f, kSplitTo = 2.0f;       // of an SM's average: split tiles above, into parts of 1 / kSplitTo
 __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys, int nsys,
                                                      const int *__restrict__ tile_base, const Ctl *__restrict__ ctl,
@@ -252,6 +252,7 @@ __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys
     }
     __syncthreads();
     const bool dense = s_extra > 0 || s_lead;
+    if (nsys == 1 && tid == 0) sys[0].err[3] = dense;
     if (!dense) {
         for (int g = tid; g < total; g += 1024) jobs[g] = make_int2(g, 1 << 8);
         if (tid < 3) meta[tid] = tid == 1 ? total : 0;
