@@ -282,6 +282,10 @@ int aap_test_pipe_wait(int64_t wait_cycles, int32_t stall);
  * or none of them dense).  Synchronises. */
 int aap_test_paths(aap_handle *h, int64_t out[4]);
 
+/* For tests: the many-steps kernel stages tiles that outgrow its shared memory
+ * in at most n scratch slices at a time (until the handle's next layout). */
+int aap_test_multi_slices(aap_handle *h, int32_t n);
+
 /* Forget the accumulated measurements (moments and histograms). */
 int aap_clear_results(aap_handle *h);
 

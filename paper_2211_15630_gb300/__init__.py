@@ -29,7 +29,7 @@ EXPORTS = (
     "aap_step_neighbours", "aap_sync", "aap_get_layout", "aap_set_timing", "aap_get_timing",
     "aap_measure", "aap_get_results", "aap_clear_results", "aap_coarse_grain", "aap_get_histograms",
     "aap_save", "aap_load", "aap_test_fail_alloc_after", "aap_test_pipe_wait",
-    "aap_test_paths", "aap_ens_test_paths", "aap_sur_test_paths",
+    "aap_test_paths", "aap_test_multi_slices", "aap_ens_test_paths", "aap_sur_test_paths",
     "aap_ens_create", "aap_ens_step", "aap_ens_measure", "aap_ens_phi_mean", "aap_ens_results",
     "aap_ens_get_state", "aap_ens_get_layout", "aap_ens_autotune", "aap_ens_info", "aap_ens_destroy",
     "aap_ens_coarse_grain",
@@ -127,6 +127,7 @@ def load(path: str = LIB_PATH):
         "aap_test_fail_alloc_after": (C.c_int, [i32]),
         "aap_test_pipe_wait": (C.c_int, [i64, i32]),
         "aap_test_paths": (C.c_int, [vp, vp]),
+        "aap_test_multi_slices": (C.c_int, [vp, i32]),
         "aap_ens_test_paths": (C.c_int, [vp, vp]),
         "aap_sur_test_paths": (C.c_int, [vp, vp]),
         "aap_load": (C.c_int, [C.c_char_p, vp, P(vp)]),
@@ -252,6 +253,11 @@ def aap_test_paths(h) -> np.ndarray:
     out = np.zeros(4, np.int64)
     _check(load().aap_test_paths(h, _p(out)))
     return out
+
+
+def aap_test_multi_slices(h, n: int) -> None:
+    """At most n scratch slices in use at a time in launches of many steps (for tests)."""
+    _check(load().aap_test_multi_slices(h, int(n)))
 
 
 def aap_ens_test_paths(e) -> np.ndarray:

@@ -410,7 +410,10 @@ int set_capacity(aap_handle *h, double factor)
     if (!h->member && p.threads == 0) {
         L.pipe_nceh = (2 * S.twmax + 4) * (S.thmax + 2);
         AAP_CK(aapk::configure_multi(L, p.nspecies > 1, S.ntiles, nsm, scap));
-        if (L.multi) L.grid_step = std::max(L.grid_step, S.ntiles);     // a scratch slice for every block
+        // scratch slices for tiles that outgrow the shared memory: one for every tile
+        // with several species, else the single-step kernels' are shared
+        if (L.multi && p.nspecies > 1) L.grid_step = std::max(L.grid_step, S.ntiles);
+        L.multi_slices = L.grid_step;
     }
     return AAP_OK;
 }
@@ -1480,6 +1483,13 @@ int aap_test_paths(aap_handle *h, int64_t out[4])
     out[0] = h->multi_launches;
     out[1] = h->multi_steps;
     return read_jobs(h->L, h->stream, out + 2);
+}
+
+int aap_test_multi_slices(aap_handle *h, int32_t n)
+{
+    if (!h || n < 1 || h->p.nspecies > 1) return fail(AAP_EINVAL, "NULL handle, n < 1 or several species");
+    h->L.multi_slices = std::min<int>(n, h->L.grid_step);
+    return AAP_OK;
 }
 
 int aap_ens_test_paths(aap_ens *e, int64_t out[4])

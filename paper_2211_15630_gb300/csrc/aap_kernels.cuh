@@ -37,7 +37,9 @@ struct LaunchCfg {
     int job_tiles;
     // many steps per launch (a small system, one block per tile, all resident)
     int multi, multi_species, multi_cap, multi_tiles, multi_threads;
-    int *multi_cnt;              // device: three private counter sets and two barrier words, zero between launches
+    int multi_slices;            // scratch slices its tiles share
+    int *multi_cnt;              // device: three private counter sets, two barrier words and a lock per slice, zero
+                                 // between launches
     // metric-free step (knn > 0): cell count, scan, scatter, k-nearest update
     int knn;
     long long mf_n, mf_ncell;
@@ -91,7 +93,7 @@ cudaError_t launch_step_pipe(const LaunchCfg &L, cudaStream_t st);
 
 // Ints of one private counter set: a line per tile and one for the spill count.
 inline int multi_stride(int ntiles) { return (ntiles + 1) * kCntStride; }
-inline size_t multi_bytes(int ntiles) { return (3 * (size_t)multi_stride(ntiles) + 4) * sizeof(int); }
+inline size_t multi_bytes(int ntiles) { return (3 * (size_t)multi_stride(ntiles) + 4 + ntiles) * sizeof(int); }
 // Decide whether a system of ntiles tiles can run many steps per launch (L.multi): all its blocks resident with at
 // least min_cap staged records each.
 cudaError_t configure_multi(LaunchCfg &L, bool species, int ntiles, int sm_count, int min_cap);

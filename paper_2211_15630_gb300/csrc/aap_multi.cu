@@ -57,7 +57,8 @@ struct MultiShared {
     int cap[kSegs];
     int4 map[kSegs];            // as RawMeta::map of the pipelined step
     int segpre[kSegs + 1];
-    int n_spill, own_spill;     // spill matches, and those of the tile's own regions
+    int n_spill, own_spill, n_list;     // spill matches, those of the tile's own regions, those listed
+    int slice;                  // scratch slice held, -1: none came free
     int warp_tot[kMultiWarps];
     int maxc;
     int ok;
@@ -131,6 +132,53 @@ __device__ __forceinline__ bool multi_barrier(unsigned *bar, unsigned target, in
     return *s_ok != 0;
 }
 
+// A free scratch slice, taken until free_slice (one thread calls; the slices are
+// fewer than the tiles of systems beyond some 300, and only dense tiles want one).  A
+// block that holds one waits for no other block, so the wait ends; it is bounded
+// all the same: -1 and ERR_TIMEOUT when the bound ran out.
+__device__ __forceinline__ int take_slice(int *locks, int slices, int *err)
+{
+    const long long t0 = clock64();
+    const long long bound = c_multi_wait_cycles > 0 ? c_multi_wait_cycles : kMultiWaitCycles;
+    for (int i = blockIdx.x % slices;; i = i + 1 == slices ? 0 : i + 1) {
+        if (atomicCAS(locks + i, 0, 1) == 0) {
+            __threadfence();
+            return i;
+        }
+        if (clock64() - t0 > bound) {
+            atomicOr(err, ERR_TIMEOUT);
+            return -1;
+        }
+    }
+}
+
+__device__ __forceinline__ void free_slice(int *locks, int i)
+{
+    __threadfence();
+    atomicExch(locks + i, 0);
+}
+
+// List the spill matches of the block's tile (entry, segment) in the staging
+// area's sorted records, which nothing uses before all records are mapped.
+template <int NT>
+__device__ __forceinline__ void list_spills(MultiShared &sh, const MultiStage &A, int cur, int nsp, int n)
+{
+    int *const spill_e = (int *)A.P;
+    unsigned char *const spill_s = (unsigned char *)(spill_e + n);
+    for (int e = threadIdx.x; e < nsp; e += NT) {
+        const int key = __ldcg(sh.S.spill_key[cur] + e);
+        for (int s = 0; s < kSegs; ++s)
+            if (sh.cidx[s] == key) {
+                const int j = atomicAdd(&sh.n_list, 1);
+                if (j < n) {
+                    spill_e[j] = e;
+                    spill_s[j] = (unsigned char)s;
+                }
+            }
+    }
+    __syncthreads();
+}
+
 // One step of the block's tile, staged in A.  m records in all, of which
 // m_seg from the segments and the rest from the spill matches; own of them
 // are the tile's own by the counters.  true when the warp updated particles.
@@ -140,10 +188,11 @@ __device__ __forceinline__ bool multi_barrier(unsigned *bar, unsigned target, in
 // halo beyond a reflecting wall is a mirror image, and no other record is.
 template <int NT, int MODEL, bool SP>
 __device__ __forceinline__ bool multi_tile(MultiShared &sh, const MultiStage &A, const MultiTables &tb, int m, int m_seg,
-                                           int own, long long step, const int *spill_e, const unsigned char *spill_s, int *wc,
-                                           int *ws, Acc &acc)
+                                           int own, long long step, int *wc, int *ws, Acc &acc)
 {
     const Sys &S = sh.S;
+    const int *const spill_e = (const int *)A.P;                // list_spills
+    const unsigned char *const spill_s = (const unsigned char *)(spill_e + (m - m_seg));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int cur = (int)(step & 1);
     const int tw = sh.O.tw, th = sh.O.th, W2 = sh.O.W2, H2 = th + 2, nce = W2 * H2;
@@ -282,15 +331,60 @@ __device__ __forceinline__ bool multi_tile(MultiShared &sh, const MultiStage &A,
     return warp * (32 / lpp) < n_own;
 }
 
+// One step of a tile that outgrows the block's shared memory, staged in a
+// slice of the scratch: the block's own, or, of fewer slices than tiles, one
+// taken for the step (several species: there is one for every tile).  false when
+// none came free.
+template <int NT, int MODEL, bool SP>
+__device__ __forceinline__ bool multi_scratch(Acc &acc, bool &any, MultiShared &sh, const MultiTables &tb, int *locks,
+                                              int slices, int tiles, unsigned char *scratch, size_t scratch_per_block,
+                                              int scratch_cap, int m, int m_seg, int own, int nsp, long long step,
+                                              int *wc, int *ws)
+{
+    const bool shared = !SP && slices < tiles;
+    int sl = blockIdx.x;
+    if (shared) {
+        if (threadIdx.x == 0) sh.slice = take_slice(locks, slices, sh.S.err);
+        __syncthreads();
+        sl = sh.slice;
+        if (sl < 0) return false;
+    }
+    const MultiStage Ag = carve_multi(scratch + scratch_per_block * sl, scratch_cap);
+    if (m > m_seg) list_spills<NT>(sh, Ag, (int)(step & 1), nsp, m - m_seg);
+    any = multi_tile<NT, MODEL, SP>(sh, Ag, tb, m, m_seg, own, step, wc, ws, acc);
+    if (shared) {
+        __syncthreads();
+        if (threadIdx.x == 0) free_slice(locks, sl);
+    }
+    return true;
+}
+
+// The same out of line with its own sums, so that its registers do not weigh
+// on the tiles in shared memory (N = 100,000: 13.5 -> 13.2 us per step; coupled species,
+// whose sums need the most registers, lose 6% by the call and inline it).
+template <int NT, int MODEL, bool SP>
+__device__ __noinline__ bool multi_scratch_call(MultiShared &sh, const MultiTables &tb, int *locks, int slices, int tiles,
+                                                unsigned char *scratch, size_t scratch_per_block, int scratch_cap, int m,
+                                                int m_seg, int own, int nsp, long long step, int *wc, int *ws)
+{
+    Acc acc = {0, 0, 0, 0, 0};
+    bool any = false;
+    const bool ok = multi_scratch<NT, MODEL, SP>(acc, any, sh, tb, locks, slices, tiles, scratch, scratch_per_block,
+                                                 scratch_cap, m, m_seg, own, nsp, step, wc, ws);
+    if (any) flush_acc<true>(acc, sh.S.acc, (int)(step & 1));
+    return ok;
+}
+
 // nsteps steps of the system from its current step; block b does tile b, and
 // one more block closes the steps (p(t), the trace, the measured moments: a
 // chain of FP64 operations that would hold up every tile's block).
 // bar[0]: barrier arrivals, bar[1]: blocks that have left (both 0 between
-// launches).  cnt3: three counter sets of `stride` ints, zero between launches.
+// launches), bar[4 + i]: whether scratch slice i is taken.  cnt3: three counter
+// sets of `stride` ints, zero between launches.
 template <int NT, int BPS, int MODEL, bool SP>
 __global__ void __launch_bounds__(NT, BPS)
 k_multi(Sys *__restrict__ sys, Ctl *ctl, int nsteps, int cap, int nceh, int hist_words, int *cnt3, int stride,
-        unsigned *bar, unsigned char *scratch, size_t scratch_per_block, int scratch_cap, int spill_list_cap)
+        unsigned *bar, unsigned char *scratch, size_t scratch_per_block, int scratch_cap, int spill_list_cap, int slices)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ MultiShared sh;
@@ -381,7 +475,7 @@ k_multi(Sys *__restrict__ sys, Ctl *ctl, int nsteps, int cap, int nceh, int hist
             // itself, the same values: no block barrier before the records)
             if (tid == 0) {
                 sh.maxc = 0;
-                sh.n_spill = sh.own_spill = 0;
+                sh.n_spill = sh.own_spill = sh.n_list = 0;
             }
             const int c = lane < kSegs ? min(__ldcg(rc + sh.cidx[lane]), sh.cap[lane])
                                        : (lane == 31 ? min(__ldcg(rs), S.spill_cap) : 0);
@@ -390,11 +484,6 @@ k_multi(Sys *__restrict__ sys, Ctl *ctl, int nsteps, int cap, int nceh, int hist
             const int m_seg = __shfl_sync(0xffffffffu, incl, kSegs - 1), nsp = __shfl_sync(0xffffffffu, c, 31);
             __syncwarp();
             int m = m_seg, own = sh.segpre[kRegions];
-            // the block's scratch slice: staging of a tile that outgrows the
-            // shared memory, then the spill matches
-            unsigned char *const mine = scratch + scratch_per_block * blockIdx.x;
-            int *const spill_e = (int *)(mine + stage_bytes(scratch_cap));
-            unsigned char *const spill_s = (unsigned char *)(spill_e + spill_list_cap);
             if (nsp > 0) {
                 // records parked in the spill list for one of the segments
                 __syncthreads();
@@ -402,12 +491,8 @@ k_multi(Sys *__restrict__ sys, Ctl *ctl, int nsteps, int cap, int nceh, int hist
                     const int key = __ldcg(S.spill_key[cur] + e);
                     for (int s = 0; s < kSegs; ++s)
                         if (sh.cidx[s] == key) {
-                            const int j = atomicAdd(&sh.n_spill, 1);
-                            if (j < spill_list_cap) {
-                                spill_e[j] = e;
-                                spill_s[j] = (unsigned char)s;
-                                if (s < kRegions) atomicAdd(&sh.own_spill, 1);
-                            }
+                            atomicAdd(&sh.n_spill, 1);
+                            if (s < kRegions) atomicAdd(&sh.own_spill, 1);
                         }
                 }
                 __syncthreads();
@@ -417,13 +502,21 @@ k_multi(Sys *__restrict__ sys, Ctl *ctl, int nsteps, int cap, int nceh, int hist
             }
             Acc acc = {0, 0, 0, 0, 0};
             bool any = false;
-            if (m <= cap)
-                any = multi_tile<NT, MODEL, SP>(sh, As, tb, m, m_seg, own, step, spill_e, spill_s, wc, ws, acc);
-            else if (m <= scratch_cap)
-                any = multi_tile<NT, MODEL, SP>(sh, carve_multi(mine, scratch_cap), tb, m, m_seg, own, step, spill_e, spill_s, wc, ws,
-                                                acc);
-            else if (tid == 0)
+            if (m <= cap) {
+                if (m > m_seg) list_spills<NT>(sh, As, cur, nsp, m - m_seg);
+                any = multi_tile<NT, MODEL, SP>(sh, As, tb, m, m_seg, own, step, wc, ws, acc);
+            } else if (m <= scratch_cap) {
+                int *const locks = (int *)(bar + 4);
+                if constexpr (SP && MODEL == 1)
+                    ok = multi_scratch<NT, MODEL, SP>(acc, any, sh, tb, locks, slices, nblk - 1, scratch, scratch_per_block,
+                                                      scratch_cap, m, m_seg, own, nsp, step, wc, ws);
+                else
+                    ok = multi_scratch_call<NT, MODEL, SP>(sh, tb, locks, slices, nblk - 1, scratch, scratch_per_block,
+                                                           scratch_cap, m, m_seg, own, nsp, step, wc, ws);
+                if (!ok) break;
+            } else if (tid == 0) {
                 atomicOr(S.err, ERR_STAGE | ERR_LOST);
+            }
             if (any) flush_acc<true>(acc, S.acc, cur);
         }
         arrived += nblk;
@@ -464,7 +557,8 @@ size_t multi_smem(int cap, int nceh, int hist_words)
            (size_t)round_up(hist_words, 4) * 4 + (size_t)round_up(nceh + 1, 8) * 2;
 }
 
-typedef void (*MultiKernel)(Sys *, Ctl *, int, int, int, int, int *, int, unsigned *, unsigned char *, size_t, int, int);
+typedef void (*MultiKernel)(Sys *, Ctl *, int, int, int, int, int *, int, unsigned *, unsigned char *, size_t, int, int,
+                            int);
 
 template <int NT, int BPS>
 MultiKernel multi_kernel_t(int model, bool species)
@@ -554,8 +648,8 @@ cudaError_t launch_multi(const LaunchCfg &L, int nsteps, cudaStream_t st)
     unsigned *bar = reinterpret_cast<unsigned *>(L.multi_cnt + 3 * (size_t)stride);
     unsigned char *scratch = L.scratch;
     size_t spb = L.scratch_per_block;
-    int scap = L.scratch_cap, slc = L.spill_list_cap;
-    void *args[] = {&sys, &ctl, &nsteps, &cap, &nceh, &hw, &cnt3, &stride, &bar, &scratch, &spb, &scap, &slc};
+    int scap = L.scratch_cap, slc = L.spill_list_cap, slices = L.multi_slices;
+    void *args[] = {&sys, &ctl, &nsteps, &cap, &nceh, &hw, &cnt3, &stride, &bar, &scratch, &spb, &scap, &slc, &slices};
     return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k), dim3(L.multi_tiles + 1), dim3(L.multi_threads), args,
                                        multi_smem(cap, nceh, hw), st);
 }

@@ -50,3 +50,34 @@ def test_ring_that_meets_in_one_half_cell(gamma, steps):
         assert np.abs(out[0][0] - (80.25 + d[0])).max() < 1e-3 and np.abs(out[0][1] - (40.5 + d[1])).max() < 1e-3
     for u, v in zip(*out):
         assert np.array_equal(u, v)
+
+
+@pytest.mark.parametrize("slices", [0, 1, 3])
+def test_dense_tiles_share_the_scratch_slices(slices):
+    """Eight rings that close in inside one call, in a system of more tiles
+    than scratch slices: their tiles outgrow the shared memory at the same time and take
+    turns at the slices (with one slice, all of them), some with spilled
+    records."""
+    m, rings, side, radius = 3000, 8, 512.0, 30
+    n = m * rings
+    g = np.random.default_rng(9)
+    th = np.concatenate([g.permutation(m) * (2.0 * np.pi / m) - np.pi for _ in range(rings)])
+    cx = np.repeat([80.25 + 128.0 * (k % 4) for k in range(rings)], m)
+    cy = np.repeat([40.5 + 256.0 * (k // 4) for k in range(rings)], m)
+    x, y = np.mod(cx - radius * np.cos(th), side), np.mod(cy - radius * np.sin(th), side)
+    out = []
+    for threads in (0, 512):
+        h = A.aap_create(params(n=n, lx=side, ly=side, model=A.AAP_LANGEVIN, v=1.0, dt=1.0, eta=0.0, gamma=1e-3, seed=31,
+                                threads=threads, tile_w=32, tile_h=16, capacity=100.0))
+        try:
+            A.aap_set_state(h, x, y, th.astype(np.float32), 0)
+            if not threads and slices:
+                A.aap_test_multi_slices(h, slices)
+            A.aap_step(h, 36)
+            assert A.aap_test_paths(h)[1] == (0 if threads else 36)
+            assert A.aap_observe(h).flags & A.AAP_FLAG_SPILLED
+            out.append(A.aap_get_state(h, n))
+        finally:
+            A.aap_destroy(h)
+    for u, v in zip(*out):
+        assert np.array_equal(u, v)
