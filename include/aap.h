@@ -279,7 +279,7 @@ int aap_test_pipe_wait(int64_t wait_cycles, int32_t stall);
  * pipelined step's last job list, the leading jobs (whole blocks do them before
  * the pipeline starts) and all jobs (more than there are tiles where dense ones
  * are split), both 0 where tiles are claimed in raster order (many tiles per SM,
- * or none of them dense).  Synchronises. */
+ * or an even state).  Synchronises. */
 int aap_test_paths(aap_handle *h, int64_t out[4]);
 
 /* For tests: the many-steps kernel stages tiles that outgrow its shared memory

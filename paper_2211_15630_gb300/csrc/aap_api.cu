@@ -853,7 +853,7 @@ void act_on_load(aap_handle *h, const int *words)
 }
 
 // Which variant of the pipelined step: the job list where the last ordering
-// found a dense tile, and always where the tile loads it reports decide when
+// found that it matters, and always where the tile loads it reports decide when
 // many steps per launch take over again.
 void act_on_order(LaunchCfg &L, int dense) { L.pipe_jobs = L.pipe_few && (L.multi || dense); }
 bool asks_order(const LaunchCfg &L) { return L.pipe && L.pipe_few && !L.multi; }

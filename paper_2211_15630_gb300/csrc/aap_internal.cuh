@@ -93,7 +93,7 @@ struct Sys {
     int bins_theta, bins_nbr;
     int *nbr_out;               // optional |Omega_i| by particle id
     int *err;                   // [4]: error bits; the largest tile load and staged set since the host looked;
-                                // whether a dense tile leads or is split (k_tile_order)
+                                // whether the order of the tiles matters (k_tile_order)
     // metric-free neighbourhoods (Sec. 2.3): one tile over the whole box whose
     // records all sit in region 0 (flat), re-sorted by cell every step
     int flat;                   // 1: every record goes to region 0 of tile 0

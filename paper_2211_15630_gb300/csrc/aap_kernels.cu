@@ -191,25 +191,32 @@ __global__ void __launch_bounds__(1024) k_finish(Sys *sys, int nsys, const int *
 // few tiles per SM (pipe_few): with many, dense tiles one after another leave
 // the pipeline's roles waiting for each other where light ones between them
 // fill the gaps (N = 2^24, clustered: 0.83 -> 0.86 ms per step).  Run every few
-// dozen steps: loads change slowly.  A state without a dense tile gets a list in
-// raster order, and the verdict that none leads or is split: the host then
-// launches the variant without the list (kernel k_step_pipe), 1 to 7% faster on
-// uniform states.
+// dozen steps: loads change slowly.  An even state gets a list in raster order, and
+// the verdict that the order does not matter: the host then launches the variant
+// without the list (kernel k_step_pipe).  A state is even while no tile leads or is
+// split and the longest is not longer than the mean by more than a share (even_share) of
+// what an SM has to do.  The list then gains about 0.3 of that excess, and its variant costs
+// VM some 5%, Langevin 2%, NVM nothing: with the list against raster order, us per step, VM
+// uniform 76.2 / 73.0 (excess 0.06), 49.1 / 51.1 (0.36), flocks 80.2 / 86.8 (0.31), at low
+// density 54.1 / 51.6 (0.14), 54.1 / 53.6 (0.45); Langevin uniform 62.9 / 61.7 (0.03), 64.9 / 67.4
+// (0.06, walls), 54.0 / 53.5 (0.06), 70.1 / 78.6 (0.17, walls); NVM uniform 92.4 / 92.1
+// (0.02), 47.3 / 47.9 (0.14).
 // jobs: [total + kMaxParts] {tile, part | parts << 8}; cost: [total] scratch;
 // meta: the number of leading jobs that whole blocks do first (tiles of more
 // own particles than own_max, two buffers of the pipeline), of all jobs, and the
 // verdict (a single system's goes to its fourth error word too).
+__device__ __forceinline__ float even_share(int model) { return model == 0 ? 0.15f : model == 1 ? 0.05f : 0.0f; }
 constexpr float kSplitAbove = 0.6f, kSplitTo = 2.0f;       // of an SM's average: split tiles above, into parts of 1 / kSplitTo
 __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys, int nsys,
                                                      const int *__restrict__ tile_base, const Ctl *__restrict__ ctl,
                                                      int own_max, int blocks, int2 *jobs, float *cost, int *meta)
 {
     constexpr int kClasses = 17;                // 0: whole blocks first
-    __shared__ float s_sum[32];
+    __shared__ float s_sum[32], s_max[32];
     __shared__ int s_cnt[kClasses], s_warp[32][kClasses], s_extra, s_kmax, s_lead;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = (int)(ctl->step & 1), total = tile_base[nsys];
-    float sum = 0.f;
+    float sum = 0.f, top = 0.f;
     for (int g = tid; g < total; g += 1024) {
         const int si = nsys > 1 ? sys_of_tile(tile_base, nsys, g) : 0;
         const Sys &S = sys[si];
@@ -222,18 +229,28 @@ __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys
         const float f = (float)own * (24.0f + 7.5f * (float)own / (float)(S.twmax * S.thmax));
         cost[g] = own > own_max ? -f : f;
         sum += f;
+        top = fmaxf(top, f);
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (lane == 0) s_sum[warp] = sum;
+    for (int o = 16; o > 0; o >>= 1) {
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+    }
+    if (lane == 0) {
+        s_sum[warp] = sum;
+        s_max[warp] = top;
+    }
     if (tid < kClasses) s_cnt[tid] = 0;
     if (tid == 0) {
         s_extra = s_lead = 0;
         s_kmax = 1;
     }
     __syncthreads();
-    float all = 0.f;
-    for (int w = 0; w < 32; ++w) all += s_sum[w];
+    float all = 0.f, longest = 0.f;
+    for (int w = 0; w < 32; ++w) {
+        all += s_sum[w];
+        longest = fmaxf(longest, s_max[w]);
+    }
     const float mean = fmaxf(all / (float)max(total, 1), 1e-20f), share = fmaxf(all / (float)blocks, 1e-20f);
     const auto cls = [&](float f, int K) {
         if (f < 0.f) return 0;
@@ -251,7 +268,7 @@ __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys
         if (cost[g] < 0.f) s_lead = 1;
     }
     __syncthreads();
-    const bool dense = s_extra > 0 || s_lead;
+    const bool dense = s_extra > 0 || s_lead || longest - mean > even_share(sys[0].model) * share;
     if (nsys == 1 && tid == 0) sys[0].err[3] = dense;
     if (!dense) {
         for (int g = tid; g < total; g += 1024) jobs[g] = make_int2(g, 1 << 8);

@@ -47,8 +47,8 @@ struct LaunchCfg {
 };
 
 // The pipelined step's jobs: up to one per tile and kMaxParts more, the tiles'
-// costs (scratch), and {leading jobs for whole blocks, jobs, whether a dense
-// tile leads or is split}.
+// costs (scratch), and {leading jobs for whole blocks, jobs, whether the order
+// matters}.
 constexpr int kMaxParts = 1024;
 constexpr int kFewPerBlock = 12;     // (2^24 at 28 tiles per SM loses 4% with the job order, 10^6 flocking at 6 to 7 gains 23%)
 inline size_t job_count(int tiles) { return (size_t)tiles + kMaxParts; }

@@ -658,13 +658,13 @@ __device__ __noinline__ void whole_block_tile_call(const Sys *__restrict__ sys, 
 // The pipelined step of one or more systems with one species each (any
 // model; the systems of one launch share it): one block of kPipeThreads
 // threads per SM.  tile_base[nsys + 1] is the prefix of the systems' tiles.
-// FEW: few tiles per SM and dense ones among them -- jobs in the order of
+// FEW: few tiles per SM and an uneven state -- jobs in the order of
 // k_tile_order, dense tiles split or done before the pipeline.  With many tiles
 // per SM these gain nothing and what they add to the kernel (the call in front
 // and its registers above all) costs 2 to 5% (N = 2^24, clustered: 870 -> 901 us
 // per step; uniform states of few tiles per SM: N = 2^20 at density 2 55.7 -> 58.8,
-// 3 10^6 at density 4 217.0 -> 229.6), so such systems, and states without a
-// dense tile, claim their tiles in raster order without them.
+// 3 10^6 at density 4 217.0 -> 229.6), so such systems, and even states, claim
+// their tiles in raster order without them.
 // The load report of the tiles is FEW's too: only systems of at most four tiles
 // per SM go by it, and one lane's few instructions between the scan and the
 // placing of every tile cost the raster variant 0.7% (N = 2^24, uniform at noise

@@ -155,17 +155,17 @@ def test_the_variant_follows_the_state_within_a_call():
     """A spot that spreads (straight paths) leaves the job list, and a ring
     that closes in takes it up: the verdicts are read every 32 steps, through
     both variants' graphs, and the states equal the whole-block kernel's."""
-    n, m, side = 100000, 8000, 330.0
+    n, m, side = 1000000, 2500, 700.0
     g = np.random.default_rng(5)
     a = g.permutation(m) * (2.0 * np.pi / m) - np.pi
     u = uniform_state(n - m, side, side, 7)
     for first, radius, out in ((True, 2.0, 1.0), (False, 100.0, -1.0)):
-        x, y = (np.concatenate([165.3 + radius * f(a), v]) for f, v in ((np.cos, u[0]), (np.sin, u[1])))
+        x, y = (np.concatenate([335.3 + radius * f(a), v]) for f, v in ((np.cos, u[0]), (np.sin, u[1])))
         th = np.concatenate([a if out > 0 else np.mod(a + 2.0 * np.pi, 2.0 * np.pi) - np.pi, u[2]]).astype(np.float32)
         states = []
         for threads in (1024, 512):
             h = A.aap_create(params(n=n, lx=side, ly=side, model=A.AAP_LANGEVIN, v=1.0, dt=1.0, eta=0.0, gamma=0.0, seed=6,
-                                    tile_w=8, tile_h=8, threads=threads))
+                                    tile_w=32, tile_h=16, threads=threads))
             try:
                 A.aap_set_state(h, x, y, th, 0)
                 if threads == 1024:
