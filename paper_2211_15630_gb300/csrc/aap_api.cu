@@ -1598,8 +1598,8 @@ int aap_observe(aap_handle *h, aap_obs *out)
     const double n = (double)h->p.n;
     const double c1 = (double)(long long)o[0] / aapk::kFix, s1 = (double)(long long)o[1] / aapk::kFix;
     const double c2 = (double)(long long)o[2] / aapk::kFix, s2 = (double)(long long)o[3] / aapk::kFix;
-    out->phi = n > 0 ? std::sqrt(c1 * c1 + s1 * s1) / n : 0.0;
-    out->q = n > 0 ? std::sqrt(c2 * c2 + s2 * s2) / n : 0.0;
+    out->phi = n > 0 ? std::sqrt(std::fma(c1, c1, s1 * s1)) / n : 0.0;
+    out->q = n > 0 ? std::sqrt(std::fma(c2, c2, s2 * s2)) / n : 0.0;
     out->mean_neighbours = h->step > 0 ? last[2] : NAN;
     out->step = h->step;
     out->flags = h->flags;

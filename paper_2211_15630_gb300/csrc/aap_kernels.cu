@@ -577,7 +577,8 @@ __global__ void __launch_bounds__(256) k_observe_all(const Sys *__restrict__ sys
 
 // Start a measurement window at the current state of every system: its p and
 // q (from the observed sums) seed last[0..1], and the steps before `until` are
-// measured.
+// measured.  The squares are added with one rounding, as aap_observe does on the
+// host, so that a window's first sample is the observed value bit for bit.
 __global__ void k_begin_measure(Sys *sys, int nsys, const unsigned long long *sums, long long until)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -587,8 +588,8 @@ __global__ void k_begin_measure(Sys *sys, int nsys, const unsigned long long *su
     const double n = (double)S.n;
     const double c1 = (double)(long long)o[0] / kFix, s1 = (double)(long long)o[1] / kFix;
     const double c2 = (double)(long long)o[2] / kFix, s2 = (double)(long long)o[3] / kFix;
-    S.last[0] = n > 0 ? sqrt(c1 * c1 + s1 * s1) / n : 0.0;
-    S.last[1] = n > 0 ? sqrt(c2 * c2 + s2 * s2) / n : 0.0;
+    S.last[0] = n > 0 ? sqrt(__fma_rn(c1, c1, __dmul_rn(s1, s1))) / n : 0.0;
+    S.last[1] = n > 0 ? sqrt(__fma_rn(c2, c2, __dmul_rn(s2, s2))) / n : 0.0;
     S.meas_until = until;
 }
 

@@ -95,6 +95,22 @@ def test_spilled_records_count_as_load():
         assert np.array_equal(a, b)
 
 
+def test_a_windows_first_sample_is_the_observed_state():
+    """p and q of a window of one step are those aap_observe gives, bit for
+    bit (the window starts on the device, the observation ends on the host)."""
+    h = A.aap_create(params(n=1000, lx=32.0, ly=32.0, eta=0.4, seed=3))
+    try:
+        for _ in range(200):
+            A.aap_step(h, 1)
+            o = A.aap_observe(h)
+            A.aap_clear_results(h)
+            A.aap_measure(h, 1)
+            r = A.aap_get_results(h)
+            assert (r.samples, r.p[0], r.q[0]) == (1, o.phi, o.q)
+    finally:
+        A.aap_destroy(h)
+
+
 def test_withheld_arrival_is_the_many_steps_kernels():
     h = A.aap_create(params(n=3000, lx=40.0, ly=40.0, eta=0.3, seed=23))
     try:
