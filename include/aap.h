@@ -94,13 +94,15 @@ typedef struct aap_params {
     int32_t  threads;    /* threads per block of the step kernel: 0 (automatic),
                             256 or 512 (whole-block tile kernel), 1024 (the
                             pipelined kernel: one block per SM with copy, sort
-                            and update warps; one species per system).
+                            and update warps; asked for by number it takes one
+                            species per system, chosen automatically a single
+                            system may have several).
                             Automatic picks 1024 where it applies, else 512,
                             and runs a system of at most four tiles per SM
-                            many steps per launch while none is dense (the same trajectory bit
-                            for bit; aap_get_layout reports the kernel of
-                            the single steps); an ensemble follows its
-                            first replica's value                           */
+                            many steps per launch while none is dense (the same
+                            trajectory bit for bit; aap_get_layout reports the
+                            kernel of the single steps); an ensemble follows
+                            its first replica's value                       */
     double   capacity;   /* tile-region capacity over the mean occupancy;
                             0 = automatic (4)                                   */
     int32_t  binnum_theta;      /* bins of the orientation histogram over

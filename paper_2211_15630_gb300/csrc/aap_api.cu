@@ -838,9 +838,12 @@ int launch_steps(const LaunchCfg &L, cudaStream_t st, long long nsteps, cudaStre
 // largest tile load and staged set; past a load of 4096 (twice that in blocks
 // of 512 threads, half of it for coupled species, whose sums cost twice as
 // much) or a staged set beyond the block's, single steps take over until both
-// have fallen by a quarter.  Per step, N = 60,000 to 100,000, many steps
-// against one: load 307: 13.3 / 31.0 us, 2138: 22.9 / 35.6, 4307: 19.5 / 30.8,
-// 7232: 38.5 / 36.4; staged beyond the block's: 84 / 38 and 611 / 131.
+// have fallen by a quarter.  Per step, us, many steps against one: in blocks of 256
+// threads (N = 60,000 to 120,000) load 439: 15.8 / 27.6, 2670: 21.6 / 30.5, 4566: 30.4 /
+// 31.4, 6995: 29.6 / 33.0, 19278: 262 / 45, staged beyond the block's 88 / 39 and 135 / 37; in
+// blocks of 512 (N = 24,000 to 40,000) 4523: 19.9 / 30.1, 10480: 27.9 / 31.2, 17066: 36.8 /
+// 31.6; coupled species in blocks of 256 (N = 60,000) 724: 25.1 / 38.2, 2148: 59 / 44, 5313:
+// 115 / 72, in blocks of 512 2466: 26.5 / 42.5, 7801: 137 / 78.
 bool use_multi(const aap_handle *h) { return h->L.multi && !h->timing && h->multi_on && !h->multi_refused; }
 
 // words: {error bits, load, staged set}

@@ -50,7 +50,12 @@ struct LaunchCfg {
 // costs (scratch), and {leading jobs for whole blocks, jobs, whether the order
 // matters}.
 constexpr int kMaxParts = 1024;
-constexpr int kFewPerBlock = 12;     // (2^24 at 28 tiles per SM loses 4% with the job order, 10^6 flocking at 6 to 7 gains 23%)
+// Up to 12 tiles per SM a list is kept.  Of uneven states, with the list / in raster
+// order, us per step: VM at 10 tiles per SM 126 / 144, at 13 153 / 167, at 18 214 / 217, at
+// 23 254 / 257, at 28 289 / 280; NVM at 13 132 / 155, at 18 170 / 192; Langevin at 20 151 /
+// 151.  So the gain ends between 23 and 28; the line is older than the verdict on
+// even states, which lost at any number, and lies on the safe side.
+constexpr int kFewPerBlock = 12;
 inline size_t job_count(int tiles) { return (size_t)tiles + kMaxParts; }
 inline size_t job_bytes(int tiles) { return job_count(tiles) * sizeof(int2) + (size_t)round_up(tiles, 4) * 4 + 16; }
 inline float *job_cost(const LaunchCfg &L) { return reinterpret_cast<float *>(L.jobs + job_count(L.job_tiles)); }

@@ -1,5 +1,6 @@
-// aap_pipe.cu -- the pipelined tile step of one system, or of an ensemble of
-// systems with one species each (sm_103a).
+// aap_pipe.cu -- the pipelined tile step of one system (of one species, or of
+// several: compiled again by aap_pipe_species.cu), or of an ensemble of systems
+// with one species each (sm_103a).
 //
 // One time step (Sec. 2 of Kuersten, "Aligning Active Particles Py
 // Package") with the arithmetic of the whole-block tile routine of
@@ -655,9 +656,10 @@ __device__ __noinline__ void whole_block_tile_call(const Sys *__restrict__ sys, 
                             spill_list_cap, step, total);
 }
 
-// The pipelined step of one or more systems with one species each (any
-// model; the systems of one launch share it): one block of kPipeThreads
-// threads per SM.  tile_base[nsys + 1] is the prefix of the systems' tiles.
+// The pipelined step of one system, or (SP false) of several systems with one
+// species each (any model; the systems of one launch share it): one block of
+// kPipeThreads threads per SM.  tile_base[nsys + 1] is the prefix of the systems'
+// tiles.
 // FEW: few tiles per SM and an uneven state -- jobs in the order of
 // k_tile_order, dense tiles split or done before the pipeline.  With many tiles
 // per SM these gain nothing and what they add to the kernel (the call in front

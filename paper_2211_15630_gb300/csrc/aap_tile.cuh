@@ -992,8 +992,10 @@ __device__ __forceinline__ void update_one(const Sys &S, const OutMeta &O, const
     warp_insert(S, nxt, act, dtile, region, rec, to.cnt(S, nxt), to.spill(S, nxt));
 }
 
-// Warp sum of v, exact for |v| < 2^43: two 32-bit warp reductions of its low
-// 16 and its high bits instead of five rounds of 64-bit shuffles.
+// Warp sum of v, exact for |v| < 2^42 (32 high parts below 2^26 fit a signed
+// word): two 32-bit warp reductions of its low 16 and its high bits instead of
+// five rounds of 64-bit shuffles.  Of a step's sums a lane holds at most 256
+// particles of 2^30 each.
 __device__ __forceinline__ long long warp_redux_ll(long long v)
 {
     const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)v & 0xffffu);
