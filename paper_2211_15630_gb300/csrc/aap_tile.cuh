@@ -1058,10 +1058,12 @@ __device__ __forceinline__ void close_sums(const Sys &S, long long step, int lan
     if (measure) {
         // on-the-fly measurement (Sec. 3.4): state t contributes the powers of
         // p(t), q(t) and of the mean neighbour number measured on it
+        // (the last product, of the fourth moment, is added without rounding it)
         const double b = lane < 4 ? p0 : (lane < 8 ? q0 : nbar);
+        const int m = lane & 3;
         double pk = b;
-        for (int k = 0; k < (lane & 3); ++k) pk *= b;
-        st += lane == 12 ? 1.0 : pk;
+        for (int k = 0; k < min(m, 2); ++k) pk = __dmul_rn(pk, b);
+        st = lane == 12 ? st + 1.0 : (m == 3 ? __fma_rn(pk, b, st) : __dadd_rn(st, pk));
         if (lane < 13) stats[lane] = st;
     }
     __syncwarp();

@@ -111,6 +111,30 @@ def test_a_windows_first_sample_is_the_observed_state():
         A.aap_destroy(h)
 
 
+@pytest.mark.parametrize("threads", [0, 512])
+def test_measured_moments_are_the_sums_of_the_trace(threads):
+    """The moments of p over a window from p(t) itself, bit for bit: powers by
+    repeated rounded products, the fourth's last product added unrounded."""
+    from fractions import Fraction
+
+    kw = dict(n=1000, lx=32.0, ly=32.0, eta=0.4, seed=3, threads=threads)
+    h1, h2 = A.aap_create(params(**kw)), A.aap_create(params(**kw))
+    try:
+        steps = 60
+        A.aap_measure(h1, steps)
+        sums = [0.0] * 4
+        for p in A.aap_phi_trace(h2, steps)[:steps].tolist():
+            sums[0] += p
+            sums[1] += p * p
+            sums[2] += p * p * p
+            sums[3] = float(Fraction(p * p * p) * Fraction(p) + Fraction(sums[3]))
+        r = A.aap_get_results(h1)
+        assert r.samples == steps and list(r.p) == [s / steps for s in sums]
+    finally:
+        A.aap_destroy(h1)
+        A.aap_destroy(h2)
+
+
 def test_withheld_arrival_is_the_many_steps_kernels():
     h = A.aap_create(params(n=3000, lx=40.0, ly=40.0, eta=0.3, seed=23))
     try:
