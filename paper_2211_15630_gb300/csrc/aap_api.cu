@@ -861,7 +861,7 @@ void act_on_load(aap_handle *h, const int *words)
 void act_on_order(LaunchCfg &L, int dense) { L.pipe_jobs = L.pipe_few && (L.multi || dense); }
 bool asks_order(const LaunchCfg &L) { return L.pipe && L.pipe_few && !L.multi; }
 
-// Copy the error and load words and the verdict on the tiles' order to
+// Copy the error and load words and whether the tiles' order matters to
 // page-locked `dst`; the load of single steps starts anew (a launch of many steps
 // starts its own).
 int copy_words(aap_handle *h, int *dst)
@@ -1331,7 +1331,7 @@ int ens_combine(aap_ens *e)
     drop_graphs(e->exec);
     int dense = 0;
     if (asks_order(L)) AAP_CK(aapk::copy_dense(L, &dense, e->stream));
-    AAP_CK(cudaStreamSynchronize(e->stream));           // the tile prefix and the verdict are locals
+    AAP_CK(cudaStreamSynchronize(e->stream));           // the tile prefix and dense are locals
     act_on_order(L, dense);
     return AAP_OK;
 }
@@ -1413,7 +1413,7 @@ int ens_poll(aap_ens *e)
     return ens_act(e, e->pinned_err);
 }
 
-// The replicas' error words and the verdict on the tiles' order to page-locked `dst` ([count + 1]).
+// The replicas' error words and whether the tiles' order matters to page-locked `dst` ([count + 1]).
 int copy_ens_words(aap_ens *e, int *dst)
 {
     const size_t count = e->m.size();

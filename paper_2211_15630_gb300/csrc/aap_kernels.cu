@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(1024) k_finish(Sys *sys, int nsys, const int *
 // the pipeline's roles waiting for each other where light ones between them
 // fill the gaps (N = 2^24, clustered: 0.83 -> 0.86 ms per step).  Run every few
 // dozen steps: loads change slowly.  An even state gets a list in raster order, and
-// the verdict that the order does not matter: the host then launches the variant
+// the finding that the order does not matter: the host then launches the variant
 // without the list (kernel k_step_pipe).  A state is even while no tile leads or is
 // split and the longest is not longer than the mean by more than a share (even_share) of
 // what an SM has to do.  The list then gains about 0.3 of that excess, and its variant costs
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(1024) k_finish(Sys *sys, int nsys, const int *
 // jobs: [total + kMaxParts] {tile, part | parts << 8}; cost: [total] scratch;
 // meta: the number of leading jobs that whole blocks do first (tiles of more
 // own particles than own_max, two buffers of the pipeline), of all jobs, and the
-// verdict (a single system's goes to its fourth error word too).
+// finding (a single system's goes to its fourth error word too).
 __device__ __forceinline__ float even_share(int model) { return model == 0 ? 0.15f : model == 1 ? 0.05f : 0.0f; }
 constexpr float kSplitAbove = 0.6f, kSplitTo = 2.0f;       // of an SM's average: split tiles above, into parts of 1 / kSplitTo
 __global__ void __launch_bounds__(1024) k_tile_order(const Sys *__restrict__ sys, int nsys,

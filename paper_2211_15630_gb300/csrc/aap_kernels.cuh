@@ -53,7 +53,7 @@ constexpr int kMaxParts = 1024;
 // Up to 12 tiles per SM a list is kept.  Of uneven states, with the list / in raster
 // order, us per step: VM at 10 tiles per SM 126 / 144, at 13 153 / 167, at 18 214 / 217, at
 // 23 254 / 257, at 28 289 / 280; NVM at 13 132 / 155, at 18 170 / 192; Langevin at 20 151 /
-// 151.  So the gain ends between 23 and 28; the line is older than the verdict on
+// 151.  So the gain ends between 23 and 28; the line is older than the check for
 // even states, which lost at any number, and lies on the safe side.
 constexpr int kFewPerBlock = 12;
 inline size_t job_count(int tiles) { return (size_t)tiles + kMaxParts; }
@@ -119,7 +119,7 @@ cudaError_t launch_insert(const Sys &S, int b, const double *x, const double *y,
                           int mode, cudaStream_t st);
 // The jobs of the pipelined step, in the order they are claimed, from the tiles' current loads.
 cudaError_t launch_tile_order(const LaunchCfg &L, cudaStream_t st);
-// Its verdict (the third word of job_meta) to host memory.
+// Whether the order matters (the third word of job_meta) to host memory.
 cudaError_t copy_dense(const LaunchCfg &L, int *dst, cudaStream_t st);
 // The largest tile load and staged set of buffer b into S.err[1] and [2].
 cudaError_t launch_tile_load(const Sys &S, int b, cudaStream_t st);

@@ -193,7 +193,7 @@ def test_job_list_for_dense_states_of_few_tiles_per_sm(side, dense, listed):
 
 def test_the_variant_follows_the_state_within_a_call():
     """A spot that spreads (straight paths) leaves the job list, and a ring
-    that closes in takes it up: the verdicts are read every 32 steps, through
+    that closes in takes it up: the state is looked at every 32 steps, through
     both variants' graphs, and the states equal the whole-block kernel's."""
     n, m, side = 1000000, 2500, 700.0
     g = np.random.default_rng(5)
